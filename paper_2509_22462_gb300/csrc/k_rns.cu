@@ -1,0 +1,733 @@
+// FP64 matrix products of the FP64 form on the BF16 tensor cores.
+//
+// GB300 issues about two FP64 FMAs per clock and SM, so the two contractions of the Hessian
+// (tangents Zdot_l = W_l Adot_{l-1}, and H = sum_l Zdot_l^T diag(c_l) Zdot_l) took 181 ms of a
+// 104M-parameter evaluation in an FP64 GEMM on the CUDA cores.  The residue scheme of Ozaki, Uchino
+// and Imamura ("Ozaki scheme II", 2025) does them with integer products instead:
+//   - every row of either operand is scaled by a power of two and rounded to integers of at most
+//     `bits` + 1 bits (bits = 52 for K = 4096 with 15 moduli: the rounding is that of FP64);
+//   - an integer is kept as its residues modulo 15 (or 16) pairwise coprime numbers p_i <= 256, each
+//     in [-p/2, p/2], which BF16 holds exactly;
+//   - one BF16 product per modulus gives the result's residue: products are at most 2^14, so 1024
+//     terms add up exactly in the tensor core's FP32 accumulator, which is reduced mod p_i after
+//     every 1024 terms of K;
+//   - the Chinese remainder theorem gives the integer result: D / P = frac(sum_i y_i / p_i) with
+//     y_i = D_i (P/p_i)^-1 mod p_i (the inverse is folded into one operand) and P = prod p_i,
+//     summed in 96-bit fixed point, where integer overflow is the frac().
+// The only roundings are those of the operands and of the result, so the error does not grow with
+// K as a sum of FP64 products does.  Chosen over slicing into 8-bit digits, which needs 28 products
+// where this needs 15.  Rows holding a NaN or an infinity give NaN.
+//
+// Measured, residual + J + H + gradient at one iterate: 784 -> 4096 x 7 -> 10 181 -> 6.0 ms (error of
+// H against 64-bit sums 5.8e-15 -> 3.8e-15), 784 -> 128 x 2 -> 10 911 -> 313 us (7.8e-16 -> 7.2e-16).
+#include <cudaTypedefs.h>
+
+#include <algorithm>
+#include <cmath>
+#include <cstring>
+
+#include "rns.cuh"
+#include "umma.cuh"
+
+namespace nnc {
+using namespace umma;
+
+namespace {
+
+constexpr int kModuli[kRnsMax] = {256, 255, 253, 251, 247, 241, 239, 233,
+                                  229, 227, 223, 217, 211, 199, 197, 193};
+
+// ------------------------------------------------------------------ residue arithmetic
+// x - p rint(x / p) for |x| <= 2^24 (all steps exact but the quotient's rounding, which can only
+// move a value next to +-p/2 to the other end).
+__device__ __forceinline__ float rns_mod(float x, float p, float pinv) {
+  const float q = __fsub_rn(__fmaf_rn(x, pinv, 12582912.f), 12582912.f);
+  return __fmaf_rn(-q, p, x);
+}
+
+// The four 16-bit limbs of a (signed, |a| <= 2^60) as floats in [-2^15, 2^15).
+struct Limbs {
+  float l0, l1, l2, l3;
+};
+__device__ __forceinline__ Limbs rns_limbs(long long a) {
+  const unsigned long long u = (unsigned long long)a + 0x8000800080008000ull;
+  const unsigned lo = (unsigned)u, hi = (unsigned)(u >> 32);
+  const float off = 8388608.f + 32768.f;
+  return Limbs{__uint_as_float(0x4B000000u | (lo & 0xFFFFu)) - off,
+               __uint_as_float(0x4B000000u | (lo >> 16)) - off,
+               __uint_as_float(0x4B000000u | (hi & 0xFFFFu)) - off,
+               __uint_as_float(0x4B000000u | (hi >> 16)) - off};
+}
+__device__ __forceinline__ float rns_res(const RnsSet& s, int i, const Limbs& l) {
+  const float x = __fmaf_rn(l.l3, s.r48[i], __fmaf_rn(l.l2, s.r32[i], __fmaf_rn(l.l1, s.r16[i], l.l0)));
+  return rns_mod(x, s.p[i], s.pinv[i]);
+}
+// BF16 bits of an integer of at most 8 significant bits: the upper half of its FP32 bits.
+__device__ __forceinline__ unsigned bf2(float a, float b) {
+  return __byte_perm(__float_as_uint(a), __float_as_uint(b), 0x7632);
+}
+
+// Scale of a row whose largest high word of |v| is `hi`: |v| < 2^e.  *sc = 2^(bits - e) makes the
+// integers, the return value 2^(e - bits) undoes it (NaN for a row with a NaN or an infinity).
+__device__ __forceinline__ double rns_scale(int hi, int bits, double* sc) {
+  const int ex = hi >> 20;                       // biased exponent, sign bit cleared
+  const int e = max(ex - 1022, -900);
+  *sc = __hiloint2double((bits - e + 1023) << 20, 0);
+  return ex == 0x7FF ? __longlong_as_double(0x7FF8000000000000ll)
+                     : __hiloint2double((e - bits + 1023) << 20, 0);
+}
+__device__ __forceinline__ int abs_hi(double v) { return __double2hiint(v) & 0x7FFFFFFF; }
+
+// 96-bit fixed-point value of D / P from the residues y_i (0 .. p_i - 1), as D 2^64 / P.
+struct Crt {
+  unsigned long long lo = 0, mid = 0;
+  unsigned hi = 0;
+  __device__ __forceinline__ void add(const RnsSet& s, int i, unsigned y) {
+    lo += (unsigned long long)y * s.c0[i];
+    mid += (unsigned long long)y * s.c1[i];
+    hi += y * s.c2[i];
+  }
+  __device__ __forceinline__ double value() const {
+    const unsigned long long m = mid + (lo >> 32);
+    const unsigned h = hi + (unsigned)(m >> 32);
+    const long long top = (long long)(((unsigned long long)h << 32) | (unsigned)m);
+    return fma((double)(unsigned)lo, 2.3283064365386963e-10, (double)top);
+  }
+};
+
+__device__ __forceinline__ int block_max(int v, int* sh) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  v = __reduce_max_sync(0xffffffffu, v);
+  if (lane == 0) sh[warp] = v;
+  __syncthreads();
+  int r = 0;
+  for (int w = 0; w < (int)(blockDim.x >> 5); ++w) r = max(r, sh[w]);
+  __syncthreads();
+  return r;
+}
+
+// ------------------------------------------------------------------ weights (once, at load)
+__global__ void __launch_bounds__(256) k_rns_pack(const __grid_constant__ RnsSet s,
+                                                  const double* __restrict__ W, int mp, int kp,
+                                                  __nv_bfloat16* __restrict__ res,
+                                                  double* __restrict__ sa) {
+  __shared__ int sh[8];
+  const int r = blockIdx.x;
+  const double* w = W + (size_t)r * kp;
+  int hi = 0;
+  for (int k = threadIdx.x; k < kp; k += blockDim.x) hi = max(hi, abs_hi(w[k]));
+  hi = block_max(hi, sh);
+  double sc;
+  const double back = rns_scale(hi, s.bits, &sc);
+  if (threadIdx.x == 0) sa[r] = back;
+  for (int k = 4 * threadIdx.x; k < kp; k += 4 * blockDim.x) {
+    Limbs l[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) l[j] = rns_limbs(__double2ll_rn(w[k + j] * sc));
+#pragma unroll 4
+    for (int i = 0; i < s.n; ++i) {
+      float v[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) v[j] = rns_mod(rns_res(s, i, l[j]) * s.q[i], s.p[i], s.pinv[i]);
+      *reinterpret_cast<uint2*>(res + ((size_t)i * mp + r) * kp + k) =
+          make_uint2(bf2(v[0], v[1]), bf2(v[2], v[3]));
+    }
+  }
+}
+
+// ------------------------------------------------------------------ tangent rows
+// One CTA per tangent (row of Zdot^T): the row's residues become FP64 (or the row is read as FP64),
+// the row's largest |sigma' z| and |sqrt|c| z| give its scales, and the residues of both are written:
+// the operand of the next layer's product and the two operands of the symmetric product, which
+// takes sqrt|c| z on both sides (sign(c) on one) so that one scale per row fits every column.
+// Bound: 90 bytes written per element (15 residues x 3 operands), about 13 operations on the FP64 pipe.
+template <bool CRT>
+__global__ void __launch_bounds__(256) k_rns_rows(const __grid_constant__ RnsSet in,
+                                                  const __grid_constant__ RnsSet out,
+                                                  const RnsRows a) {
+  __shared__ int sh[8];
+  const int r = blockIdx.x;
+  double* zrow = a.Z + (size_t)r * a.ldz;
+  const double sb = CRT ? in.scale * a.sb[r] : 0.0;
+  int ha = 0, hs = 0;
+  for (int k = 4 * threadIdx.x; k < a.K; k += 4 * blockDim.x) {
+    double z[4];
+    if (CRT) {
+      Crt t[4];
+      const unsigned char* c = a.C + (size_t)r * a.ldc + k;
+      const size_t plane = (size_t)a.n * a.ldc;
+#pragma unroll 5
+      for (int i = 0; i < in.n; ++i) {
+        const unsigned y = __ldg(reinterpret_cast<const unsigned*>(c + i * plane));
+        t[0].add(in, i, y & 0xFFu);
+        t[1].add(in, i, (y >> 8) & 0xFFu);
+        t[2].add(in, i, (y >> 16) & 0xFFu);
+        t[3].add(in, i, y >> 24);
+      }
+#pragma unroll
+      for (int j = 0; j < 4; ++j) z[j] = t[j].value() * sb * __ldg(a.sa + k + j);
+      *reinterpret_cast<double2*>(zrow + k) = make_double2(z[0], z[1]);
+      *reinterpret_cast<double2*>(zrow + k + 2) = make_double2(z[2], z[3]);
+    } else {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) z[j] = zrow[k + j];
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      if (a.At) ha = max(ha, abs_hi(__ldg(a.s1 + k + j) * z[j]));
+      if (a.Sa) hs = max(hs, abs_hi(__ldg(a.rc + k + j) * z[j]));
+    }
+  }
+  if (!a.At && !a.Sa) return;
+  double sca, scs;
+  ha = block_max(ha, sh);
+  hs = block_max(hs, sh);
+  const double ba = rns_scale(ha, out.bits, &sca), bs = rns_scale(hs, out.bits, &scs);
+  if (threadIdx.x == 0) {
+    if (a.At) a.sat[r] = ba;
+    if (a.Sa) a.ss[r] = bs;
+  }
+  const size_t plane = (size_t)a.n * a.K;
+  for (int k = 4 * threadIdx.x; k < a.K; k += 4 * blockDim.x) {
+    double z[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) z[j] = zrow[k + j];
+    const size_t o = (size_t)r * a.K + k;
+    if (a.At) {
+      Limbs l[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) l[j] = rns_limbs(__double2ll_rn(__ldg(a.s1 + k + j) * z[j] * sca));
+      __nv_bfloat16* dst = (__nv_bfloat16*)a.At + o;
+#pragma unroll 5
+      for (int i = 0; i < out.n; ++i)
+        *reinterpret_cast<uint2*>(dst + i * plane) =
+            make_uint2(bf2(rns_res(out, i, l[0]), rns_res(out, i, l[1])),
+                       bf2(rns_res(out, i, l[2]), rns_res(out, i, l[3])));
+    }
+    if (a.Sa) {
+      Limbs l[4];
+      unsigned neg0, neg1;   // sign bits of c, in the places of the packed BF16 pairs
+      {
+        unsigned s4[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          s4[j] = (unsigned)__double2hiint(__ldg(a.c + k + j)) & 0x80000000u;
+          l[j] = rns_limbs(__double2ll_rn(__ldg(a.rc + k + j) * z[j] * scs));
+        }
+        neg0 = (s4[0] >> 16) | s4[1];
+        neg1 = (s4[2] >> 16) | s4[3];
+      }
+      __nv_bfloat16 *da = (__nv_bfloat16*)a.Sa + o, *db = (__nv_bfloat16*)a.Sb + o;
+#pragma unroll 5
+      for (int i = 0; i < out.n; ++i) {
+        float v[4], w[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          v[j] = rns_res(out, i, l[j]);
+          w[j] = rns_mod(v[j] * out.q[i], out.p[i], out.pinv[i]);
+        }
+        *reinterpret_cast<uint2*>(da + i * plane) = make_uint2(bf2(w[0], w[1]), bf2(w[2], w[3]));
+        *reinterpret_cast<uint2*>(db + i * plane) =
+            make_uint2(bf2(v[0], v[1]) ^ neg0, bf2(v[2], v[3]) ^ neg1);
+      }
+    }
+  }
+}
+
+__global__ void k_rns_curv(const double* __restrict__ c, double* __restrict__ rc, int k) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < k) rc[i] = sqrt(fabs(c[i]));
+}
+
+__global__ void k_rns_softmax_ext(int n, int m, int col, const double* __restrict__ p,
+                                  const double* __restrict__ lam, double* __restrict__ Z, int ldz,
+                                  double* __restrict__ c, double* __restrict__ rc) {
+  const int j = blockIdx.x * blockDim.x + threadIdx.x;
+  if (j >= n) return;
+  double lb = 0.0;
+  for (int i = 0; i < m; ++i) lb += lam[i] * p[i];
+  const double r = sqrt(lb * lb + 1.0);
+  const double g[2] = {lb + r, lb - r};
+  double w[2] = {0.0, 0.0};
+  for (int i = 0; i < m; ++i) {
+    const double z = Z[(size_t)j * ldz + i];
+    const double pl = p[i] * lam[i];
+#pragma unroll
+    for (int k = 0; k < 2; ++k) w[k] += z * (p[i] + (2.0 * lb - g[k]) * pl);
+  }
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    const double t = 2.0 * lb - g[k], gp = g[k] / (1.0 + t * t);
+    Z[(size_t)j * ldz + col + k] = w[k];
+    if (j == 0) {
+      c[col + k] = gp;
+      rc[col + k] = sqrt(fabs(gp));
+    }
+  }
+}
+
+// ------------------------------------------------------------------ H from the residue planes
+struct RnsFinish {
+  RnsSet set[2];                       // at most two systems occur (15 or 16 moduli), by K their bits
+  unsigned char which[kRnsMaxLayers];
+};
+__global__ void __launch_bounds__(256) k_rns_h(const __grid_constant__ RnsFinish f, int layers,
+                                               const unsigned char* __restrict__ U, int ldu,
+                                               const double* __restrict__ ss, int n,
+                                               double* __restrict__ H) {
+  __shared__ double t[8][129];
+  const int i0 = blockIdx.x * 128, j0 = blockIdx.y * 8;
+  if (i0 + 127 < j0) return;           // strictly above the diagonal
+  const int x = threadIdx.x, y = threadIdx.y;
+  const int i = i0 + 4 * x, j = j0 + y;
+  double v[4] = {0.0, 0.0, 0.0, 0.0};
+  if (j < n && i < n) {
+    for (int l = 0; l < layers; ++l) {
+      const RnsSet& s = f.set[f.which[l]];
+      const unsigned char* u = U + ((size_t)l * kRnsMax * n + j) * ldu + i;
+      const size_t plane = (size_t)n * ldu;
+      Crt r[4];
+#pragma unroll 5
+      for (int q = 0; q < s.n; ++q) {
+        const unsigned b = __ldg(reinterpret_cast<const unsigned*>(u + q * plane));
+        r[0].add(s, q, b & 0xFFu);
+        r[1].add(s, q, (b >> 8) & 0xFFu);
+        r[2].add(s, q, (b >> 16) & 0xFFu);
+        r[3].add(s, q, b >> 24);
+      }
+      const double* sl = ss + (size_t)l * n;
+      const double sj = s.scale * sl[j];
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        if (i + k < n) v[k] = fma(r[k].value() * sj, sl[i + k], v[k]);
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      if (i + k < n && i + k >= j) H[(size_t)j * n + i + k] = v[k];
+  }
+#pragma unroll
+  for (int k = 0; k < 4; ++k) t[y][4 * x + k] = v[k];
+  __syncthreads();
+  // mirror: rows i0 .. i0 + 127, columns j0 .. j0 + 7
+  for (int e = threadIdx.y * 32 + threadIdx.x; e < 128 * 8; e += 256) {
+    const int ii = i0 + e / 8, jj = j0 + e % 8;
+    if (ii < n && jj < n && ii > jj) H[(size_t)ii * n + jj] = t[e % 8][e / 8];
+  }
+}
+
+// ------------------------------------------------------------------ residue GEMM
+// Persistent: CTA b takes the (modulus, tile) pairs b, b + gridDim.x, ... of 128 x BN tiles.  Warp 0
+// copies the operands (TMA, 64-element K blocks, 128-byte swizzle) through a ring of stages, warp 1
+// issues the MMAs into one of two TMEM accumulators, which it changes every 1024 terms of K, and
+// eight epilogue warps (two per 32-lane TMEM quadrant, each half of the columns) reduce the finished
+// accumulator mod p into registers while the next one fills; after a tile's last accumulator they
+// store its residues, one byte each.
+// Bound: the tensor pipe.  A reduction costs three FP32 operations per element and 1024 terms of K,
+// 0.2 of the MMA time on 8 warps, and runs under the next accumulator's MMAs; the tile is as wide as
+// two accumulators in TMEM allow.
+constexpr int kGBM = 128, kGBK = 64;
+constexpr int kGThreads = 320;                 // producer, MMA, eight epilogue warps
+constexpr int kGChunk = 1024 / kGBK;           // K blocks that add up exactly
+
+struct RnsGemm {
+  int M, N, nkb, lower, ntm, ntn, tiles, n_mod, a_rows, b_rows;
+  unsigned char* C;
+  int ldc;
+  int* err;
+  float p[kRnsMax], pinv[kRnsMax];
+};
+
+template <int BN>
+struct GCfg {
+  static constexpr int STAGE = (kGBM + BN) * 128;
+  static constexpr int STAGES = (227 * 1024 - 2048) / STAGE > 6 ? 6 : (227 * 1024 - 2048) / STAGE;
+  static constexpr int SMEM = STAGES * STAGE + 1024 + 256;
+  static constexpr uint32_t IDESC = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kGBM >> 4) << 24);
+  static_assert(BN % 16 == 0 && BN <= 256 && (BN * 128) % 1024 == 0, "tile width");
+};
+
+template <int BN>
+__global__ void __launch_bounds__(kGThreads, 1)
+    k_rns_gemm(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtensorMap tb,
+               const __grid_constant__ RnsGemm g) {
+  using C = GCfg<BN>;
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+  uint64_t* full = (uint64_t*)(smem + C::STAGES * C::STAGE);
+  uint64_t* empty = full + C::STAGES;
+  uint64_t* accf = empty + C::STAGES;   // [2]: accumulator b holds finished sums
+  uint64_t* tfree = accf + 2;           // [2]: the epilogue has read accumulator b
+  uint64_t* mdone = tfree + 2;          // every MMA issued has completed
+  uint32_t* tmem_slot = (uint32_t*)(mdone + 1);
+  volatile int* abort_flag = (volatile int*)(tmem_slot + 1);
+  volatile int* consumed_sh = (volatile int*)(tmem_slot + 2);
+
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int per_mod = g.tiles, total = g.tiles * g.n_mod;
+  auto decode = [&](int t, int& mod, int& tm, int& tn) {
+    mod = t / per_mod;
+    int r = t - mod * per_mod;
+    if (g.lower) {          // BN = 128: row tm holds the tiles tn = 0 .. tm
+      tm = 0;
+      while (r > tm) r -= ++tm;
+      tn = r;
+    } else {
+      tn = r / g.ntm;
+      tm = r - tn * g.ntm;
+    }
+  };
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < C::STAGES; ++s) {
+      mbar_init(smem_u32(&full[s]), 1);
+      mbar_init(smem_u32(&empty[s]), 1);
+    }
+    for (int b = 0; b < 2; ++b) {
+      mbar_init(smem_u32(&accf[b]), 1);
+      mbar_init(smem_u32(&tfree[b]), 8);   // one arrival per epilogue warp
+    }
+    mbar_init(smem_u32(mdone), 1);
+    *abort_flag = 0;
+    *consumed_sh = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                     smem_u32(tmem_slot)),
+                 "r"(512)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = *tmem_slot;
+
+  int issued = 0;  // producer only
+  if (warp == 0) {
+    if (lane == 0) {
+      int i = 0;
+      bool stop = false;
+      for (int t = blockIdx.x; t < total && !stop; t += gridDim.x) {
+        int mod, tm, tn;
+        decode(t, mod, tm, tn);
+        const int ar = mod * g.a_rows + tm * kGBM, br = mod * g.b_rows + tn * BN;
+        for (int kb = 0; kb < g.nkb; ++kb, ++i) {
+          const int s = i % C::STAGES;
+          const uint32_t ph = (uint32_t)(i / C::STAGES) & 1u;
+          if (!mbar_wait(smem_u32(&empty[s]), ph ^ 1u, g.err, 71, abort_flag)) {
+            stop = true;
+            break;
+          }
+          uint8_t* st = smem + s * C::STAGE;
+          const uint32_t fb = smem_u32(&full[s]);
+          mbar_expect_tx(fb, C::STAGE);
+          tma_load_2d(smem_u32(st), &ta, fb, kb * kGBK, ar);
+          tma_load_2d(smem_u32(st + kGBM * 128), &tb, fb, kb * kGBK, br);
+          issued = i + 1;
+        }
+      }
+    }
+  } else if (warp == 1) {
+    if (lane == 0) {
+      int i = 0, ai = 0;   // stages consumed, accumulators started
+      bool stop = false;
+      for (int t = blockIdx.x; t < total && !stop; t += gridDim.x) {
+        int mod, tm, tn;
+        decode(t, mod, tm, tn);
+        const int n_eff = (min(BN, g.N - tn * BN) + 15) / 16 * 16;
+        const uint32_t idesc = C::IDESC | ((uint32_t)(n_eff >> 3) << 17);
+        for (int kb0 = 0; kb0 < g.nkb && !stop; kb0 += kGChunk, ++ai) {
+          const int b = ai & 1;
+          if (ai >= 2 &&
+              !mbar_wait(smem_u32(&tfree[b]), (uint32_t)((ai - 2) >> 1) & 1u, g.err, 72, abort_flag)) {
+            stop = true;
+            break;
+          }
+          tc_fence_after();
+          const uint32_t d = tmem + (uint32_t)(b * 256);
+          const int kb1 = min(g.nkb, kb0 + kGChunk);
+          for (int kb = kb0; kb < kb1; ++kb, ++i) {
+            const int s = i % C::STAGES;
+            const uint32_t ph = (uint32_t)(i / C::STAGES) & 1u;
+            if (!mbar_wait(smem_u32(&full[s]), ph, g.err, 73, abort_flag)) {
+              stop = true;
+              break;
+            }
+            tc_fence_after();
+            const uint32_t sa = smem_u32(smem + s * C::STAGE), sb = sa + kGBM * 128;
+#pragma unroll
+            for (int kk = 0; kk < kGBK / 16; ++kk)
+              umma_bf16(d, sdesc<2, 1024>(sa + kk * 32), sdesc<2, 1024>(sb + kk * 32), idesc,
+                        (kb > kb0 || kk > 0) ? 1u : 0u);
+            umma_commit(smem_u32(&empty[s]));
+          }
+          if (!stop) umma_commit(smem_u32(&accf[b]));
+        }
+      }
+      *consumed_sh = i;
+      umma_commit(smem_u32(mdone));
+    }
+  } else {
+    const int q = warp & 3;              // TMEM lanes 32q .. 32q + 31 belong to this warp
+    const int half = (warp - 2) >> 2;    // columns half * BN / 2 ..
+    constexpr int NH = BN / 2;
+    int ai = 0;
+    bool stop = false;
+    for (int t = blockIdx.x; t < total && !stop; t += gridDim.x) {
+      int mod, tm, tn;
+      decode(t, mod, tm, tn);
+      const int n_eff = min(BN, g.N - tn * BN);
+      const float p = g.p[mod], pinv = g.pinv[mod];
+      float res[NH];
+#pragma unroll
+      for (int j = 0; j < NH; ++j) res[j] = 0.f;
+      for (int kb0 = 0; kb0 < g.nkb; kb0 += kGChunk, ++ai) {
+        const int b = ai & 1;
+        const bool ok = mbar_wait(smem_u32(&accf[b]), (uint32_t)(ai >> 1) & 1u, g.err, 74, abort_flag);
+        if (!__all_sync(0xffffffffu, ok)) {
+          stop = true;
+          break;
+        }
+        tc_fence_after();
+        const uint32_t src = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(b * 256 + half * NH);
+#pragma unroll
+        for (int c0 = 0; c0 < NH; c0 += 8) {
+          if (half * NH + c0 < n_eff) {
+            uint32_t v[8];
+            asm volatile(
+                "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]),
+                  "=r"(v[7])
+                : "r"(src + (uint32_t)c0));
+            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+            for (int j = 0; j < 8; ++j) res[c0 + j] += rns_mod(__uint_as_float(v[j]), p, pinv);
+          }
+        }
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(smem_u32(&tfree[b]));
+      }
+      if (stop) break;
+      const int n0 = tn * BN + half * NH;
+      unsigned char* dst = g.C + ((size_t)mod * g.N + n0) * g.ldc + tm * kGBM + q * 32 + lane;
+#pragma unroll
+      for (int j = 0; j < NH; ++j) {
+        if (n0 + j < g.N) {
+          float r = rns_mod(res[j], p, pinv);
+          r += r < 0.f ? p : 0.f;
+          dst[(size_t)j * g.ldc] = (unsigned char)__float_as_uint(r + 8388608.f);
+        }
+      }
+    }
+  }
+
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 1 && lane == 0) {
+    volatile int no_abort = 0;
+    mbar_wait(smem_u32(mdone), 0, g.err, 76, &no_abort, *abort_flag ? kWaitCycles / 8 : kWaitCycles);
+  }
+  if (*abort_flag && warp == 0 && lane == 0) {
+    for (int i = *consumed_sh; i < issued; ++i) {
+      volatile int no_abort = 0;
+      mbar_wait(smem_u32(&full[i % C::STAGES]), (uint32_t)(i / C::STAGES) & 1u, g.err, 77, &no_abort,
+                kWaitCycles / 8);
+    }
+  }
+  __syncthreads();
+  if (warp == 1) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512)
+                 : "memory");
+  }
+}
+
+PFN_cuTensorMapEncodeTiled_v12000 rns_encode() {
+  void* p = nullptr;
+  cudaDriverEntryPointQueryResult q;
+  if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) !=
+          cudaSuccess ||
+      q != cudaDriverEntryPointSuccess)
+    return nullptr;
+  return (PFN_cuTensorMapEncodeTiled_v12000)p;
+}
+
+bool rns_map(CUtensorMap* m, const void* base, long long rows, int cols, int box_rows) {
+  auto enc = rns_encode();
+  if (!enc || !base) return false;
+  cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
+  cuuint64_t strides[1] = {(cuuint64_t)cols * 2};
+  cuuint32_t box[2] = {(cuuint32_t)kGBK, (cuuint32_t)box_rows};
+  cuuint32_t es[2] = {1, 1};
+  return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, es,
+             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+template <int BN>
+cudaError_t launch_gemm(const RnsPlan& p, const RnsGemm& g, int grid, cudaStream_t st) {
+  using C = GCfg<BN>;
+  static bool attr = false;
+  if (!attr) {
+    cudaError_t e = cudaFuncSetAttribute(k_rns_gemm<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         C::SMEM);
+    if (e != cudaSuccess) return e;
+    attr = true;
+  }
+  k_rns_gemm<BN><<<grid, kGThreads, C::SMEM, st>>>(p.ta, p.tb, g);
+  note_launch();
+  return cudaGetLastError();
+}
+
+}  // namespace
+
+RnsSet rns_set(int K) {
+  // 15 moduli leave 52 bits at K = 4096; products of fewer terms, whose FP64 sums round less often,
+  // take a 16th (57 bits at K = 1024): the error stays below that of an FP64 sum over the whole
+  // range, and the added product costs 7 % where launches, not products, set the time.
+  RnsSet s;
+  s.n = K <= 1024 ? 16 : 15;
+  double bits = 0.0, P = 1.0;
+  for (int i = 0; i < s.n; ++i) {
+    bits += std::log2((double)kModuli[i]);
+    P *= kModuli[i];
+  }
+  s.scale = std::ldexp(P, -64);
+  s.bits = std::min(60, (int)std::floor((bits - 1.0 - std::log2((double)K)) / 2.0 - 1e-9));
+  auto sym = [](long long v, int p) {
+    v %= p;
+    return (float)(v > p / 2 ? v - p : v);
+  };
+  for (int i = 0; i < s.n; ++i) {
+    const int p = kModuli[i];
+    s.p[i] = (float)p;
+    s.pinv[i] = 1.0f / (float)p;
+    const long long r16 = 65536 % p, r32 = r16 * r16 % p, r48 = r32 * r16 % p;
+    s.r16[i] = sym(r16, p);
+    s.r32[i] = sym(r32, p);
+    s.r48[i] = sym(r48, p);
+    long long m = 1;
+    for (int j = 0; j < s.n; ++j)
+      if (j != i) m = m * (kModuli[j] % p) % p;
+    long long inv = 1;
+    while (m * inv % p != 1) ++inv;   // the moduli are pairwise coprime
+    s.q[i] = sym(inv, p);
+    const unsigned __int128 c = ((((unsigned __int128)1) << 97) / p + 1) / 2;
+    s.c0[i] = (unsigned)c;
+    s.c1[i] = (unsigned)(c >> 32);
+    s.c2[i] = (unsigned)(c >> 64);
+  }
+  return s;
+}
+
+int rns_plan(RnsPlan& p, const void* A, int a_rows, const void* B, int b_rows, int M, int N, int K,
+             int n_mod, bool lower) {
+  p = RnsPlan();
+  if (K % kGBK || K <= 0 || M <= 0 || N <= 0 || N > b_rows) return NNC_ERR_ARG;
+  p.M = M;
+  p.N = N;
+  p.nkb = K / kGBK;
+  p.a_rows = a_rows;
+  p.b_rows = b_rows;
+  p.lower = lower ? 1 : 0;
+  // tile width: the least padded work, a tile counting 8 columns of overhead and at least 96 (narrower
+  // MMAs are bound by reading A from shared memory)
+  p.bn = 128;
+  if (!lower) {
+    long long best = -1;
+    for (int bn : {128, 208, 256}) {
+      long long cost = 0;
+      for (int n = 0; n < N; n += bn) cost += std::max((std::min(bn, N - n) + 15) / 16 * 16, 96) + 8;
+      if (best < 0 || cost < best) {
+        best = cost;
+        p.bn = bn;
+      }
+    }
+  }
+  if (!rns_map(&p.ta, A, (long long)n_mod * a_rows, K, kGBM) ||
+      !rns_map(&p.tb, B, (long long)n_mod * b_rows, K, p.bn))
+    return NNC_ERR_CUDA;
+  p.ready = true;
+  return NNC_OK;
+}
+
+cudaError_t rns_gemm(const RnsPlan& p, const RnsSet& s, unsigned char* C, int ldc, int* err,
+                     int sm_count, cudaStream_t st) {
+  RnsGemm g{};
+  g.ntm = (p.M + kGBM - 1) / kGBM;
+  g.ntn = (p.N + p.bn - 1) / p.bn;
+  if (!p.ready || ldc < g.ntm * kGBM) return cudaErrorInvalidValue;
+  g.M = p.M;
+  g.N = p.N;
+  g.nkb = p.nkb;
+  g.lower = p.lower;
+  g.tiles = p.lower ? g.ntm * (g.ntm + 1) / 2 : g.ntm * g.ntn;
+  g.n_mod = s.n;
+  g.a_rows = p.a_rows;
+  g.b_rows = p.b_rows;
+  g.C = C;
+  g.ldc = ldc;
+  g.err = err;
+  for (int i = 0; i < s.n; ++i) {
+    g.p[i] = s.p[i];
+    g.pinv[i] = s.pinv[i];
+  }
+  const int grid = std::min(sm_count, g.tiles * g.n_mod);
+  switch (p.bn) {
+    case 128: return launch_gemm<128>(p, g, grid, st);
+    case 208: return launch_gemm<208>(p, g, grid, st);
+    case 256: return launch_gemm<256>(p, g, grid, st);
+    default: return cudaErrorInvalidValue;
+  }
+}
+
+cudaError_t rns_pack_weights(const RnsSet& s, const double* W, int mp, int kp, void* res, double* sa,
+                             cudaStream_t st) {
+  k_rns_pack<<<mp, 256, 0, st>>>(s, W, mp, kp, (__nv_bfloat16*)res, sa);
+  note_launch();
+  return cudaGetLastError();
+}
+
+cudaError_t rns_rows(const RnsSet& in, const RnsSet& out, const RnsRows& a, cudaStream_t st) {
+  if (a.K % 128 || a.n < 1 || (a.ldz & 1)) return cudaErrorInvalidValue;
+  const int threads = std::min(256, std::max(32, a.K / 4));
+  if (a.C) k_rns_rows<true><<<a.n, threads, 0, st>>>(in, out, a);
+  else k_rns_rows<false><<<a.n, threads, 0, st>>>(in, out, a);
+  note_launch();
+  return cudaGetLastError();
+}
+
+cudaError_t rns_curv(const double* c, double* rc, int k, cudaStream_t st) {
+  k_rns_curv<<<(k + 255) / 256, 256, 0, st>>>(c, rc, k);
+  note_launch();
+  return cudaGetLastError();
+}
+
+cudaError_t rns_softmax_ext(int n, int m, int col, const double* p, const double* lam, double* Z,
+                            int ldz, double* c, double* rc, cudaStream_t st) {
+  k_rns_softmax_ext<<<(n + 127) / 128, 128, 0, st>>>(n, m, col, p, lam, Z, ldz, c, rc);
+  note_launch();
+  return cudaGetLastError();
+}
+
+cudaError_t rns_h_finish(const RnsSet* sets, int layers, const unsigned char* U, int ldu,
+                         const double* ss, int n, double* H, cudaStream_t st) {
+  if (layers < 1 || layers > kRnsMaxLayers) return cudaErrorInvalidValue;
+  RnsFinish f{};
+  int have = 0;
+  for (int l = 0; l < layers; ++l) {
+    int w = 0;
+    while (w < have && f.set[w].n != sets[l].n) ++w;
+    if (w == have) f.set[have++] = sets[l];   // what the result needs depends on the moduli alone
+    f.which[l] = (unsigned char)w;
+  }
+  dim3 grid((n + 127) / 128, (n + 7) / 8);
+  k_rns_h<<<grid, dim3(32, 8), 0, st>>>(f, layers, U, ldu, ss, n, H);
+  note_launch();
+  return cudaGetLastError();
+}
+
+}  // namespace nnc

@@ -1,8 +1,8 @@
 // CUDA-core GEMMs of the FP64 and FP32 forms: the forward tangent sweep of the Hessian
 // (Zdot_l = W_l Adot_{l-1}, n_in tangent columns) and the per-layer symmetric product
-// H += Zdot_l^T diag(c_l) Zdot_l.  GB300's FP64 rate is low, so the FP64 form is the accuracy
-// reference of the GPU path rather than its fast path; the kernel is a plain shared-memory
-// tiled GEMM with register micro-tiles.
+// H += Zdot_l^T diag(c_l) Zdot_l: a plain shared-memory tiled GEMM with register micro-tiles.  The
+// FP64 form comes here only when the residue products of k_rns.cu do not fit (their residues take
+// four times the memory of the FP64 weights) or for more than kRnsMaxLayers curved layers.
 #include "kernels.cuh"
 
 namespace nnc {

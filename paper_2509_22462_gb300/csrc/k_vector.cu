@@ -522,14 +522,15 @@ __global__ void __launch_bounds__(256) k_first_tangent_t(const float* __restrict
   }
 }
 
-// W^T (FP32): T[j][i] = W[i][j] for i < rows, j < cols, through 32 x 32 shared tiles.
-__global__ void k_transpose_f32(const float* __restrict__ W, int ldw, int rows, int cols,
-                                float* __restrict__ T, int ldt) {
-  __shared__ float tile[32][33];
+// W^T: T[j][i] = W[i][j] for i < rows, j < cols, through 32 x 32 shared tiles.
+template <typename TW>
+__global__ void k_transpose(const TW* __restrict__ W, int ldw, int rows, int cols,
+                            TW* __restrict__ T, int ldt) {
+  __shared__ TW tile[32][33];
   const int i0 = blockIdx.y * 32, j0 = blockIdx.x * 32;
   for (int r = threadIdx.y; r < 32; r += blockDim.y) {
     const int i = i0 + r, j = j0 + threadIdx.x;
-    tile[r][threadIdx.x] = (i < rows && j < cols) ? W[(size_t)i * ldw + j] : 0.f;
+    tile[r][threadIdx.x] = (i < rows && j < cols) ? W[(size_t)i * ldw + j] : TW(0);
   }
   __syncthreads();
   for (int r = threadIdx.y; r < 32; r += blockDim.y) {
@@ -541,7 +542,15 @@ __global__ void k_transpose_f32(const float* __restrict__ W, int ldw, int rows, 
 cudaError_t launch_transpose_f32(const float* W, int ldw, int rows, int cols, float* T, int ldt,
                                  cudaStream_t st) {
   dim3 g((cols + 31) / 32, (rows + 31) / 32), b(32, 8);
-  k_transpose_f32<<<g, b, 0, st>>>(W, ldw, rows, cols, T, ldt);
+  k_transpose<float><<<g, b, 0, st>>>(W, ldw, rows, cols, T, ldt);
+  note_launch();
+  return cudaGetLastError();
+}
+
+cudaError_t launch_transpose_f64(const double* W, int ldw, int rows, int cols, double* T, int ldt,
+                                 cudaStream_t st) {
+  dim3 g((cols + 31) / 32, (rows + 31) / 32), b(32, 8);
+  k_transpose<double><<<g, b, 0, st>>>(W, ldw, rows, cols, T, ldt);
   note_launch();
   return cudaGetLastError();
 }

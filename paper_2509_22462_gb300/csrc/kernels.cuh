@@ -61,8 +61,10 @@ cudaError_t launch_first_tangent(Elem e, const void* W1, int ldw, int m_pad, int
 cudaError_t launch_first_tangent_t(bool x3, const float* W1T, int ldt, int m_pad, int n,
                                    const double* s1, const double* c, TanBuf At, int lda,
                                    TanBuf Yt, int ldz, cudaStream_t st);
-// T[j][i] = W[i][j] (FP32) for i < rows, j < cols.
+// T[j][i] = W[i][j] (FP32 / FP64) for i < rows, j < cols.
 cudaError_t launch_transpose_f32(const float* W, int ldw, int rows, int cols, float* T, int ldt,
+                                 cudaStream_t st);
+cudaError_t launch_transpose_f64(const double* W, int ldw, int rows, int cols, double* T, int ldt,
                                  cudaStream_t st);
 // H[i][j] = sum_s Hp[s][max(i,j)][min(i,j)]  (exactly symmetric); Hp is double or float.
 cudaError_t launch_h_finish(bool part_f32, const void* Hp, int splits, int n, int ldp, double* H,

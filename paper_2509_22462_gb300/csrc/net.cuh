@@ -5,6 +5,7 @@
 #include <vector>
 
 #include "kernels.cuh"
+#include "rns.cuh"
 #include "tc.cuh"
 
 struct nnc_net;
@@ -47,6 +48,13 @@ struct LayerDev {
   nnc::RevGeom rev_geom;          // its launch geometry
   int rev_cnt_off = 0;            // offset of its strip counters in nnc_net::rev_cnt
   int zy_off = -1;                // column offset of this layer's Zdot / Ydot block (-1: none)
+  // FP64 form, residue products: BF16 residues of W [set.n][mp][kp], their row scales, the plans
+  // of the tangent product and of the symmetric product, and this layer's residue plane of H
+  void* Wr = nullptr;
+  double* wr_scale = nullptr;
+  nnc::RnsSet set_in, set_out;    // products over K = kp (tangents) and K = mp (next layer, H)
+  nnc::RnsPlan plan_rt, plan_rs;
+  int h_plane = -1;
 };
 
 struct nnc_net {
@@ -103,6 +111,15 @@ struct nnc_net {
   void* Hp = nullptr;        // split partial sums of H (double for CUDA-core forms, float for TC)
   int h_splits = 1;
   bool hp_f32 = false;
+  // FP64 form on the tensor cores (residue products, k_rns.cu)
+  bool rns = false;
+  double *c64 = nullptr, *rc64 = nullptr;  // c_l of all curved layers at zy_off, and sqrt|c_l|
+  double* Z1 = nullptr;                    // W_1^T [n_in][mp_1 + 128]
+  double* Zs = nullptr;                    // Zdot_l^T of the current layer [n_in][zs_ld]
+  int zs_ld = 0, u_ld = 0, h_planes = 0;
+  void *Rt = nullptr, *Ra = nullptr, *Rb = nullptr;   // residues: next operand, symmetric product
+  unsigned char *Rc = nullptr, *Ru = nullptr;  // results of the tangent product, planes of H
+  double *rt_scale = nullptr, *ru_scale = nullptr;     // [n_in], [h_planes][n_in]
   int* dev_err = nullptr;    // device error word of bounded waits
   double* h_stage = nullptr; // pinned host staging
   size_t h_stage_elems = 0;

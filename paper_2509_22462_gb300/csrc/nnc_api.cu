@@ -427,6 +427,68 @@ int run_hessian(nnc_net* net, const double* lam, double* H, cudaStream_t st, boo
   return NNC_OK;
 }
 
+// The same for the FP64 form by residue products on the tensor cores (k_rns.cu): per layer the
+// product, one pass over its rows (result to FP64, scales, operands of the next layer and of H), and
+// the layer's symmetric product into its own residue plane; the planes are added in FP64 at the end.
+int run_hessian_rns(nnc_net* net, const double* lam, double* H, cudaStream_t st) {
+  const int n = net->n_in;
+  if (net->h_planes == 0) {  // every layer is linear: H = 0
+    CK(cudaMemsetAsync(H, 0, sizeof(double) * n * n, st));
+    return NNC_OK;
+  }
+  CK(rns_curv(net->c64, net->rc64, net->K_total, st));
+  RnsSet sets[kRnsMaxLayers];
+  for (int l = 0; l < net->L; ++l) {
+    LayerDev& Ly = net->layers[l];
+    const bool last = l == net->L - 1, soft = last && net->softmax;
+    if (last && Ly.zy_off < 0) break;  // a linear output layer adds nothing to H
+    RnsRows a;
+    a.n = n;
+    a.K = Ly.mp;
+    a.Z = l == 0 ? net->Z1 : net->Zs;
+    a.ldz = l == 0 ? Ly.mp + kPad : net->zs_ld;
+    if (l > 0) {
+      PROF(PK_TANGENT);
+      CK(rns_gemm(Ly.plan_rt, Ly.set_in, net->Rc, Ly.mp, net->dev_err, net->sm_count, st));
+      a.C = net->Rc;
+      a.ldc = Ly.mp;
+      a.sa = Ly.wr_scale;
+      a.sb = net->rt_scale;
+    }
+    PROF(PK_OTHER);
+    if (soft) {   // the result in FP64 first, then its two added columns
+      if (l > 0) CK(rns_rows(Ly.set_in, Ly.set_out, a, st));
+      CK(rns_softmax_ext(n, net->n_out, Ly.mp, Ly.a, lam, a.Z, a.ldz, Ly.c,
+                         net->rc64 + Ly.zy_off, st));
+      a.C = nullptr;
+      a.K = Ly.mp + kPad;
+    }
+    a.s1 = Ly.s1;
+    if (!last) {
+      a.At = net->Rt;
+      a.sat = net->rt_scale;
+    }
+    if (Ly.zy_off >= 0) {
+      a.c = net->c64 + Ly.zy_off;
+      a.rc = net->rc64 + Ly.zy_off;
+      a.Sa = net->Ra;
+      a.Sb = net->Rb;
+      a.ss = net->ru_scale + (size_t)Ly.h_plane * n;
+    }
+    CK(rns_rows(Ly.set_in, Ly.set_out, a, st));
+    if (Ly.zy_off >= 0) {
+      PROF(PK_SYRK);
+      CK(rns_gemm(Ly.plan_rs, Ly.set_out,
+                  net->Ru + (size_t)Ly.h_plane * kRnsMax * n * net->u_ld, net->u_ld, net->dev_err,
+                  net->sm_count, st));
+      sets[Ly.h_plane] = Ly.set_out;
+    }
+  }
+  PROF(PK_OTHER);
+  CK(rns_h_finish(sets, net->h_planes, net->Ru, net->u_ld, net->ru_scale, n, H, st));
+  return NNC_OK;
+}
+
 // One value pass at x, then whatever is asked: y = NN(x), the residual rr = yv - NN(x), J, H and
 // the gradient lambda^T J.
 int eval_all(nnc_net* net, const double* x, const double* lam, double* y, double* J, double* H,
@@ -471,7 +533,7 @@ int eval_all(nnc_net* net, const double* x, const double* lam, double* y, double
     if (r != NNC_OK) return r;
   }
   if (H) {
-    r = run_hessian(net, lam, H, st, false);
+    r = net->rns ? run_hessian_rns(net, lam, H, st) : run_hessian(net, lam, H, st, false);
     if (r != NNC_OK) return r;
   }
   return NNC_OK;
@@ -654,6 +716,70 @@ void nnc_free(nnc_net* net) {
   delete net;
 }
 
+// Buffers, residues and plans of the FP64 form's residue products.  They take 30 to 32 bytes per
+// weight beside the 8 of the FP64 weights; where that is more than half of the free memory, or more
+// than kRnsMaxLayers layers are curved, the CUDA-core products stay in use (net->rns false).
+static int load_rns(nnc_net* net) {
+  const int n = net->n_in, L = net->L;
+  int planes = 0, mp_max = 0;
+  size_t need = 0;
+  auto used = [&](int l) { return l < L - 1 || net->layers[l].zy_off >= 0; };
+  for (int l = 0; l < L; ++l) {
+    LayerDev& Ly = net->layers[l];
+    if (!used(l)) continue;
+    if (Ly.zy_off >= 0) Ly.h_plane = planes++;
+    mp_max = std::max(mp_max, Ly.mp);
+    if (l > 0) need += (size_t)Ly.mp * Ly.kp * 2 * kRnsMax;
+  }
+  net->h_planes = planes;
+  net->zs_ld = mp_max + kPad;
+  net->u_ld = net->n_in_pad;
+  const size_t row_elems = (size_t)n * net->zs_ld;
+  need += row_elems * (kRnsMax * 7 + 16) + (size_t)planes * kRnsMax * n * net->u_ld;
+  size_t free_b = 0, total_b = 0;
+  CK(cudaMemGetInfo(&free_b, &total_b));
+  if (planes > kRnsMaxLayers || need > free_b / 2) return NNC_OK;
+  net->rns = true;
+  AL(net->c64, std::max(net->K_total, kPad));
+  AL(net->rc64, std::max(net->K_total, kPad));
+  if (planes == 0) return NNC_OK;
+  unsigned char* p;
+  AL(net->Z1, (size_t)n * (net->layers[0].mp + kPad));
+  AL(net->Zs, row_elems);
+  AL(p, row_elems * 2 * kRnsMax);
+  net->Rt = p;
+  AL(p, row_elems * 2 * kRnsMax);
+  net->Ra = p;
+  AL(p, row_elems * 2 * kRnsMax);
+  net->Rb = p;
+  AL(net->Rc, row_elems * kRnsMax);
+  AL(net->Ru, (size_t)planes * kRnsMax * n * net->u_ld);
+  AL(net->rt_scale, n);
+  AL(net->ru_scale, (size_t)planes * n);
+  for (int l = 0; l < L; ++l) {
+    LayerDev& Ly = net->layers[l];
+    if (!used(l)) break;
+    if (Ly.zy_off >= 0) Ly.c = net->c64 + Ly.zy_off;
+    const int ko = Ly.mp + (l == L - 1 && net->softmax ? kPad : 0);
+    Ly.set_in = rns_set(Ly.kp);
+    Ly.set_out = rns_set(ko);
+    int r = NNC_OK;
+    if (l > 0) {
+      AL(p, (size_t)Ly.set_in.n * Ly.mp * Ly.kp * 2);
+      Ly.Wr = p;
+      AL(Ly.wr_scale, Ly.mp);
+      CK(rns_pack_weights(Ly.set_in, Ly.W64, Ly.mp, Ly.kp, Ly.Wr, Ly.wr_scale, net->stream));
+      r = rns_plan(Ly.plan_rt, Ly.Wr, Ly.mp, net->Rt, n, Ly.mp, n, Ly.kp, Ly.set_in.n, false);
+    } else {
+      CK(launch_transpose_f64(Ly.W64, Ly.kp, Ly.mp, n, net->Z1, Ly.mp + kPad, net->stream));
+    }
+    if (r == NNC_OK && Ly.zy_off >= 0)
+      r = rns_plan(Ly.plan_rs, net->Ra, n, net->Rb, n, n, n, ko, Ly.set_out.n, true);
+    if (r != NNC_OK) return fail(r, "plan of the residue products failed");
+  }
+  return NNC_OK;
+}
+
 static int load_impl(nnc_net* net, int n_layers, const int* widths, const int* act,
                      const double* const* W, const double* const* b) {
   cudaDeviceProp prop;
@@ -795,12 +921,16 @@ static int load_impl(nnc_net* net, int n_layers, const int* widths, const int* a
         cudaEventCreateWithFlags(&net->ev_join, cudaEventDisableTiming) != cudaSuccess)
       return fail(NNC_ERR_CUDA, "side stream or events could not be created");
   }
+  if (prec == NNC_FP64) {
+    int r = load_rns(net);
+    if (r != NNC_OK) return r;
+  }
   const size_t tan_elems = (size_t)n * mp_max;
   const size_t zy_elems = (size_t)n * std::max(net->K_total, kPad);
   const size_t es = elem_size(prec);
   const bool x3 = prec == NNC_BF16X3;
   unsigned char* p;
-  for (int pp = 0; pp < 2; ++pp) {
+  for (int pp = 0; pp < 2 && !net->rns; ++pp) {
     AL(p, tan_elems * es);
     net->At[pp][0] = p;
     if (x3) {
@@ -808,7 +938,7 @@ static int load_impl(nnc_net* net, int n_layers, const int* widths, const int* a
       net->At[pp][1] = p;
     }
   }
-  for (int part = 0; part < (x3 ? 2 : 1); ++part) {
+  for (int part = 0; part < (x3 ? 2 : 1) && !net->rns; ++part) {
     AL(p, zy_elems * es);
     net->Zt[part] = p;
     AL(p, zy_elems * es);
@@ -913,7 +1043,7 @@ static int load_impl(nnc_net* net, int n_layers, const int* widths, const int* a
     float* hp;
     AL(hp, (size_t)splits * n * n);
     net->Hp = hp;
-  } else {
+  } else if (!net->rns) {
     const int tile = prec == NNC_FP64 ? 64 : 128;
     const int T = (n + tile - 1) / tile;
     const int tiles = T * (T + 1) / 2;

@@ -1,0 +1,74 @@
+// FP64 matrix products on the BF16 tensor cores by a residue number system (k_rns.cu), host side.
+#pragma once
+#include <cuda.h>
+
+#include "common.cuh"
+
+namespace nnc {
+
+constexpr int kRnsMax = 16;     // residues per number at most
+
+// Moduli and the constants of one product's number system, passed to the kernels by value.
+struct RnsSet {
+  int n = 0;                    // moduli in use
+  int bits = 0;                 // operands are integers of magnitude <= 2^bits
+  float p[kRnsMax], pinv[kRnsMax];
+  float r16[kRnsMax], r32[kRnsMax], r48[kRnsMax];   // 2^16, 2^32, 2^48 mod p, in [-p/2, p/2]
+  float q[kRnsMax];             // (P / p)^-1 mod p, in [-p/2, p/2]
+  unsigned c0[kRnsMax], c1[kRnsMax], c2[kRnsMax];   // round(2^96 / p), low word first
+  double scale = 0.0;           // P 2^-64
+};
+// The system of a product over K terms (K <= 65664).
+RnsSet rns_set(int K);
+
+struct RnsPlan {
+  CUtensorMap ta, tb;
+  int M = 0, N = 0, nkb = 0, bn = 0, lower = 0, a_rows = 0, b_rows = 0;
+  bool ready = false;
+};
+// D = A B^T for every residue: A [set.n][a_rows][K] and B [set.n][b_rows][K] (BF16 integers, K-major,
+// row stride K, a multiple of 64); M <= a_rows rounded up to 128, N <= b_rows.  lower: only the
+// tiles on and below the diagonal.
+int rns_plan(RnsPlan& p, const void* A, int a_rows, const void* B, int b_rows, int M, int N, int K,
+             int n_mod, bool lower);
+// C[i][n][m] = (sum_k A_i[m][k] B_i[n][k]) mod p_i, one byte each, rows of ldc (>= M rounded up to
+// 128) bytes, N rows per residue.
+cudaError_t rns_gemm(const RnsPlan& p, const RnsSet& s, unsigned char* C, int ldc, int* err,
+                     int sm_count, cudaStream_t st);
+
+// Weights W [mp][kp] (FP64): residues [set.n][mp][kp] with q folded in, and the row scales sa[mp].
+cudaError_t rns_pack_weights(const RnsSet& s, const double* W, int mp, int kp, void* res, double* sa,
+                             cudaStream_t st);
+
+// One layer's tangents, row by row (n rows of K = mp columns).
+struct RnsRows {
+  // source: residues C [in.n][n][ldc] of Zdot with the scales sa[m], sb[row], or FP64 Z
+  const unsigned char* C = nullptr;
+  int ldc = 0;
+  const double *sa = nullptr, *sb = nullptr;
+  double* Z = nullptr;          // [n][ldz]: read if C is NULL, else written
+  int ldz = 0;
+  int n = 0, K = 0;             // K: columns handled (a multiple of 128)
+  const double* s1 = nullptr;   // sigma' of the layer
+  const double *c = nullptr, *rc = nullptr;   // curvature weight and sqrt|c|
+  void* At = nullptr;           // residues of s1 * Z [out.n][n][K], or NULL
+  double* sat = nullptr;        // their row scales [n]
+  void *Sa = nullptr, *Sb = nullptr;   // residues of rc Z (q folded in) and sign(c) rc Z, or NULL
+  double* ss = nullptr;         // their row scales [n]
+};
+cudaError_t rns_rows(const RnsSet& in, const RnsSet& out, const RnsRows& a, cudaStream_t st);
+
+// rc = sqrt|c| (k entries)
+cudaError_t rns_curv(const double* c, double* rc, int k, cudaStream_t st);
+// The rank-two part of a softmax layer's curvature as two more columns m, m + 1 of its block:
+// Z[j][m + k] = w_k[j], c[m + k] = g'_k, rc likewise (see k_softmax_ext).
+cudaError_t rns_softmax_ext(int n, int m, int col, const double* p, const double* lam, double* Z,
+                            int ldz, double* c, double* rc, cudaStream_t st);
+
+// H[i][j] = H[j][i] = sum_l ss_l[i] ss_l[j] D_l[i][j] over `layers` residue planes
+// U [layers][kRnsMax][n][ldu] (entry [j][i], i >= j), ss [layers][n], sets[l] the system of plane l.
+constexpr int kRnsMaxLayers = 64;
+cudaError_t rns_h_finish(const RnsSet* sets, int layers, const unsigned char* U, int ldu,
+                         const double* ss, int n, double* H, cudaStream_t st);
+
+}  // namespace nnc
