@@ -14,18 +14,22 @@
 //   - the Chinese remainder theorem gives the integer result: D / P = frac(sum_i y_i / p_i) with
 //     y_i = D_i (P/p_i)^-1 mod p_i (the inverse is folded into one operand) and P = prod p_i,
 //     summed in 96-bit fixed point, where integer overflow is the frac().
+// The adjoints of the reverse sweep, W_l^T Zbar, take the same residues of W (REV below): n_out + 1
+// FP64 FMAs per weight would be 2.5 ms of the same evaluation.
 // The only roundings are those of the operands and of the result, so the error does not grow with
 // K as a sum of FP64 products does.  Chosen over slicing into 8-bit digits, which needs 28 products
 // where this needs 15.  Rows holding a NaN or an infinity give NaN.
 //
-// Measured, residual + J + H + gradient at one iterate: 784 -> 4096 x 7 -> 10 181 -> 6.0 ms (error of
-// H against 64-bit sums 5.8e-15 -> 3.8e-15), 784 -> 128 x 2 -> 10 911 -> 313 us (7.8e-16 -> 7.2e-16).
+// Measured, residual + J + H + gradient at one iterate: 784 -> 4096 x 7 -> 10 181 -> 6.0 ms with the
+// Hessian's products and 4.1 ms with the reverse sweep's too (error of H against 64-bit sums 5.6e-15
+// -> 4.3e-15), 784 -> 128 x 2 -> 10 911 -> 313 -> 183 us (7.8e-16 both).
 #include <cudaTypedefs.h>
 
 #include <algorithm>
 #include <cmath>
 #include <cstring>
 
+#include "async.cuh"
 #include "rns.cuh"
 #include "umma.cuh"
 
@@ -142,13 +146,12 @@ __global__ void __launch_bounds__(256) k_rns_pack(const __grid_constant__ RnsSet
 // takes sqrt|c| z on both sides (sign(c) on one) so that one scale per row fits every column.
 // Bound: 90 bytes written per element (15 residues x 3 operands), about 13 operations on the FP64 pipe.
 template <bool CRT>
-__global__ void __launch_bounds__(256) k_rns_rows(const __grid_constant__ RnsSet in,
-                                                  const __grid_constant__ RnsSet out,
+__global__ void __launch_bounds__(256) k_rns_rows(const __grid_constant__ RnsSet set,
                                                   const RnsRows a) {
   __shared__ int sh[8];
   const int r = blockIdx.x;
   double* zrow = a.Z + (size_t)r * a.ldz;
-  const double sb = CRT ? in.scale * a.sb[r] : 0.0;
+  const double sb = CRT ? set.scale * a.sb[r] : 0.0;
   int ha = 0, hs = 0;
   for (int k = 4 * threadIdx.x; k < a.K; k += 4 * blockDim.x) {
     double z[4];
@@ -157,12 +160,12 @@ __global__ void __launch_bounds__(256) k_rns_rows(const __grid_constant__ RnsSet
       const unsigned char* c = a.C + (size_t)r * a.ldc + k;
       const size_t plane = (size_t)a.n * a.ldc;
 #pragma unroll 5
-      for (int i = 0; i < in.n; ++i) {
+      for (int i = 0; i < set.n; ++i) {
         const unsigned y = __ldg(reinterpret_cast<const unsigned*>(c + i * plane));
-        t[0].add(in, i, y & 0xFFu);
-        t[1].add(in, i, (y >> 8) & 0xFFu);
-        t[2].add(in, i, (y >> 16) & 0xFFu);
-        t[3].add(in, i, y >> 24);
+        t[0].add(set, i, y & 0xFFu);
+        t[1].add(set, i, (y >> 8) & 0xFFu);
+        t[2].add(set, i, (y >> 16) & 0xFFu);
+        t[3].add(set, i, y >> 24);
       }
 #pragma unroll
       for (int j = 0; j < 4; ++j) z[j] = t[j].value() * sb * __ldg(a.sa + k + j);
@@ -182,7 +185,7 @@ __global__ void __launch_bounds__(256) k_rns_rows(const __grid_constant__ RnsSet
   double sca, scs;
   ha = block_max(ha, sh);
   hs = block_max(hs, sh);
-  const double ba = rns_scale(ha, out.bits, &sca), bs = rns_scale(hs, out.bits, &scs);
+  const double ba = rns_scale(ha, set.bits, &sca), bs = rns_scale(hs, set.bits, &scs);
   if (threadIdx.x == 0) {
     if (a.At) a.sat[r] = ba;
     if (a.Sa) a.ss[r] = bs;
@@ -199,10 +202,10 @@ __global__ void __launch_bounds__(256) k_rns_rows(const __grid_constant__ RnsSet
       for (int j = 0; j < 4; ++j) l[j] = rns_limbs(__double2ll_rn(__ldg(a.s1 + k + j) * z[j] * sca));
       __nv_bfloat16* dst = (__nv_bfloat16*)a.At + o;
 #pragma unroll 5
-      for (int i = 0; i < out.n; ++i)
+      for (int i = 0; i < set.n; ++i)
         *reinterpret_cast<uint2*>(dst + i * plane) =
-            make_uint2(bf2(rns_res(out, i, l[0]), rns_res(out, i, l[1])),
-                       bf2(rns_res(out, i, l[2]), rns_res(out, i, l[3])));
+            make_uint2(bf2(rns_res(set, i, l[0]), rns_res(set, i, l[1])),
+                       bf2(rns_res(set, i, l[2]), rns_res(set, i, l[3])));
     }
     if (a.Sa) {
       Limbs l[4];
@@ -219,18 +222,111 @@ __global__ void __launch_bounds__(256) k_rns_rows(const __grid_constant__ RnsSet
       }
       __nv_bfloat16 *da = (__nv_bfloat16*)a.Sa + o, *db = (__nv_bfloat16*)a.Sb + o;
 #pragma unroll 5
-      for (int i = 0; i < out.n; ++i) {
+      for (int i = 0; i < set.n; ++i) {
         float v[4], w[4];
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-          v[j] = rns_res(out, i, l[j]);
-          w[j] = rns_mod(v[j] * out.q[i], out.p[i], out.pinv[i]);
+          v[j] = rns_res(set, i, l[j]);
+          w[j] = rns_mod(v[j] * set.q[i], set.p[i], set.pinv[i]);
         }
         *reinterpret_cast<uint2*>(da + i * plane) = make_uint2(bf2(w[0], w[1]), bf2(w[2], w[3]));
         *reinterpret_cast<uint2*>(db + i * plane) =
             make_uint2(bf2(v[0], v[1]) ^ neg0, bf2(v[2], v[3]) ^ neg1);
       }
     }
+  }
+}
+
+// ------------------------------------------------------------------ reverse rows
+// One cluster of eight CTAs per seed column s: Abar[k][s] from the residue planes of W_l^T Zbar (or,
+// for the output layer, the seeds), then sigma' Abar of the layer below as residues, one scale per
+// seed (the row scales of that layer's weights are multiplied in, since its product sums over rows).
+// First layer: J and the gradient instead.  Eight SMs share a seed because its 4096 entries cost ten
+// operations each on the FP64 pipe, 10 us on one SM.
+constexpr int kRevCl = 8;
+__global__ void __launch_bounds__(256) k_rns_rev_rows(const __grid_constant__ RnsSet set,
+                                                      const RnsRev a) {
+  __shared__ int sh[8], mine;
+  const int s = blockIdx.y;
+  const int kb = blockIdx.x * 4 * blockDim.x, step = gridDim.x * 4 * blockDim.x;
+  const bool is_lam = s == a.lam_col;
+  double* zrow = a.Zs + (size_t)s * a.K;
+  int hi = 0;
+  for (int k = kb + 4 * threadIdx.x; k < a.K; k += step) {
+    double v[4];
+    if (a.C) {
+      Crt t[4];
+      const double sb = set.scale * a.sb[s];
+      const unsigned char* c = a.C + (size_t)s * a.K + k;
+      const size_t plane = (size_t)a.seeds * a.K;
+#pragma unroll 3
+      for (int i = 0; i < set.n; ++i) {
+        float y[4] = {0.f, 0.f, 0.f, 0.f};
+        for (int ch = 0; ch < a.chunks; ++ch) {
+          const unsigned w = __ldg(reinterpret_cast<const unsigned*>(c + (size_t)(ch * set.n + i) * plane));
+#pragma unroll
+          for (int j = 0; j < 4; ++j) y[j] += __uint_as_float(0x4B000000u | ((w >> (8 * j)) & 0xFFu)) - 8388608.f;
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          float r = rns_mod(y[j], set.p[i], set.pinv[i]);
+          r += r < 0.f ? set.p[i] : 0.f;
+          t[j].add(set, i, __float_as_uint(r + 8388608.f) & 0x1FFu);
+        }
+      }
+#pragma unroll
+      for (int j = 0; j < 4; ++j) v[j] = t[j].value() * sb;
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int kk = k + j;
+      double z;
+      if (a.C) {
+        if (a.s1) {
+          z = a.s1[kk] * v[j];
+          if (is_lam) {
+            const double cv = a.s2[kk] * v[j];
+            a.c_out[kk] = cv;
+          }
+        } else {
+          if (kk < a.kvalid) {
+            if (a.J && s < a.nJ) a.J[(size_t)s * a.kvalid + kk] = v[j];
+            if (a.g && is_lam) a.g[kk] = v[j];
+          }
+          continue;
+        }
+      } else {
+        double cv = 0.0;
+        z = kk < a.kvalid ? out_seed(kk, s, a.kvalid, a.nJ, a.lam_col, a.s1, a.s2, a.lam, a.soft_p, &cv) : 0.0;
+        if (is_lam) a.c_out[kk] = cv;
+      }
+      z *= a.sa[kk];
+      hi = max(hi, abs_hi(z));
+      zrow[kk] = z;
+    }
+  }
+  if (a.C && !a.s1) return;   // the whole cluster: nothing is exchanged on the first layer
+  hi = block_max(hi, sh);
+  if (threadIdx.x == 0) mine = hi;
+  __syncthreads();
+  async::cluster_sync();
+  for (int q = 0; q < kRevCl; ++q)
+    hi = max(hi, __float_as_int(async::ld_dsmem_f32(smem_u32(&mine), (uint32_t)q)));
+  async::cluster_sync();      // no CTA leaves while another still reads its shared memory
+  double sc;
+  const double back = rns_scale(hi, set.bits, &sc);
+  if (blockIdx.x == 0 && threadIdx.x == 0) a.sb_out[s] = back;
+  for (int k = kb + 4 * threadIdx.x; k < a.K; k += step) {
+    Limbs l[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) l[j] = rns_limbs(__double2ll_rn(zrow[k + j] * sc));
+    __nv_bfloat16* dst = (__nv_bfloat16*)a.Zr + (size_t)s * a.K + k;
+    const size_t plane = (size_t)a.seeds * a.K;
+#pragma unroll 5
+    for (int i = 0; i < set.n; ++i)
+      *reinterpret_cast<uint2*>(dst + i * plane) =
+          make_uint2(bf2(rns_res(set, i, l[0]), rns_res(set, i, l[1])),
+                     bf2(rns_res(set, i, l[2]), rns_res(set, i, l[3])));
   }
 }
 
@@ -267,11 +363,7 @@ __global__ void k_rns_softmax_ext(int n, int m, int col, const double* __restric
 }
 
 // ------------------------------------------------------------------ H from the residue planes
-struct RnsFinish {
-  RnsSet set[2];                       // at most two systems occur (15 or 16 moduli), by K their bits
-  unsigned char which[kRnsMaxLayers];
-};
-__global__ void __launch_bounds__(256) k_rns_h(const __grid_constant__ RnsFinish f, int layers,
+__global__ void __launch_bounds__(256) k_rns_h(const __grid_constant__ RnsSet s, int layers,
                                                const unsigned char* __restrict__ U, int ldu,
                                                const double* __restrict__ ss, int n,
                                                double* __restrict__ H) {
@@ -283,7 +375,6 @@ __global__ void __launch_bounds__(256) k_rns_h(const __grid_constant__ RnsFinish
   double v[4] = {0.0, 0.0, 0.0, 0.0};
   if (j < n && i < n) {
     for (int l = 0; l < layers; ++l) {
-      const RnsSet& s = f.set[f.which[l]];
       const unsigned char* u = U + ((size_t)l * kRnsMax * n + j) * ldu + i;
       const size_t plane = (size_t)n * ldu;
       Crt r[4];
@@ -325,11 +416,18 @@ __global__ void __launch_bounds__(256) k_rns_h(const __grid_constant__ RnsFinish
 // Bound: the tensor pipe.  A reduction costs three FP32 operations per element and 1024 terms of K,
 // 0.2 of the MMA time on 8 warps, and runs under the next accumulator's MMAs; the tile is as wide as
 // two accumulators in TMEM allow.
+//
+// REV: the reverse sweep's product W^T Zbar over the rows of W, BN = 16, 32 or 48 seed columns.  A is
+// the same residue array read the other way round: its stages are two boxes of 64 rows x 64 columns,
+// which the MMA takes as an MN-major operand.  Each item is one 128-column strip of one modulus and
+// one chunk of up to 1024 rows, whose residues go to a plane of their own (the reader adds the
+// chunks).  Bound: HBM, 30 bytes per weight; up to 12 stages of 18 KB keep 200 KB per SM in flight.
 constexpr int kGBM = 128, kGBK = 64;
 constexpr int kGThreads = 320;                 // producer, MMA, eight epilogue warps
 constexpr int kGChunk = 1024 / kGBK;           // K blocks that add up exactly
 
 struct RnsGemm {
+  int chunks;            // REV: chunks of 1024 rows
   int M, N, nkb, lower, ntm, ntn, tiles, n_mod, a_rows, b_rows;
   unsigned char* C;
   int ldc;
@@ -337,20 +435,30 @@ struct RnsGemm {
   float p[kRnsMax], pinv[kRnsMax];
 };
 
-template <int BN>
+template <int BN, bool REV>
 struct GCfg {
   static constexpr int STAGE = (kGBM + BN) * 128;
-  static constexpr int STAGES = (227 * 1024 - 2048) / STAGE > 6 ? 6 : (227 * 1024 - 2048) / STAGE;
+  static constexpr int FIT = (227 * 1024 - 2048) / STAGE, CAP = REV ? 12 : 6;
+  static constexpr int STAGES = FIT > CAP ? CAP : FIT;
   static constexpr int SMEM = STAGES * STAGE + 1024 + 256;
-  static constexpr uint32_t IDESC = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kGBM >> 4) << 24);
+  static_assert((2 * STAGES + 5) * 8 + 12 <= 256, "barriers fit behind the stages");
+  // FP32 sums of BF16 products, A MN-major (bit 15) in the reverse sweep
+  static constexpr uint32_t IDESC = (1u << 4) | (1u << 7) | (1u << 10) | (REV ? 1u << 15 : 0u) |
+                                    ((uint32_t)(kGBM >> 4) << 24);
   static_assert(BN % 16 == 0 && BN <= 256 && (BN * 128) % 1024 == 0, "tile width");
 };
 
-template <int BN>
+// Descriptor of an MN-major operand in 128-byte swizzled rows of 64 elements: 8 rows of K per KB
+// (stride byte offset 1024), the next 64 elements of M `lbo` bytes on.
+__device__ __forceinline__ uint64_t sdesc_mn(uint32_t addr, uint32_t lbo) {
+  return sdesc<2, 1024>(addr) | ((uint64_t)(lbo >> 4) << 16);
+}
+
+template <int BN, bool REV>
 __global__ void __launch_bounds__(kGThreads, 1)
     k_rns_gemm(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtensorMap tb,
                const __grid_constant__ RnsGemm g) {
-  using C = GCfg<BN>;
+  using C = GCfg<BN, REV>;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   uint64_t* full = (uint64_t*)(smem + C::STAGES * C::STAGE);
@@ -364,6 +472,7 @@ __global__ void __launch_bounds__(kGThreads, 1)
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int per_mod = g.tiles, total = g.tiles * g.n_mod;
+  // REV: tn is the chunk of rows
   auto decode = [&](int t, int& mod, int& tm, int& tn) {
     mod = t / per_mod;
     int r = t - mod * per_mod;
@@ -412,8 +521,11 @@ __global__ void __launch_bounds__(kGThreads, 1)
       for (int t = blockIdx.x; t < total && !stop; t += gridDim.x) {
         int mod, tm, tn;
         decode(t, mod, tm, tn);
-        const int ar = mod * g.a_rows + tm * kGBM, br = mod * g.b_rows + tn * BN;
-        for (int kb = 0; kb < g.nkb; ++kb, ++i) {
+        const int kb_beg = REV ? tn * kGChunk : 0;
+        const int kb_end = REV ? min(g.nkb, kb_beg + kGChunk) : g.nkb;
+        const int ar = mod * g.a_rows + (REV ? 0 : tm * kGBM);
+        const int br = mod * g.b_rows + (REV ? 0 : tn * BN);
+        for (int kb = kb_beg; kb < kb_end; ++kb, ++i) {
           const int s = i % C::STAGES;
           const uint32_t ph = (uint32_t)(i / C::STAGES) & 1u;
           if (!mbar_wait(smem_u32(&empty[s]), ph ^ 1u, g.err, 71, abort_flag)) {
@@ -423,7 +535,12 @@ __global__ void __launch_bounds__(kGThreads, 1)
           uint8_t* st = smem + s * C::STAGE;
           const uint32_t fb = smem_u32(&full[s]);
           mbar_expect_tx(fb, C::STAGE);
-          tma_load_2d(smem_u32(st), &ta, fb, kb * kGBK, ar);
+          if (REV) {
+            tma_load_2d(smem_u32(st), &ta, fb, tm * kGBM, ar + kb * kGBK);
+            tma_load_2d(smem_u32(st + kGBK * 128), &ta, fb, tm * kGBM + 64, ar + kb * kGBK);
+          } else {
+            tma_load_2d(smem_u32(st), &ta, fb, kb * kGBK, ar);
+          }
           tma_load_2d(smem_u32(st + kGBM * 128), &tb, fb, kb * kGBK, br);
           issued = i + 1;
         }
@@ -436,9 +553,11 @@ __global__ void __launch_bounds__(kGThreads, 1)
       for (int t = blockIdx.x; t < total && !stop; t += gridDim.x) {
         int mod, tm, tn;
         decode(t, mod, tm, tn);
-        const int n_eff = (min(BN, g.N - tn * BN) + 15) / 16 * 16;
+        const int n_eff = REV ? BN : (min(BN, g.N - tn * BN) + 15) / 16 * 16;
         const uint32_t idesc = C::IDESC | ((uint32_t)(n_eff >> 3) << 17);
-        for (int kb0 = 0; kb0 < g.nkb && !stop; kb0 += kGChunk, ++ai) {
+        const int kb_beg = REV ? tn * kGChunk : 0;
+        const int kb_end = REV ? min(g.nkb, kb_beg + kGChunk) : g.nkb;
+        for (int kb0 = kb_beg; kb0 < kb_end && !stop; kb0 += kGChunk, ++ai) {
           const int b = ai & 1;
           if (ai >= 2 &&
               !mbar_wait(smem_u32(&tfree[b]), (uint32_t)((ai - 2) >> 1) & 1u, g.err, 72, abort_flag)) {
@@ -459,7 +578,8 @@ __global__ void __launch_bounds__(kGThreads, 1)
             const uint32_t sa = smem_u32(smem + s * C::STAGE), sb = sa + kGBM * 128;
 #pragma unroll
             for (int kk = 0; kk < kGBK / 16; ++kk)
-              umma_bf16(d, sdesc<2, 1024>(sa + kk * 32), sdesc<2, 1024>(sb + kk * 32), idesc,
+              umma_bf16(d, REV ? sdesc_mn(sa + kk * 16 * 128, kGBK * 128) : sdesc<2, 1024>(sa + kk * 32),
+                        sdesc<2, 1024>(sb + kk * 32), idesc,
                         (kb > kb0 || kk > 0) ? 1u : 0u);
             umma_commit(smem_u32(&empty[s]));
           }
@@ -478,12 +598,14 @@ __global__ void __launch_bounds__(kGThreads, 1)
     for (int t = blockIdx.x; t < total && !stop; t += gridDim.x) {
       int mod, tm, tn;
       decode(t, mod, tm, tn);
-      const int n_eff = min(BN, g.N - tn * BN);
+      const int n_eff = REV ? g.N : min(BN, g.N - tn * BN);
       const float p = g.p[mod], pinv = g.pinv[mod];
       float res[NH];
 #pragma unroll
       for (int j = 0; j < NH; ++j) res[j] = 0.f;
-      for (int kb0 = 0; kb0 < g.nkb; kb0 += kGChunk, ++ai) {
+      const int kb_beg = REV ? tn * kGChunk : 0;
+      const int kb_end = REV ? min(g.nkb, kb_beg + kGChunk) : g.nkb;
+      for (int kb0 = kb_beg; kb0 < kb_end; kb0 += kGChunk, ++ai) {
         const int b = ai & 1;
         const bool ok = mbar_wait(smem_u32(&accf[b]), (uint32_t)(ai >> 1) & 1u, g.err, 74, abort_flag);
         if (!__all_sync(0xffffffffu, ok)) {
@@ -511,8 +633,9 @@ __global__ void __launch_bounds__(kGThreads, 1)
         if (lane == 0) mbar_arrive(smem_u32(&tfree[b]));
       }
       if (stop) break;
-      const int n0 = tn * BN + half * NH;
-      unsigned char* dst = g.C + ((size_t)mod * g.N + n0) * g.ldc + tm * kGBM + q * 32 + lane;
+      const int n0 = (REV ? 0 : tn * BN) + half * NH;
+      const size_t plane = REV ? (size_t)(tn * g.n_mod + mod) * BN : (size_t)mod * g.N;
+      unsigned char* dst = g.C + (plane + n0) * g.ldc + tm * kGBM + q * 32 + lane;
 #pragma unroll
       for (int j = 0; j < NH; ++j) {
         if (n0 + j < g.N) {
@@ -555,7 +678,7 @@ PFN_cuTensorMapEncodeTiled_v12000 rns_encode() {
   return (PFN_cuTensorMapEncodeTiled_v12000)p;
 }
 
-bool rns_map(CUtensorMap* m, const void* base, long long rows, int cols, int box_rows) {
+bool rns_map(CUtensorMap* m, const void* base, long long rows, int cols, int box_rows) {   // 64-column boxes
   auto enc = rns_encode();
   if (!enc || !base) return false;
   cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
@@ -567,17 +690,17 @@ bool rns_map(CUtensorMap* m, const void* base, long long rows, int cols, int box
              CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-template <int BN>
+template <int BN, bool REV = false>
 cudaError_t launch_gemm(const RnsPlan& p, const RnsGemm& g, int grid, cudaStream_t st) {
-  using C = GCfg<BN>;
+  using C = GCfg<BN, REV>;
   static bool attr = false;
   if (!attr) {
-    cudaError_t e = cudaFuncSetAttribute(k_rns_gemm<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaError_t e = cudaFuncSetAttribute(k_rns_gemm<BN, REV>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          C::SMEM);
     if (e != cudaSuccess) return e;
     attr = true;
   }
-  k_rns_gemm<BN><<<grid, kGThreads, C::SMEM, st>>>(p.ta, p.tb, g);
+  k_rns_gemm<BN, REV><<<grid, kGThreads, C::SMEM, st>>>(p.ta, p.tb, g);
   note_launch();
   return cudaGetLastError();
 }
@@ -654,11 +777,29 @@ int rns_plan(RnsPlan& p, const void* A, int a_rows, const void* B, int b_rows, i
   return NNC_OK;
 }
 
+int rns_plan_rev(RnsPlan& p, const void* W, int mp, int kp, const void* Z, int seeds, int n_mod) {
+  p = RnsPlan();
+  if (mp % 128 || kp % 128 || seeds < 1 || seeds > 48) return NNC_ERR_ARG;
+  p.M = kp;
+  p.nkb = mp / kGBK;
+  p.bn = (seeds + 15) / 16 * 16;
+  p.N = p.bn;
+  p.a_rows = mp;
+  p.b_rows = p.bn;
+  p.rev = 1;
+  if (!rns_map(&p.ta, W, (long long)n_mod * mp, kp, kGBK) ||
+      !rns_map(&p.tb, Z, (long long)n_mod * p.bn, mp, p.bn))
+    return NNC_ERR_CUDA;
+  p.ready = true;
+  return NNC_OK;
+}
+
 cudaError_t rns_gemm(const RnsPlan& p, const RnsSet& s, unsigned char* C, int ldc, int* err,
                      int sm_count, cudaStream_t st) {
   RnsGemm g{};
   g.ntm = (p.M + kGBM - 1) / kGBM;
-  g.ntn = (p.N + p.bn - 1) / p.bn;
+  g.chunks = (p.nkb + kGChunk - 1) / kGChunk;
+  g.ntn = p.rev ? g.chunks : (p.N + p.bn - 1) / p.bn;
   if (!p.ready || ldc < g.ntm * kGBM) return cudaErrorInvalidValue;
   g.M = p.M;
   g.N = p.N;
@@ -676,7 +817,10 @@ cudaError_t rns_gemm(const RnsPlan& p, const RnsSet& s, unsigned char* C, int ld
     g.pinv[i] = s.pinv[i];
   }
   const int grid = std::min(sm_count, g.tiles * g.n_mod);
-  switch (p.bn) {
+  switch (p.rev ? -p.bn : p.bn) {
+    case -16: return launch_gemm<16, true>(p, g, grid, st);
+    case -32: return launch_gemm<32, true>(p, g, grid, st);
+    case -48: return launch_gemm<48, true>(p, g, grid, st);
     case 128: return launch_gemm<128>(p, g, grid, st);
     case 208: return launch_gemm<208>(p, g, grid, st);
     case 256: return launch_gemm<256>(p, g, grid, st);
@@ -691,13 +835,31 @@ cudaError_t rns_pack_weights(const RnsSet& s, const double* W, int mp, int kp, v
   return cudaGetLastError();
 }
 
-cudaError_t rns_rows(const RnsSet& in, const RnsSet& out, const RnsRows& a, cudaStream_t st) {
+cudaError_t rns_rows(const RnsSet& s, const RnsRows& a, cudaStream_t st) {
   if (a.K % 128 || a.n < 1 || (a.ldz & 1)) return cudaErrorInvalidValue;
   const int threads = std::min(256, std::max(32, a.K / 4));
-  if (a.C) k_rns_rows<true><<<a.n, threads, 0, st>>>(in, out, a);
-  else k_rns_rows<false><<<a.n, threads, 0, st>>>(in, out, a);
+  if (a.C) k_rns_rows<true><<<a.n, threads, 0, st>>>(s, a);
+  else k_rns_rows<false><<<a.n, threads, 0, st>>>(s, a);
   note_launch();
   return cudaGetLastError();
+}
+
+cudaError_t rns_rev_rows(const RnsSet& s, const RnsRev& a, int S, cudaStream_t st) {
+  if (a.K % 128 || S < 1 || S > a.seeds) return cudaErrorInvalidValue;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(kRevCl, S);
+  cfg.blockDim = dim3(std::min(256, std::max(32, (a.K / (4 * kRevCl) + 31) / 32 * 32)));
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = kRevCl;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, k_rns_rev_rows, s, a);
+  note_launch();
+  return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 cudaError_t rns_curv(const double* c, double* rc, int k, cudaStream_t st) {
@@ -713,19 +875,10 @@ cudaError_t rns_softmax_ext(int n, int m, int col, const double* p, const double
   return cudaGetLastError();
 }
 
-cudaError_t rns_h_finish(const RnsSet* sets, int layers, const unsigned char* U, int ldu,
+cudaError_t rns_h_finish(const RnsSet& s, int layers, const unsigned char* U, int ldu,
                          const double* ss, int n, double* H, cudaStream_t st) {
-  if (layers < 1 || layers > kRnsMaxLayers) return cudaErrorInvalidValue;
-  RnsFinish f{};
-  int have = 0;
-  for (int l = 0; l < layers; ++l) {
-    int w = 0;
-    while (w < have && f.set[w].n != sets[l].n) ++w;
-    if (w == have) f.set[have++] = sets[l];   // what the result needs depends on the moduli alone
-    f.which[l] = (unsigned char)w;
-  }
   dim3 grid((n + 127) / 128, (n + 7) / 8);
-  k_rns_h<<<grid, dim3(32, 8), 0, st>>>(f, layers, U, ldu, ss, n, H);
+  k_rns_h<<<grid, dim3(32, 8), 0, st>>>(s, layers, U, ldu, ss, n, H);
   note_launch();
   return cudaGetLastError();
 }

@@ -2,7 +2,7 @@
 // (Zdot_l = W_l Adot_{l-1}, n_in tangent columns) and the per-layer symmetric product
 // H += Zdot_l^T diag(c_l) Zdot_l: a plain shared-memory tiled GEMM with register micro-tiles.  The
 // FP64 form comes here only when the residue products of k_rns.cu do not fit (their residues take
-// four times the memory of the FP64 weights) or for more than kRnsMaxLayers curved layers.
+// four times the memory of the FP64 weights).
 #include "kernels.cuh"
 
 namespace nnc {

@@ -48,12 +48,11 @@ struct LayerDev {
   nnc::RevGeom rev_geom;          // its launch geometry
   int rev_cnt_off = 0;            // offset of its strip counters in nnc_net::rev_cnt
   int zy_off = -1;                // column offset of this layer's Zdot / Ydot block (-1: none)
-  // FP64 form, residue products: BF16 residues of W [set.n][mp][kp], their row scales, the plans
-  // of the tangent product and of the symmetric product, and this layer's residue plane of H
+  // FP64 form, residue products: BF16 residues of W [rset.n][mp][kp], their row scales, the
+  // plans of its products, and its residue plane of H
   void* Wr = nullptr;
   double* wr_scale = nullptr;
-  nnc::RnsSet set_in, set_out;    // products over K = kp (tangents) and K = mp (next layer, H)
-  nnc::RnsPlan plan_rt, plan_rs;
+  nnc::RnsPlan plan_rt, plan_rs, plan_rr;   // tangents, symmetric product, reverse
   int h_plane = -1;
 };
 
@@ -113,6 +112,11 @@ struct nnc_net {
   bool hp_f32 = false;
   // FP64 form on the tensor cores (residue products, k_rns.cu)
   bool rns = false;
+  nnc::RnsSet rset;                        // one number system for every product of the net
+  double* Zv = nullptr;                    // reverse seeds, scaled [S_max][mp_max]
+  void* Zr = nullptr;                      // their residues [rset.n][S_max to 16][mp_max]
+  double* zr_scale = nullptr;              // their scales, ping-pong [2][48]
+  unsigned char* Cv = nullptr;             // results of the reverse product
   double *c64 = nullptr, *rc64 = nullptr;  // c_l of all curved layers at zy_off, and sqrt|c_l|
   double* Z1 = nullptr;                    // W_1^T [n_in][mp_1 + 128]
   double* Zs = nullptr;                    // Zdot_l^T of the current layer [n_in][zs_ld]

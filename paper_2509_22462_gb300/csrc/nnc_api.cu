@@ -64,16 +64,16 @@ size_t elem_size(int prec) { return prec == NNC_FP64 ? 8 : prec == NNC_FP32 ? 4 
   } while (0)
 
 template <typename T>
-int dalloc(nnc_net* net, T** p, size_t n) {
+int dalloc(nnc_net* net, T** p, size_t n, bool zero = true) {
   void* q = nullptr;
   const size_t bytes = std::max<size_t>(n, 1) * sizeof(T);
   cudaError_t e = cudaMalloc(&q, bytes);
   if (e != cudaSuccess)
     return fail(NNC_ERR_OOM, std::string("cudaMalloc(") + std::to_string(bytes) + "): " +
                                  cudaGetErrorString(e));
-  e = cudaMemsetAsync(q, 0, bytes, net->stream);
-  if (e != cudaSuccess) return fail(NNC_ERR_CUDA, cudaGetErrorString(e));
+  if (zero) e = cudaMemsetAsync(q, 0, bytes, net->stream);
   net->allocs.push_back(q);
+  if (e != cudaSuccess) return fail(NNC_ERR_CUDA, cudaGetErrorString(e));
   net->bytes += bytes;
   *p = (T*)q;
   return NNC_OK;
@@ -82,6 +82,12 @@ int dalloc(nnc_net* net, T** p, size_t n) {
 #define AL(p, n)                                    \
   do {                                              \
     int r_ = dalloc(net, &(p), (n));                \
+    if (r_ != NNC_OK) return r_;                    \
+  } while (0)
+// an array whose every element is written before it is read
+#define AL_RAW(p, n)                                \
+  do {                                              \
+    int r_ = dalloc(net, &(p), (n), false);         \
     if (r_ != NNC_OK) return r_;                    \
   } while (0)
 
@@ -220,6 +226,45 @@ int run_reverse(nnc_net* net, bool fp64, int nJ, bool with_lam, const double* la
   const bool tc = is_tc(net->prec);
   LayerDev& Lo = net->layers.back();
   const double* soft_p = net->softmax ? Lo.a : nullptr;   // softmax probabilities (value pass)
+  if (net->rns) {
+    // residue products; between two of them one kernel adds the result up, applies the layer boundary
+    // and makes the residues of the next seeds
+    RnsRev a;
+    a.seeds = (net->S_max + 15) / 16 * 16;
+    a.nJ = nJ;
+    a.lam_col = lam_col;
+    a.Zs = net->Zv;
+    a.Zr = net->Zr;
+    a.K = Lo.mp;
+    a.kvalid = Lo.m;
+    a.s1 = Lo.s1;
+    a.s2 = Lo.s2;
+    a.lam = lam;
+    a.soft_p = soft_p;
+    a.sa = Lo.wr_scale;
+    a.c_out = Lo.c;
+    a.sb_out = net->zr_scale;
+    CK(rns_rev_rows(net->rset, a, S, st));
+    for (int l = net->L - 1; l >= 0; --l) {
+      LayerDev& Ly = net->layers[l];
+      PROF(PK_REV);
+      CK(rns_gemm(Ly.plan_rr, net->rset, net->Cv, Ly.kp, net->dev_err, net->sm_count, st));
+      a.C = net->Cv;
+      a.chunks = (Ly.mp + 1023) / 1024;
+      a.sb = a.sb_out;
+      a.sb_out = net->zr_scale + (l % 2 == net->L % 2 ? 0 : 48);
+      a.K = Ly.kp;
+      a.kvalid = Ly.k;
+      a.s1 = l > 0 ? net->layers[l - 1].s1 : nullptr;
+      a.s2 = l > 0 ? net->layers[l - 1].s2 : nullptr;
+      a.sa = l > 0 ? net->layers[l - 1].wr_scale : nullptr;
+      a.c_out = l > 0 ? net->layers[l - 1].c : nullptr;
+      a.J = l > 0 ? nullptr : J;
+      a.g = l > 0 ? nullptr : g;
+      CK(rns_rev_rows(net->rset, a, S, st));
+    }
+    return NNC_OK;
+  }
   if (net->tc_rev) {
     // seeds^T in three BF16 parts, then per layer: split-K tensor-core product W_l^T Zbar and a reduce
     // that forms the next seeds (or J and the gradient on the first layer)
@@ -437,7 +482,6 @@ int run_hessian_rns(nnc_net* net, const double* lam, double* H, cudaStream_t st)
     return NNC_OK;
   }
   CK(rns_curv(net->c64, net->rc64, net->K_total, st));
-  RnsSet sets[kRnsMaxLayers];
   for (int l = 0; l < net->L; ++l) {
     LayerDev& Ly = net->layers[l];
     const bool last = l == net->L - 1, soft = last && net->softmax;
@@ -449,7 +493,7 @@ int run_hessian_rns(nnc_net* net, const double* lam, double* H, cudaStream_t st)
     a.ldz = l == 0 ? Ly.mp + kPad : net->zs_ld;
     if (l > 0) {
       PROF(PK_TANGENT);
-      CK(rns_gemm(Ly.plan_rt, Ly.set_in, net->Rc, Ly.mp, net->dev_err, net->sm_count, st));
+      CK(rns_gemm(Ly.plan_rt, net->rset, net->Rc, Ly.mp, net->dev_err, net->sm_count, st));
       a.C = net->Rc;
       a.ldc = Ly.mp;
       a.sa = Ly.wr_scale;
@@ -457,7 +501,7 @@ int run_hessian_rns(nnc_net* net, const double* lam, double* H, cudaStream_t st)
     }
     PROF(PK_OTHER);
     if (soft) {   // the result in FP64 first, then its two added columns
-      if (l > 0) CK(rns_rows(Ly.set_in, Ly.set_out, a, st));
+      if (l > 0) CK(rns_rows(net->rset, a, st));
       CK(rns_softmax_ext(n, net->n_out, Ly.mp, Ly.a, lam, a.Z, a.ldz, Ly.c,
                          net->rc64 + Ly.zy_off, st));
       a.C = nullptr;
@@ -475,17 +519,16 @@ int run_hessian_rns(nnc_net* net, const double* lam, double* H, cudaStream_t st)
       a.Sb = net->Rb;
       a.ss = net->ru_scale + (size_t)Ly.h_plane * n;
     }
-    CK(rns_rows(Ly.set_in, Ly.set_out, a, st));
+    CK(rns_rows(net->rset, a, st));
     if (Ly.zy_off >= 0) {
       PROF(PK_SYRK);
-      CK(rns_gemm(Ly.plan_rs, Ly.set_out,
+      CK(rns_gemm(Ly.plan_rs, net->rset,
                   net->Ru + (size_t)Ly.h_plane * kRnsMax * n * net->u_ld, net->u_ld, net->dev_err,
                   net->sm_count, st));
-      sets[Ly.h_plane] = Ly.set_out;
     }
   }
   PROF(PK_OTHER);
-  CK(rns_h_finish(sets, net->h_planes, net->Ru, net->u_ld, net->ru_scale, n, H, st));
+  CK(rns_h_finish(net->rset, net->h_planes, net->Ru, net->u_ld, net->ru_scale, n, H, st));
   return NNC_OK;
 }
 
@@ -717,64 +760,68 @@ void nnc_free(nnc_net* net) {
 }
 
 // Buffers, residues and plans of the FP64 form's residue products.  They take 30 to 32 bytes per
-// weight beside the 8 of the FP64 weights; where that is more than half of the free memory, or more
-// than kRnsMaxLayers layers are curved, the CUDA-core products stay in use (net->rns false).
+// weight beside the 8 of the FP64 weights; where that is more than half of the free memory, the
+// CUDA-core products stay in use (net->rns false).
 static int load_rns(nnc_net* net) {
   const int n = net->n_in, L = net->L;
-  int planes = 0, mp_max = 0;
-  size_t need = 0;
-  auto used = [&](int l) { return l < L - 1 || net->layers[l].zy_off >= 0; };
+  int planes = 0, k_max = net->n_in_pad;
+  size_t need = 0, cv = 0;
+  const int seeds = (net->S_max + 15) / 16 * 16;
   for (int l = 0; l < L; ++l) {
     LayerDev& Ly = net->layers[l];
-    if (!used(l)) continue;
     if (Ly.zy_off >= 0) Ly.h_plane = planes++;
-    mp_max = std::max(mp_max, Ly.mp);
-    if (l > 0) need += (size_t)Ly.mp * Ly.kp * 2 * kRnsMax;
+    k_max = std::max(k_max, Ly.mp);
+    need += (size_t)Ly.mp * Ly.kp * 2 * kRnsMax;
+    cv = std::max(cv, (size_t)((Ly.mp + 1023) / 1024) * kRnsMax * seeds * Ly.kp);
   }
   net->h_planes = planes;
-  net->zs_ld = mp_max + kPad;
+  net->zs_ld = k_max + kPad;
   net->u_ld = net->n_in_pad;
-  const size_t row_elems = (size_t)n * net->zs_ld;
-  need += row_elems * (kRnsMax * 7 + 16) + (size_t)planes * kRnsMax * n * net->u_ld;
+  net->rset = rns_set(net->zs_ld);
+  const size_t row_elems = (size_t)n * net->zs_ld, rs = net->rset.n;
+  need += row_elems * (kRnsMax * 7 + 16) + (size_t)planes * kRnsMax * n * net->u_ld + cv +
+          (size_t)seeds * k_max * (8 + 2 * kRnsMax);
   size_t free_b = 0, total_b = 0;
   CK(cudaMemGetInfo(&free_b, &total_b));
-  if (planes > kRnsMaxLayers || need > free_b / 2) return NNC_OK;
+  if (need > free_b / 2) return NNC_OK;
   net->rns = true;
+  unsigned char* p;
   AL(net->c64, std::max(net->K_total, kPad));
   AL(net->rc64, std::max(net->K_total, kPad));
-  if (planes == 0) return NNC_OK;
-  unsigned char* p;
-  AL(net->Z1, (size_t)n * (net->layers[0].mp + kPad));
-  AL(net->Zs, row_elems);
-  AL(p, row_elems * 2 * kRnsMax);
-  net->Rt = p;
-  AL(p, row_elems * 2 * kRnsMax);
-  net->Ra = p;
-  AL(p, row_elems * 2 * kRnsMax);
-  net->Rb = p;
-  AL(net->Rc, row_elems * kRnsMax);
-  AL(net->Ru, (size_t)planes * kRnsMax * n * net->u_ld);
-  AL(net->rt_scale, n);
-  AL(net->ru_scale, (size_t)planes * n);
+  AL(net->Zv, (size_t)seeds * k_max);
+  AL(p, (size_t)seeds * k_max * 2 * rs);
+  net->Zr = p;
+  AL(net->zr_scale, 96);
+  AL_RAW(net->Cv, cv);
+  if (planes > 0) {
+    AL(net->Z1, (size_t)n * (net->layers[0].mp + kPad));
+    AL(net->Zs, row_elems);
+    AL_RAW(p, row_elems * 2 * rs);
+    net->Rt = p;
+    AL_RAW(p, row_elems * 2 * rs);
+    net->Ra = p;
+    AL_RAW(p, row_elems * 2 * rs);
+    net->Rb = p;
+    AL_RAW(net->Rc, row_elems * rs);
+    AL_RAW(net->Ru, (size_t)planes * kRnsMax * n * net->u_ld);
+    AL(net->rt_scale, n);
+    AL(net->ru_scale, (size_t)planes * n);
+    LayerDev& L1 = net->layers[0];
+    CK(launch_transpose_f64(L1.W64, L1.kp, L1.mp, n, net->Z1, L1.mp + kPad, net->stream));
+  }
   for (int l = 0; l < L; ++l) {
     LayerDev& Ly = net->layers[l];
-    if (!used(l)) break;
     if (Ly.zy_off >= 0) Ly.c = net->c64 + Ly.zy_off;
-    const int ko = Ly.mp + (l == L - 1 && net->softmax ? kPad : 0);
-    Ly.set_in = rns_set(Ly.kp);
-    Ly.set_out = rns_set(ko);
-    int r = NNC_OK;
-    if (l > 0) {
-      AL(p, (size_t)Ly.set_in.n * Ly.mp * Ly.kp * 2);
-      Ly.Wr = p;
-      AL(Ly.wr_scale, Ly.mp);
-      CK(rns_pack_weights(Ly.set_in, Ly.W64, Ly.mp, Ly.kp, Ly.Wr, Ly.wr_scale, net->stream));
-      r = rns_plan(Ly.plan_rt, Ly.Wr, Ly.mp, net->Rt, n, Ly.mp, n, Ly.kp, Ly.set_in.n, false);
-    } else {
-      CK(launch_transpose_f64(Ly.W64, Ly.kp, Ly.mp, n, net->Z1, Ly.mp + kPad, net->stream));
-    }
+    AL_RAW(p, rs * Ly.mp * Ly.kp * 2);
+    Ly.Wr = p;
+    AL(Ly.wr_scale, Ly.mp);
+    CK(rns_pack_weights(net->rset, Ly.W64, Ly.mp, Ly.kp, Ly.Wr, Ly.wr_scale, net->stream));
+    int r = rns_plan_rev(Ly.plan_rr, Ly.Wr, Ly.mp, Ly.kp, net->Zr, net->S_max, net->rset.n);
+    if (r == NNC_OK && planes > 0 && l > 0)
+      r = rns_plan(Ly.plan_rt, Ly.Wr, Ly.mp, net->Rt, n, Ly.mp, n, Ly.kp, net->rset.n, false);
     if (r == NNC_OK && Ly.zy_off >= 0)
-      r = rns_plan(Ly.plan_rs, net->Ra, n, net->Rb, n, n, n, ko, Ly.set_out.n, true);
+      r = rns_plan(Ly.plan_rs, net->Ra, n, net->Rb, n, n, n,
+                   Ly.mp + (l == L - 1 && net->softmax ? kPad : 0), net->rset.n, true);
     if (r != NNC_OK) return fail(r, "plan of the residue products failed");
   }
   return NNC_OK;

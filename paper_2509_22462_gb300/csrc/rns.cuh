@@ -23,7 +23,7 @@ RnsSet rns_set(int K);
 
 struct RnsPlan {
   CUtensorMap ta, tb;
-  int M = 0, N = 0, nkb = 0, bn = 0, lower = 0, a_rows = 0, b_rows = 0;
+  int M = 0, N = 0, nkb = 0, bn = 0, lower = 0, rev = 0, a_rows = 0, b_rows = 0;
   bool ready = false;
 };
 // D = A B^T for every residue: A [set.n][a_rows][K] and B [set.n][b_rows][K] (BF16 integers, K-major,
@@ -56,7 +56,28 @@ struct RnsRows {
   void *Sa = nullptr, *Sb = nullptr;   // residues of rc Z (q folded in) and sign(c) rc Z, or NULL
   double* ss = nullptr;         // their row scales [n]
 };
-cudaError_t rns_rows(const RnsSet& in, const RnsSet& out, const RnsRows& a, cudaStream_t st);
+cudaError_t rns_rows(const RnsSet& s, const RnsRows& a, cudaStream_t st);
+
+// One step between two reverse products: seeds s < S, K columns (the output layer's rows, or the
+// columns of the layer just multiplied, padded).
+struct RnsRev {
+  const unsigned char* C = nullptr;   // planes of rns_gemm on an rns_plan_rev plan, or NULL: seeds
+  int chunks = 0, seeds = 0;          // seeds: rows of a plane (S rounded up to 16)
+  const double* sb = nullptr;         // scales of the seeds that were multiplied [S]
+  int K = 0, kvalid = 0, nJ = 0, lam_col = -1;
+  const double *s1 = nullptr, *s2 = nullptr;   // of the layer that owns the K columns; NULL: x
+  const double *lam = nullptr, *soft_p = nullptr;   // seeds (out_seed)
+  const double* sa = nullptr;         // that layer's row scales of W
+  double* c_out = nullptr;            // its curvature weights (lambda column)
+  double *J = nullptr, *g = nullptr;  // x: J [nJ][kvalid], gradient (each may be NULL)
+  double* Zs = nullptr;               // scratch [S][K]
+  void* Zr = nullptr;                 // residues [n][seeds][K] of the scaled seeds
+  double* sb_out = nullptr;           // their scales [S]
+};
+cudaError_t rns_rev_rows(const RnsSet& s, const RnsRev& a, int S, cudaStream_t st);
+// Product W^T Z over the mp rows of the residues W [n][mp][kp], Z [n][seeds rounded up to 16][mp].
+// rns_gemm then writes C[chunk][i][seed][k] (rows of kp bytes), chunks = rows / 1024 rounded up.
+int rns_plan_rev(RnsPlan& p, const void* W, int mp, int kp, const void* Z, int seeds, int n_mod);
 
 // rc = sqrt|c| (k entries)
 cudaError_t rns_curv(const double* c, double* rc, int k, cudaStream_t st);
@@ -66,9 +87,8 @@ cudaError_t rns_softmax_ext(int n, int m, int col, const double* p, const double
                             int ldz, double* c, double* rc, cudaStream_t st);
 
 // H[i][j] = H[j][i] = sum_l ss_l[i] ss_l[j] D_l[i][j] over `layers` residue planes
-// U [layers][kRnsMax][n][ldu] (entry [j][i], i >= j), ss [layers][n], sets[l] the system of plane l.
-constexpr int kRnsMaxLayers = 64;
-cudaError_t rns_h_finish(const RnsSet* sets, int layers, const unsigned char* U, int ldu,
+// U [layers][kRnsMax][n][ldu] (entry [j][i], i >= j), ss [layers][n].
+cudaError_t rns_h_finish(const RnsSet& s, int layers, const unsigned char* U, int ldu,
                          const double* ss, int n, double* H, cudaStream_t st);
 
 }  // namespace nnc

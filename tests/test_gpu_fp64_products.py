@@ -1,7 +1,7 @@
 """The FP64 form's residue products (csrc/k_rns.cu) against the FP64 oracle at the sizes where they
-change shape: the edges of tiles and column blocks, 16 and 15 moduli (K <= 1024 and above), one and
-several exact accumulations of 1024 terms, softmax columns, and the CUDA-core products that stay for
-nets of more than 64 curved layers.
+change shape: the edges of tiles and column blocks, 16 and 15 moduli, one and several exact
+accumulations of 1024 terms, 16, 32 and 48 seed columns, softmax columns, and the CUDA-core products
+that stay where the residues do not fit in memory.
 
 Tolerance (relative Frobenius).  Every row of an operand is rounded to 52 bits or more of its largest
 entry, so a product is off by at most 2 * 2^-52 * t of its terms' size, t = largest / rms entry of a
@@ -56,6 +56,7 @@ NETS = [
     ([209, 127, 384, 15], ["gelu", "identity", "softmax"]),
     ([257, 1023, 1025, 2], ["tanh", "tanh", "identity"]),
     ([40, 2049, 1152, 47], ["sigmoid", "tanh", "softmax"]),
+    ([1025, 200, 16], ["tanh", "identity"]),
     ([130, 33], ["softmax"]),
     ([12, 7], ["tanh"]),
     ([5] + [8] * 66 + [2], ["tanh"] * 66 + ["identity"]),
@@ -92,6 +93,21 @@ def test_row_scales(lib):
     Hs = net.hessian_lag(x / s, lam)
     net.free()
     assert np.array_equal(Hs / np.outer(s, s), H)   # powers of two: not one bit differs
+
+
+def test_no_room_for_residues(lib):
+    """With little free memory the net keeps the CUDA-core products."""
+    import torch
+    mlp = make_mlp(MLPSpec([300, 140, 130, 3], ["tanh", "gelu", "softmax"]), seed=5, tag="rns-room")
+    torch.cuda.empty_cache()
+    free = torch.cuda.mem_get_info()[0]
+    hold = torch.empty(free - (48 << 20), dtype=torch.uint8, device="cuda")   # residues need 31 of 24
+    try:
+        check(lib, mlp, 5)
+    finally:
+        del hold
+        torch.cuda.empty_cache()
+    check(lib, mlp, 5)
 
 
 def test_nan_weight(lib):
