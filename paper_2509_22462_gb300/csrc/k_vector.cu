@@ -674,85 +674,70 @@ cudaError_t launch_first_tangent(Elem e, const void* W1, int ldw, int m_pad, int
 }
 
 // ------------------------------------------------------------------ Hessian finish
-// H[i][j] = sum_s Hp[s][max(i,j)][min(i,j)]: the split partial sums hold the lower triangle; a
-// 32 x 32 tile of H and its mirror tile are read coalesced and written coalesced.
-template <typename TP>
-__global__ void k_h_finish(const TP* __restrict__ Hp, int splits, int n, int ldp,
-                           double* __restrict__ H) {
-  __shared__ double t[32][33];
-  const int bi = blockIdx.y, bj = blockIdx.x;   // tile row / column of H
-  const int i0 = bi * 32, j0 = bj * 32;
-  // source tile: lower-triangle storage of block (max, min)
-  const int r0 = bi >= bj ? i0 : j0, c0 = bi >= bj ? j0 : i0;
-  for (int rr = threadIdx.y; rr < 32; rr += blockDim.y) {
-    const int r = r0 + rr, c = c0 + threadIdx.x;
-    double v = 0.0;
-    if (r < n && c < n) {
-      const int R = r >= c ? r : c, C = r >= c ? c : r;
-#pragma unroll 4
-      for (int s = 0; s < splits; ++s) v += (double)Hp[((size_t)s * n + R) * ldp + C];
-    }
-    t[rr][threadIdx.x] = v;
-  }
-  __syncthreads();
-  for (int rr = threadIdx.y; rr < 32; rr += blockDim.y) {
-    const int i = i0 + rr, j = j0 + threadIdx.x;
-    if (i < n && j < n) H[(size_t)i * n + j] = bi >= bj ? t[rr][threadIdx.x] : t[threadIdx.x][rr];
-  }
-}
-
-// FP32 partials (tensor-core forms): one block of 32 x 8 threads per lower 32 x 32 tile (bi >= bj)
-// sums the splits in FP32 (GB300's FP64 rate is a small fraction of FP32's; the partials carry
-// FP32 accuracy anyway), four rows per thread with every split's load issued before the adds,
-// then writes the tile and its mirror, each coalesced.  Only R >= C entries of the partials are
-// read (the upper triangle of a diagonal tile is not written by the product).
-__global__ void __launch_bounds__(256) k_h_finish_f32(const float* __restrict__ Hp, int splits,
-                                                      int n, int ldp, double* __restrict__ H) {
-  __shared__ float t[32][33];
-  int b = blockIdx.x, bi = 0;
+// H[i][j] = sum_s Hp[s][max(i,j)][min(i,j)]: the split partial sums hold the lower triangle.
+// Blocks of 32 x 8 threads, R rows per thread, 4 / R blocks per lower 32 x 32 tile (bi >= bj), sum the
+// splits in order in the partials' type (GB300's FP64 rate is a small fraction of FP32's; FP32 partials
+// carry FP32 accuracy anyway), 16 or 32 loads in flight, then write their rows of the tile and of its
+// mirror, each coalesced.  Only R >= C entries of the partials are read (the upper triangle of a diagonal
+// tile is not written by the product).
+// R = 4 for up to 16 splits.  Few inputs leave few tiles and many splits, where the loads' latency is
+// the time: n = 117, 107 splits took 52 us with R = 4 and one split's four loads in flight on 10 CTAs, 23
+// so.  FP64 partials of n = 784, 11 splits: 21 us when every tile of the full square was summed.
+template <typename TP, int R>
+__global__ void __launch_bounds__(256) k_h_finish(const TP* __restrict__ Hp, int splits, int n, int ldp,
+                                                  double* __restrict__ H) {
+  __shared__ TP t[8 * R][33];
+  int b = blockIdx.x / (4 / R), bi = 0;
+  const int sub = blockIdx.x % (4 / R) * 8 * R;   // first row of this block in the tile
   while (b > bi) b -= ++bi;          // lower-tile index -> (bi, bj), bj = b <= bi
   const int bj = b;
-  const int i0 = bi * 32, j0 = bj * 32, x = threadIdx.x, y = threadIdx.y;
+  const int i0 = bi * 32 + sub, j0 = bj * 32, x = threadIdx.x, y = threadIdx.y;
   const size_t plane = (size_t)n * ldp;
-  const float* p[4];
-  bool in[4];
-  float v[4];
+  const TP* p[R];
+  bool in[R];
+  TP v[R];
 #pragma unroll
-  for (int k = 0; k < 4; ++k) {
+  for (int k = 0; k < R; ++k) {
     const int r = i0 + y + 8 * k, c = j0 + x;
     in[k] = r < n && c < n;
-    const int R = r >= c ? r : c, C = r >= c ? c : r;
-    p[k] = Hp + (size_t)R * ldp + C;
-    v[k] = 0.f;
+    const int Rr = r >= c ? r : c, C = r >= c ? c : r;
+    p[k] = Hp + (size_t)Rr * ldp + C;
+    v[k] = TP(0);
   }
-  for (int s = 0; s < splits; ++s)
+  constexpr int U = R == 1 ? 32 : 4;
+  for (int s = 0; s < splits; s += U) {
+    TP q[U][R];
 #pragma unroll
-    for (int k = 0; k < 4; ++k)
-      if (in[k]) v[k] += __ldg(p[k] + s * plane);
+    for (int u = 0; u < U; ++u)
 #pragma unroll
-  for (int k = 0; k < 4; ++k) t[y + 8 * k][x] = v[k];
+      for (int k = 0; k < R; ++k) q[u][k] = in[k] && s + u < splits ? __ldg(p[k] + (s + u) * plane) : TP(0);
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+#pragma unroll
+      for (int k = 0; k < R; ++k)
+        if (s + u < splits) v[k] += q[u][k];
+  }
+#pragma unroll
+  for (int k = 0; k < R; ++k) {
+    t[y + 8 * k][x] = v[k];
+    if (in[k]) H[(size_t)(i0 + y + 8 * k) * n + j0 + x] = (double)v[k];
+  }
+  if (bi == bj) return;
   __syncthreads();
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    const int rr = y + 8 * k;
-    const int i = i0 + rr, j = j0 + x;
-    if (i < n && j < n) H[(size_t)i * n + j] = (double)t[rr][x];
-    if (bi != bj) {
-      const int i2 = j0 + rr, j2 = i0 + x;   // mirror tile H[j0..][i0..]
-      if (i2 < n && j2 < n) H[(size_t)i2 * n + j2] = (double)t[x][rr];
-    }
+  // mirror: rows j0 .. j0 + 31, columns i0 .. i0 + 8 R - 1
+  for (int e = y * 32 + x; e < 32 * 8 * R; e += 256) {
+    const int jj = e / (8 * R), ii = e % (8 * R);
+    if (i0 + ii < n) H[(size_t)(j0 + jj) * n + i0 + ii] = (double)t[ii][jj];
   }
 }
 
 cudaError_t launch_h_finish(bool part_f32, const void* Hp, int splits, int n, int ldp, double* H,
                             cudaStream_t st) {
-  const int T = (n + 31) / 32;
-  if (part_f32) {
-    k_h_finish_f32<<<T * (T + 1) / 2, dim3(32, 8), 0, st>>>((const float*)Hp, splits, n, ldp, H);
-  } else {
-    dim3 grid(T, T), block(32, 8);
-    k_h_finish<double><<<grid, block, 0, st>>>((const double*)Hp, splits, n, ldp, H);
-  }
+  const int T = (n + 31) / 32, tiles = T * (T + 1) / 2;
+  const dim3 block(32, 8);
+  if (!part_f32) k_h_finish<double, 4><<<tiles, block, 0, st>>>((const double*)Hp, splits, n, ldp, H);
+  else if (splits > 16) k_h_finish<float, 1><<<4 * tiles, block, 0, st>>>((const float*)Hp, splits, n, ldp, H);
+  else k_h_finish<float, 4><<<tiles, block, 0, st>>>((const float*)Hp, splits, n, ldp, H);
   note_launch();
   return cudaGetLastError();
 }
@@ -956,18 +941,33 @@ cudaError_t launch_rev_seed_t(int m, int S, int nJ, int lam_col, const double* s
 // Sum the split partials P[sp][k][0..bn) of W_l^T Zbar; then either the next seeds (transposed,
 // three BF16 parts: Zb[s][k] = s1[k] * Abar[k][s]) and c = s2 * Abar[:, lam_col], or, on the first
 // layer, J_out[s][k] (s < nJ) and g_out[k] (s = lam_col) for k < kvalid.
-__global__ void k_rev_reduce_t(const float* __restrict__ P, int splits, int kcols, int bn, int S,
-                               int kvalid, const double* __restrict__ s1,
-                               const double* __restrict__ s2, int lam_col, int nJ,
-                               __nv_bfloat16* __restrict__ z0, __nv_bfloat16* __restrict__ z1,
-                               __nv_bfloat16* __restrict__ z2, int ld, double* __restrict__ c_out,
-                               float* __restrict__ c_f,
-                               double* __restrict__ J_out, double* __restrict__ g_out) {
-  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= kcols * S) return;
+// Rows of blockDim.y threads share the splits of an output (FP64 sums, added up in order of the row).
+// One row for few splits; with few columns and many splits (the first layer of a net of few inputs: 128
+// columns, 128 splits) one row was latency, split after split on 19 CTAs, 34 us.
+__global__ void __launch_bounds__(256) k_rev_reduce_t(
+    const float* __restrict__ P, int splits, int kcols, int bn, int S, int kvalid,
+    const double* __restrict__ s1, const double* __restrict__ s2, int lam_col, int nJ,
+    __nv_bfloat16* __restrict__ z0, __nv_bfloat16* __restrict__ z1, __nv_bfloat16* __restrict__ z2, int ld,
+    double* __restrict__ c_out, float* __restrict__ c_f, double* __restrict__ J_out,
+    double* __restrict__ g_out) {
+  __shared__ double t[8][32];
+  const int idx = blockIdx.x * blockDim.x + threadIdx.x, rows = blockDim.y;
+  const bool in = idx < kcols * S;
   const int k = idx / S, s = idx % S;
   double v = 0.0;
-  for (int sp = 0; sp < splits; ++sp) v += (double)P[((size_t)sp * kcols + k) * bn + s];
+  if (in) {
+    const float* q = P + (size_t)k * bn + s;
+    const size_t plane = (size_t)kcols * bn;
+#pragma unroll 8
+    for (int sp = threadIdx.y; sp < splits; sp += rows) v += (double)q[sp * plane];
+  }
+  if (rows > 1) {   // blocks of 32 x 8
+    t[threadIdx.y][threadIdx.x] = v;
+    __syncthreads();
+    if (threadIdx.y > 0) return;
+    for (int r = 1; r < rows; ++r) v += t[r][threadIdx.x];
+  }
+  if (!in) return;
   if (s1) {
     __nv_bfloat16 a, b, c;
     split3_bf16(s1[k] * v, a, b, c);
@@ -992,9 +992,10 @@ cudaError_t launch_rev_reduce_t(const float* P, int splits, int kcols, int bn, i
   __nv_bfloat16* z0 = z ? (__nv_bfloat16*)z[0] : nullptr;
   __nv_bfloat16* z1 = z ? (__nv_bfloat16*)z[1] : nullptr;
   __nv_bfloat16* z2 = z ? (__nv_bfloat16*)z[2] : nullptr;
-  k_rev_reduce_t<<<(kcols * S + 255) / 256, 256, 0, st>>>(P, splits, kcols, bn, S, kvalid, s1, s2,
-                                                          lam_col, nJ, z0, z1, z2, ld, c_out, c_f,
-                                                          J_out, g_out);
+  const dim3 block = splits > 16 ? dim3(32, 8) : dim3(256, 1);
+  k_rev_reduce_t<<<(kcols * S + block.x - 1) / block.x, block, 0, st>>>(P, splits, kcols, bn, S, kvalid, s1, s2,
+                                                                        lam_col, nJ, z0, z1, z2, ld, c_out,
+                                                                        c_f, J_out, g_out);
   note_launch();
   return cudaGetLastError();
 }
