@@ -193,7 +193,6 @@ int batch_eval(nnc_batch* b, const double* x, const double* lam, double* y, doub
     BCK(cudaMemsetAsync(H, 0, sizeof(double) * b->h_sum, st));
     return NNC_OK;
   }
-  BCK(cudaMemsetAsync(b->Hp, 0, sizeof(float) * b->h_sum * b->plan_syrk.splits, st));
   BCK(tc_syrk_grouped(b->plan_syrk, b->n_work, b->d_work, b->d_gn, b->d_goff, b->d_hoff, b->h_sum,
                       b->Hp, b->dev_err, st));
   BCK(launch_bh_finish(b->Hp, b->plan_syrk.splits, b->h_sum, K, b->d_gn, b->d_hoff, H, st));

@@ -279,9 +279,9 @@ __global__ void k_bh_finish(const float* __restrict__ Hp, int splits, long long 
   const int g = blockIdx.y;
   const int n = gn[g];
   const long long base = hoff[g];
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < (long long)n * n;
-       e += (long long)gridDim.x * blockDim.x) {
-    const int i = (int)(e / n), j = (int)(e % n);
+  for (unsigned e = blockIdx.x * blockDim.x + threadIdx.x; e < (unsigned)(n * n);   // n <= 256
+       e += gridDim.x * blockDim.x) {
+    const int i = (int)(e / (unsigned)n), j = (int)(e % (unsigned)n);
     const int r = i > j ? i : j, cc = i > j ? j : i;
     double v = 0.0;
     for (int s = 0; s < splits; ++s) v += (double)Hp[s * ldh_split + base + (long long)r * n + cc];

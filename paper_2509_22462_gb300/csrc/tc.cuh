@@ -89,7 +89,7 @@ cudaError_t tc_plain(const PlainPlan& p, const float* bias, float* C, int ldc, b
 // part[split][k][0..bn) (FP32, bn = 16 or 48).
 cudaError_t tc_rev(const TcPlan& p, float* part, int* err, cudaStream_t st);
 
-// Hp: splits x N x N floats (row stride N); partial sums of the lower triangle are added.
+// Hp: splits x N x N floats (row stride N); partial sums of the lower triangle are written.
 cudaError_t tc_syrk(const TcPlan& p, float* Hp, int* err, cudaStream_t st);
 
 // Grouped forms for a batch of networks of equal hidden widths (stacked buffers): group g's
