@@ -1571,9 +1571,12 @@ int tc_plan_make(TcPlan& p, int kind, int prec, const void* a_hi, const void* a_
     const int cands[4] = {256, 208, 128, 112};
     const int ntm = M / BM;
     for (int bn : cands) {
-      // waves of full tiles; the narrow remainder tile counts as a full one
+      // waves of full tiles; the narrow remainder tile counts as a full one.  A tile takes its columns
+      // plus 60 (set-up, first copies, epilogue: 9 us at K = 4096), at least 188 (narrower MMAs are bound
+      // by reading A).  Evaluation, BF16, tiles of 112 / 128 / 208 / 256: 784 -> 8192 x 3 -> 10 670 / 669 /
+      // 599 / 627 us; 784 -> 4096 x 7 -> 10 578 / 572 / 496 / 506; 784 -> 1024 x 3 -> 10 119 / 119 / 122 / 122.
       const int ctas = ntm * ((N + bn - 1) / bn);
-      const double cost = (double)((ctas + sm_count - 1) / sm_count) * (bn + 24);
+      const double cost = (double)((ctas + sm_count - 1) / sm_count) * std::max(bn + 60, 188);
       if (cost < best - 1e-9) {
         best = cost;
         best_bn = bn;

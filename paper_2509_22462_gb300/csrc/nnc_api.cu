@@ -1014,16 +1014,21 @@ static int load_impl(nnc_net* net, int n_layers, const int* widths, const int* a
     for (int l = 1; l < n_layers; ++l) {
       LayerDev& Ly = net->layers[l];
       const int cur = (l - 1) % 2;
+      // split form, wide layers: SM pairs, each of which copies half of the tangent tile (784 -> 4096 x 7
+      // -> 10: 705 us against 717 with one SM per tile)
+      const bool pair = prec == NNC_BF16X3 && Ly.mp % 256 == 0 && Ly.mp >= 2048 && n > 256;
       int r = prec == NNC_FP8
                   ? tc_plan_make(Ly.plan_tan, TC_TANGENT, prec, Ly.W8, nullptr, Ly.mp, Ly.kp, net->A8,
                                  nullptr, n, Ly.kp, Ly.mp, n, Ly.kp, net->sm_count)
                   : tc_plan_make(Ly.plan_tan, TC_TANGENT, prec, Ly.Whi, Ly.Wlo, Ly.mp, Ly.kp,
                                  net->At[cur][0], net->At[cur][1], n, Ly.kp, Ly.mp, n, Ly.kp,
-                                 net->sm_count);
+                                 net->sm_count, pair ? -208 : 0);
       if (r != NNC_OK) return fail(r, "tensor-core tangent plan failed");
     }
     // the persistent chain: every tangent GEMM of an evaluation in one launch (not FP8, whose
-    // tangent operand is re-quantized between layers)
+    // tangent operand is re-quantized between layers).  Only where the caller or the autotuner asks for
+    // it: its resident CTAs keep the reverse sweep off the SMs (evaluation of 784 -> 4096 x 7 -> 10, BF16:
+    // 572 us against 496 us with one launch per layer; 784 -> 1024 x 3 -> 10: 127 against 122 us).
     if (prec == NNC_BF16 || prec == NNC_BF16X3) {
       int nl = 0;
       for (int l = 1; l < n_layers; ++l) {
@@ -1046,7 +1051,6 @@ static int load_impl(nnc_net* net, int n_layers, const int* widths, const int* a
           AL(cnt, (size_t)nl * net->chain_plans[0].ntn);
           net->chain_cnt = cnt;
           net->chain_nl = nl;
-          net->use_chain = true;
         } else {
           net->chain_plans.clear();
         }
