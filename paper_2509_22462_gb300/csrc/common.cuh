@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 #include <cuda_bf16.h>
 #include <cstdint>
+#include <utility>
 
 #include "../../include/nnc.h"
 
@@ -14,6 +15,26 @@ inline int pad_up(int v, int p = kPad) { return (v + p - 1) / p * p; }
 
 // Host-side launch counter (every kernel launch of the library goes through note_launch()).
 void note_launch(int n = 1);
+
+// Launch with programmatic dependent launch: the kernel may be scheduled while the one before it in the
+// stream still runs, and waits for its results itself (griddepcontrol.wait before its first access to
+// memory that another kernel writes).
+template <typename... P, typename... A>
+cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
+  note_launch();
+  return e != cudaSuccess ? e : cudaGetLastError();
+}
 
 // sigma, sigma' and sigma'' of Eq. 3's activations, in FP64.  The derivatives follow from
 // the definitions: tanh' = 1 - t^2, tanh'' = -2 t (1 - t^2); sigmoid' = s (1 - s),

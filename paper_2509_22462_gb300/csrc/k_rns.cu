@@ -20,9 +20,12 @@
 // K as a sum of FP64 products does.  Chosen over slicing into 8-bit digits, which needs 28 products
 // where this needs 15.  Rows holding a NaN or an infinity give NaN.
 //
+// Every kernel waits for the one before it itself (programmatic dependent launch): a small net's evaluation
+// is twenty short launches.
+//
 // Measured, residual + J + H + gradient at one iterate: 784 -> 4096 x 7 -> 10 181 -> 6.0 ms with the
-// Hessian's products and 4.1 ms with the reverse sweep's too (error of H against 64-bit sums 5.6e-15
-// -> 4.3e-15), 784 -> 128 x 2 -> 10 911 -> 313 -> 183 us (7.8e-16 both).
+// Hessian's products, 4.1 ms with the reverse sweep's too and 3.84 ms with the integer helpers below (error of
+// H against 64-bit sums 5.7e-15 -> 4.1e-15), 784 -> 128 x 2 -> 10 912 -> 313 -> 182 -> 125 us (8e-16 both).
 #include <cudaTypedefs.h>
 
 #include <algorithm>
@@ -71,16 +74,41 @@ __device__ __forceinline__ unsigned bf2(float a, float b) {
   return __byte_perm(__float_as_uint(a), __float_as_uint(b), 0x7632);
 }
 
-// Scale of a row whose largest high word of |v| is `hi`: |v| < 2^e.  *sc = 2^(bits - e) makes the
-// integers, the return value 2^(e - bits) undoes it (NaN for a row with a NaN or an infinity).
-__device__ __forceinline__ double rns_scale(int hi, int bits, double* sc) {
-  const int ex = hi >> 20;                       // biased exponent, sign bit cleared
+// Scale of a row whose values are below 2^(ex - 1022) in size (ex: biased exponent, 0x7FF for a row
+// with a NaN or an infinity).  *sh = bits - e makes the integers v 2^sh, the return value 2^-sh undoes it
+// (NaN for a row with a NaN or an infinity).
+__device__ __forceinline__ double rns_scale(int ex, int bits, int* sh) {
   const int e = max(ex - 1022, -900);
-  *sc = __hiloint2double((bits - e + 1023) << 20, 0);
+  *sh = bits - e;
   return ex == 0x7FF ? __longlong_as_double(0x7FF8000000000000ll)
                      : __hiloint2double((e - bits + 1023) << 20, 0);
 }
-__device__ __forceinline__ int abs_hi(double v) { return __double2hiint(v) & 0x7FFFFFFF; }
+__device__ __forceinline__ int expo(double v) { return (__double2hiint(v) >> 20) & 0x7FF; }
+
+// GB300 issues one FP64 instruction of a warp every 16 clocks of an SM; the helpers below do in a dozen
+// integer instructions (a clock or less each) what would be two or three FP64 ones per element.
+
+// Biased exponent that bounds |a b| < 2^(e - 1022) (0x7FF: a NaN, an infinity or an overflow): from the
+// top 21 bits of both mantissas, rounded up.
+__device__ __forceinline__ int prod_expo(double a, double b) {
+  const int ha = __double2hiint(a), hb = __double2hiint(b);
+  const int ea = (ha >> 20) & 0x7FF, eb = (hb >> 20) & 0x7FF;
+  const unsigned p = __umulhi(((unsigned)ha << 11) | 0x800007FFu, ((unsigned)hb << 11) | 0x800007FFu);
+  const int e = ea + eb - 1023 + (p >= 0x7FFFFFFCu ? 1 : 0);
+  return max(ea, eb) == 0x7FF ? 0x7FF : min(max(e, 0), 0x7FF);
+}
+// v 2^sh as an integer, to nearest; |v 2^sh| <= 2^60.
+__device__ __forceinline__ long long to_int(double v, int sh) {
+  const long long u = __double_as_longlong(v);
+  const int e = (int)(u >> 52) & 0x7FF;
+  const unsigned long long m = ((unsigned long long)u & 0xFFFFFFFFFFFFFull) | 0x10000000000000ull;
+  const int s = e - 1075 + sh;   // |v| 2^sh = m 2^s
+  const int t = min(max(-s, 0), 63);
+  const unsigned long long half = t > 0 ? 1ull << (t - 1) : 0ull;
+  unsigned long long r = s >= 0 ? m << min(s, 8) : (m + half) >> t;
+  if (e == 0) r = 0;
+  return u < 0 ? -(long long)r : (long long)r;
+}
 
 // 96-bit fixed-point value of D / P from the residues y_i (0 .. p_i - 1), as D 2^64 / P.
 struct Crt {
@@ -91,11 +119,26 @@ struct Crt {
     mid += (unsigned long long)y * s.c1[i];
     hi += y * s.c2[i];
   }
+  // rounded to nearest by hand: sign and size, 64 leading bits, 53 of them
   __device__ __forceinline__ double value() const {
     const unsigned long long m = mid + (lo >> 32);
     const unsigned h = hi + (unsigned)(m >> 32);
-    const long long top = (long long)(((unsigned long long)h << 32) | (unsigned)m);
-    return fma((double)(unsigned)lo, 2.3283064365386963e-10, (double)top);
+    unsigned long long t = ((unsigned long long)h << 32) | (unsigned)m;
+    unsigned l = (unsigned)lo;
+    const bool neg = (int)h < 0;
+    if (neg) {   // ones' complement: off by 2^-32 of a unit of t
+      t = ~t;
+      l = ~l;
+    }
+    if (t == 0) {   // below 2^-64 P
+      const double v = (double)l * 2.3283064365386963e-10;
+      return neg ? -v : v;
+    }
+    const int z = __clzll((long long)t);
+    t = z ? (t << z) | (((unsigned long long)l << 32) >> (64 - z)) : t;
+    t = (t >> 11) + ((t >> 10) & 1ull);   // 2^52 .. 2^53, times 2^(11 - z)
+    t += ((unsigned long long)(1085 - z)) << 52;
+    return __longlong_as_double((long long)(t | (neg ? 0x8000000000000000ull : 0ull)));
   }
 };
 
@@ -118,16 +161,14 @@ __global__ void __launch_bounds__(256) k_rns_pack(const __grid_constant__ RnsSet
   __shared__ int sh[8];
   const int r = blockIdx.x;
   const double* w = W + (size_t)r * kp;
-  int hi = 0;
-  for (int k = threadIdx.x; k < kp; k += blockDim.x) hi = max(hi, abs_hi(w[k]));
-  hi = block_max(hi, sh);
-  double sc;
-  const double back = rns_scale(hi, s.bits, &sc);
+  int ex = 0, sc;
+  for (int k = threadIdx.x; k < kp; k += blockDim.x) ex = max(ex, expo(w[k]));
+  const double back = rns_scale(block_max(ex, sh), s.bits, &sc);
   if (threadIdx.x == 0) sa[r] = back;
   for (int k = 4 * threadIdx.x; k < kp; k += 4 * blockDim.x) {
     Limbs l[4];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) l[j] = rns_limbs(__double2ll_rn(w[k + j] * sc));
+    for (int j = 0; j < 4; ++j) l[j] = rns_limbs(to_int(w[k + j], sc));
 #pragma unroll 4
     for (int i = 0; i < s.n; ++i) {
       float v[4];
@@ -144,13 +185,16 @@ __global__ void __launch_bounds__(256) k_rns_pack(const __grid_constant__ RnsSet
 // the row's largest |sigma' z| and |sqrt|c| z| give its scales, and the residues of both are written:
 // the operand of the next layer's product and the two operands of the symmetric product, which
 // takes sqrt|c| z on both sides (sign(c) on one) so that one scale per row fits every column.
-// Bound: 90 bytes written per element (15 residues x 3 operands), about 13 operations on the FP64 pipe.
+// Bound: 90 bytes written per element (15 residues x 3 operands) and about 450 instructions; four of them
+// on the FP64 pipe.
 template <bool CRT>
 __global__ void __launch_bounds__(256) k_rns_rows(const __grid_constant__ RnsSet set,
                                                   const RnsRows a) {
   __shared__ int sh[8];
   const int r = blockIdx.x;
   double* zrow = a.Z + (size_t)r * a.ldz;
+  griddep_wait();
+  griddep_launch();
   const double sb = CRT ? set.scale * a.sb[r] : 0.0;
   int ha = 0, hs = 0;
   for (int k = 4 * threadIdx.x; k < a.K; k += 4 * blockDim.x) {
@@ -177,12 +221,12 @@ __global__ void __launch_bounds__(256) k_rns_rows(const __grid_constant__ RnsSet
     }
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-      if (a.At) ha = max(ha, abs_hi(__ldg(a.s1 + k + j) * z[j]));
-      if (a.Sa) hs = max(hs, abs_hi(__ldg(a.rc + k + j) * z[j]));
+      if (a.At) ha = max(ha, prod_expo(__ldg(a.s1 + k + j), z[j]));
+      if (a.Sa) hs = max(hs, prod_expo(__ldg(a.rc + k + j), z[j]));
     }
   }
   if (!a.At && !a.Sa) return;
-  double sca, scs;
+  int sca, scs;
   ha = block_max(ha, sh);
   hs = block_max(hs, sh);
   const double ba = rns_scale(ha, set.bits, &sca), bs = rns_scale(hs, set.bits, &scs);
@@ -199,7 +243,7 @@ __global__ void __launch_bounds__(256) k_rns_rows(const __grid_constant__ RnsSet
     if (a.At) {
       Limbs l[4];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) l[j] = rns_limbs(__double2ll_rn(__ldg(a.s1 + k + j) * z[j] * sca));
+      for (int j = 0; j < 4; ++j) l[j] = rns_limbs(to_int(__ldg(a.s1 + k + j) * z[j], sca));
       __nv_bfloat16* dst = (__nv_bfloat16*)a.At + o;
 #pragma unroll 5
       for (int i = 0; i < set.n; ++i)
@@ -215,7 +259,7 @@ __global__ void __launch_bounds__(256) k_rns_rows(const __grid_constant__ RnsSet
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
           s4[j] = (unsigned)__double2hiint(__ldg(a.c + k + j)) & 0x80000000u;
-          l[j] = rns_limbs(__double2ll_rn(__ldg(a.rc + k + j) * z[j] * scs));
+          l[j] = rns_limbs(to_int(__ldg(a.rc + k + j) * z[j], scs));
         }
         neg0 = (s4[0] >> 16) | s4[1];
         neg1 = (s4[2] >> 16) | s4[3];
@@ -241,104 +285,102 @@ __global__ void __launch_bounds__(256) k_rns_rows(const __grid_constant__ RnsSet
 // One cluster of eight CTAs per seed column s: Abar[k][s] from the residue planes of W_l^T Zbar (or,
 // for the output layer, the seeds), then sigma' Abar of the layer below as residues, one scale per
 // seed (the row scales of that layer's weights are multiplied in, since its product sums over rows).
-// First layer: J and the gradient instead.  Eight SMs share a seed because its 4096 entries cost ten
-// operations each on the FP64 pipe, 10 us on one SM.
+// First layer: J and the gradient instead.  Bound: latency, so a thread has one column up to 4096, and
+// its loads, twenty at a time, are in flight together.
 constexpr int kRevCl = 8;
-__global__ void __launch_bounds__(256) k_rns_rev_rows(const __grid_constant__ RnsSet set,
+__global__ void __launch_bounds__(512) k_rns_rev_rows(const __grid_constant__ RnsSet set,
                                                       const RnsRev a) {
-  __shared__ int sh[8], mine;
+  __shared__ int sh[16], mine;
   const int s = blockIdx.y;
-  const int kb = blockIdx.x * 4 * blockDim.x, step = gridDim.x * 4 * blockDim.x;
+  const int k0 = blockIdx.x * blockDim.x + threadIdx.x, step = gridDim.x * blockDim.x;
   const bool is_lam = s == a.lam_col;
   double* zrow = a.Zs + (size_t)s * a.K;
-  int hi = 0;
-  for (int k = kb + 4 * threadIdx.x; k < a.K; k += step) {
-    double v[4];
+  griddep_wait();
+  griddep_launch();
+  int ex = 0;
+  double keep = 0.0;   // of column k0
+  for (int k = k0; k < a.K; k += step) {
+    double z;
     if (a.C) {
-      Crt t[4];
-      const double sb = set.scale * a.sb[s];
+      Crt t;
       const unsigned char* c = a.C + (size_t)s * a.K + k;
       const size_t plane = (size_t)a.seeds * a.K;
-#pragma unroll 3
-      for (int i = 0; i < set.n; ++i) {
-        float y[4] = {0.f, 0.f, 0.f, 0.f};
-        for (int ch = 0; ch < a.chunks; ++ch) {
-          const unsigned w = __ldg(reinterpret_cast<const unsigned*>(c + (size_t)(ch * set.n + i) * plane));
+      for (int i0 = 0; i0 < set.n; i0 += 5) {
+        unsigned y[5] = {0, 0, 0, 0, 0};
+        for (int c0 = 0; c0 < a.chunks; c0 += 4) {
+          unsigned q[5][4];
 #pragma unroll
-          for (int j = 0; j < 4; ++j) y[j] += __uint_as_float(0x4B000000u | ((w >> (8 * j)) & 0xFFu)) - 8388608.f;
+          for (int u = 0; u < 5; ++u)
+#pragma unroll
+            for (int w = 0; w < 4; ++w)
+              q[u][w] = i0 + u < set.n && c0 + w < a.chunks
+                            ? __ldg(c + (size_t)((c0 + w) * set.n + i0 + u) * plane) : 0u;
+#pragma unroll
+          for (int u = 0; u < 5; ++u) y[u] += q[u][0] + q[u][1] + q[u][2] + q[u][3];
         }
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          float r = rns_mod(y[j], set.p[i], set.pinv[i]);
-          r += r < 0.f ? set.p[i] : 0.f;
-          t[j].add(set, i, __float_as_uint(r + 8388608.f) & 0x1FFu);
+        for (int u = 0; u < 5; ++u) {
+          if (i0 + u < set.n) {
+            float r = rns_mod((float)y[u], set.p[i0 + u], set.pinv[i0 + u]);
+            r += r < 0.f ? set.p[i0 + u] : 0.f;
+            t.add(set, i0 + u, __float_as_uint(r + 8388608.f) & 0x1FFu);
+          }
         }
       }
-#pragma unroll
-      for (int j = 0; j < 4; ++j) v[j] = t[j].value() * sb;
-    }
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int kk = k + j;
-      double z;
-      if (a.C) {
-        if (a.s1) {
-          z = a.s1[kk] * v[j];
-          if (is_lam) {
-            const double cv = a.s2[kk] * v[j];
-            a.c_out[kk] = cv;
-          }
-        } else {
-          if (kk < a.kvalid) {
-            if (a.J && s < a.nJ) a.J[(size_t)s * a.kvalid + kk] = v[j];
-            if (a.g && is_lam) a.g[kk] = v[j];
-          }
-          continue;
+      const double v = t.value() * (set.scale * a.sb[s]);
+      if (!a.s1) {
+        if (k < a.kvalid) {
+          if (a.J && s < a.nJ) a.J[(size_t)s * a.kvalid + k] = v;
+          if (a.g && is_lam) a.g[k] = v;
         }
-      } else {
-        double cv = 0.0;
-        z = kk < a.kvalid ? out_seed(kk, s, a.kvalid, a.nJ, a.lam_col, a.s1, a.s2, a.lam, a.soft_p, &cv) : 0.0;
-        if (is_lam) a.c_out[kk] = cv;
+        continue;
       }
-      z *= a.sa[kk];
-      hi = max(hi, abs_hi(z));
-      zrow[kk] = z;
+      z = a.s1[k] * v;
+      if (is_lam) {
+        const double cv = a.s2[k] * v;
+        a.c_out[k] = cv;
+        if (a.rc_out) a.rc_out[k] = sqrt(fabs(cv));
+      }
+    } else {
+      double cv = 0.0;
+      z = k < a.kvalid ? out_seed(k, s, a.kvalid, a.nJ, a.lam_col, a.s1, a.s2, a.lam, a.soft_p, &cv) : 0.0;
+      if (is_lam) {
+        a.c_out[k] = cv;
+        if (a.rc_out) a.rc_out[k] = sqrt(fabs(cv));
+      }
     }
+    z *= a.sa[k];
+    ex = max(ex, expo(z));
+    if (k == k0) keep = z;
+    else zrow[k] = z;
   }
   if (a.C && !a.s1) return;   // the whole cluster: nothing is exchanged on the first layer
-  hi = block_max(hi, sh);
-  if (threadIdx.x == 0) mine = hi;
+  ex = block_max(ex, sh);
+  if (threadIdx.x == 0) mine = ex;
   __syncthreads();
   async::cluster_sync();
   for (int q = 0; q < kRevCl; ++q)
-    hi = max(hi, __float_as_int(async::ld_dsmem_f32(smem_u32(&mine), (uint32_t)q)));
+    ex = max(ex, __float_as_int(async::ld_dsmem_f32(smem_u32(&mine), (uint32_t)q)));
   async::cluster_sync();      // no CTA leaves while another still reads its shared memory
-  double sc;
-  const double back = rns_scale(hi, set.bits, &sc);
+  int sc;
+  const double back = rns_scale(ex, set.bits, &sc);
   if (blockIdx.x == 0 && threadIdx.x == 0) a.sb_out[s] = back;
-  for (int k = kb + 4 * threadIdx.x; k < a.K; k += step) {
-    Limbs l[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) l[j] = rns_limbs(__double2ll_rn(zrow[k + j] * sc));
+  for (int k = k0; k < a.K; k += step) {
+    const Limbs l = rns_limbs(to_int(k == k0 ? keep : zrow[k], sc));
     __nv_bfloat16* dst = (__nv_bfloat16*)a.Zr + (size_t)s * a.K + k;
     const size_t plane = (size_t)a.seeds * a.K;
 #pragma unroll 5
     for (int i = 0; i < set.n; ++i)
-      *reinterpret_cast<uint2*>(dst + i * plane) =
-          make_uint2(bf2(rns_res(set, i, l[0]), rns_res(set, i, l[1])),
-                     bf2(rns_res(set, i, l[2]), rns_res(set, i, l[3])));
+      dst[i * plane] = __ushort_as_bfloat16((unsigned short)(__float_as_uint(rns_res(set, i, l)) >> 16));
   }
-}
-
-__global__ void k_rns_curv(const double* __restrict__ c, double* __restrict__ rc, int k) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < k) rc[i] = sqrt(fabs(c[i]));
 }
 
 __global__ void k_rns_softmax_ext(int n, int m, int col, const double* __restrict__ p,
                                   const double* __restrict__ lam, double* __restrict__ Z, int ldz,
                                   double* __restrict__ c, double* __restrict__ rc) {
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
+  griddep_wait();
+  griddep_launch();
   if (j >= n) return;
   double lb = 0.0;
   for (int i = 0; i < m; ++i) lb += lam[i] * p[i];
@@ -369,6 +411,8 @@ __global__ void __launch_bounds__(256) k_rns_h(const __grid_constant__ RnsSet s,
                                                double* __restrict__ H) {
   __shared__ double t[8][129];
   const int i0 = blockIdx.x * 128, j0 = blockIdx.y * 8;
+  griddep_wait();
+  griddep_launch();
   if (i0 + 127 < j0) return;           // strictly above the diagonal
   const int x = threadIdx.x, y = threadIdx.y;
   const int i = i0 + 4 * x, j = j0 + y;
@@ -512,6 +556,8 @@ __global__ void __launch_bounds__(kGThreads, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
+  griddep_wait();     // the operands are written, and the last reader of C is done
+  griddep_launch();
 
   int issued = 0;  // producer only
   if (warp == 0) {
@@ -700,9 +746,7 @@ cudaError_t launch_gemm(const RnsPlan& p, const RnsGemm& g, int grid, cudaStream
     if (e != cudaSuccess) return e;
     attr = true;
   }
-  k_rns_gemm<BN, REV><<<grid, kGThreads, C::SMEM, st>>>(p.ta, p.tb, g);
-  note_launch();
-  return cudaGetLastError();
+  return launch_pdl(k_rns_gemm<BN, REV>, dim3(grid), dim3(kGThreads), C::SMEM, st, p.ta, p.tb, g);
 }
 
 }  // namespace
@@ -838,49 +882,40 @@ cudaError_t rns_pack_weights(const RnsSet& s, const double* W, int mp, int kp, v
 cudaError_t rns_rows(const RnsSet& s, const RnsRows& a, cudaStream_t st) {
   if (a.K % 128 || a.n < 1 || (a.ldz & 1)) return cudaErrorInvalidValue;
   const int threads = std::min(256, std::max(32, a.K / 4));
-  if (a.C) k_rns_rows<true><<<a.n, threads, 0, st>>>(s, a);
-  else k_rns_rows<false><<<a.n, threads, 0, st>>>(s, a);
-  note_launch();
-  return cudaGetLastError();
+  return a.C ? launch_pdl(k_rns_rows<true>, dim3(a.n), dim3(threads), 0, st, s, a)
+             : launch_pdl(k_rns_rows<false>, dim3(a.n), dim3(threads), 0, st, s, a);
 }
 
 cudaError_t rns_rev_rows(const RnsSet& s, const RnsRev& a, int S, cudaStream_t st) {
   if (a.K % 128 || S < 1 || S > a.seeds) return cudaErrorInvalidValue;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(kRevCl, S);
-  cfg.blockDim = dim3(std::min(256, std::max(32, (a.K / (4 * kRevCl) + 31) / 32 * 32)));
+  cfg.blockDim = dim3(std::min(512, std::max(32, (a.K / kRevCl + 31) / 32 * 32)));
   cfg.stream = st;
-  cudaLaunchAttribute at[1];
+  cudaLaunchAttribute at[2];
+  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[1].val.programmaticStreamSerializationAllowed = 1;
   at[0].id = cudaLaunchAttributeClusterDimension;
   at[0].val.clusterDim.x = kRevCl;
   at[0].val.clusterDim.y = 1;
   at[0].val.clusterDim.z = 1;
   cfg.attrs = at;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = 2;
   const cudaError_t e = cudaLaunchKernelEx(&cfg, k_rns_rev_rows, s, a);
   note_launch();
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 
-cudaError_t rns_curv(const double* c, double* rc, int k, cudaStream_t st) {
-  k_rns_curv<<<(k + 255) / 256, 256, 0, st>>>(c, rc, k);
-  note_launch();
-  return cudaGetLastError();
-}
-
 cudaError_t rns_softmax_ext(int n, int m, int col, const double* p, const double* lam, double* Z,
                             int ldz, double* c, double* rc, cudaStream_t st) {
-  k_rns_softmax_ext<<<(n + 127) / 128, 128, 0, st>>>(n, m, col, p, lam, Z, ldz, c, rc);
-  note_launch();
-  return cudaGetLastError();
+  return launch_pdl(k_rns_softmax_ext, dim3((n + 127) / 128), dim3(128), 0, st, n, m, col, p, lam, Z, ldz, c,
+                    rc);
 }
 
 cudaError_t rns_h_finish(const RnsSet& s, int layers, const unsigned char* U, int ldu,
                          const double* ss, int n, double* H, cudaStream_t st) {
   dim3 grid((n + 127) / 128, (n + 7) / 8);
-  k_rns_h<<<grid, dim3(32, 8), 0, st>>>(s, layers, U, ldu, ss, n, H);
-  note_launch();
-  return cudaGetLastError();
+  return launch_pdl(k_rns_h, grid, dim3(32, 8), 0, st, s, layers, U, ldu, ss, n, H);
 }
 
 }  // namespace nnc

@@ -9,38 +9,22 @@
 namespace nnc {
 
 // ------------------------------------------------------------------ forward value pass
-// One warp per output row.  FP32 weights are multiplied in FP32 with four independent
-// partial sums per lane (32 terms each for k = 4096), which are summed in FP64.
-template <typename TW>
-__global__ void __launch_bounds__(256) k_gemv_fwd(const TW* __restrict__ W, int ldw,
+// FP64 form: one warp per output row, eight rows to a CTA, whose activations one warp evaluates
+// together.  Bound: the FP64 pipe, on which an instruction takes as long for one lane as for 32 (16
+// clocks of an SM): 29 us of FMAs for 4096 x 4096, and the 100 instructions of an activation were half
+// as much again when every warp evaluated its own.
+__global__ void __launch_bounds__(256) k_gemv_fwd(const double* __restrict__ W, int ldw,
                                                   const double* __restrict__ bias,
-                                                  const void* __restrict__ a_in_v, int m, int k,
-                                                  int act, double* __restrict__ a_out,
-                                                  float* __restrict__ a_out_f,
-                                                  double* __restrict__ s1, double* __restrict__ s2) {
-  const int row = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  if (row >= m) return;
-  double acc;
-  if constexpr (std::is_same<TW, float>::value) {
-    // FP32 weights meet the FP32 copy of the activations (no FP64 conversions in the loop).
-    const float4* r4 = reinterpret_cast<const float4*>(W + (size_t)row * ldw);
-    const float4* a4 = reinterpret_cast<const float4*>(a_in_v);
-    const int nk4 = (k + 3) >> 2;
-    float p0 = 0.f, p1 = 0.f, p2 = 0.f, p3 = 0.f;
-#pragma unroll 8
-    for (int j = lane; j < nk4; j += 32) {
-      const float4 w = __ldg(r4 + j);
-      const float4 a = a4[j];
-      p0 = fmaf(w.x, a.x, p0);
-      p1 = fmaf(w.y, a.y, p1);
-      p2 = fmaf(w.z, a.z, p2);
-      p3 = fmaf(w.w, a.w, p3);
-    }
-    acc = ((double)p0 + (double)p1) + ((double)p2 + (double)p3);
-  } else {
+                                                  const double* __restrict__ a_in, int m, int k, int act,
+                                                  double* __restrict__ a_out, double* __restrict__ s1,
+                                                  double* __restrict__ s2) {
+  __shared__ double zs[8];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  int row = blockIdx.x * 8 + warp;
+  async::griddep_wait();
+  async::griddep_launch();
+  if (row < m) {
     const double2* r2 = reinterpret_cast<const double2*>(W + (size_t)row * ldw);
-    const double* a_in = reinterpret_cast<const double*>(a_in_v);
     const int nk2 = (k + 1) >> 1;
     double q0 = 0.0, q1 = 0.0;
 #pragma unroll 4
@@ -50,33 +34,24 @@ __global__ void __launch_bounds__(256) k_gemv_fwd(const TW* __restrict__ W, int 
       q0 = fma(w.x, a.x, q0);
       q1 = fma(w.y, a.y, q1);
     }
-    acc = q0 + q1;
+    const double acc = warp_sum(q0 + q1);
+    if (lane == 0) zs[warp] = acc;
   }
-  acc = warp_sum(acc);
-  if (lane == 0) {
-    const double z = acc + (bias ? bias[row] : 0.0);
+  __syncthreads();
+  row = blockIdx.x * 8 + threadIdx.x;
+  if (threadIdx.x < 8 && row < m) {
+    const double z = zs[threadIdx.x] + (bias ? bias[row] : 0.0);
     double a, d1, d2;
     act_eval(act, z, a, d1, d2);
     a_out[row] = a;
-    if (a_out_f) a_out_f[row] = (float)a;
     if (s1) s1[row] = d1;
     if (s2) s2[row] = d2;
   }
 }
 
-cudaError_t launch_gemv_fwd(bool fp64, const void* W, int ldw, const double* b, const void* a_in,
-                            int m, int k, int act, double* a_out, float* a_out_f, double* s1,
-                            double* s2, cudaStream_t st) {
-  const int threads = 256;
-  const int blocks = (m * 32 + threads - 1) / threads;
-  if (fp64)
-    k_gemv_fwd<double><<<blocks, threads, 0, st>>>((const double*)W, ldw, b, a_in, m, k, act, a_out,
-                                                   a_out_f, s1, s2);
-  else
-    k_gemv_fwd<float><<<blocks, threads, 0, st>>>((const float*)W, ldw, b, a_in, m, k, act, a_out,
-                                                  a_out_f, s1, s2);
-  note_launch();
-  return cudaGetLastError();
+cudaError_t launch_gemv_fwd(const double* W, int ldw, const double* b, const double* a_in, int m, int k,
+                            int act, double* a_out, double* s1, double* s2, cudaStream_t st) {
+  return launch_pdl(k_gemv_fwd, dim3((m + 7) / 8), dim3(256), 0, st, W, ldw, b, a_in, m, k, act, a_out, s1, s2);
 }
 
 // ------------------------------------------------------------------ reverse sweep
@@ -274,6 +249,8 @@ __device__ __forceinline__ void put_tan(TanBuf b, size_t i, float v) {
 // maximum subtracted before exp.  m <= 64; one warp.
 __global__ void k_softmax_head(int m, double* __restrict__ z) {
   const int lane = threadIdx.x;
+  async::griddep_wait();
+  async::griddep_launch();
   double v0 = lane < m ? z[lane] : -INFINITY, v1 = lane + 32 < m ? z[lane + 32] : -INFINITY;
   double mx = fmax(v0, v1);
   for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
@@ -285,9 +262,7 @@ __global__ void k_softmax_head(int m, double* __restrict__ z) {
 
 cudaError_t launch_softmax_head(int m, double* z, cudaStream_t st) {
   if (m > 64) return cudaErrorInvalidValue;
-  k_softmax_head<<<1, 32, 0, st>>>(m, z);
-  note_launch();
-  return cudaGetLastError();
+  return launch_pdl(k_softmax_head, dim3(1), dim3(32), 0, st, m, z);
 }
 
 // The softmax layer's curvature grad_z^2(lambda^T p) = diag(p (lambda - lambar)) + U C U^T with
@@ -744,17 +719,19 @@ cudaError_t launch_h_finish(bool part_f32, const void* Hp, int splits, int n, in
 
 __global__ void k_sub(const double* y, const double* a, double* r, int n) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  async::griddep_wait();
+  async::griddep_launch();
   if (i < n) r[i] = y[i] - a[i];
 }
 
 cudaError_t launch_sub(const double* y, const double* a, double* r, int n, cudaStream_t st) {
-  k_sub<<<(n + 255) / 256, 256, 0, st>>>(y, a, r, n);
-  note_launch();
-  return cudaGetLastError();
+  return launch_pdl(k_sub, dim3((n + 255) / 256), dim3(256), 0, st, y, a, r, n);
 }
 
 __global__ void k_copy_pad(const double* src, double* dst, float2* dst2, int n, int n_pad) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  async::griddep_wait();
+  async::griddep_launch();
   if (i < n_pad) {
     const double v = i < n ? src[i] : 0.0;
     dst[i] = v;
@@ -767,9 +744,7 @@ __global__ void k_copy_pad(const double* src, double* dst, float2* dst2, int n, 
 
 cudaError_t launch_copy_pad(const double* src, double* dst, void* dst2, int n, int n_pad,
                             cudaStream_t st) {
-  k_copy_pad<<<(n_pad + 255) / 256, 256, 0, st>>>(src, dst, (float2*)dst2, n, n_pad);
-  note_launch();
-  return cudaGetLastError();
+  return launch_pdl(k_copy_pad, dim3((n_pad + 255) / 256), dim3(256), 0, st, src, dst, (float2*)dst2, n, n_pad);
 }
 
 }  // namespace nnc

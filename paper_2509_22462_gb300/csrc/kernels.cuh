@@ -18,11 +18,10 @@ struct TanBuf {
 enum class Elem { F64, F32, BF16, BF16X3 };
 
 // ---- vector kernels (k_vector.cu)
-// Forward layer: z = W a_in + b, a_out = sigma(z), s1 = sigma'(z), s2 = sigma''(z).
-// a_in is double (fp64) or float (FP32 weights); a_out_f (may be NULL) receives a float copy.
-cudaError_t launch_gemv_fwd(bool fp64, const void* W, int ldw, const double* b, const void* a_in,
-                            int m, int k, int act, double* a_out, float* a_out_f, double* s1,
-                            double* s2, cudaStream_t st);
+// FP64 forward layer: z = W a_in + b, a_out = sigma(z), s1 = sigma'(z), s2 = sigma''(z) (each of the
+// last two may be NULL).
+cudaError_t launch_gemv_fwd(const double* W, int ldw, const double* b, const double* a_in, int m, int k,
+                            int act, double* a_out, double* s1, double* s2, cudaStream_t st);
 // Reverse layer with S seed columns: part[c][kk][s] = sum over row chunk c of W[r][kk] Zbar[r][s]
 // (part is double for FP64 weights, float for FP32 weights).
 cudaError_t launch_gemv_rev(bool fp64, const void* W, int ldw, int m, int kcols, const double* Zbar,

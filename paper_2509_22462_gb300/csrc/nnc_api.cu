@@ -166,8 +166,7 @@ int run_forward(nnc_net* net, bool fp64, cudaStream_t st, int l0 = 0, int l1 = -
     const double* a_in = net->x;
     for (auto& Ly : net->layers) {
       PROF(PK_FWD);
-      CK(launch_gemv_fwd(true, Ly.W64, Ly.kp, Ly.b, a_in, Ly.m, Ly.kp, Ly.act, Ly.a, nullptr, Ly.s1,
-                         Ly.s2, st));
+      CK(launch_gemv_fwd(Ly.W64, Ly.kp, Ly.b, a_in, Ly.m, Ly.kp, Ly.act, Ly.a, Ly.s1, Ly.s2, st));
       a_in = Ly.a;
     }
     if (net->softmax) CK(launch_softmax_head(net->n_out, net->layers.back().a, st));
@@ -198,8 +197,7 @@ int run_forward_fp64_values(nnc_net* net, const double* x, cudaStream_t st) {
     const double* a_in = net->xr;
     for (auto& Ly : net->layers) {
       PROF(PK_FWD);
-      CK(launch_gemv_fwd(true, Ly.W64, Ly.kp, Ly.b, a_in, Ly.m, Ly.kp, Ly.act, Ly.ra, nullptr,
-                         nullptr, nullptr, st));
+      CK(launch_gemv_fwd(Ly.W64, Ly.kp, Ly.b, a_in, Ly.m, Ly.kp, Ly.act, Ly.ra, nullptr, nullptr, st));
       a_in = Ly.ra;
     }
   } else {
@@ -242,7 +240,9 @@ int run_reverse(nnc_net* net, bool fp64, int nJ, bool with_lam, const double* la
     a.lam = lam;
     a.soft_p = soft_p;
     a.sa = Lo.wr_scale;
+    auto rc = [&](const LayerDev& Ly) { return Ly.zy_off >= 0 ? net->rc64 + Ly.zy_off : nullptr; };
     a.c_out = Lo.c;
+    a.rc_out = rc(Lo);
     a.sb_out = net->zr_scale;
     CK(rns_rev_rows(net->rset, a, S, st));
     for (int l = net->L - 1; l >= 0; --l) {
@@ -259,6 +259,7 @@ int run_reverse(nnc_net* net, bool fp64, int nJ, bool with_lam, const double* la
       a.s2 = l > 0 ? net->layers[l - 1].s2 : nullptr;
       a.sa = l > 0 ? net->layers[l - 1].wr_scale : nullptr;
       a.c_out = l > 0 ? net->layers[l - 1].c : nullptr;
+      a.rc_out = l > 0 ? rc(net->layers[l - 1]) : nullptr;
       a.J = l > 0 ? nullptr : J;
       a.g = l > 0 ? nullptr : g;
       CK(rns_rev_rows(net->rset, a, S, st));
@@ -481,7 +482,6 @@ int run_hessian_rns(nnc_net* net, const double* lam, double* H, cudaStream_t st)
     CK(cudaMemsetAsync(H, 0, sizeof(double) * n * n, st));
     return NNC_OK;
   }
-  CK(rns_curv(net->c64, net->rc64, net->K_total, st));
   for (int l = 0; l < net->L; ++l) {
     LayerDev& Ly = net->layers[l];
     const bool last = l == net->L - 1, soft = last && net->softmax;

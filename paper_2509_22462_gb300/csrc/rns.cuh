@@ -68,7 +68,7 @@ struct RnsRev {
   const double *s1 = nullptr, *s2 = nullptr;   // of the layer that owns the K columns; NULL: x
   const double *lam = nullptr, *soft_p = nullptr;   // seeds (out_seed)
   const double* sa = nullptr;         // that layer's row scales of W
-  double* c_out = nullptr;            // its curvature weights (lambda column)
+  double *c_out = nullptr, *rc_out = nullptr;   // its curvature weights c (lambda column), and sqrt|c| or NULL
   double *J = nullptr, *g = nullptr;  // x: J [nJ][kvalid], gradient (each may be NULL)
   double* Zs = nullptr;               // scratch [S][K]
   void* Zr = nullptr;                 // residues [n][seeds][K] of the scaled seeds
@@ -79,8 +79,6 @@ cudaError_t rns_rev_rows(const RnsSet& s, const RnsRev& a, int S, cudaStream_t s
 // rns_gemm then writes C[chunk][i][seed][k] (rows of kp bytes), chunks = rows / 1024 rounded up.
 int rns_plan_rev(RnsPlan& p, const void* W, int mp, int kp, const void* Z, int seeds, int n_mod);
 
-// rc = sqrt|c| (k entries)
-cudaError_t rns_curv(const double* c, double* rc, int k, cudaStream_t st);
 // The rank-two part of a softmax layer's curvature as two more columns m, m + 1 of its block:
 // Z[j][m + k] = w_k[j], c[m + k] = g'_k, rc likewise (see k_softmax_ext).
 cudaError_t rns_softmax_ext(int n, int m, int col, const double* p, const double* lam, double* Z,
