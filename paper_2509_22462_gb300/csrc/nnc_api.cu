@@ -588,7 +588,9 @@ int check_net(const nnc_net* net) {
 }
 
 // Host-pointer wrapper: copy inputs in, run, copy outputs out, wait.  An output in page-locked
-// memory is written there by the kernel that forms it (no device buffer, no transfer after it).
+// memory is written there by the kernel that forms it (no device buffer, no transfer after it).  So are
+// the outputs of a small net (up to 256 KB together), into the net's own pinned staging and from there to
+// the caller's pageable arrays: a transfer to pageable memory waits for the device each time.
 int host_call(nnc_net* net, const double* x, const double* lam, double* y, double* J, double* H,
               double* g, const double* yv = nullptr, double* rr = nullptr) {
   int r = check_net(net);
@@ -613,9 +615,27 @@ int host_call(nnc_net* net, const double* x, const double* lam, double* y, doubl
   const size_t n_copy = rr ? (size_t)(hy - hs) + net->n_out
                         : lam ? (size_t)(hl - hs) + net->n_out : (size_t)net->n_in;
   CK(cudaMemcpyAsync(net->xin, hs, sizeof(double) * n_copy, cudaMemcpyHostToDevice, st));
-  // each output: written in place if pinned, else through its device buffer and a copy
-  auto direct = [](double* h) { return h ? (double*)pinned_dev_ptr(h) : nullptr; };
-  double *y_d = direct(y), *J_d = direct(J), *H_d = direct(H), *g_d = direct(g), *r_d = direct(rr);
+  // each output: written in place if pinned, through the pinned staging if there is one, else through
+  // its device buffer and a copy
+  double* stage = net->h_out;
+  struct Back {
+    double* h;
+    const double* from;
+    size_t n;
+  } staged[5];
+  int n_staged = 0;
+  auto direct = [&](double* h, size_t n) -> double* {
+    if (!h) return nullptr;
+    double* d = (double*)pinned_dev_ptr(h);
+    if (d || !stage) return d;
+    d = net->h_out_dev + (stage - net->h_out);
+    staged[n_staged++] = Back{h, stage, n};
+    stage += n;
+    return d;
+  };
+  const size_t n_o = net->n_out, n_i = net->n_in;
+  double *y_d = direct(y, n_o), *J_d = direct(J, n_o * n_i), *H_d = direct(H, n_i * n_i),
+         *g_d = direct(g, n_i), *r_d = direct(rr, n_o);
   r = eval_all(net, net->xin, lam ? net->lam : nullptr, y_d ? y_d : y ? net->ydev : nullptr,
                J_d ? J_d : J ? net->Jdev : nullptr, H_d ? H_d : H ? net->Hdev : nullptr,
                g_d ? g_d : g ? net->gdev : nullptr, st, rr ? net->yres : nullptr,
@@ -630,7 +650,10 @@ int host_call(nnc_net* net, const double* x, const double* lam, double* y, doubl
   CK(back(J, J_d, net->Jdev, (size_t)net->n_out * net->n_in));
   CK(back(H, H_d, net->Hdev, (size_t)net->n_in * net->n_in));
   CK(back(g, g_d, net->gdev, net->n_in));
-  return sync_check(net, st);   // the error word of the bounded waits comes back with the outputs
+  r = sync_check(net, st);   // the error word of the bounded waits comes back with the outputs
+  for (int i = 0; i < n_staged && r == NNC_OK; ++i)
+    std::memcpy(staged[i].h, staged[i].from, sizeof(double) * staged[i].n);
+  return r;
 }
 
 }  // namespace
@@ -749,6 +772,7 @@ void nnc_free(nnc_net* net) {
   for (void* p : net->allocs) cudaFree(p);
   for (cudaEvent_t e : net->ev_pool) cudaEventDestroy(e);
   if (net->h_stage) cudaFreeHost(net->h_stage);
+  if (net->h_out) cudaFreeHost(net->h_out);
   if (net->side_stream) {
     cudaStreamSynchronize(net->side_stream);
     cudaStreamDestroy(net->side_stream);
@@ -1109,6 +1133,11 @@ static int load_impl(nnc_net* net, int n_layers, const int* widths, const int* a
   // pinned staging of the host calls: x [n_in_pad] | lambda [n_out] | y [n_out] | error word
   net->h_stage_elems = (size_t)net->n_in_pad + 2 * (size_t)net->n_out + 1;
   CK(cudaMallocHost(&net->h_stage, sizeof(double) * net->h_stage_elems));
+  const size_t n_out_all = (size_t)n * n + (size_t)(net->n_out + 1) * n + 2 * (size_t)net->n_out;
+  if (n_out_all * sizeof(double) <= 256 * 1024) {
+    CK(cudaMallocHost(&net->h_out, sizeof(double) * n_out_all));
+    CK(cudaHostGetDevicePointer((void**)&net->h_out_dev, net->h_out, 0));
+  }
   CK(cudaStreamSynchronize(net->stream));
   return NNC_OK;
 }
