@@ -1179,19 +1179,12 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_chain(const __grid_constant_
 // C = A B^T for the learned warm start's small dense layers (forward Z = X W^T, backward
 // dH = dZ W and dW = dZ^T X with transposed operand copies): one 128 x BN tile per CTA, the
 // producer / MMA / epilogue warps of k_tc_gemm, single BF16 product into an FP32 TMEM tile.
-// Epilogue: C[m][n] = acc + bias[n] for m < M, n < N (FP32, row stride ldc); with gelu also
-// Hf = GELU(C) (FP32), Hl = GELU(C) (BF16, row stride ldc) and, when Ht is given, the transposed
-// BF16 copy Ht[n][m] (row stride ldt), the operand layout of the next backward product.
+// Epilogue: C[m][n] = acc + bias[n] for m < M, n < N (FP32, row stride ldc).
 struct PlainArgs {
   int M, N, nkb, ntn;
   const float* bias;
   float* C;
   int ldc;
-  int gelu;
-  float* Hf;
-  __nv_bfloat16* Hl;
-  __nv_bfloat16* Ht;
-  int ldt;
   int* err;
 };
 
@@ -1292,17 +1285,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           for (int j = 0; j < 16; ++j) {
             const int n = n0 + c0 + j;
             if (n < args.N) {
-              const float z = v[j] + (args.bias ? args.bias[n] : 0.f);
-              const size_t o = (size_t)m * args.ldc + n;
-              args.C[o] = z;
-              if (args.gelu) {
-                double a, d1, d2;
-                act_eval(NNC_GELU, (double)z, a, d1, d2);
-                args.Hf[o] = (float)a;
-                const __nv_bfloat16 hb = __float2bfloat16_rn((float)a);
-                args.Hl[o] = hb;
-                if (args.Ht) args.Ht[(size_t)n * args.ldt + m] = hb;
-              }
+              args.C[(size_t)m * args.ldc + n] = v[j] + (args.bias ? args.bias[n] : 0.f);
             }
           }
         }
@@ -1686,8 +1669,10 @@ int tc_plain_plan(PlainPlan& p, const void* A, int a_rows, int lda, const void* 
   p.M = M;
   p.N = N;
   p.K = K;
-  p.bn = N <= 128 ? 128 : 256;
   p.ntm = (M + BM - 1) / BM;
+  // small products are bound by latency, most of it one CTA's epilogue: 32-column tiles while they fit
+  // the chip in one wave
+  p.bn = p.ntm * ((N + 31) / 32) <= 152 ? 32 : N <= 128 ? 128 : 256;
   p.ntn = (N + p.bn - 1) / p.bn;
   if (!make_map(&p.ta, A, a_rows, K, lda, BM, 64) || !make_map(&p.tb, B, b_rows, K, ldb, p.bn, 64))
     return NNC_ERR_CUDA;
@@ -1709,12 +1694,13 @@ cudaError_t launch_plain_t(const PlainPlan& p, const PlainArgs& a, cudaStream_t 
   return cudaGetLastError();
 }
 
-cudaError_t tc_plain(const PlainPlan& p, const float* bias, float* Cout, int ldc, bool gelu, float* Hf,
-                     void* Hl, void* Ht, int ldt, int* err, cudaStream_t st) {
-  if (!p.ready || !Cout || (gelu && (!Hf || !Hl))) return cudaErrorInvalidValue;
-  PlainArgs a{p.M, p.N, p.K / 64, p.ntn, bias, Cout, ldc, gelu ? 1 : 0, Hf, (__nv_bfloat16*)Hl,
-              (__nv_bfloat16*)Ht, ldt, err};
-  return p.bn == 128 ? launch_plain_t<128>(p, a, st) : launch_plain_t<256>(p, a, st);
+cudaError_t tc_plain(const PlainPlan& p, const float* bias, float* Cout, int ldc, int* err,
+                     cudaStream_t st) {
+  if (!p.ready || !Cout) return cudaErrorInvalidValue;
+  PlainArgs a{p.M, p.N, p.K / 64, p.ntn, bias, Cout, ldc, err};
+  return p.bn == 32    ? launch_plain_t<32>(p, a, st)
+         : p.bn == 128 ? launch_plain_t<128>(p, a, st)
+                       : launch_plain_t<256>(p, a, st);
 }
 
 template <int BN, int MODE>

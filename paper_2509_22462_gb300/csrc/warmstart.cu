@@ -8,10 +8,8 @@
 //             dH_{l-1} = dZ_l W_l; dZ = dH * GELU'(Z)
 //   Adam      (Kingma & Ba) on FP32 master weights, FP32 moments, BF16 operand copies.
 // GEMMs: in the BF16 form the products run on the tcgen05 tensor cores (tc_plain: TMA-fed BF16
-// operands, FP32 accumulation in tensor memory, bias / GELU fused into the epilogue, which also
-// writes the transposed BF16 copy of each activation that the weight gradient dW = dZ^T H reads);
-// the backward products take transposed operand copies written by the loss, GELU-derivative and
-// Adam kernels.  Shapes the tensor cores cannot take (a batch that is not a multiple of 64 in the
+// operands, FP32 accumulation in tensor memory, bias added in the epilogue); the backward products
+// take transposed operand copies written by the GELU, loss, GELU-derivative and Adam kernels.  Shapes the tensor cores cannot take (a batch that is not a multiple of 64 in the
 // weight-gradient products, widths that are not multiples of 64) and the FP32 form use a
 // shared-memory tiled CUDA-core kernel.
 #include <algorithm>
@@ -41,166 +39,249 @@ __device__ __forceinline__ float ld(const T* p) {
   else return __bfloat162float(*p);
 }
 
+// One 32 x 32 tile per CTA, 2 x 2 outputs a thread, the next K slice in registers while this one is
+// multiplied.  Bound: latency (the products are small); 32 x 32 tiles give a 64 x 256 product 16 CTAs
+// where 64 x 64 tiles gave it 4.
 template <typename T>
 __global__ void __launch_bounds__(256) k_ws_gemm(const T* __restrict__ A, long sam, long sak,
                                                  const T* __restrict__ B, long sbk, long sbn, int M,
                                                  int N, int K, const float* __restrict__ bias,
-                                                 float* __restrict__ C, int ldc, int gelu,
-                                                 float* __restrict__ Hf, T* __restrict__ Hl,
-                                                 int accumulate) {
-  __shared__ float As[16][65];
-  __shared__ float Bs[16][65];
-  const int m0 = blockIdx.y * 64, n0 = blockIdx.x * 64;
+                                                 float* __restrict__ C, int ldc) {
+  __shared__ float As[32][33], Bs[32][33];
+  const int m0 = blockIdx.y * 32, n0 = blockIdx.x * 32;
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  float acc[4][4] = {};
-  for (int k0 = 0; k0 < K; k0 += 16) {
-    for (int i = threadIdx.x; i < 64 * 16; i += 256) {
-      const int r = i >> 4, kk = i & 15;
-      const int gm = m0 + r, gk = k0 + kk;
-      As[kk][r] = (gm < M && gk < K) ? ld(A + gm * sam + gk * sak) : 0.f;
-      const int gn = n0 + r;
-      Bs[kk][r] = (gn < N && gk < K) ? ld(B + gk * sbk + gn * sbn) : 0.f;
+  const int lo = threadIdx.x & 31, hi = threadIdx.x >> 5;   // neighbouring threads: neighbouring addresses
+  float ra[4], rb[4];
+  auto load = [&](int k0) {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int o = hi + 8 * j;
+      const int ak = k0 + (sak == 1 ? lo : o), am = m0 + (sak == 1 ? o : lo);
+      ra[j] = am < M && ak < K ? ld(A + am * sam + ak * sak) : 0.f;
+      const int bk = k0 + (sbk == 1 ? lo : o), bn = n0 + (sbk == 1 ? o : lo);
+      rb[j] = bn < N && bk < K ? ld(B + bk * sbk + bn * sbn) : 0.f;
+    }
+  };
+  float acc[2][2] = {};
+  load(0);
+  for (int k0 = 0; k0 < K; k0 += 32) {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int o = hi + 8 * j;
+      if (sak == 1) As[lo][o] = ra[j];
+      else As[o][lo] = ra[j];
+      if (sbk == 1) Bs[lo][o] = rb[j];
+      else Bs[o][lo] = rb[j];
     }
     __syncthreads();
+    if (k0 + 32 < K) load(k0 + 32);
 #pragma unroll
-    for (int kk = 0; kk < 16; ++kk) {
-      float a[4], b[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) a[i] = As[kk][tx + 16 * i];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) b[j] = Bs[kk][ty + 16 * j];
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
+    for (int kk = 0; kk < 32; ++kk) {
+      const float a0 = As[kk][tx], a1 = As[kk][tx + 16], b0 = Bs[kk][ty], b1 = Bs[kk][ty + 16];
+      acc[0][0] = fmaf(a0, b0, acc[0][0]);
+      acc[0][1] = fmaf(a0, b1, acc[0][1]);
+      acc[1][0] = fmaf(a1, b0, acc[1][0]);
+      acc[1][1] = fmaf(a1, b1, acc[1][1]);
     }
     __syncthreads();
   }
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
+  for (int i = 0; i < 2; ++i) {
     const int m = m0 + tx + 16 * i;
-    if (m >= M) continue;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
+    for (int j = 0; j < 2; ++j) {
       const int n = n0 + ty + 16 * j;
-      if (n >= N) continue;
-      float v = acc[i][j] + (bias ? bias[n] : 0.f);
-      const size_t o = (size_t)m * ldc + n;
-      if (accumulate) v += C[o];
-      C[o] = v;
-      if (gelu) {
-        double a, d1, d2;
-        act_eval(NNC_GELU, (double)v, a, d1, d2);
-        Hf[o] = (float)a;
-        if constexpr (std::is_same<T, float>::value) Hl[o] = (float)a;
-        else Hl[o] = __float2bfloat16_rn((float)a);
-      }
+      if (m < M && n < N) C[(size_t)m * ldc + n] = acc[i][j] + (bias ? bias[n] : 0.f);
     }
   }
 }
 
 template <typename T>
 void gemm(const T* A, long sam, long sak, const T* B, long sbk, long sbn, int M, int N, int K,
-          const float* bias, float* C, int ldc, bool gelu, float* Hf, T* Hl, cudaStream_t st) {
-  dim3 grid((N + 63) / 64, (M + 63) / 64);
-  k_ws_gemm<T><<<grid, 256, 0, st>>>(A, sam, sak, B, sbk, sbn, M, N, K, bias, C, ldc, gelu ? 1 : 0,
-                                     Hf, Hl, 0);
+          const float* bias, float* C, int ldc, cudaStream_t st) {
+  dim3 grid((N + 31) / 32, (M + 31) / 32);
+  k_ws_gemm<T><<<grid, 256, 0, st>>>(A, sam, sak, B, sbk, sbn, M, N, K, bias, C, ldc);
   note_launch();
 }
 
-// dZ = dH * GELU'(Z), stored in FP32 and in the operand type.
 template <typename T>
-__global__ void k_ws_gelu_back(const float* __restrict__ dH, const float* __restrict__ Z, int n,
-                               float* __restrict__ dZ, T* __restrict__ dZl, int cols,
-                               __nv_bfloat16* __restrict__ dZt, int ldt) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+__device__ __forceinline__ T to_op(float v) {
+  if constexpr (std::is_same<T, float>::value) return v;
+  else return __float2bfloat16_rn(v);
+}
+
+// H = GELU(Z) in the operand type (and, for the tensor-core backward products, its transposed copy) and
+// D1 = GELU'(Z).  Bound: the FP64 pipe, two FMAs per clock and SM, so the elements are spread over the
+// whole chip in CTAs of 64.  In the epilogue of the product the 64 x 256 values were one SM's work, and
+// with them a training step of 64 rows (512 -> 256 -> 256 -> 713) took 1.1 ms; now at most 0.1 ms.
+template <typename T>
+__global__ void __launch_bounds__(64) k_ws_gelu(const float* __restrict__ Z, int n, T* __restrict__ Hl,
+                                                float* __restrict__ D1, int cols,
+                                                __nv_bfloat16* __restrict__ Ht, int ldt) {
+  const int i = blockIdx.x * 64 + threadIdx.x;
   if (i >= n) return;
   double a, d1, d2;
   act_eval(NNC_GELU, (double)Z[i], a, d1, d2);
-  const float v = dH[i] * (float)d1;
-  dZ[i] = v;
-  if constexpr (std::is_same<T, float>::value) dZl[i] = v;
-  else dZl[i] = __float2bfloat16_rn(v);
-  if (dZt) dZt[(size_t)(i % cols) * ldt + i / cols] = __float2bfloat16_rn(v);   // transposed copy
+  const T h = to_op<T>((float)a);
+  Hl[i] = h;
+  D1[i] = (float)d1;
+  if constexpr (!std::is_same<T, float>::value)
+    if (Ht) Ht[(size_t)(i % cols) * ldt + i / cols] = h;
 }
 
-// dP = 2 (P - T) / (B n_out); loss partial sums per block into part[blockIdx.x].
+// Writes v of rows b .. b + 7 of one column of a transposed copy (16 bytes; ldt and b multiples of 8).
+__device__ __forceinline__ void put8(__nv_bfloat16* dst, const float (&v)[8]) {
+  __nv_bfloat162 h[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) h[j] = __floats2bfloat162_rn(v[2 * j], v[2 * j + 1]);
+  *reinterpret_cast<uint4*>(dst) = *reinterpret_cast<const uint4*>(h);
+}
+
+// dZ = dH * GELU'(Z) in the operand type and transposed, db[j] = sum_b dZ[b][j]: one thread per column,
+// rows in order, eight loads in flight.
 template <typename T>
-__global__ void k_ws_loss(const float* __restrict__ P, const float* __restrict__ Tt, int n,
-                          float scale, float* __restrict__ dP, T* __restrict__ dPl,
-                          double* __restrict__ part, int cols, __nv_bfloat16* __restrict__ dPp,
-                          int ldp, __nv_bfloat16* __restrict__ dPt, int ldt) {
-  __shared__ double red[256];
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  double s = 0.0;
-  if (i < n) {
-    const float d = P[i] - Tt[i];
-    s = (double)d * d;
-    const float g = 2.f * d * scale;
-    dP[i] = g;
-    if constexpr (std::is_same<T, float>::value) dPl[i] = g;
-    else dPl[i] = __float2bfloat16_rn(g);
-    // tensor-core operands: dP with its row stride padded to a multiple of 64 (the padding stays
-    // zero) and dP^T
-    const int r = i / cols, c = i % cols;
-    if (dPp) dPp[(size_t)r * ldp + c] = __float2bfloat16_rn(g);
-    if (dPt) dPt[(size_t)c * ldt + r] = __float2bfloat16_rn(g);
-  }
-  red[threadIdx.x] = s;
-  __syncthreads();
-  for (int o = 128; o > 0; o >>= 1) {
-    if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) part[blockIdx.x] = red[0];
-}
-
-// db[j] = sum_b dZ[b][j]
-__global__ void k_ws_colsum(const float* __restrict__ dZ, int B, int N, float* __restrict__ db) {
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= N) return;
+__global__ void __launch_bounds__(32) k_ws_gelu_back(const float* __restrict__ dH,
+                                                     const float* __restrict__ D1, int B, int cols,
+                                                     T* __restrict__ dZl, float* __restrict__ db,
+                                                     __nv_bfloat16* __restrict__ dZt, int ldt) {
+  const int j = blockIdx.x * 32 + threadIdx.x;
+  if (j >= cols) return;
   float s = 0.f;
-  for (int b = 0; b < B; ++b) s += dZ[(size_t)b * N + j];
+  for (int b0 = 0; b0 < B; b0 += 8) {
+    float v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const size_t o = (size_t)(b0 + u) * cols + j;
+      v[u] = b0 + u < B ? __fmul_rn(dH[o], D1[o]) : 0.f;   // rounded before it is summed
+    }
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      if (b0 + u < B) {
+        s += v[u];
+        dZl[(size_t)(b0 + u) * cols + j] = to_op<T>(v[u]);
+      }
+    }
+    if (dZt) put8(dZt + (size_t)j * ldt + b0, v);
+  }
   db[j] = s;
 }
 
-// Adam on one flat parameter array; refreshes the operand copy (and, for a weight matrix of
-// `cols` columns with wt given, its transposed BF16 copy, row stride ldt).
+// dP = 2 (P - T) / (B n_out) in the operand type and in the layouts of the tensor-core products (row
+// stride padded to a multiple of 64, the padding stays zero; transposed), its column sums db and the
+// loss's column sums part[j]: one thread per column as above.
 template <typename T>
-__global__ void k_ws_adam(float* __restrict__ w, const float* __restrict__ g, float* __restrict__ m,
-                          float* __restrict__ v, T* __restrict__ wl, int n, float lr, float b1,
-                          float b2, float eps, float c1, float c2, int cols,
-                          __nv_bfloat16* __restrict__ wt, int ldt) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const float gi = g[i];
-  const float mi = b1 * m[i] + (1.f - b1) * gi;
-  const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
-  m[i] = mi;
-  v[i] = vi;
-  const float wi = w[i] - lr * (mi / c1) / (sqrtf(vi / c2) + eps);
-  w[i] = wi;
-  if (wl) {
-    if constexpr (std::is_same<T, float>::value) wl[i] = wi;
-    else wl[i] = __float2bfloat16_rn(wi);
+__global__ void __launch_bounds__(32) k_ws_loss(const float* __restrict__ P, const float* __restrict__ Tt,
+                                                int B, int cols, float scale, T* __restrict__ dPl,
+                                                float* __restrict__ db, double* __restrict__ part,
+                                                __nv_bfloat16* __restrict__ dPp, int ldp,
+                                                __nv_bfloat16* __restrict__ dPt, int ldt) {
+  const int j = blockIdx.x * 32 + threadIdx.x;
+  if (j >= cols) return;
+  double l = 0.0;
+  float s = 0.f;
+  for (int b0 = 0; b0 < B; b0 += 8) {
+    float v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const size_t o = (size_t)(b0 + u) * cols + j;
+      v[u] = b0 + u < B ? P[o] - Tt[o] : 0.f;
+    }
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      l += (double)v[u] * v[u];
+      v[u] = __fmul_rn(2.f * v[u], scale);
+      if (b0 + u < B) {
+        s += v[u];
+        if (dPp) dPp[(size_t)(b0 + u) * ldp + j] = __float2bfloat16_rn(v[u]);
+        else dPl[(size_t)(b0 + u) * cols + j] = to_op<T>(v[u]);
+      }
+    }
+    if (dPt) put8(dPt + (size_t)j * ldt + b0, v);
   }
-  if (wt) wt[(size_t)(i % cols) * ldt + i / cols] = __float2bfloat16_rn(wi);
+  part[j] = l;
+  db[j] = s;
 }
 
+// Adam on the six parameter arrays in one launch; refreshes a weight matrix's operand copy wl and, with
+// wt given, its transposed BF16 copy (`cols` columns, row stride ldt).
+struct AdamSeg {
+  float *w, *m, *v;
+  const float* g;
+  void* wl;
+  __nv_bfloat16* wt;
+  int n, cols, ldt, blk0;   // blk0: the array's first block of 256 elements
+};
+struct AdamArgs {
+  AdamSeg a[6];
+  float lr, b1, b2, eps, c1, c2;
+};
 template <typename T>
-__global__ void k_ws_gather(const float* __restrict__ src, const int* __restrict__ idx, int rows,
-                            int cols, float* __restrict__ dst, T* __restrict__ dstl,
-                            __nv_bfloat16* __restrict__ dstt = nullptr, int ldt = 0) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= rows * cols) return;
-  const int r = i / cols, c = i % cols;
-  const float v = src[(size_t)idx[r] * cols + c];
-  if (dst) dst[i] = v;
-  if (dstl) {
-    if constexpr (std::is_same<T, float>::value) dstl[i] = v;
-    else dstl[i] = __float2bfloat16_rn(v);
+__global__ void __launch_bounds__(256) k_ws_adam(const __grid_constant__ AdamArgs p) {
+  int k = 5;
+  while ((int)blockIdx.x < p.a[k].blk0) --k;
+  const AdamSeg& q = p.a[k];
+  const int i = ((int)blockIdx.x - q.blk0) * 256 + threadIdx.x;
+  if (i >= q.n) return;
+  const float gi = q.g[i];
+  const float mi = fmaf(1.f - p.b1, gi, __fmul_rn(p.b1, q.m[i]));
+  const float vi = fmaf(__fmul_rn(1.f - p.b2, gi), gi, __fmul_rn(p.b2, q.v[i]));
+  q.m[i] = mi;
+  q.v[i] = vi;
+  const float wi = q.w[i] - p.lr * (mi / p.c1) / (sqrtf(vi / p.c2) + p.eps);
+  q.w[i] = wi;
+  if (q.wl) ((T*)q.wl)[i] = to_op<T>(wi);
+  if (q.wt) q.wt[(size_t)(i % q.cols) * q.ldt + i / q.cols] = __float2bfloat16_rn(wi);
+}
+
+// One batch: rows idx[0 .. B) of the standardized inputs (operand type, transposed copy) and targets.
+template <typename T>
+__global__ void __launch_bounds__(256) k_ws_gather(const float* __restrict__ Ud, const float* __restrict__ Td,
+                                                   const int* __restrict__ idx, int n_in, int n_out,
+                                                   T* __restrict__ Ul, __nv_bfloat16* __restrict__ Ut,
+                                                   int ldt, float* __restrict__ Tt) {
+  const int r = blockIdx.x, c = blockIdx.y * 256 + threadIdx.x;
+  const size_t row = idx[r];
+  if (c < n_in) {
+    const float v = Ud[row * n_in + c];
+    Ul[(size_t)r * n_in + c] = to_op<T>(v);
+    if (Ut) Ut[(size_t)c * ldt + r] = __float2bfloat16_rn(v);
+  } else if (c < n_in + n_out) {
+    Tt[(size_t)r * n_out + c - n_in] = Td[row * n_out + c - n_in];
   }
-  if (dstt) dstt[(size_t)c * ldt + r] = __float2bfloat16_rn(v);
+}
+
+// Mean and standard deviation of each column of X [N][cols], rows in order, 16 loads in flight.
+__global__ void __launch_bounds__(32) k_ws_stats(const double* __restrict__ X, int N, int cols,
+                                                 double* __restrict__ mean, double* __restrict__ sd) {
+  const int j = blockIdx.x * 32 + threadIdx.x;
+  if (j >= cols) return;
+  double mu = 0.0, sq = 0.0;
+#pragma unroll 1
+  for (int pass = 0; pass < 2; ++pass) {
+    for (int r0 = 0; r0 < N; r0 += 16) {
+      double v[16];
+#pragma unroll
+      for (int u = 0; u < 16; ++u) v[u] = r0 + u < N ? X[(size_t)(r0 + u) * cols + j] : 0.0;
+#pragma unroll
+      for (int u = 0; u < 16; ++u) {
+        if (r0 + u >= N) break;
+        if (pass == 0) mu += v[u];
+        else sq += (v[u] - mu) * (v[u] - mu);
+      }
+    }
+    if (pass == 0) mu /= N;
+  }
+  mean[j] = mu;
+  sd[j] = fmax(sqrt(sq / N), 1e-12);
+}
+__global__ void __launch_bounds__(256) k_ws_standardize(const double* __restrict__ X, int cols,
+                                                        const double* __restrict__ mean,
+                                                        const double* __restrict__ sd,
+                                                        float* __restrict__ Y) {
+  const int c = blockIdx.y * 256 + threadIdx.x;
+  if (c >= cols) return;
+  const size_t o = (size_t)blockIdx.x * cols + c;
+  Y[o] = (float)((X[o] - mean[c]) / sd[c]);
 }
 
 // dst = src in the operand type; with dstt also the transposed BF16 copy of a rows x cols matrix
@@ -238,12 +319,15 @@ struct nnc_ws {
   long long step = 0;
   // batch workspace (capacity cap rows)
   int cap = 0;
-  float *U = nullptr, *Tt = nullptr, *Z1 = nullptr, *H1 = nullptr, *Z2 = nullptr, *H2 = nullptr,
-        *P = nullptr, *dP = nullptr, *dH = nullptr, *dZ = nullptr;
+  float *U = nullptr, *Tt = nullptr, *Z1 = nullptr, *D1 = nullptr, *Z2 = nullptr, *D2 = nullptr,
+        *P = nullptr, *dH = nullptr;   // D1, D2: GELU' of the two hidden layers
   void *Ul = nullptr, *H1l = nullptr, *H2l = nullptr, *dPl = nullptr, *dZl = nullptr;
-  double* part = nullptr;
-  int* idx = nullptr;
-  float *Ud = nullptr, *Td = nullptr;   // standardized dataset on the device
+  double* part = nullptr;   // [n_out] the loss's column sums
+  // training set on the device (capacity nd rows): as given, standardized, the epoch's order, and the
+  // means and deviations of the columns [2][n_in + n_out]
+  double *Ur = nullptr, *Tr = nullptr, *stats = nullptr;
+  float *Ud = nullptr, *Td = nullptr;
+  int* perm = nullptr;
   int nd = 0;
   // tensor-core path (BF16 form with n_in, h1, h2 multiples of 64): transposed BF16 operand copies
   // (row stride cap), dP with its row stride padded to n_out_p, W2^T and W3^T, and the plans of
@@ -284,21 +368,18 @@ int ensure_cap(nnc_ws* s, int B) {
   WAL(s->U, big);
   WAL(s->Tt, big);
   WAL(s->Z1, big);
-  WAL(s->H1, big);
+  WAL(s->D1, big);
   WAL(s->Z2, big);
-  WAL(s->H2, big);
+  WAL(s->D2, big);
   WAL(s->P, big);
-  WAL(s->dP, big);
   WAL(s->dH, big);
-  WAL(s->dZ, big);
   unsigned char* q;
   WAL(q, big * esz(s)); s->Ul = q;
   WAL(q, big * esz(s)); s->H1l = q;
   WAL(q, big * esz(s)); s->H2l = q;
   WAL(q, big * esz(s)); s->dPl = q;
   WAL(q, big * esz(s)); s->dZl = q;
-  WAL(s->part, (big + 255) / 256 + 1);
-  WAL(s->idx, B);
+  WAL(s->part, s->n_out);
   if (s->tc) {
     WAL(s->Ut, (size_t)s->n_in * B);
     WAL(s->H1t, (size_t)s->h1 * B);
@@ -309,6 +390,29 @@ int ensure_cap(nnc_ws* s, int B) {
   }
   s->cap = B;
   s->plan_rows = -1;
+  return NNC_OK;
+}
+
+// training-set buffers for N rows; a larger set replaces them
+int ensure_set(nnc_ws* s, int N) {
+  if (N <= s->nd) return NNC_OK;
+  WCK(cudaStreamSynchronize(s->stream));
+  for (void* p : {(void*)s->Ur, (void*)s->Tr, (void*)s->Ud, (void*)s->Td, (void*)s->perm}) {
+    if (!p) continue;
+    s->allocs.erase(std::find(s->allocs.begin(), s->allocs.end(), p));
+    cudaFree(p);
+  }
+  s->Ur = s->Tr = nullptr;
+  s->Ud = s->Td = nullptr;
+  s->perm = nullptr;
+  s->nd = 0;
+  WAL(s->Ur, (size_t)N * s->n_in);
+  WAL(s->Tr, (size_t)N * s->n_out);
+  WAL(s->Ud, (size_t)N * s->n_in);
+  WAL(s->Td, (size_t)N * s->n_out);
+  WAL(s->perm, N);
+  if (!s->stats) WAL(s->stats, 2 * (size_t)(s->n_in + s->n_out));
+  s->nd = N;
   return NNC_OK;
 }
 
@@ -340,7 +444,13 @@ int make_plans(nnc_ws* s, int B) {
     if (e_ != cudaSuccess) return wfail(NNC_ERR_CUDA, std::string(#expr) + ": " + cudaGetErrorString(e_)); \
   } while (0)
 
-// forward on the first B rows of s->U (FP32) / s->Ul (operand type): P = net(U)
+template <typename T>
+void gelu(nnc_ws* s, const float* Z, int B, int cols, void* Hl, float* D1, __nv_bfloat16* Ht) {
+  k_ws_gelu<T><<<(B * cols + 63) / 64, 64, 0, s->stream>>>(Z, B * cols, (T*)Hl, D1, cols, Ht, s->cap);
+  note_launch();
+}
+
+// forward on the first B rows of s->Ul (operand type): P = net(U)
 template <typename T>
 int forward(nnc_ws* s, int B) {
   cudaStream_t st = s->stream;
@@ -348,19 +458,22 @@ int forward(nnc_ws* s, int B) {
     if (s->tc) {
       int r = make_plans(s, B);
       if (r) return r;
-      TCK(nnc::tc_plain(s->pl[0], s->w[1], s->Z1, s->h1, true, s->H1, s->H1l, s->H1t, s->cap, s->d_err, st));
-      TCK(nnc::tc_plain(s->pl[1], s->w[3], s->Z2, s->h2, true, s->H2, s->H2l, s->H2t, s->cap, s->d_err, st));
-      TCK(nnc::tc_plain(s->pl[2], s->w[5], s->P, s->n_out, false, nullptr, nullptr, nullptr, 0, s->d_err, st));
+      TCK(nnc::tc_plain(s->pl[0], s->w[1], s->Z1, s->h1, s->d_err, st));
+      gelu<T>(s, s->Z1, B, s->h1, s->H1l, s->D1, s->H1t);
+      TCK(nnc::tc_plain(s->pl[1], s->w[3], s->Z2, s->h2, s->d_err, st));
+      gelu<T>(s, s->Z2, B, s->h2, s->H2l, s->D2, s->H2t);
+      TCK(nnc::tc_plain(s->pl[2], s->w[5], s->P, s->n_out, s->d_err, st));
       return NNC_OK;
     }
   }
-  T* Ul = (T*)s->Ul;
-  gemm<T>(Ul, s->n_in, 1, (const T*)s->wl[0], 1, s->n_in, B, s->h1, s->n_in, s->w[1], s->Z1, s->h1,
-          true, s->H1, (T*)s->H1l, st);
-  gemm<T>((const T*)s->H1l, s->h1, 1, (const T*)s->wl[2], 1, s->h1, B, s->h2, s->h1, s->w[3], s->Z2,
-          s->h2, true, s->H2, (T*)s->H2l, st);
+  gemm<T>((const T*)s->Ul, s->n_in, 1, (const T*)s->wl[0], 1, s->n_in, B, s->h1, s->n_in, s->w[1], s->Z1,
+          s->h1, st);
+  gelu<T>(s, s->Z1, B, s->h1, s->H1l, s->D1, nullptr);
+  gemm<T>((const T*)s->H1l, s->h1, 1, (const T*)s->wl[2], 1, s->h1, B, s->h2, s->h1, s->w[3], s->Z2, s->h2,
+          st);
+  gelu<T>(s, s->Z2, B, s->h2, s->H2l, s->D2, nullptr);
   gemm<T>((const T*)s->H2l, s->h2, 1, (const T*)s->wl[4], 1, s->h2, B, s->n_out, s->h2, s->w[5], s->P,
-          s->n_out, false, nullptr, (T*)nullptr, st);
+          s->n_out, st);
   return NNC_OK;
 }
 
@@ -371,56 +484,43 @@ int loss_grad(nnc_ws* s, int B, double* loss) {
   int rf = forward<T>(s, B);
   if (rf) return rf;
   const int nP = B * s->n_out;
-  const int nb = (nP + 255) / 256;
   // tensor-core backward products need the batch (their K) to be a multiple of 64
   const bool tcb = !std::is_same<T, float>::value && s->tc && B % 64 == 0;
-  k_ws_loss<T><<<nb, 256, 0, st>>>(s->P, s->Tt, nP, 1.f / (float)nP, s->dP, (T*)s->dPl, s->part,
-                                   s->n_out, tcb ? s->dPp : nullptr, s->n_out_p,
-                                   tcb ? s->dPt : nullptr, s->cap);
+  __nv_bfloat16* dZt = tcb ? s->dZt : nullptr;
+  auto back = [&](const float* D, int cols, float* db) {
+    k_ws_gelu_back<T><<<(cols + 31) / 32, 32, 0, st>>>(s->dH, D, B, cols, (T*)s->dZl, db, dZt, s->cap);
+    note_launch();
+  };
+  k_ws_loss<T><<<(s->n_out + 31) / 32, 32, 0, st>>>(s->P, s->Tt, B, s->n_out, 1.f / (float)nP, (T*)s->dPl,
+                                                    s->g[5], s->part, tcb ? s->dPp : nullptr, s->n_out_p,
+                                                    tcb ? s->dPt : nullptr, s->cap);
   note_launch();
+  // layer by layer: dW = dZ^T H (db with dZ), dH = dZ W, dZ = dH * GELU'
   if (tcb) {
-    // layer 3: dW3 = dP^T H2, db3 = colsum dP, dH2 = dP W3
-    TCK(nnc::tc_plain(s->pl[3], nullptr, s->g[4], s->h2, false, nullptr, nullptr, nullptr, 0, s->d_err, st));
-    k_ws_colsum<<<(s->n_out + 255) / 256, 256, 0, st>>>(s->dP, B, s->n_out, s->g[5]);
-    TCK(nnc::tc_plain(s->pl[4], nullptr, s->dH, s->h2, false, nullptr, nullptr, nullptr, 0, s->d_err, st));
-    k_ws_gelu_back<T><<<(B * s->h2 + 255) / 256, 256, 0, st>>>(s->dH, s->Z2, B * s->h2, s->dZ, (T*)s->dZl,
-                                                              s->h2, s->dZt, s->cap);
-    // layer 2
-    TCK(nnc::tc_plain(s->pl[5], nullptr, s->g[2], s->h1, false, nullptr, nullptr, nullptr, 0, s->d_err, st));
-    k_ws_colsum<<<(s->h2 + 255) / 256, 256, 0, st>>>(s->dZ, B, s->h2, s->g[3]);
-    TCK(nnc::tc_plain(s->pl[6], nullptr, s->dH, s->h1, false, nullptr, nullptr, nullptr, 0, s->d_err, st));
-    k_ws_gelu_back<T><<<(B * s->h1 + 255) / 256, 256, 0, st>>>(s->dH, s->Z1, B * s->h1, s->dZ, (T*)s->dZl,
-                                                              s->h1, s->dZt, s->cap);
-    // layer 1
-    TCK(nnc::tc_plain(s->pl[7], nullptr, s->g[0], s->n_in, false, nullptr, nullptr, nullptr, 0, s->d_err, st));
-    k_ws_colsum<<<(s->h1 + 255) / 256, 256, 0, st>>>(s->dZ, B, s->h1, s->g[1]);
-    note_launch(5);
+    TCK(nnc::tc_plain(s->pl[3], nullptr, s->g[4], s->h2, s->d_err, st));
+    TCK(nnc::tc_plain(s->pl[4], nullptr, s->dH, s->h2, s->d_err, st));
+    back(s->D2, s->h2, s->g[3]);
+    TCK(nnc::tc_plain(s->pl[5], nullptr, s->g[2], s->h1, s->d_err, st));
+    TCK(nnc::tc_plain(s->pl[6], nullptr, s->dH, s->h1, s->d_err, st));
+    back(s->D1, s->h1, s->g[1]);
+    TCK(nnc::tc_plain(s->pl[7], nullptr, s->g[0], s->n_in, s->d_err, st));
   } else {
-  // layer 3: dW3 = dP^T H2, db3 = colsum dP, dH2 = dP W3
-  gemm<T>((const T*)s->dPl, 1, s->n_out, (const T*)s->H2l, s->h2, 1, s->n_out, s->h2, B, nullptr,
-          s->g[4], s->h2, false, nullptr, (T*)nullptr, st);
-  k_ws_colsum<<<(s->n_out + 255) / 256, 256, 0, st>>>(s->dP, B, s->n_out, s->g[5]);
-  gemm<T>((const T*)s->dPl, s->n_out, 1, (const T*)s->wl[4], s->h2, 1, B, s->h2, s->n_out, nullptr,
-          s->dH, s->h2, false, nullptr, (T*)nullptr, st);
-  k_ws_gelu_back<T><<<(B * s->h2 + 255) / 256, 256, 0, st>>>(s->dH, s->Z2, B * s->h2, s->dZ, (T*)s->dZl,
-                                                            s->h2, nullptr, 0);
-  // layer 2
-  gemm<T>((const T*)s->dZl, 1, s->h2, (const T*)s->H1l, s->h1, 1, s->h2, s->h1, B, nullptr, s->g[2],
-          s->h1, false, nullptr, (T*)nullptr, st);
-  k_ws_colsum<<<(s->h2 + 255) / 256, 256, 0, st>>>(s->dZ, B, s->h2, s->g[3]);
-  gemm<T>((const T*)s->dZl, s->h2, 1, (const T*)s->wl[2], s->h1, 1, B, s->h1, s->h2, nullptr, s->dH,
-          s->h1, false, nullptr, (T*)nullptr, st);
-  k_ws_gelu_back<T><<<(B * s->h1 + 255) / 256, 256, 0, st>>>(s->dH, s->Z1, B * s->h1, s->dZ, (T*)s->dZl,
-                                                            s->h1, nullptr, 0);
-  // layer 1
-  gemm<T>((const T*)s->dZl, 1, s->h1, (const T*)s->Ul, s->n_in, 1, s->h1, s->n_in, B, nullptr, s->g[0],
-          s->n_in, false, nullptr, (T*)nullptr, st);
-  k_ws_colsum<<<(s->h1 + 255) / 256, 256, 0, st>>>(s->dZ, B, s->h1, s->g[1]);
-  note_launch(5);
+    gemm<T>((const T*)s->dPl, 1, s->n_out, (const T*)s->H2l, s->h2, 1, s->n_out, s->h2, B, nullptr, s->g[4],
+            s->h2, st);
+    gemm<T>((const T*)s->dPl, s->n_out, 1, (const T*)s->wl[4], s->h2, 1, B, s->h2, s->n_out, nullptr, s->dH,
+            s->h2, st);
+    back(s->D2, s->h2, s->g[3]);
+    gemm<T>((const T*)s->dZl, 1, s->h2, (const T*)s->H1l, s->h1, 1, s->h2, s->h1, B, nullptr, s->g[2], s->h1,
+            st);
+    gemm<T>((const T*)s->dZl, s->h2, 1, (const T*)s->wl[2], s->h1, 1, B, s->h1, s->h2, nullptr, s->dH, s->h1,
+            st);
+    back(s->D1, s->h1, s->g[1]);
+    gemm<T>((const T*)s->dZl, 1, s->h1, (const T*)s->Ul, s->n_in, 1, s->h1, s->n_in, B, nullptr, s->g[0],
+            s->n_in, st);
   }
   if (loss) {
-    std::vector<double> h(nb);
-    WCK(cudaMemcpyAsync(h.data(), s->part, sizeof(double) * nb, cudaMemcpyDeviceToHost, st));
+    std::vector<double> h(s->n_out);
+    WCK(cudaMemcpyAsync(h.data(), s->part, sizeof(double) * s->n_out, cudaMemcpyDeviceToHost, st));
     WCK(cudaStreamSynchronize(st));
     double t = 0;
     for (double x : h) t += x;
@@ -432,17 +532,23 @@ int loss_grad(nnc_ws* s, int B, double* loss) {
 template <typename T>
 void adam(nnc_ws* s, float lr, float b1, float b2, float eps) {
   s->step += 1;
-  const float c1 = 1.f - std::pow(b1, (float)s->step), c2 = 1.f - std::pow(b2, (float)s->step);
+  AdamArgs p{};
+  p.lr = lr;
+  p.b1 = b1;
+  p.b2 = b2;
+  p.eps = eps;
+  p.c1 = 1.f - std::pow(b1, (float)s->step);
+  p.c2 = 1.f - std::pow(b2, (float)s->step);
+  int blocks = 0;
   for (int i = 0; i < 6; ++i) {
     // W2^T and W3^T feed the tensor-core backward products
     __nv_bfloat16* wt = !s->tc ? nullptr : i == 2 ? s->W2t : i == 4 ? s->W3t : nullptr;
-    const int cols = i == 2 ? s->h1 : i == 4 ? s->h2 : 1;
-    const int ldt = i == 2 ? s->h2 : i == 4 ? s->n_out_p : 0;
-    k_ws_adam<T><<<(s->sizes[i] + 255) / 256, 256, 0, s->stream>>>(
-        s->w[i], s->g[i], s->m[i], s->v[i], (i % 2 == 0) ? (T*)s->wl[i] : (T*)nullptr, s->sizes[i], lr,
-        b1, b2, eps, c1, c2, cols, wt, ldt);
+    p.a[i] = AdamSeg{s->w[i], s->m[i], s->v[i], s->g[i], i % 2 == 0 ? s->wl[i] : nullptr, wt, s->sizes[i],
+                     i == 2 ? s->h1 : i == 4 ? s->h2 : 1, i == 2 ? s->h2 : i == 4 ? s->n_out_p : 0, blocks};
+    blocks += (s->sizes[i] + 255) / 256;
   }
-  note_launch(6);
+  k_ws_adam<T><<<blocks, 256, 0, s->stream>>>(p);
+  note_launch();
 }
 
 template <typename T>
@@ -620,62 +726,50 @@ int nnc_ws_train(nnc_ws* s, const double* U, const double* Tt, int N, int epochs
                  double lr, double beta1, double beta2, double eps, unsigned long long seed,
                  double* final_loss) {
   if (!s || !U || !Tt || N < 1 || epochs < 0 || batch < 1) return wfail(NNC_ERR_ARG, "nnc_ws_train: bad arguments");
-  // standardize inputs and targets per coordinate over the data set
-  for (int c = 0; c < s->n_in; ++c) {
-    double mu = 0, sq = 0;
-    for (int r = 0; r < N; ++r) mu += U[(size_t)r * s->n_in + c];
-    mu /= N;
-    for (int r = 0; r < N; ++r) sq += (U[(size_t)r * s->n_in + c] - mu) * (U[(size_t)r * s->n_in + c] - mu);
-    s->in_mean[c] = mu;
-    s->in_std[c] = std::max(std::sqrt(sq / N), 1e-12);
-  }
-  for (int c = 0; c < s->n_out; ++c) {
-    double mu = 0, sq = 0;
-    for (int r = 0; r < N; ++r) mu += Tt[(size_t)r * s->n_out + c];
-    mu /= N;
-    for (int r = 0; r < N; ++r) sq += (Tt[(size_t)r * s->n_out + c] - mu) * (Tt[(size_t)r * s->n_out + c] - mu);
-    s->out_mean[c] = mu;
-    s->out_std[c] = std::max(std::sqrt(sq / N), 1e-12);
-  }
-  // the standardized data set stays on the device; batches are gathered by index
-  std::vector<float> hu((size_t)N * s->n_in), ht((size_t)N * s->n_out);
-  for (int r = 0; r < N; ++r) {
-    for (int c = 0; c < s->n_in; ++c)
-      hu[(size_t)r * s->n_in + c] = (float)((U[(size_t)r * s->n_in + c] - s->in_mean[c]) / s->in_std[c]);
-    for (int c = 0; c < s->n_out; ++c)
-      ht[(size_t)r * s->n_out + c] = (float)((Tt[(size_t)r * s->n_out + c] - s->out_mean[c]) / s->out_std[c]);
-  }
-  if (N > s->nd) {
-    int r = walloc(s, &s->Ud, hu.size());
-    if (!r) r = walloc(s, &s->Td, ht.size());
-    if (r) return r;
-    s->nd = N;
-  }
-  WCK(cudaMemcpyAsync(s->Ud, hu.data(), sizeof(float) * hu.size(), cudaMemcpyHostToDevice, s->stream));
-  WCK(cudaMemcpyAsync(s->Td, ht.data(), sizeof(float) * ht.size(), cudaMemcpyHostToDevice, s->stream));
-  const int B = std::min(batch, N);
+  const int B = std::min(batch, N), n_in = s->n_in, n_out = s->n_out, nc = n_in + n_out;
   int r = ensure_cap(s, B);
+  if (!r) r = ensure_set(s, N);
   if (r) return r;
+  cudaStream_t st = s->stream;
+  // the data set goes to the device as given and is standardized there, per coordinate; batches are
+  // gathered by index
+  WCK(cudaMemcpyAsync(s->Ur, U, sizeof(double) * (size_t)N * n_in, cudaMemcpyHostToDevice, st));
+  WCK(cudaMemcpyAsync(s->Tr, Tt, sizeof(double) * (size_t)N * n_out, cudaMemcpyHostToDevice, st));
+  double *mean = s->stats, *sd = s->stats + nc;
+  k_ws_stats<<<(n_in + 31) / 32, 32, 0, st>>>(s->Ur, N, n_in, mean, sd);
+  k_ws_stats<<<(n_out + 31) / 32, 32, 0, st>>>(s->Tr, N, n_out, mean + n_in, sd + n_in);
+  k_ws_standardize<<<dim3(N, (n_in + 255) / 256), 256, 0, st>>>(s->Ur, n_in, mean, sd, s->Ud);
+  k_ws_standardize<<<dim3(N, (n_out + 255) / 256), 256, 0, st>>>(s->Tr, n_out, mean + n_in, sd + n_in, s->Td);
+  note_launch(4);
+  std::vector<double> h(2 * (size_t)nc);
+  WCK(cudaMemcpyAsync(h.data(), s->stats, sizeof(double) * h.size(), cudaMemcpyDeviceToHost, st));
+  WCK(cudaStreamSynchronize(st));
+  std::copy_n(h.begin(), n_in, s->in_mean.begin());
+  std::copy_n(h.begin() + n_in, n_out, s->out_mean.begin());
+  std::copy_n(h.begin() + nc, n_in, s->in_std.begin());
+  std::copy_n(h.begin() + nc + n_in, n_out, s->out_std.begin());
   std::mt19937_64 rng(seed);
   std::vector<int> perm(N);
   std::iota(perm.begin(), perm.end(), 0);
   double last = 0.0;
+  const dim3 gg(B, (nc + 255) / 256);
   for (int e = 0; e < epochs; ++e) {
     std::shuffle(perm.begin(), perm.end(), rng);
+    WCK(cudaMemcpyAsync(s->perm, perm.data(), sizeof(int) * N, cudaMemcpyHostToDevice, st));
+    WCK(cudaStreamSynchronize(st));   // `perm` is shuffled again
     for (int b0 = 0; b0 + B <= N; b0 += B) {
-      WCK(cudaMemcpyAsync(s->idx, perm.data() + b0, sizeof(int) * B, cudaMemcpyHostToDevice, s->stream));
       const bool want = (e == epochs - 1) && (b0 + 2 * B > N);
       if (s->prec == NNC_FP32) {
-        k_ws_gather<float><<<(B * s->n_in + 255) / 256, 256, 0, s->stream>>>(s->Ud, s->idx, B, s->n_in, s->U, (float*)s->Ul);
-        k_ws_gather<float><<<(B * s->n_out + 255) / 256, 256, 0, s->stream>>>(s->Td, s->idx, B, s->n_out, s->Tt, (float*)nullptr);
-        note_launch(2);
+        k_ws_gather<float><<<gg, 256, 0, st>>>(s->Ud, s->Td, s->perm + b0, n_in, n_out, (float*)s->Ul,
+                                               nullptr, 0, s->Tt);
+        note_launch();
         r = loss_grad<float>(s, B, want ? &last : nullptr);
         adam<float>(s, (float)lr, (float)beta1, (float)beta2, (float)eps);
       } else {
-        k_ws_gather<__nv_bfloat16><<<(B * s->n_in + 255) / 256, 256, 0, s->stream>>>(
-            s->Ud, s->idx, B, s->n_in, s->U, (__nv_bfloat16*)s->Ul, s->tc ? s->Ut : nullptr, s->cap);
-        k_ws_gather<__nv_bfloat16><<<(B * s->n_out + 255) / 256, 256, 0, s->stream>>>(s->Td, s->idx, B, s->n_out, s->Tt, (__nv_bfloat16*)nullptr);
-        note_launch(2);
+        k_ws_gather<__nv_bfloat16><<<gg, 256, 0, st>>>(s->Ud, s->Td, s->perm + b0, n_in, n_out,
+                                                       (__nv_bfloat16*)s->Ul, s->tc ? s->Ut : nullptr,
+                                                       s->cap, s->Tt);
+        note_launch();
         r = loss_grad<__nv_bfloat16>(s, B, want ? &last : nullptr);
         adam<__nv_bfloat16>(s, (float)lr, (float)beta1, (float)beta2, (float)eps);
       }

@@ -143,3 +143,48 @@ def test_warm_started_ipm_matches_oracle(nnc):
     b.free()
     for n in nets:
         n.free()
+
+
+@pytest.mark.parametrize("prec,shape", [
+    ("fp32", (1, 1, 1, 1, 1)),          # one element of every kernel
+    ("fp32", (33, 31, 65, 17, 7)),      # past the 32-wide tiles and column blocks, rows not in eights
+    ("fp32", (64, 32, 96, 32, 40)),     # whole tiles
+    ("bf16", (31, 33, 64, 65, 9)),      # BF16 operands on the CUDA cores
+    ("bf16", (64, 64, 64, 33, 64)),     # one K block, a second 32-column tile of one column
+    ("bf16", (64, 192, 64, 713, 1920)),  # more 32-column tiles than SMs: the wide tiles
+])
+def test_gradient_kernels_at_edges(nnc, prec, shape):
+    """Loss and gradients at the edges of tiles, column blocks and row groups (tolerances of the file)."""
+    n_in, h1, h2, n_out, B = shape
+    p = synth.warmstart_params(n_in, h1, h2, n_out, seed=B)
+    p = [np.float32(x).astype(np.float64) for x in p]
+    rng = np.random.default_rng(B)
+    U = np.float32(rng.standard_normal((B, n_in))).astype(np.float64)
+    T = np.float32(rng.standard_normal((B, n_out))).astype(np.float64)
+    tol = 1e-5 if prec == "fp32" else 3e-2
+    ws = nnc.WarmStart(p, precision=prec)
+    loss, g = ws.loss_grad(U, T)
+    ws.free()
+    lo, go = ows.loss(p, U, T), ows.grad(p, U, T)
+    assert abs(loss - lo) <= tol * lo
+    assert max(rel(a, b) for a, b in zip(g, go)) < tol
+
+
+@pytest.mark.parametrize("n", [1, 15, 16, 33, 300])
+def test_standardization(nnc, n):
+    """train() with no epochs leaves the scaling of its data set: predictions are those of the initial
+    network on standardized inputs, scaled back.  FP32 products of 40 terms on standardized values,
+    mapped back by deviations and means of order one: 1e-5."""
+    p, _, _ = _data()
+    rng = np.random.default_rng(n)
+    U, T = 3.0 + 2.0 * rng.standard_normal((n, 40)), -1.0 + 0.5 * rng.standard_normal((n, 23))
+    ws = nnc.WarmStart(p, precision="fp32")
+    for _ in range(2):   # a second, larger set replaces the first one's buffers
+        ws.train(U, T, 0)
+        mu, sd = U.mean(0), np.maximum(U.std(0), 1e-12)
+        to, so = T.mean(0), np.maximum(T.std(0), 1e-12)
+        V = U + 0.1 * sd
+        want = ows.forward(p, (V - mu) / sd)[0] * so + to
+        assert rel(ws.predict(V), want) < 1e-5
+        U, T = np.concatenate([U, 2.0 * U + 1.0]), np.concatenate([T, 0.3 - T])
+    ws.free()
