@@ -456,7 +456,7 @@ int run_hessian(nnc_net* net, const double* lam, double* H, cudaStream_t st, boo
   }
   {
     PROF(PK_SYRK);
-    if (!tc)  // the tensor-core product stores its partials; the CUDA-core one adds to them
+    if (prec == NNC_FP64)  // the other products store their partials; the FP64 one adds to them
       CK(cudaMemsetAsync(net->Hp, 0, (size_t)net->h_splits * n * n * 8, st));
     if (tc)
       CK(tc_syrk(net->plan_syrk, (float*)net->Hp, net->dev_err, st));
