@@ -1233,6 +1233,9 @@ __global__ void __launch_bounds__(kThreads, 1)
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
 
+  griddep_wait();   // the operands are written, and the last reader of C is done
+  griddep_launch();
+
   int issued = 0;
   if (warp == 0) {
     if (lane == 0) {
@@ -1689,9 +1692,7 @@ cudaError_t launch_plain_t(const PlainPlan& p, const PlainArgs& a, cudaStream_t 
     if (e != cudaSuccess) return e;
     attr = true;
   }
-  k_tc_plain<BN><<<p.ntm * p.ntn, kThreads, C::SMEM, st>>>(p.ta, p.tb, a);
-  note_launch();
-  return cudaGetLastError();
+  return launch_pdl(k_tc_plain<BN>, dim3(p.ntm * p.ntn), dim3(kThreads), C::SMEM, st, p.ta, p.tb, a);
 }
 
 cudaError_t tc_plain(const PlainPlan& p, const float* bias, float* Cout, int ldc, int* err,

@@ -21,6 +21,7 @@
 #include <vector>
 
 #include "../../include/nnc.h"
+#include "async.cuh"
 #include "common.cuh"
 #include "tc.cuh"
 
@@ -28,6 +29,8 @@ namespace nnc {
 void set_last_error(const std::string& msg);
 }
 using namespace nnc;
+using async::griddep_launch;
+using async::griddep_wait;
 
 namespace {
 
@@ -63,6 +66,8 @@ __global__ void __launch_bounds__(256) k_ws_gemm(const T* __restrict__ A, long s
     }
   };
   float acc[2][2] = {};
+  griddep_wait();
+  griddep_launch();
   load(0);
   for (int k0 = 0; k0 < K; k0 += 32) {
 #pragma unroll
@@ -100,8 +105,7 @@ template <typename T>
 void gemm(const T* A, long sam, long sak, const T* B, long sbk, long sbn, int M, int N, int K,
           const float* bias, float* C, int ldc, cudaStream_t st) {
   dim3 grid((N + 31) / 32, (M + 31) / 32);
-  k_ws_gemm<T><<<grid, 256, 0, st>>>(A, sam, sak, B, sbk, sbn, M, N, K, bias, C, ldc);
-  note_launch();
+  launch_pdl(k_ws_gemm<T>, grid, dim3(256), 0, st, A, sam, sak, B, sbk, sbn, M, N, K, bias, C, ldc);
 }
 
 template <typename T>
@@ -113,11 +117,13 @@ __device__ __forceinline__ T to_op(float v) {
 // H = GELU(Z) in the operand type (and, for the tensor-core backward products, its transposed copy) and
 // D1 = GELU'(Z).  Bound: the FP64 pipe, two FMAs per clock and SM, so the elements are spread over the
 // whole chip in CTAs of 64.  In the epilogue of the product the 64 x 256 values were one SM's work, and
-// with them a training step of 64 rows (512 -> 256 -> 256 -> 713) took 1.1 ms; now at most 0.1 ms.
+// with them a training step of 64 rows (512 -> 256 -> 256 -> 713) took 1.1 ms; now 0.08 ms.
 template <typename T>
 __global__ void __launch_bounds__(64) k_ws_gelu(const float* __restrict__ Z, int n, T* __restrict__ Hl,
                                                 float* __restrict__ D1, int cols,
                                                 __nv_bfloat16* __restrict__ Ht, int ldt) {
+  griddep_wait();
+  griddep_launch();
   const int i = blockIdx.x * 64 + threadIdx.x;
   if (i >= n) return;
   double a, d1, d2;
@@ -144,6 +150,8 @@ __global__ void __launch_bounds__(32) k_ws_gelu_back(const float* __restrict__ d
                                                      const float* __restrict__ D1, int B, int cols,
                                                      T* __restrict__ dZl, float* __restrict__ db,
                                                      __nv_bfloat16* __restrict__ dZt, int ldt) {
+  griddep_wait();
+  griddep_launch();
   const int j = blockIdx.x * 32 + threadIdx.x;
   if (j >= cols) return;
   float s = 0.f;
@@ -175,6 +183,8 @@ __global__ void __launch_bounds__(32) k_ws_loss(const float* __restrict__ P, con
                                                 float* __restrict__ db, double* __restrict__ part,
                                                 __nv_bfloat16* __restrict__ dPp, int ldp,
                                                 __nv_bfloat16* __restrict__ dPt, int ldt) {
+  griddep_wait();
+  griddep_launch();
   const int j = blockIdx.x * 32 + threadIdx.x;
   if (j >= cols) return;
   double l = 0.0;
@@ -217,6 +227,8 @@ struct AdamArgs {
 };
 template <typename T>
 __global__ void __launch_bounds__(256) k_ws_adam(const __grid_constant__ AdamArgs p) {
+  griddep_wait();
+  griddep_launch();
   int k = 5;
   while ((int)blockIdx.x < p.a[k].blk0) --k;
   const AdamSeg& q = p.a[k];
@@ -239,6 +251,8 @@ __global__ void __launch_bounds__(256) k_ws_gather(const float* __restrict__ Ud,
                                                    const int* __restrict__ idx, int n_in, int n_out,
                                                    T* __restrict__ Ul, __nv_bfloat16* __restrict__ Ut,
                                                    int ldt, float* __restrict__ Tt) {
+  griddep_wait();
+  griddep_launch();
   const int r = blockIdx.x, c = blockIdx.y * 256 + threadIdx.x;
   const size_t row = idx[r];
   if (c < n_in) {
@@ -446,8 +460,8 @@ int make_plans(nnc_ws* s, int B) {
 
 template <typename T>
 void gelu(nnc_ws* s, const float* Z, int B, int cols, void* Hl, float* D1, __nv_bfloat16* Ht) {
-  k_ws_gelu<T><<<(B * cols + 63) / 64, 64, 0, s->stream>>>(Z, B * cols, (T*)Hl, D1, cols, Ht, s->cap);
-  note_launch();
+  launch_pdl(k_ws_gelu<T>, dim3((B * cols + 63) / 64), dim3(64), 0, s->stream, Z, B * cols, (T*)Hl, D1, cols, Ht,
+             s->cap);
 }
 
 // forward on the first B rows of s->Ul (operand type): P = net(U)
@@ -488,13 +502,12 @@ int loss_grad(nnc_ws* s, int B, double* loss) {
   const bool tcb = !std::is_same<T, float>::value && s->tc && B % 64 == 0;
   __nv_bfloat16* dZt = tcb ? s->dZt : nullptr;
   auto back = [&](const float* D, int cols, float* db) {
-    k_ws_gelu_back<T><<<(cols + 31) / 32, 32, 0, st>>>(s->dH, D, B, cols, (T*)s->dZl, db, dZt, s->cap);
-    note_launch();
+    launch_pdl(k_ws_gelu_back<T>, dim3((cols + 31) / 32), dim3(32), 0, st, s->dH, D, B, cols, (T*)s->dZl, db, dZt,
+               s->cap);
   };
-  k_ws_loss<T><<<(s->n_out + 31) / 32, 32, 0, st>>>(s->P, s->Tt, B, s->n_out, 1.f / (float)nP, (T*)s->dPl,
-                                                    s->g[5], s->part, tcb ? s->dPp : nullptr, s->n_out_p,
-                                                    tcb ? s->dPt : nullptr, s->cap);
-  note_launch();
+  launch_pdl(k_ws_loss<T>, dim3((s->n_out + 31) / 32), dim3(32), 0, st, s->P, s->Tt, B, s->n_out,
+             1.f / (float)nP, (T*)s->dPl, s->g[5], s->part, tcb ? s->dPp : nullptr, s->n_out_p,
+             tcb ? s->dPt : nullptr, s->cap);
   // layer by layer: dW = dZ^T H (db with dZ), dH = dZ W, dZ = dH * GELU'
   if (tcb) {
     TCK(nnc::tc_plain(s->pl[3], nullptr, s->g[4], s->h2, s->d_err, st));
@@ -547,8 +560,7 @@ void adam(nnc_ws* s, float lr, float b1, float b2, float eps) {
                      i == 2 ? s->h1 : i == 4 ? s->h2 : 1, i == 2 ? s->h2 : i == 4 ? s->n_out_p : 0, blocks};
     blocks += (s->sizes[i] + 255) / 256;
   }
-  k_ws_adam<T><<<blocks, 256, 0, s->stream>>>(p);
-  note_launch();
+  launch_pdl(k_ws_adam<T>, dim3(blocks), dim3(256), 0, s->stream, p);
 }
 
 template <typename T>
@@ -760,16 +772,13 @@ int nnc_ws_train(nnc_ws* s, const double* U, const double* Tt, int N, int epochs
     for (int b0 = 0; b0 + B <= N; b0 += B) {
       const bool want = (e == epochs - 1) && (b0 + 2 * B > N);
       if (s->prec == NNC_FP32) {
-        k_ws_gather<float><<<gg, 256, 0, st>>>(s->Ud, s->Td, s->perm + b0, n_in, n_out, (float*)s->Ul,
-                                               nullptr, 0, s->Tt);
-        note_launch();
+        launch_pdl(k_ws_gather<float>, gg, dim3(256), 0, st, s->Ud, s->Td, s->perm + b0, n_in, n_out, (float*)s->Ul,
+                   nullptr, 0, s->Tt);
         r = loss_grad<float>(s, B, want ? &last : nullptr);
         adam<float>(s, (float)lr, (float)beta1, (float)beta2, (float)eps);
       } else {
-        k_ws_gather<__nv_bfloat16><<<gg, 256, 0, st>>>(s->Ud, s->Td, s->perm + b0, n_in, n_out,
-                                                       (__nv_bfloat16*)s->Ul, s->tc ? s->Ut : nullptr,
-                                                       s->cap, s->Tt);
-        note_launch();
+        launch_pdl(k_ws_gather<__nv_bfloat16>, gg, dim3(256), 0, st, s->Ud, s->Td, s->perm + b0, n_in, n_out,
+                   (__nv_bfloat16*)s->Ul, s->tc ? s->Ut : nullptr, s->cap, s->Tt);
         r = loss_grad<__nv_bfloat16>(s, B, want ? &last : nullptr);
         adam<__nv_bfloat16>(s, (float)lr, (float)beta1, (float)beta2, (float)eps);
       }
