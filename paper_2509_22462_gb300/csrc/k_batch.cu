@@ -6,6 +6,7 @@
 #include <algorithm>
 #include <type_traits>
 
+#include "async.cuh"
 #include "batch.cuh"
 
 namespace nnc {
@@ -20,6 +21,8 @@ __device__ __forceinline__ double bwarp_sum(double v) {
 __global__ void k_bx_scatter(const double* __restrict__ xcat, const int* __restrict__ gn,
                              const int* __restrict__ goff, int kp, double* __restrict__ xs,
                              float* __restrict__ xf) {
+  async::griddep_wait();
+  async::griddep_launch();
   const int g = blockIdx.y;
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= kp) return;
@@ -31,8 +34,7 @@ __global__ void k_bx_scatter(const double* __restrict__ xcat, const int* __restr
 cudaError_t launch_bx_scatter(const double* xcat, const int* gn, const int* goff, int kp, int groups,
                               double* xs, float* xf, cudaStream_t st) {
   dim3 grid((kp + 255) / 256, groups);
-  k_bx_scatter<<<grid, 256, 0, st>>>(xcat, gn, goff, kp, xs, xf);
-  note_launch();
+  launch_pdl(k_bx_scatter, grid, dim3(256), 0, st, xcat, gn, goff, kp, xs, xf);
   return cudaGetLastError();
 }
 
@@ -48,6 +50,8 @@ __global__ void __launch_bounds__(256) k_bgemv_rev(const float* __restrict__ W, 
                                                    int m, const double* __restrict__ Zbar, int S,
                                                    int chunks, float* __restrict__ part,
                                                    const int* __restrict__ gcols) {
+  async::griddep_wait();
+  async::griddep_launch();
   __shared__ float zs[kBRowsMax][SMAX];
   const int rows = brev_rows(ldw);
   const int g = blockIdx.z;
@@ -99,12 +103,11 @@ cudaError_t launch_bgemv_rev(const float* W, int ldw, int mp, int m, int groups,
   const int threads = std::min(256, (ldw / 4 + 31) / 32 * 32);
   dim3 grid((ldw + 4 * threads - 1) / (4 * threads), chunks, groups);
   if (S <= 2)
-    k_bgemv_rev<2><<<grid, threads, 0, st>>>(W, ldw, mp, m, Zbar, S, chunks, part, gcols);
+    launch_pdl(k_bgemv_rev<2>, grid, dim3(threads), 0, st, W, ldw, mp, m, Zbar, S, chunks, part, gcols);
   else if (S <= 4)
-    k_bgemv_rev<4><<<grid, threads, 0, st>>>(W, ldw, mp, m, Zbar, S, chunks, part, gcols);
+    launch_pdl(k_bgemv_rev<4>, grid, dim3(threads), 0, st, W, ldw, mp, m, Zbar, S, chunks, part, gcols);
   else
     return cudaErrorInvalidValue;
-  note_launch();
   return cudaGetLastError();
 }
 
@@ -118,6 +121,8 @@ __global__ void k_brev_reduce(const float* __restrict__ part, int chunks, int kc
                               double* __restrict__ c_out, float* __restrict__ c_f,
                               const int* __restrict__ gn, const int* __restrict__ goff,
                               double* __restrict__ J_cat, double* __restrict__ g_cat) {
+  async::griddep_wait();
+  async::griddep_launch();
   const int g = blockIdx.y;
   const int idx = blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= kcols * S) return;
@@ -150,9 +155,8 @@ cudaError_t launch_brev_reduce(const float* part, int chunks, int kcols, int mp_
                                double* Zbar_out, double* c_out, float* c_f, const int* gn,
                                const int* goff, double* J_cat, double* g_cat, cudaStream_t st) {
   dim3 grid((kcols * S + 255) / 256, groups);
-  k_brev_reduce<<<grid, 256, 0, st>>>(part, chunks, kcols, mp_out, S, s1, s2, lam_col, nJ, Zbar_out,
-                                      c_out, c_f, gn, goff, J_cat, g_cat);
-  note_launch();
+  launch_pdl(k_brev_reduce, grid, dim3(256), 0, st, part, chunks, kcols, mp_out, S, s1, s2, lam_col,
+             nJ, Zbar_out, c_out, c_f, gn, goff, J_cat, g_cat);
   return cudaGetLastError();
 }
 
@@ -161,6 +165,8 @@ __global__ void k_brev_seed(int m, int mp, int S, int nJ, int lam_col, const dou
                             const double* __restrict__ s2, const double* __restrict__ lam,
                             double* __restrict__ Zbar, double* __restrict__ c_out,
                             float* __restrict__ c_f) {
+  async::griddep_wait();
+  async::griddep_launch();
   const int g = blockIdx.y;
   const int idx = blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= m * S) return;
@@ -180,8 +186,7 @@ cudaError_t launch_brev_seed(int m, int mp, int groups, int S, int nJ, int lam_c
                              const double* s2, const double* lam, double* Zbar, double* c_out,
                              float* c_f, cudaStream_t st) {
   dim3 grid((m * S + 255) / 256, groups);
-  k_brev_seed<<<grid, 256, 0, st>>>(m, mp, S, nJ, lam_col, s1, s2, lam, Zbar, c_out, c_f);
-  note_launch();
+  launch_pdl(k_brev_seed, grid, dim3(256), 0, st, m, mp, S, nJ, lam_col, s1, s2, lam, Zbar, c_out, c_f);
   return cudaGetLastError();
 }
 
@@ -199,6 +204,8 @@ __global__ void __launch_bounds__(256) k_bfirst_tangent(const float* __restrict_
                                                         int lda, __nv_bfloat16* zt_hi,
                                                         __nv_bfloat16* zt_lo, __nv_bfloat16* yt_hi,
                                                         __nv_bfloat16* yt_lo, int ldz, int x3) {
+  async::griddep_wait();
+  async::griddep_launch();
   __shared__ float tile[64][33];
   const int g = blockIdx.z;
   const int n_g = gn[g];
@@ -264,11 +271,9 @@ cudaError_t launch_bfirst_tangent(const float* W1, int ldw, int mp, int groups, 
       !al8(yt_hi) || !al8(yt_lo) || (zt_hi && !yt_hi))
     return cudaErrorInvalidValue;
   dim3 grid((n_max + 31) / 32, mp / 64, groups);
-  k_bfirst_tangent<<<grid, 256, 0, st>>>(
-      W1, ldw, mp, gn, goff, s1, c, (__nv_bfloat16*)at_hi, (__nv_bfloat16*)at_lo, lda,
-      (__nv_bfloat16*)zt_hi, (__nv_bfloat16*)zt_lo, (__nv_bfloat16*)yt_hi, (__nv_bfloat16*)yt_lo, ldz,
-      x3 ? 1 : 0);
-  note_launch();
+  launch_pdl(k_bfirst_tangent, grid, dim3(256), 0, st, W1, ldw, mp, gn, goff, s1, c,
+             (__nv_bfloat16*)at_hi, (__nv_bfloat16*)at_lo, lda, (__nv_bfloat16*)zt_hi,
+             (__nv_bfloat16*)zt_lo, (__nv_bfloat16*)yt_hi, (__nv_bfloat16*)yt_lo, ldz, x3 ? 1 : 0);
   return cudaGetLastError();
 }
 
@@ -276,6 +281,8 @@ cudaError_t launch_bfirst_tangent(const float* W1, int ldw, int mp, int groups, 
 __global__ void k_bh_finish(const float* __restrict__ Hp, int splits, long long ldh_split,
                             const int* __restrict__ gn, const long long* __restrict__ hoff,
                             double* __restrict__ H) {
+  async::griddep_wait();
+  async::griddep_launch();
   const int g = blockIdx.y;
   const int n = gn[g];
   const long long base = hoff[g];
@@ -292,13 +299,14 @@ __global__ void k_bh_finish(const float* __restrict__ Hp, int splits, long long 
 cudaError_t launch_bh_finish(const float* Hp, int splits, long long ldh_split, int groups,
                              const int* gn, const long long* hoff, double* H, cudaStream_t st) {
   dim3 grid(32, groups);
-  k_bh_finish<<<grid, 256, 0, st>>>(Hp, splits, ldh_split, gn, hoff, H);
-  note_launch();
+  launch_pdl(k_bh_finish, grid, dim3(256), 0, st, Hp, splits, ldh_split, gn, hoff, H);
   return cudaGetLastError();
 }
 
 // r_cat[g*m + i] = y_cat[g*m + i] - a[g*mp + i]
 __global__ void k_bsub(const double* y, const double* a, int m, int mp, int groups, double* r) {
+  async::griddep_wait();
+  async::griddep_launch();
   const int idx = blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= m * groups) return;
   const int g = idx / m, i = idx % m;
@@ -307,21 +315,21 @@ __global__ void k_bsub(const double* y, const double* a, int m, int mp, int grou
 
 cudaError_t launch_bsub(const double* y, const double* a, int m, int mp, int groups, double* r,
                         cudaStream_t st) {
-  k_bsub<<<(m * groups + 255) / 256, 256, 0, st>>>(y, a, m, mp, groups, r);
-  note_launch();
+  launch_pdl(k_bsub, dim3((m * groups + 255) / 256), dim3(256), 0, st, y, a, m, mp, groups, r);
   return cudaGetLastError();
 }
 
 // y_cat[g*m + i] = a[g*mp + i]
 __global__ void k_bgather(const double* a, int m, int mp, int groups, double* y) {
+  async::griddep_wait();
+  async::griddep_launch();
   const int idx = blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= m * groups) return;
   y[idx] = a[(size_t)(idx / m) * mp + idx % m];
 }
 
 cudaError_t launch_bgather(const double* a, int m, int mp, int groups, double* y, cudaStream_t st) {
-  k_bgather<<<(m * groups + 255) / 256, 256, 0, st>>>(a, m, mp, groups, y);
-  note_launch();
+  launch_pdl(k_bgather, dim3((m * groups + 255) / 256), dim3(256), 0, st, a, m, mp, groups, y);
   return cudaGetLastError();
 }
 

@@ -238,6 +238,7 @@ __global__ void k_rev_seed_f(int m, int S, int SM, int nJ, int lam_col, const do
                              const double* __restrict__ s2, const double* __restrict__ lam,
                              const double* __restrict__ p, float* __restrict__ Zf,
                              double* __restrict__ c_out, float* __restrict__ c_f) {
+  griddep_wait();
   griddep_launch();
   const int idx = blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= m * SM) return;
@@ -330,9 +331,8 @@ cudaError_t launch_rev_seed_f(int m, int S, int nJ, int lam_col, const double* s
                               const double* lam, const double* p, float* Zf, double* c_out,
                               float* c_f, cudaStream_t st) {
   const int SM = rev_stream_sm(S);
-  k_rev_seed_f<<<(m * SM + 255) / 256, 256, 0, st>>>(m, S, SM, nJ, lam_col, s1, s2, lam, p, Zf,
-                                                     c_out, c_f);
-  note_launch();
+  launch_pdl(k_rev_seed_f, dim3((m * SM + 255) / 256), dim3(256), 0, st, m, S, SM, nJ, lam_col, s1, s2,
+             lam, p, Zf, c_out, c_f);
   return cudaGetLastError();
 }
 

@@ -317,9 +317,9 @@ __global__ void __launch_bounds__(kThreads, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
-  // tangent chain (launched with programmatic dependent launch): the previous layer's outputs,
-  // this layer's B operand, are complete before any copy or store of this CTA
-  if (KIND == TC_TANGENT) griddep_wait();
+  // programmatic dependent launch: the previous launch's outputs, this one's B operand, are complete
+  // before any copy or store of this CTA
+  griddep_wait();
 
   int issued = 0;  // producer only
   if (warp == 0) {
@@ -387,7 +387,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     const bool ok = epi_all(mbar_wait(smem_u32(accf), 0, args.err, 3, abort_flag));
     tc_fence_after();
     // the next layer may be queued now: its CTAs take SMs as this grid's epilogues end
-    if (KIND == TC_TANGENT && threadIdx.x == 64) griddep_launch();
+    if (threadIdx.x == 64) griddep_launch();
     if (ok && KIND == TC_REV) {
       // split-K partial of W_l^T Zbar: P[split][k][0..BN) for row k of this tile
       const int k = m0 + row;
@@ -800,6 +800,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
+  griddep_wait();
+  griddep_launch();
 
   int issued = 0;  // producer only
   if (warp == 0) {
@@ -1384,26 +1386,9 @@ cudaError_t launch_t(const TcPlan& p, const TcArgs& a, dim3 grid, cudaStream_t s
     if (e != cudaSuccess) return e;
     attr = true;
   }
-  if (KIND == TC_TANGENT) {
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = grid;
-    cfg.blockDim = dim3(kThreads);
-    cfg.dynamicSmemBytes = C::SMEM;
-    cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, k_tc_gemm<BN, MODE, KIND>, p.ta_hi, p.ta_lo,
-                                             p.tb_hi, p.tb_lo, p.ta_p2, p.tb_p2, a);
-    note_launch();
-    return e;
-  }
-  k_tc_gemm<BN, MODE, KIND><<<grid, kThreads, C::SMEM, st>>>(p.ta_hi, p.ta_lo, p.tb_hi, p.tb_lo, p.ta_p2,
-                                                             p.tb_p2, a);
-  note_launch();
-  return cudaGetLastError();
+  return launch_pdl(k_tc_gemm<BN, MODE, KIND>, grid, dim3(kThreads), C::SMEM, st, p.ta_hi, p.ta_lo,
+                    p.tb_hi,
+                    p.tb_lo, p.ta_p2, p.tb_p2, a);
 }
 
 template <int BNP, int MODE>
@@ -1652,9 +1637,9 @@ cudaError_t launch_gtan_t(const TcPlan& p, const TcArgs& a, int groups, int grid
     if (e != cudaSuccess) return e;
     attr = true;
   }
-  k_tc_gtan<BN, MODE><<<grid, kThreads, C::SMEM, st>>>(p.ta_hi, p.ta_lo, p.tb_hi, p.tb_lo, a, groups);
-  note_launch();
-  return cudaGetLastError();
+  return launch_pdl(k_tc_gtan<BN, MODE>, dim3(grid), dim3(kThreads), C::SMEM, st, p.ta_hi, p.ta_lo,
+                    p.tb_hi, p.tb_lo,
+                    a, groups);
 }
 
 template <int BN>

@@ -51,7 +51,8 @@ __global__ void __launch_bounds__(256) k_gemv_fwd(const double* __restrict__ W, 
 
 cudaError_t launch_gemv_fwd(const double* W, int ldw, const double* b, const double* a_in, int m, int k,
                             int act, double* a_out, double* s1, double* s2, cudaStream_t st) {
-  return launch_pdl(k_gemv_fwd, dim3((m + 7) / 8), dim3(256), 0, st, W, ldw, b, a_in, m, k, act, a_out, s1, s2);
+  return launch_pdl(k_gemv_fwd, dim3((m + 7) / 8), dim3(256), 0, st, W, ldw, b, a_in, m, k, act, a_out,
+                    s1, s2);
 }
 
 // ------------------------------------------------------------------ reverse sweep
@@ -291,6 +292,8 @@ __device__ __forceinline__ void set_tan(TanBuf b, size_t i, double v) {
 template <Elem E>
 __global__ void k_softmax_ext(int n, int m, const double* __restrict__ p, const double* __restrict__ lam,
                               TanBuf ZL, TanBuf Zx, TanBuf Yx, int ldz) {
+  async::griddep_wait();
+  async::griddep_launch();
   const int j = blockIdx.x * blockDim.x + threadIdx.x;   // tangent (row of Zdot^T)
   if (j >= n) return;
   double lb = 0.0;
@@ -317,14 +320,17 @@ cudaError_t launch_softmax_ext(Elem e, int n, int m, const double* p, const doub
                                TanBuf Zx, TanBuf Yx, int ldz, cudaStream_t st) {
   const int blocks = (n + 127) / 128;
   switch (e) {
-    case Elem::F64: k_softmax_ext<Elem::F64><<<blocks, 128, 0, st>>>(n, m, p, lam, ZL, Zx, Yx, ldz); break;
-    case Elem::F32: k_softmax_ext<Elem::F32><<<blocks, 128, 0, st>>>(n, m, p, lam, ZL, Zx, Yx, ldz); break;
-    case Elem::BF16: k_softmax_ext<Elem::BF16><<<blocks, 128, 0, st>>>(n, m, p, lam, ZL, Zx, Yx, ldz); break;
+    case Elem::F64: launch_pdl(k_softmax_ext<Elem::F64>, dim3(blocks), dim3(128), 0, st, n, m, p, lam,
+                               ZL, Zx, Yx, ldz); break;
+    case Elem::F32: launch_pdl(k_softmax_ext<Elem::F32>, dim3(blocks), dim3(128), 0, st, n, m, p, lam,
+                               ZL, Zx, Yx, ldz); break;
+    case Elem::BF16: launch_pdl(k_softmax_ext<Elem::BF16>, dim3(blocks), dim3(128), 0, st, n, m, p,
+                                lam, ZL, Zx, Yx, ldz); break;
     case Elem::BF16X3:
-      k_softmax_ext<Elem::BF16X3><<<blocks, 128, 0, st>>>(n, m, p, lam, ZL, Zx, Yx, ldz);
+      launch_pdl(k_softmax_ext<Elem::BF16X3>, dim3(blocks), dim3(128), 0, st, n, m, p, lam, ZL, Zx, Yx,
+                 ldz);
       break;
   }
-  note_launch();
   return cudaGetLastError();
 }
 
@@ -332,6 +338,8 @@ template <Elem E, typename TW>
 __global__ void k_first_tangent(const TW* __restrict__ W1, int ldw, int m_pad, int n,
                                 const double* __restrict__ s1, const double* __restrict__ c,
                                 TanBuf At, int lda, TanBuf Zt, TanBuf Yt, int ldz) {
+  async::griddep_wait();
+  async::griddep_launch();
   __shared__ TW tile[32][33];
   const int m0 = blockIdx.y * 32, n0 = blockIdx.x * 32;
   for (int r = threadIdx.y; r < 32; r += blockDim.y) {
@@ -443,6 +451,8 @@ __global__ void __launch_bounds__(256) k_first_tangent_t(const float* __restrict
                                                          const double* __restrict__ s1,
                                                          const double* __restrict__ c, TanBuf At,
                                                          int lda, TanBuf Yt, int ldz) {
+  async::griddep_wait();
+  async::griddep_launch();
   const int mb = 8 * (blockIdx.x * blockDim.x + threadIdx.x);
   if (mb >= m_pad) return;
   const int n0 = blockIdx.y * kFtN;
@@ -536,10 +546,11 @@ cudaError_t launch_first_tangent_t(bool x3, const float* W1T, int ldt, int m_pad
   if (m_pad % 8 || ldt % 4 || lda % 8 || ldz % 8 || ((uintptr_t)W1T & 15)) return cudaErrorInvalidValue;
   const dim3 grid((m_pad / 8 + 255) / 256, (n + kFtN - 1) / kFtN);
   if (x3)
-    k_first_tangent_t<true><<<grid, 256, 0, st>>>(W1T, ldt, m_pad, n, s1, c, At, lda, Yt, ldz);
+    launch_pdl(k_first_tangent_t<true>, grid, dim3(256), 0, st, W1T, ldt, m_pad, n, s1, c, At, lda, Yt,
+               ldz);
   else
-    k_first_tangent_t<false><<<grid, 256, 0, st>>>(W1T, ldt, m_pad, n, s1, c, At, lda, Yt, ldz);
-  note_launch();
+    launch_pdl(k_first_tangent_t<false>, grid, dim3(256), 0, st, W1T, ldt, m_pad, n, s1, c, At, lda,
+               Yt, ldz);
   return cudaGetLastError();
 }
 
@@ -628,23 +639,22 @@ cudaError_t launch_first_tangent(Elem e, const void* W1, int ldw, int m_pad, int
   const float* Wf = (const float*)W1;
   switch (e) {
     case Elem::F64:
-      k_first_tangent<Elem::F64, double><<<grid, block, 0, st>>>((const double*)W1, ldw, m_pad, n, s1,
-                                                                 c, At, lda, Zt, Yt, ldz);
+      launch_pdl(k_first_tangent<Elem::F64, double>, grid, block, 0, st, (const double*)W1, ldw, m_pad,
+                 n, s1, c, At, lda, Zt, Yt, ldz);
       break;
     case Elem::F32:
-      k_first_tangent<Elem::F32, float><<<grid, block, 0, st>>>(Wf, ldw, m_pad, n, s1, c, At, lda, Zt,
-                                                                Yt, ldz);
+      launch_pdl(k_first_tangent<Elem::F32, float>, grid, block, 0, st, Wf, ldw, m_pad, n, s1, c, At,
+                 lda, Zt, Yt, ldz);
       break;
     case Elem::BF16:
-      k_first_tangent<Elem::BF16, float><<<grid, block, 0, st>>>(Wf, ldw, m_pad, n, s1, c, At, lda,
-                                                                 Zt, Yt, ldz);
+      launch_pdl(k_first_tangent<Elem::BF16, float>, grid, block, 0, st, Wf, ldw, m_pad, n, s1, c, At,
+                 lda, Zt, Yt, ldz);
       break;
     case Elem::BF16X3:
-      k_first_tangent<Elem::BF16X3, float><<<grid, block, 0, st>>>(Wf, ldw, m_pad, n, s1, c, At, lda,
-                                                                   Zt, Yt, ldz);
+      launch_pdl(k_first_tangent<Elem::BF16X3, float>, grid, block, 0, st, Wf, ldw, m_pad, n, s1, c,
+                 At, lda, Zt, Yt, ldz);
       break;
   }
-  note_launch();
   return cudaGetLastError();
 }
 
@@ -661,6 +671,8 @@ cudaError_t launch_first_tangent(Elem e, const void* W1, int ldw, int m_pad, int
 template <typename TP, int R>
 __global__ void __launch_bounds__(256) k_h_finish(const TP* __restrict__ Hp, int splits, int n, int ldp,
                                                   double* __restrict__ H) {
+  async::griddep_wait();
+  async::griddep_launch();
   __shared__ TP t[8 * R][33];
   int b = blockIdx.x / (4 / R), bi = 0;
   const int sub = blockIdx.x % (4 / R) * 8 * R;   // first row of this block in the tile
@@ -710,10 +722,11 @@ cudaError_t launch_h_finish(bool part_f32, const void* Hp, int splits, int n, in
                             cudaStream_t st) {
   const int T = (n + 31) / 32, tiles = T * (T + 1) / 2;
   const dim3 block(32, 8);
-  if (!part_f32) k_h_finish<double, 4><<<tiles, block, 0, st>>>((const double*)Hp, splits, n, ldp, H);
-  else if (splits > 16) k_h_finish<float, 1><<<4 * tiles, block, 0, st>>>((const float*)Hp, splits, n, ldp, H);
-  else k_h_finish<float, 4><<<tiles, block, 0, st>>>((const float*)Hp, splits, n, ldp, H);
-  note_launch();
+  if (!part_f32) launch_pdl(k_h_finish<double, 4>, dim3(tiles), block, 0, st, (const double*)Hp,
+                            splits, n, ldp, H);
+  else if (splits > 16) launch_pdl(k_h_finish<float, 1>, dim3(4 * tiles), block, 0, st,
+                                   (const float*)Hp, splits, n, ldp, H);
+  else launch_pdl(k_h_finish<float, 4>, dim3(tiles), block, 0, st, (const float*)Hp, splits, n, ldp, H);
   return cudaGetLastError();
 }
 
@@ -744,7 +757,8 @@ __global__ void k_copy_pad(const double* src, double* dst, float2* dst2, int n, 
 
 cudaError_t launch_copy_pad(const double* src, double* dst, void* dst2, int n, int n_pad,
                             cudaStream_t st) {
-  return launch_pdl(k_copy_pad, dim3((n_pad + 255) / 256), dim3(256), 0, st, src, dst, (float2*)dst2, n, n_pad);
+  return launch_pdl(k_copy_pad, dim3((n_pad + 255) / 256), dim3(256), 0, st, src, dst, (float2*)dst2,
+                    n, n_pad);
 }
 
 }  // namespace nnc
@@ -886,6 +900,8 @@ __global__ void k_rev_seed_t(int m, int S, int nJ, int lam_col, const double* __
                              const double* __restrict__ p, __nv_bfloat16* __restrict__ z0,
                              __nv_bfloat16* __restrict__ z1, __nv_bfloat16* __restrict__ z2, int ld,
                              double* __restrict__ c_out, float* __restrict__ c_f) {
+  async::griddep_wait();
+  async::griddep_launch();
   const int idx = blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= m * S) return;
   const int i = idx / S, s = idx % S;
@@ -906,10 +922,8 @@ __global__ void k_rev_seed_t(int m, int S, int nJ, int lam_col, const double* __
 cudaError_t launch_rev_seed_t(int m, int S, int nJ, int lam_col, const double* s1, const double* s2,
                               const double* lam, const double* p, void* const z[3], int ld,
                               double* c_out, float* c_f, cudaStream_t st) {
-  k_rev_seed_t<<<(m * S + 255) / 256, 256, 0, st>>>(m, S, nJ, lam_col, s1, s2, lam, p,
-                                                    (__nv_bfloat16*)z[0], (__nv_bfloat16*)z[1],
-                                                    (__nv_bfloat16*)z[2], ld, c_out, c_f);
-  note_launch();
+  launch_pdl(k_rev_seed_t, dim3((m * S + 255) / 256), dim3(256), 0, st, m, S, nJ, lam_col, s1, s2, lam,
+             p, (__nv_bfloat16*)z[0], (__nv_bfloat16*)z[1], (__nv_bfloat16*)z[2], ld, c_out, c_f);
   return cudaGetLastError();
 }
 
@@ -925,6 +939,8 @@ __global__ void __launch_bounds__(256) k_rev_reduce_t(
     __nv_bfloat16* __restrict__ z0, __nv_bfloat16* __restrict__ z1, __nv_bfloat16* __restrict__ z2, int ld,
     double* __restrict__ c_out, float* __restrict__ c_f, double* __restrict__ J_out,
     double* __restrict__ g_out) {
+  async::griddep_wait();
+  async::griddep_launch();
   __shared__ double t[8][32];
   const int idx = blockIdx.x * blockDim.x + threadIdx.x, rows = blockDim.y;
   const bool in = idx < kcols * S;
@@ -968,10 +984,8 @@ cudaError_t launch_rev_reduce_t(const float* P, int splits, int kcols, int bn, i
   __nv_bfloat16* z1 = z ? (__nv_bfloat16*)z[1] : nullptr;
   __nv_bfloat16* z2 = z ? (__nv_bfloat16*)z[2] : nullptr;
   const dim3 block = splits > 16 ? dim3(32, 8) : dim3(256, 1);
-  k_rev_reduce_t<<<(kcols * S + block.x - 1) / block.x, block, 0, st>>>(P, splits, kcols, bn, S, kvalid, s1, s2,
-                                                                        lam_col, nJ, z0, z1, z2, ld, c_out,
-                                                                        c_f, J_out, g_out);
-  note_launch();
+  launch_pdl(k_rev_reduce_t, dim3((kcols * S + block.x - 1) / block.x), block, 0, st, P, splits, kcols,
+             bn, S, kvalid, s1, s2, lam_col, nJ, z0, z1, z2, ld, c_out, c_f, J_out, g_out);
   return cudaGetLastError();
 }
 
@@ -985,6 +999,8 @@ namespace nnc {
 // hi + lo of two FP32 numbers, hi = fl32(v), lo = fl32(v - hi).
 // (hi, lo) float pairs of an FP64 array (weights at load time, the network input per call).
 __global__ void k_split_df(const double* __restrict__ src, size_t n, float2* __restrict__ dst) {
+  async::griddep_wait();
+  async::griddep_launch();
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
     const double v = src[i];
     const float h = (float)v;
@@ -995,8 +1011,7 @@ __global__ void k_split_df(const double* __restrict__ src, size_t n, float2* __r
 cudaError_t launch_split_df(const double* src, size_t n, void* dst, cudaStream_t st) {
   size_t blocks = (n + 255) / 256;
   if (blocks > 4096) blocks = 4096;
-  k_split_df<<<(unsigned)blocks, 256, 0, st>>>(src, n, (float2*)dst);
-  note_launch();
+  launch_pdl(k_split_df, dim3((unsigned)blocks), dim3(256), 0, st, src, n, (float2*)dst);
   return cudaGetLastError();
 }
 

@@ -460,7 +460,8 @@ int make_plans(nnc_ws* s, int B) {
 
 template <typename T>
 void gelu(nnc_ws* s, const float* Z, int B, int cols, void* Hl, float* D1, __nv_bfloat16* Ht) {
-  launch_pdl(k_ws_gelu<T>, dim3((B * cols + 63) / 64), dim3(64), 0, s->stream, Z, B * cols, (T*)Hl, D1, cols, Ht,
+  launch_pdl(k_ws_gelu<T>, dim3((B * cols + 63) / 64), dim3(64), 0, s->stream, Z, B * cols, (T*)Hl, D1,
+             cols, Ht,
              s->cap);
 }
 
@@ -502,7 +503,8 @@ int loss_grad(nnc_ws* s, int B, double* loss) {
   const bool tcb = !std::is_same<T, float>::value && s->tc && B % 64 == 0;
   __nv_bfloat16* dZt = tcb ? s->dZt : nullptr;
   auto back = [&](const float* D, int cols, float* db) {
-    launch_pdl(k_ws_gelu_back<T>, dim3((cols + 31) / 32), dim3(32), 0, st, s->dH, D, B, cols, (T*)s->dZl, db, dZt,
+    launch_pdl(k_ws_gelu_back<T>, dim3((cols + 31) / 32), dim3(32), 0, st, s->dH, D, B, cols,
+               (T*)s->dZl, db, dZt,
                s->cap);
   };
   launch_pdl(k_ws_loss<T>, dim3((s->n_out + 31) / 32), dim3(32), 0, st, s->P, s->Tt, B, s->n_out,
@@ -772,12 +774,14 @@ int nnc_ws_train(nnc_ws* s, const double* U, const double* Tt, int N, int epochs
     for (int b0 = 0; b0 + B <= N; b0 += B) {
       const bool want = (e == epochs - 1) && (b0 + 2 * B > N);
       if (s->prec == NNC_FP32) {
-        launch_pdl(k_ws_gather<float>, gg, dim3(256), 0, st, s->Ud, s->Td, s->perm + b0, n_in, n_out, (float*)s->Ul,
+        launch_pdl(k_ws_gather<float>, gg, dim3(256), 0, st, s->Ud, s->Td, s->perm + b0, n_in, n_out,
+                   (float*)s->Ul,
                    nullptr, 0, s->Tt);
         r = loss_grad<float>(s, B, want ? &last : nullptr);
         adam<float>(s, (float)lr, (float)beta1, (float)beta2, (float)eps);
       } else {
-        launch_pdl(k_ws_gather<__nv_bfloat16>, gg, dim3(256), 0, st, s->Ud, s->Td, s->perm + b0, n_in, n_out,
+        launch_pdl(k_ws_gather<__nv_bfloat16>, gg, dim3(256), 0, st, s->Ud, s->Td, s->perm + b0, n_in,
+                   n_out,
                    (__nv_bfloat16*)s->Ul, s->tc ? s->Ut : nullptr, s->cap, s->Tt);
         r = loss_grad<__nv_bfloat16>(s, B, want ? &last : nullptr);
         adam<__nv_bfloat16>(s, (float)lr, (float)beta1, (float)beta2, (float)eps);
