@@ -208,8 +208,12 @@ __global__ void __launch_bounds__(kRvThreads, SM <= 12 ? 2 : 1) k_rev_stream(con
   const int n_cl = gridDim.y / cl;
   const uint32_t cbase = smem_u32(cpart);
   for (int idx = i0 + threadIdx.x; idx < i1; idx += kRvThreads) {
-    float v = 0.f;
-    for (int q = 0; q < cl; ++q) v += ld_dsmem_f32(cbase + idx * 4, (uint32_t)q);
+    float t[kRvMaxCluster], v = 0.f;   // the loads together, the sum in rank order
+#pragma unroll
+    for (int q = 0; q < kRvMaxCluster; ++q) t[q] = q < cl ? ld_dsmem_f32(cbase + idx * 4, (uint32_t)q) : 0.f;
+#pragma unroll
+    for (int q = 0; q < kRvMaxCluster; ++q)
+      if (q < cl) v += t[q];
     if (n_cl == 1)
       rv_boundary<SM>(a, k0 + idx / SM, idx % SM, v);
     else
