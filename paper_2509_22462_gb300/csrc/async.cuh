@@ -92,6 +92,18 @@ __device__ __forceinline__ void named_sync(int id, int threads) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
 }
 
+// The same with the barrier's number known at compile time (a number in a register reserves all 16
+// barriers, which limits the CTAs of an SM), and arriving there without waiting: the thread's earlier
+// shared-memory accesses are seen after the barrier.
+template <int ID>
+__device__ __forceinline__ void named_sync(int threads) {
+  asm volatile("bar.sync %0, %1;" ::"n"(ID), "r"(threads) : "memory");
+}
+template <int ID>
+__device__ __forceinline__ void named_arrive(int threads) {
+  asm volatile("bar.arrive %0, %1;" ::"n"(ID), "r"(threads) : "memory");
+}
+
 // Thread-block clusters: rank of this CTA, a full cluster barrier (release / acquire: shared
 // memory written before it is visible to the other CTAs after it), and a load from the shared
 // memory of CTA `rank` of the cluster at the address that `local` has in this CTA.

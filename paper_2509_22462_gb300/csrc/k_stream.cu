@@ -6,9 +6,11 @@
 // shared-memory stages with bulk asynchronous copies (cp.async.bulk completing on an mbarrier),
 // refilling a stage as soon as it has read it.  The warp's slice of the activation vector is
 // held in registers for the whole kernel, so the inner loop is shared-memory loads and FMAs only.
-// Per row each warp leaves one partial sum in shared memory; after every batch of up to 32 rows
-// the CTA synchronises and warp 0 adds the partials (in a fixed order), applies the bias and the
-// activation and writes the outputs.
+// Per row each warp leaves one partial sum in shared memory; after every batch of up to 32 rows one
+// warp adds the partials (in a fixed order), applies the bias and the activation and writes the outputs.
+// In CTAs of four warps or more that is one more warp, and the others stream on: the hundred dependent
+// FP64 operations of an activation take 2 to 3 us (70 clocks each).  Smaller CTAs have no registers to
+// spare for it; their warp 0 does it while the others wait.
 //
 // Launches use programmatic dependent launch: a layer's kernel issues its first weight copies
 // (which depend on nothing computed in the step), then waits for the previous kernel's
@@ -32,9 +34,10 @@ using namespace async;
 constexpr int kSvGroup = 512;      // bytes of a row one warp instruction covers (32 lanes x 16 B)
 constexpr int kSvMaxGroups = 8;    // groups per warp slice (4 KB)
 constexpr int kSvMaxWarps = 16;
-constexpr int kSvMaxStages = 4;
+constexpr int kSvStages = 2;       // per warp; what brings the stream to HBM speed is enough warps per SM
 constexpr int kSvBatch = 32;       // rows between CTA-wide reductions
 constexpr int kSvSlice = kSvMaxGroups * kSvGroup;
+constexpr int kSvWarpBytes = kSvStages * kSvSlice + 2 * kSvBatch * (int)sizeof(double);
 
 struct SvArgs {
   const void* W;        // [m][ldw] (hi, lo) float2 weights
@@ -48,9 +51,8 @@ struct SvArgs {
   double* s1;           // [m] sigma'(z) or NULL
   double* s2;           // [m] sigma''(z) or NULL
   int* err;             // device error word (bounded waits)
-  int nw;               // warps per CTA (= blockDim.x / 32)
+  int nw;               // streaming warps per CTA
   int gw;               // 512-byte groups per warp slice (<= kSvMaxGroups)
-  int ns;               // ring stages per warp (<= kSvMaxStages)
   int rows_per_cta;
   // grouped rows (a batch of networks stacked by rows): rows [g group_rows, (g + 1) group_rows)
   // belong to group g, whose first group_m are valid and whose activation vector starts at
@@ -61,10 +63,12 @@ struct SvArgs {
   const int* gcols;
 };
 
-__global__ void __launch_bounds__(kSvMaxWarps * 32) k_gemv_stream(const SvArgs p) {
+// NW: streaming warps at most; FIN: one more warp finishes the rows; CTAS: CTAs per SM that the registers
+// have to leave room for.
+template <int NW, bool FIN, int CTAS>
+__global__ void __launch_bounds__((NW + FIN) * 32, CTAS) k_gemv_stream(const SvArgs p) {
   extern __shared__ __align__(128) unsigned char sv_smem[];
-  __shared__ __align__(8) uint64_t full[kSvMaxWarps][kSvMaxStages];
-  __shared__ double part[kSvBatch][kSvMaxWarps];
+  __shared__ __align__(8) uint64_t full[NW][kSvStages];
   __shared__ volatile int abort_flag;
   constexpr int EB = 8;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -80,29 +84,69 @@ __global__ void __launch_bounds__(kSvMaxWarps * 32) k_gemv_stream(const SvArgs p
       (p.group_rows && p.gcols) ? min(groups, (p.gcols[grp] * EB + kSvGroup - 1) / kSvGroup) : groups;
   const int ng = max(0, min(groups_used, g0 + p.gw) - g0);  // this warp's groups
   const int slice_bytes = ng * kSvGroup;
-  unsigned char* ring = sv_smem + warp * (p.ns * kSvSlice);
-  if (p.ns < 1 || p.ns > kSvMaxStages || p.nw * 32 != (int)blockDim.x || p.nw > kSvMaxWarps ||
+  unsigned char* ring = sv_smem + warp * (kSvStages * kSvSlice);
+  double* part = reinterpret_cast<double*>(sv_smem + p.nw * kSvStages * kSvSlice);   // [2][kSvBatch][nw]
+  const int threads = blockDim.x;
+  if ((p.nw + FIN) * 32 != threads || p.nw > NW ||
       p.gw < 1 || p.gw > kSvMaxGroups)
     return;  // the launcher never builds such a configuration
 
   if (threadIdx.x == 0) abort_flag = 0;
-  if (lane == 0) {
-    for (int s = 0; s < p.ns; ++s) mbar_init(smem_u32(&full[warp][s]), 1);
+  if (lane == 0 && warp < p.nw) {
+    for (int s = 0; s < kSvStages; ++s) mbar_init(smem_u32(&full[warp][s]), 1);
     fence_mbar_init();
   }
   __syncthreads();
-  auto issue = [&](int i) {  // this warp's slice of row r0 + i into stage i % ns
-    const int s = i % p.ns;
-    const uint32_t bar = smem_u32(&full[warp][s]);
-    mbar_expect_tx(bar, (uint32_t)slice_bytes);
-    bulk_g2s(smem_u32(ring + s * kSvSlice),
-             (const unsigned char*)p.W + (size_t)(r0 + i) * row_bytes + (size_t)g0 * kSvGroup,
-             (uint32_t)slice_bytes, bar);
+  // rows r0 + b0 .. + nb of batch buffer b, one per lane
+  auto finish = [&](int b0, int nb, int b) {
+    if (lane >= nb) return;
+    const int row = r0 + b0 + lane;
+    const double* q = part + (size_t)(b * kSvBatch + lane) * p.nw;
+    double z = p.bias ? p.bias[row] : 0.0;
+    for (int w = 0; w < p.nw; ++w) z += q[w];
+    double a, d1, d2;
+    act_eval(p.act, z, a, d1, d2);
+    if (p.a_df) {
+      const float ah = (float)a;
+      p.a_df[row] = make_float2(ah, (float)(a - (double)ah));
+    }
+    if (p.a_out) p.a_out[row] = a;
+    if (p.s1) p.s1[row] = d1;
+    if (p.s2) p.s2[row] = d2;
   };
-  const int total = ng > 0 ? nrows : 0;
-  int issued = 0;  // meaningful on lane 0 only
+  // FIN: batch b's partials go to buffer b & 1; barrier 1 + (b & 1) says that they are there, 3 + (b & 1)
+  // that they have been read.  Every warp meets every barrier, also after a wait that ran out.
+  if (FIN && warp == p.nw) {
+    griddep_wait();
+    griddep_launch();
+    for (int b0 = 0, b = 0; b0 < nrows; b0 += kSvBatch, b ^= 1) {
+      if (b) named_sync<2>(threads);
+      else named_sync<1>(threads);
+      if (!abort_flag) finish(b0, min(kSvBatch, nrows - b0), b);
+      __syncwarp();
+      if (b0 + 2 * kSvBatch < nrows) {
+        if (b) named_arrive<4>(threads);
+        else named_arrive<3>(threads);
+      }
+    }
+    return;
+  }
+  // lane 0: copies of this warp's slice of successive rows, stage after stage
+  int left = ng > 0 ? nrows : 0, in_stage = 0, issued = 0;
+  const unsigned char* src =
+      (const unsigned char*)p.W + (size_t)r0 * row_bytes + (size_t)g0 * kSvGroup;
+  const uint32_t bar0 = smem_u32(&full[warp][0]), ring0 = smem_u32(ring);
+  auto issue = [&]() {
+    if (left == 0) return;
+    mbar_expect_tx(bar0 + in_stage * 8, (uint32_t)slice_bytes);
+    bulk_g2s(ring0 + in_stage * kSvSlice, src, (uint32_t)slice_bytes, bar0 + in_stage * 8);
+    src += row_bytes;
+    in_stage ^= 1;
+    --left;
+    ++issued;
+  };
   if (lane == 0)
-    for (; issued < total && issued < p.ns; ++issued) issue(issued);
+    for (int s = 0; s < kSvStages; ++s) issue();
 
   griddep_wait();    // the previous layer's activations are complete and visible
   griddep_launch();  // the next kernel in the stream may start issuing its own copies
@@ -115,14 +159,18 @@ __global__ void __launch_bounds__(kSvMaxWarps * 32) k_gemv_stream(const SvArgs p
     act[g] = g < ng ? __ldg(a4 + g * 32) : make_float4(0.f, 0.f, 0.f, 0.f);
 
   int i = 0;  // rows consumed by this warp
-  for (int b0 = 0; b0 < nrows; b0 += kSvBatch) {
-    const int nb = min(kSvBatch, nrows - b0);
-    for (int r = 0; r < nb && !abort_flag; ++r) {
+  bool ok = true;
+  for (int b0 = 0, b = 0; b0 < nrows; b0 += kSvBatch, b ^= 1) {
+    const int nb = min(kSvBatch, nrows - b0), buf = FIN ? b : 0;
+    if (FIN && b0 >= 2 * kSvBatch) {
+      if (b) named_sync<4>(threads);
+      else named_sync<3>(threads);
+    }
+    for (int r = 0; r < nb && ok; ++r) {
       float q0 = 0.f, q1 = 0.f, q2 = 0.f, q3 = 0.f;
       if (ng > 0) {
-        const int s = i % p.ns;
-        bool ok = mbar_wait(smem_u32(&full[warp][s]), (uint32_t)(i / p.ns) & 1u, p.err, 21);
-        ok = __all_sync(0xffffffffu, ok);
+        const uint32_t s = (uint32_t)i & 1u;
+        ok = __all_sync(0xffffffffu, mbar_wait(bar0 + s * 8, (uint32_t)(i >> 1) & 1u, p.err, 21));
         if (!ok) {
           abort_flag = 1;
           break;
@@ -138,42 +186,47 @@ __global__ void __launch_bounds__(kSvMaxWarps * 32) k_gemv_stream(const SvArgs p
         }
         __syncwarp();
         ++i;
-        if (lane == 0 && issued < total) {  // refill the stage just read
+        if (lane == 0) {  // refill the stage just read
           fence_proxy_async();
-          issue(issued);
-          ++issued;
+          issue();
         }
       }
       // warp reduction of the two double-float sums (q0, q1), (q2, q3) in FP32 operations
       df_add(q0, q1, q2, q3);
       warp_sum_df(q0, q1);
-      if (lane == 0) part[r][warp] = (double)q0 + (double)q1;
+      if (lane == 0) part[(size_t)(buf * kSvBatch + r) * p.nw + warp] = (double)q0 + (double)q1;
     }
-    __syncthreads();
-    if (abort_flag) break;
-    if (warp == 0 && lane < nb) {
-      const int row = r0 + b0 + lane;
-      double z = p.bias ? p.bias[row] : 0.0;
-      for (int w = 0; w < p.nw; ++w) z += part[lane][w];
-      double a, d1, d2;
-      act_eval(p.act, z, a, d1, d2);
-      if (p.a_out) p.a_out[row] = a;
-      if (p.a_df) {
-        const float ah = (float)a;
-        p.a_df[row] = make_float2(ah, (float)(a - (double)ah));
-      }
-      if (p.s1) p.s1[row] = d1;
-      if (p.s2) p.s2[row] = d2;
+    __syncwarp();
+    if (FIN) {
+      if (b) named_arrive<2>(threads);
+      else named_arrive<1>(threads);
+    } else {
+      __syncthreads();
+      if (warp == 0 && !abort_flag) finish(b0, nb, 0);
+      __syncthreads();
     }
-    __syncthreads();
   }
-  if (abort_flag && lane == 0) {
+  if (!ok && lane == 0) {
     // a wait ran out: let this warp's copies still in flight land (short bound) before the
     // stages go away
     for (int k = i; k < issued; ++k)
-      mbar_wait(smem_u32(&full[warp][k % p.ns]), (uint32_t)(k / p.ns) & 1u, p.err, 22,
-                kWaitCycles / 8);
+      mbar_wait(bar0 + (k & 1) * 8, (uint32_t)(k >> 1) & 1u, p.err, 22, kWaitCycles / 8);
   }
+}
+
+template <int NW, bool FIN, int CTAS>
+cudaError_t launch_sv_t(const SvArgs& a, int grid, int smem, cudaStream_t st) {
+  static bool attr = false;
+  if (!attr) {
+    cudaError_t e = cudaFuncSetAttribute(k_gemv_stream<NW, FIN, CTAS>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, NW * kSvWarpBytes);
+    if (e != cudaSuccess) return e;
+    e = cudaFuncSetAttribute(k_gemv_stream<NW, FIN, CTAS>,
+                             cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+    if (e != cudaSuccess) return e;
+    attr = true;
+  }
+  return launch_pdl(k_gemv_stream<NW, FIN, CTAS>, dim3(grid), dim3((a.nw + FIN) * 32), smem, st, a);
 }
 
 cudaError_t launch_sv(SvArgs a, int sm_count, cudaStream_t st) {
@@ -185,24 +238,11 @@ cudaError_t launch_sv(SvArgs a, int sm_count, cudaStream_t st) {
   // Two stages per warp suffice; what brings the stream to HBM speed is enough warps per SM
   // (3-4 CTAs): measured at 6.3 TB/s on a 1 GB matrix (6.6 TB/s with FP32 weights).  (Four stages
   // for one-warp CTAs, the 2 KB rows of a batch's first layer, measured slower: 216 against 154 us.)
-  a.ns = 2;
-  const int smem = a.nw * a.ns * kSvSlice;
-  static bool attr = false;
-  if (!attr) {
-    cudaError_t e = cudaFuncSetAttribute(k_gemv_stream,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         kSvMaxWarps * 3 * kSvSlice);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k_gemv_stream, cudaFuncAttributePreferredSharedMemoryCarveout,
-                             100);
-    if (e != cudaSuccess) return e;
-    attr = true;
-  }
-  if (smem > kSvMaxWarps * 3 * kSvSlice || a.ns > kSvMaxStages || a.gw > kSvMaxGroups)
-    return cudaErrorInvalidValue;
+  const int smem = a.nw * kSvWarpBytes;
+  if (a.gw > kSvMaxGroups) return cudaErrorInvalidValue;
   // CTAs per SM from shared memory (about 200 KB usable with the static part) and warps: layers
   // with short rows (few warps per CTA) get more CTAs per SM, so more copies are in flight
-  const int per_sm = std::max(1, std::min({12, 200 * 1024 / smem, 48 / a.nw}));
+  const int per_sm = std::max(1, std::min({12, 208 * 1024 / smem, 48 / a.nw}));
   int used;
   if (a.group_rows > 0) {
     // grouped: rows per CTA a power of two dividing group_rows (a multiple of 128), chosen so
@@ -227,19 +267,9 @@ cudaError_t launch_sv(SvArgs a, int sm_count, cudaStream_t st) {
     a.rows_per_cta = (a.m + grid - 1) / grid;
     used = (a.m + a.rows_per_cta - 1) / a.rows_per_cta;
   }
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(used);
-  cfg.blockDim = dim3(a.nw * 32);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  const cudaError_t e = cudaLaunchKernelEx(&cfg, k_gemv_stream, a);
-  note_launch();
-  return e != cudaSuccess ? e : cudaGetLastError();
+  if (a.nw < 4) return launch_sv_t<3, false, 8>(a, used, smem, st);
+  if (a.nw <= 8) return launch_sv_t<8, true, 3>(a, used, smem, st);
+  return launch_sv_t<kSvMaxWarps, true, 1>(a, used, smem, st);
 }
 
 // Self-test of the bounded wait: an mbarrier that nothing arrives on, waited for `limit` cycles;
@@ -267,7 +297,7 @@ cudaError_t launch_gemv_stream_df(const void* W2, int ldw, int m, const double* 
                                   int act, double* a_out, void* a_df, double* s1, double* s2,
                                   int* err, int sm_count, cudaStream_t st) {
   if (ldw % kPad) return cudaErrorInvalidValue;
-  SvArgs a{W2, ldw, m, b, a_in2, act, a_out, (float2*)a_df, s1, s2, err, 0, 0, 0, 0, 0, 0, 0,
+  SvArgs a{W2, ldw, m, b, a_in2, act, a_out, (float2*)a_df, s1, s2, err, 0, 0, 0, 0, 0, 0,
            nullptr};
   return launch_sv(a, sm_count, st);
 }
@@ -278,7 +308,7 @@ cudaError_t launch_gemv_stream_df_grouped(const void* W2, int ldw, int groups, i
                                           int* err, int sm_count, cudaStream_t st, const int* gcols) {
   if (ldw % kPad || mp % kPad || ld_in % kPad || groups < 1 || m < 1 || m > mp)
     return cudaErrorInvalidValue;
-  SvArgs a{W2, ldw, groups * mp, b, a_in2, act, a_out, (float2*)a_df, s1, s2, err, 0, 0, 0, 0,
+  SvArgs a{W2, ldw, groups * mp, b, a_in2, act, a_out, (float2*)a_df, s1, s2, err, 0, 0, 0,
            mp, m, ld_in, gcols};
   return launch_sv(a, sm_count, st);
 }
