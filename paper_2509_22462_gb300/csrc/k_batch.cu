@@ -42,7 +42,8 @@ cudaError_t launch_bx_scatter(const double* xcat, const int* gn, const int* goff
 // Reverse step of every group: part[g][c][kk][s] = sum_{r in chunk c} W_g[r][kk] Zbar_g[r][s]
 // (FP32 weights, FP32 seeds), up to 256 threads x 4 columns per block (fewer for short rows, so
 // that no thread of a block is idle), 64 rows per chunk.  Larger chunks cut the partial-sum
-// traffic but leave too few blocks to stream the weights at full rate.
+// traffic but leave too few blocks to stream the weights at full rate.  Eight rows' loads are in flight, the
+// first ones before the seeds are there.
 constexpr int kBRowsMax = 64;
 __host__ __device__ constexpr int brev_rows(int) { return 64; }
 template <int SMAX>
@@ -50,14 +51,24 @@ __global__ void __launch_bounds__(256) k_bgemv_rev(const float* __restrict__ W, 
                                                    int m, const double* __restrict__ Zbar, int S,
                                                    int chunks, float* __restrict__ part,
                                                    const int* __restrict__ gcols) {
-  async::griddep_wait();
-  async::griddep_launch();
   __shared__ float zs[kBRowsMax][SMAX];
   const int rows = brev_rows(ldw);
   const int g = blockIdx.z;
   const int c0 = (blockIdx.x * blockDim.x + threadIdx.x) * 4;
   const int r0 = blockIdx.y * rows;
   const int nr = min(rows, m - r0);
+  // columns past the net's own (zero padding of a first layer): zero partials, no weight reads
+  const bool any = nr > 0 && c0 < ldw && !(gcols && c0 >= gcols[g]);
+  const float* wp = W + ((size_t)g * mp + r0) * ldw + c0;
+  float4 w[8];
+  auto load = [&](int r) {
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      if (r + u < nr) w[u] = __ldg(reinterpret_cast<const float4*>(wp + (size_t)(r + u) * ldw));
+  };
+  if (any) load(0);   // the weights depend on nothing computed before
+  async::griddep_wait();
+  async::griddep_launch();
   const double* zg = Zbar + (size_t)g * mp * S;
   for (int i = threadIdx.x; i < rows * SMAX; i += blockDim.x) {
     const int r = i / SMAX, s = i % SMAX;
@@ -66,8 +77,7 @@ __global__ void __launch_bounds__(256) k_bgemv_rev(const float* __restrict__ W, 
   __syncthreads();
   if (c0 >= ldw) return;
   float* out = part + (((size_t)g * chunks + blockIdx.y) * ldw + c0) * S;
-  // columns past the net's own (zero padding of a first layer): zero partials, no weight reads
-  if (nr <= 0 || (gcols && c0 >= gcols[g])) {
+  if (!any) {
     for (int i = 0; i < 4 * S; ++i) out[i] = 0.f;
     return;
   }
@@ -76,18 +86,21 @@ __global__ void __launch_bounds__(256) k_bgemv_rev(const float* __restrict__ W, 
   for (int v = 0; v < 4; ++v)
 #pragma unroll
     for (int s = 0; s < SMAX; ++s) acc[v][s] = 0.f;
-  const float* wp = W + ((size_t)g * mp + r0) * ldw + c0;
-#pragma unroll 4
-  for (int r = 0; r < nr; ++r) {
-    const float4 w = __ldg(reinterpret_cast<const float4*>(wp + (size_t)r * ldw));
+  for (int r = 0; r < nr; r += 8) {
 #pragma unroll
-    for (int s = 0; s < SMAX; ++s) {
-      const float z = zs[r][s];
-      acc[0][s] = fmaf(w.x, z, acc[0][s]);
-      acc[1][s] = fmaf(w.y, z, acc[1][s]);
-      acc[2][s] = fmaf(w.z, z, acc[2][s]);
-      acc[3][s] = fmaf(w.w, z, acc[3][s]);
+    for (int u = 0; u < 8; ++u) {
+      if (r + u < nr) {
+#pragma unroll
+        for (int s = 0; s < SMAX; ++s) {
+          const float z = zs[r + u][s];
+          acc[0][s] = fmaf(w[u].x, z, acc[0][s]);
+          acc[1][s] = fmaf(w[u].y, z, acc[1][s]);
+          acc[2][s] = fmaf(w[u].z, z, acc[2][s]);
+          acc[3][s] = fmaf(w[u].w, z, acc[3][s]);
+        }
+      }
     }
+    load(r + 8);
   }
 #pragma unroll
   for (int v = 0; v < 4; ++v)
