@@ -127,7 +127,7 @@ struct nnc_net {
   int* dev_err = nullptr;    // device error word of bounded waits
   double* h_stage = nullptr; // pinned host staging
   size_t h_stage_elems = 0;
-  // pinned staging of a small net's host outputs (y, J, H, gradient, residual), and its device address
+  // behind it, pinned staging of a small net's host outputs, and its device address
   double *h_out = nullptr, *h_out_dev = nullptr;
   size_t bytes = 0;
   // optional per-kernel-kind CUDA-event timing (nnc_profile)

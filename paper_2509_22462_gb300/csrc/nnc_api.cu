@@ -772,7 +772,6 @@ void nnc_free(nnc_net* net) {
   for (void* p : net->allocs) cudaFree(p);
   for (cudaEvent_t e : net->ev_pool) cudaEventDestroy(e);
   if (net->h_stage) cudaFreeHost(net->h_stage);
-  if (net->h_out) cudaFreeHost(net->h_out);
   if (net->side_stream) {
     cudaStreamSynchronize(net->side_stream);
     cudaStreamDestroy(net->side_stream);
@@ -1130,12 +1129,15 @@ static int load_impl(nnc_net* net, int n_layers, const int* widths, const int* a
     AL(hp, (size_t)splits * n * n);
     net->Hp = hp;
   }
-  // pinned staging of the host calls: x [n_in_pad] | lambda [n_out] | y [n_out] | error word
+  // pinned staging of the host calls: x [n_in_pad] | lambda [n_out] | y [n_out] | error word, and, where
+  // they take at most 256 KB, the outputs y, J, H, gradient and residual (one block: page-locking costs
+  // a millisecond a call)
   net->h_stage_elems = (size_t)net->n_in_pad + 2 * (size_t)net->n_out + 1;
-  CK(cudaMallocHost(&net->h_stage, sizeof(double) * net->h_stage_elems));
-  const size_t n_out_all = (size_t)n * n + (size_t)(net->n_out + 1) * n + 2 * (size_t)net->n_out;
-  if (n_out_all * sizeof(double) <= 256 * 1024) {
-    CK(cudaMallocHost(&net->h_out, sizeof(double) * n_out_all));
+  size_t n_outs = (size_t)n * n + (size_t)(net->n_out + 1) * n + 2 * (size_t)net->n_out;
+  if (n_outs * sizeof(double) > 256 * 1024) n_outs = 0;
+  CK(cudaMallocHost(&net->h_stage, sizeof(double) * (net->h_stage_elems + n_outs)));
+  if (n_outs > 0) {
+    net->h_out = net->h_stage + net->h_stage_elems;
     CK(cudaHostGetDevicePointer((void**)&net->h_out_dev, net->h_out, 0));
   }
   CK(cudaStreamSynchronize(net->stream));
