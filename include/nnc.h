@@ -50,7 +50,14 @@ typedef enum {
 } nnc_status;
 
 /* Number format of the network evaluation (Section 5.1 leaves it unstated).
- *   NNC_FP64   : every kernel in FP64 (value, Jacobian, Hessian).  The reference form.
+ *   NNC_FP64   : FP64 weights, value pass and outputs; the reference form.  The products of the
+ *                Jacobian, the gradient and the Hessian run on the tensor cores by residues: operands
+ *                are integers of 50 (65536-wide layers) to 57 bits (up to 1024) below the largest entry
+ *                of a row, after powers of two have evened out the weights' columns, and the integer
+ *                sums are exact.  The error of a column is that of an FP64 sum of normally distributed
+ *                terms, whatever the units of inputs, hidden units and outputs.  Weights that powers of
+ *                two do not even out, such as sparse ones, and nets whose residues do not fit in
+ *                memory have FP64 products instead.
  *   NNC_FP32   : FP32 weights and tangents on CUDA cores, FP32 products, FP64 outputs.
  *   NNC_BF16   : value/Jacobian/adjoint in FP32; Hessian sweep on tcgen05 tensor cores with
  *                BF16 operands and FP32 accumulation (one product per tile).

@@ -5,7 +5,12 @@
 // 104M-parameter evaluation in an FP64 GEMM on the CUDA cores.  The residue scheme of Ozaki, Uchino
 // and Imamura ("Ozaki scheme II", 2025) does them with integer products instead:
 //   - every row of either operand is scaled by a power of two and rounded to integers of at most
-//     `bits` + 1 bits (bits = 52 for K = 4096 with 15 moduli: the rounding is that of FP64);
+//     `bits` + 1 bits below its largest entry (bits = 57 for K <= 1024 with 16 moduli, 52 for K = 4096
+//     with 15);
+//   - so an entry 2^j below its row's largest has j bits fewer.  Powers of two even out the columns of the
+//     weights beforehand (k_rns_colsum), which makes the rounding independent of the units in which
+//     inputs, hidden units and outputs are measured; weights that stay uneven (k_rns_spread) keep the
+//     FP64 products;
 //   - an integer is kept as its residues modulo 15 (or 16) pairwise coprime numbers p_i <= 256, each
 //     in [-p/2, p/2], which BF16 holds exactly;
 //   - one BF16 product per modulus gives the result's residue: products are at most 2^14, so 1024
@@ -142,6 +147,11 @@ struct Crt {
   }
 };
 
+// The biased exponent of v 2^d from that of v.
+__device__ __forceinline__ int shift_expo(int e, int d) {
+  return e == 0x7FF ? e : min(max(e + d, 0), 0x7FF);
+}
+
 __device__ __forceinline__ int block_max(int v, int* sh) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   v = __reduce_max_sync(0xffffffffu, v);
@@ -152,23 +162,142 @@ __device__ __forceinline__ int block_max(int v, int* sh) {
   __syncthreads();
   return r;
 }
+__device__ __forceinline__ int block_sum(int v, int* sh) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  v = __reduce_add_sync(0xffffffffu, v);
+  if (lane == 0) sh[warp] = v;
+  __syncthreads();
+  int r = 0;
+  for (int w = 0; w < (int)(blockDim.x >> 5); ++w) r += sh[w];
+  __syncthreads();
+  return r;
+}
 
 // ------------------------------------------------------------------ weights (once, at load)
+// Column exponents.  A row of W is rounded relative to its largest entry, so a column that is small in
+// every row (an input in small units, the outgoing weights of a hidden unit in large ones) would lose
+// what it is smaller by: inputs spread over 2^40 left 1e-6 of a column of J, where FP64 products leave
+// 2e-15.  2^de[k] is the geometric mean of column k's entries in units of the first column's, which sees
+// through rows of any size.  The mean is taken of 16 bits of mantissa behind the exponent, in integers, so
+// that the order of the sums does not matter.  A matrix whose means all lie within 2^2.5 of the first one,
+// as those of evenly scaled weights do, stays as it is (784 -> 128 x 2 -> 10 takes 129 us with its
+// exponents of -1, 0 and 1, 126 without).
+struct RnsEven {
+  unsigned long long* sum;   // [k] of the nonzero entries' logarithms, times 2^16
+  int *cnt, *small;          // [k] nonzero entries; entries in nonzero rows that are small there
+  unsigned long long* total; // [3] entries looked at, small ones, nonzero rows
+};
+constexpr int kEvenRows = 256;   // rows of W per CTA
+
+__global__ void __launch_bounds__(256) k_rns_colsum(const double* __restrict__ W, int ldw, int m, int k,
+                                                    const RnsEven e, int* __restrict__ flags) {
+  __shared__ unsigned long long s[8][32];
+  __shared__ int c[8][32];
+  const int col = blockIdx.x * 32 + threadIdx.x, y = threadIdx.y;
+  const int r1 = min(m, (int)(blockIdx.y + 1) * kEvenRows);
+  unsigned long long sum = 0;
+  int cnt = 0;
+  bool odd = false;
+  if (col < k) {
+    for (int r = blockIdx.y * kEvenRows + y; r < r1; r += 8) {
+      const double w = W[(size_t)r * ldw + col];
+      const int ex = expo(w);
+      // the exponents of products and scales stay in range for weights of 2^-200 to 2^200
+      odd |= w != 0.0 && (ex < 1023 - 200 || ex > 1023 + 200);
+      if (ex > 0) {
+        sum += (unsigned)(__double2hiint(w) & 0x7FFFFFFF) >> 4;
+        ++cnt;
+      }
+    }
+  }
+  if (odd) atomicOr(flags, kRnsUneven);
+  s[y][threadIdx.x] = sum;
+  c[y][threadIdx.x] = cnt;
+  __syncthreads();
+  if (y > 0 || col >= k) return;
+  for (int j = 1; j < 8; ++j) {
+    sum += s[j][threadIdx.x];
+    cnt += c[j][threadIdx.x];
+  }
+  atomicAdd(e.sum + col, sum);
+  atomicAdd(e.cnt + col, cnt);
+}
+
+__global__ void __launch_bounds__(256) k_rns_colexp(int k, const RnsEven e, int* __restrict__ de,
+                                                    int* __restrict__ flags) {
+  const int col = blockIdx.x * 256 + threadIdx.x;
+  if (col >= k) return;
+  int q = 0;   // the first column that is not zero
+  while (q < k - 1 && e.cnt[q] == 0) ++q;
+  int d = 0;
+  if (e.cnt[col] > 0) {   // sum / cnt against sum_q / cnt_q, to nearest: |difference| < 2^59
+    const long long c = e.cnt[col], cq = e.cnt[q], den = c * cq << 16;
+    const long long num = 2 * ((long long)e.sum[col] * cq - (long long)e.sum[q] * c) + den;
+    d = (int)(num >= 0 ? num / (2 * den) : -((2 * den - 1 - num) / (2 * den)));
+  }
+  de[col] = d;
+  if (abs(d) > 2) atomicOr(flags, kRnsScaled);
+}
+
+// How uneven W 2^-de is: an entry is small if it lies more than 2^(bits - 44) below its row's largest, so
+// that fewer than 44 of its bits are kept.  Sums in which such entries are outnumbered lose nothing to
+// speak of (a few percent of normally distributed entries are small); a row or column that consists of
+// them would.  So of 64 entries or more in a row or a column at most a quarter may be small, of 16 or
+// more half, and of the whole matrix a quarter.  Rows and columns of zeros do not count.
+__device__ __forceinline__ bool rns_uneven(int small, int n) {
+  return n >= 64 ? 4 * (long long)small > n : n >= 16 && 2 * small > n;
+}
+__global__ void __launch_bounds__(256) k_rns_spread(const double* __restrict__ W, int ldw, int k, int bits,
+                                                    const int* __restrict__ de, const RnsEven e,
+                                                    int* __restrict__ flags) {
+  __shared__ int sh[8];
+  const double* w = W + (size_t)blockIdx.x * ldw;
+  int ex = 0;
+  for (int j = threadIdx.x; j < k; j += 256)
+    if (expo(w[j]) > 0) ex = max(ex, expo(w[j]) - de[j]);
+  ex = block_max(ex, sh);
+  if (ex <= 0) return;   // a row of zeros
+  int small = 0, n = 0;
+  for (int j = threadIdx.x; j < k; j += 256) {
+    if (e.cnt[j] == 0) continue;
+    ++n;
+    if (expo(w[j]) == 0 || expo(w[j]) - de[j] < ex - (bits - 44)) {
+      ++small;
+      atomicAdd(e.small + j, 1);
+    }
+  }
+  n = block_sum(n, sh);
+  small = block_sum(small, sh);
+  if (threadIdx.x == 0) {
+    if (rns_uneven(small, n)) atomicOr(flags, kRnsUneven);
+    atomicAdd(e.total, (unsigned long long)n);
+    atomicAdd(e.total + 1, (unsigned long long)small);
+    atomicAdd(e.total + 2, 1ull);
+  }
+}
+__global__ void __launch_bounds__(256) k_rns_colspread(int k, const RnsEven e, int* __restrict__ flags) {
+  const int col = blockIdx.x * 256 + threadIdx.x;
+  if (col < k && rns_uneven(e.small[col], (int)e.total[2])) atomicOr(flags, kRnsUneven);
+  if (col == 0 && 4 * e.total[1] > e.total[0]) atomicOr(flags, kRnsUneven);
+}
+
 __global__ void __launch_bounds__(256) k_rns_pack(const __grid_constant__ RnsSet s,
                                                   const double* __restrict__ W, int mp, int kp,
+                                                  const int* __restrict__ de,
                                                   __nv_bfloat16* __restrict__ res,
                                                   double* __restrict__ sa) {
   __shared__ int sh[8];
   const int r = blockIdx.x;
   const double* w = W + (size_t)r * kp;
   int ex = 0, sc;
-  for (int k = threadIdx.x; k < kp; k += blockDim.x) ex = max(ex, expo(w[k]));
+  for (int k = threadIdx.x; k < kp; k += blockDim.x)
+    if (expo(w[k]) > 0) ex = max(ex, expo(w[k]) - (de ? de[k] : 0));
   const double back = rns_scale(block_max(ex, sh), s.bits, &sc);
   if (threadIdx.x == 0) sa[r] = back;
   for (int k = 4 * threadIdx.x; k < kp; k += 4 * blockDim.x) {
     Limbs l[4];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) l[j] = rns_limbs(to_int(w[k + j], sc));
+    for (int j = 0; j < 4; ++j) l[j] = rns_limbs(to_int(w[k + j], sc - (de ? de[k + j] : 0)));
 #pragma unroll 4
     for (int i = 0; i < s.n; ++i) {
       float v[4];
@@ -187,7 +316,8 @@ __global__ void __launch_bounds__(256) k_rns_pack(const __grid_constant__ RnsSet
 // takes sqrt|c| z on both sides (sign(c) on one) so that one scale per row fits every column.
 // Bound: 90 bytes written per element (15 residues x 3 operands) and about 450 instructions; four of them
 // on the FP64 pipe.
-template <bool CRT>
+// DE: the next layer's weights have column exponents.
+template <bool CRT, bool DE>
 __global__ void __launch_bounds__(256) k_rns_rows(const __grid_constant__ RnsSet set,
                                                   const RnsRows a) {
   __shared__ int sh[8];
@@ -219,9 +349,14 @@ __global__ void __launch_bounds__(256) k_rns_rows(const __grid_constant__ RnsSet
 #pragma unroll
       for (int j = 0; j < 4; ++j) z[j] = zrow[k + j];
     }
+    int d[4];
+    if (DE) *reinterpret_cast<int4*>(d) = __ldg(reinterpret_cast<const int4*>(a.de + k));
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-      if (a.At) ha = max(ha, prod_expo(__ldg(a.s1 + k + j), z[j]));
+      if (a.At) {
+        const int e = prod_expo(__ldg(a.s1 + k + j), z[j]);
+        ha = max(ha, DE ? shift_expo(e, d[j]) : e);
+      }
       if (a.Sa) hs = max(hs, prod_expo(__ldg(a.rc + k + j), z[j]));
     }
   }
@@ -242,8 +377,10 @@ __global__ void __launch_bounds__(256) k_rns_rows(const __grid_constant__ RnsSet
     const size_t o = (size_t)r * a.K + k;
     if (a.At) {
       Limbs l[4];
+      int d[4] = {0, 0, 0, 0};
+      if (DE) *reinterpret_cast<int4*>(d) = __ldg(reinterpret_cast<const int4*>(a.de + k));
 #pragma unroll
-      for (int j = 0; j < 4; ++j) l[j] = rns_limbs(to_int(__ldg(a.s1 + k + j) * z[j], sca));
+      for (int j = 0; j < 4; ++j) l[j] = rns_limbs(to_int(__ldg(a.s1 + k + j) * z[j], sca + d[j]));
       __nv_bfloat16* dst = (__nv_bfloat16*)a.At + o;
 #pragma unroll 5
       for (int i = 0; i < set.n; ++i)
@@ -287,7 +424,9 @@ __global__ void __launch_bounds__(256) k_rns_rows(const __grid_constant__ RnsSet
 // seed (the row scales of that layer's weights are multiplied in, since its product sums over rows).
 // First layer: J and the gradient instead.  Bound: latency, so a thread has one column up to 4096, and
 // its loads, twenty at a time, are in flight together.
+// DE: the weights just multiplied have column exponents.
 constexpr int kRevCl = 8;
+template <bool DE>
 __global__ void __launch_bounds__(512) k_rns_rev_rows(const __grid_constant__ RnsSet set,
                                                       const RnsRev a) {
   __shared__ int sh[16], mine;
@@ -302,6 +441,7 @@ __global__ void __launch_bounds__(512) k_rns_rev_rows(const __grid_constant__ Rn
   for (int k = k0; k < a.K; k += step) {
     double z;
     if (a.C) {
+      const int de = DE ? __ldg(a.de + k) : 0;
       Crt t;
       const unsigned char* c = a.C + (size_t)s * a.K + k;
       const size_t plane = (size_t)a.seeds * a.K;
@@ -327,7 +467,8 @@ __global__ void __launch_bounds__(512) k_rns_rev_rows(const __grid_constant__ Rn
           }
         }
       }
-      const double v = t.value() * (set.scale * a.sb[s]);
+      double v = t.value() * (set.scale * a.sb[s]);
+      if (DE) v *= __hiloint2double((de + 1023) << 20, 0);
       if (!a.s1) {
         if (k < a.kvalid) {
           if (a.J && s < a.nJ) a.J[(size_t)s * a.kvalid + k] = v;
@@ -753,8 +894,8 @@ cudaError_t launch_gemm(const RnsPlan& p, const RnsGemm& g, int grid, cudaStream
 
 RnsSet rns_set(int K) {
   // 15 moduli leave 52 bits at K = 4096; products of fewer terms, whose FP64 sums round less often,
-  // take a 16th (57 bits at K = 1024): the error stays below that of an FP64 sum over the whole
-  // range, and the added product costs 7 % where launches, not products, set the time.
+  // take a 16th (57 bits at K = 1024): with even rows (k_rns_spread) the error stays near that of an FP64
+  // sum, and the added product costs 7 % where launches, not products, set the time.
   RnsSet s;
   s.n = K <= 1024 ? 16 : 15;
   double bits = 0.0, P = 1.0;
@@ -872,9 +1013,29 @@ cudaError_t rns_gemm(const RnsPlan& p, const RnsSet& s, unsigned char* C, int ld
   }
 }
 
-cudaError_t rns_pack_weights(const RnsSet& s, const double* W, int mp, int kp, void* res, double* sa,
-                             cudaStream_t st) {
-  k_rns_pack<<<mp, 256, 0, st>>>(s, W, mp, kp, (__nv_bfloat16*)res, sa);
+size_t rns_even_scratch(int k) { return (size_t)k * 16 + 24; }
+
+cudaError_t rns_even_out(const RnsSet& s, const double* W, int ldw, int m, int k, void* scratch, int* de,
+                         int* flags, cudaStream_t st) {
+  RnsEven e;
+  e.sum = (unsigned long long*)scratch;
+  e.total = e.sum + k;
+  e.cnt = (int*)(e.total + 3);
+  e.small = e.cnt + k;
+  const cudaError_t r = cudaMemsetAsync(scratch, 0, rns_even_scratch(k), st);
+  if (r != cudaSuccess) return r;
+  k_rns_colsum<<<dim3((k + 31) / 32, (m + kEvenRows - 1) / kEvenRows), dim3(32, 8), 0, st>>>(W, ldw, m, k, e,
+                                                                                             flags);
+  k_rns_colexp<<<(k + 255) / 256, 256, 0, st>>>(k, e, de, flags);
+  k_rns_spread<<<m, 256, 0, st>>>(W, ldw, k, s.bits, de, e, flags);
+  k_rns_colspread<<<(k + 255) / 256, 256, 0, st>>>(k, e, flags);
+  note_launch(4);
+  return cudaGetLastError();
+}
+
+cudaError_t rns_pack_weights(const RnsSet& s, const double* W, int mp, int kp, const int* de, void* res,
+                             double* sa, cudaStream_t st) {
+  k_rns_pack<<<mp, 256, 0, st>>>(s, W, mp, kp, de, (__nv_bfloat16*)res, sa);
   note_launch();
   return cudaGetLastError();
 }
@@ -882,8 +1043,9 @@ cudaError_t rns_pack_weights(const RnsSet& s, const double* W, int mp, int kp, v
 cudaError_t rns_rows(const RnsSet& s, const RnsRows& a, cudaStream_t st) {
   if (a.K % 128 || a.n < 1 || (a.ldz & 1)) return cudaErrorInvalidValue;
   const int threads = std::min(256, std::max(32, a.K / 4));
-  return a.C ? launch_pdl(k_rns_rows<true>, dim3(a.n), dim3(threads), 0, st, s, a)
-             : launch_pdl(k_rns_rows<false>, dim3(a.n), dim3(threads), 0, st, s, a);
+  auto kernel = a.At && a.de ? (a.C ? k_rns_rows<true, true> : k_rns_rows<false, true>)
+                             : (a.C ? k_rns_rows<true, false> : k_rns_rows<false, false>);
+  return launch_pdl(kernel, dim3(a.n), dim3(threads), 0, st, s, a);
 }
 
 cudaError_t rns_rev_rows(const RnsSet& s, const RnsRev& a, int S, cudaStream_t st) {
@@ -901,7 +1063,7 @@ cudaError_t rns_rev_rows(const RnsSet& s, const RnsRev& a, int S, cudaStream_t s
   at[0].val.clusterDim.z = 1;
   cfg.attrs = at;
   cfg.numAttrs = 2;
-  const cudaError_t e = cudaLaunchKernelEx(&cfg, k_rns_rev_rows, s, a);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, a.C && a.de ? k_rns_rev_rows<true> : k_rns_rev_rows<false>, s, a);
   note_launch();
   return e != cudaSuccess ? e : cudaGetLastError();
 }

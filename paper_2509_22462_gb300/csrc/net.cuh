@@ -52,6 +52,7 @@ struct LayerDev {
   // plans of its products, and its residue plane of H
   void* Wr = nullptr;
   double* wr_scale = nullptr;
+  int* wr_de = nullptr;           // exponents of its columns [kp], NULL if all are zero
   nnc::RnsPlan plan_rt, plan_rs, plan_rr;   // tangents, symmetric product, reverse
   int h_plane = -1;
 };

@@ -250,6 +250,7 @@ int run_reverse(nnc_net* net, bool fp64, int nJ, bool with_lam, const double* la
       PROF(PK_REV);
       CK(rns_gemm(Ly.plan_rr, net->rset, net->Cv, Ly.kp, net->dev_err, net->sm_count, st));
       a.C = net->Cv;
+      a.de = Ly.wr_de;
       a.chunks = (Ly.mp + 1023) / 1024;
       a.sb = a.sb_out;
       a.sb_out = net->zr_scale + (l % 2 == net->L % 2 ? 0 : 48);
@@ -511,6 +512,7 @@ int run_hessian_rns(nnc_net* net, const double* lam, double* H, cudaStream_t st)
     if (!last) {
       a.At = net->Rt;
       a.sat = net->rt_scale;
+      a.de = net->layers[l + 1].wr_de;
     }
     if (Ly.zy_off >= 0) {
       a.c = net->c64 + Ly.zy_off;
@@ -783,8 +785,9 @@ void nnc_free(nnc_net* net) {
 }
 
 // Buffers, residues and plans of the FP64 form's residue products.  They take 30 to 32 bytes per
-// weight beside the 8 of the FP64 weights; where that is more than half of the free memory, the
-// CUDA-core products stay in use (net->rns false).
+// weight beside the 8 of the FP64 weights; where that is more than half of the free memory, or where the
+// residues of the weights would keep too few bits (rns_even_out), the CUDA-core products stay in use
+// (net->rns false).
 static int load_rns(nnc_net* net) {
   const int n = net->n_in, L = net->L;
   int planes = 0, k_max = net->n_in_pad;
@@ -807,8 +810,25 @@ static int load_rns(nnc_net* net) {
   size_t free_b = 0, total_b = 0;
   CK(cudaMemGetInfo(&free_b, &total_b));
   if (need > free_b / 2) return NNC_OK;
-  net->rns = true;
   unsigned char* p;
+  // the layers' column exponents, and whether the weights are even enough
+  int *flags, *de;
+  std::vector<int> hflags(L);
+  AL(flags, L);
+  AL(p, rns_even_scratch(k_max));
+  for (int l = 0; l < L; ++l) {
+    LayerDev& Ly = net->layers[l];
+    AL(de, Ly.kp);
+    Ly.wr_de = de;
+    CK(rns_even_out(net->rset, Ly.W64, Ly.kp, Ly.m, Ly.k, p, de, flags + l, net->stream));
+  }
+  CK(cudaMemcpyAsync(hflags.data(), flags, sizeof(int) * L, cudaMemcpyDeviceToHost, net->stream));
+  CK(cudaStreamSynchronize(net->stream));
+  for (int l = 0; l < L; ++l) {
+    if (hflags[l] & kRnsUneven) return NNC_OK;
+    if (!(hflags[l] & kRnsScaled)) net->layers[l].wr_de = nullptr;
+  }
+  net->rns = true;
   AL(net->c64, std::max(net->K_total, kPad));
   AL(net->rc64, std::max(net->K_total, kPad));
   AL(net->Zv, (size_t)seeds * k_max);
@@ -838,7 +858,7 @@ static int load_rns(nnc_net* net) {
     AL_RAW(p, rs * Ly.mp * Ly.kp * 2);
     Ly.Wr = p;
     AL(Ly.wr_scale, Ly.mp);
-    CK(rns_pack_weights(net->rset, Ly.W64, Ly.mp, Ly.kp, Ly.Wr, Ly.wr_scale, net->stream));
+    CK(rns_pack_weights(net->rset, Ly.W64, Ly.mp, Ly.kp, Ly.wr_de, Ly.Wr, Ly.wr_scale, net->stream));
     int r = rns_plan_rev(Ly.plan_rr, Ly.Wr, Ly.mp, Ly.kp, net->Zr, net->S_max, net->rset.n);
     if (r == NNC_OK && planes > 0 && l > 0)
       r = rns_plan(Ly.plan_rt, Ly.Wr, Ly.mp, net->Rt, n, Ly.mp, n, Ly.kp, net->rset.n, false);

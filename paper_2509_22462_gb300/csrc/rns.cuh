@@ -36,9 +36,20 @@ int rns_plan(RnsPlan& p, const void* A, int a_rows, const void* B, int b_rows, i
 cudaError_t rns_gemm(const RnsPlan& p, const RnsSet& s, unsigned char* C, int ldc, int* err,
                      int sm_count, cudaStream_t st);
 
-// Weights W [mp][kp] (FP64): residues [set.n][mp][kp] with q folded in, and the row scales sa[mp].
-cudaError_t rns_pack_weights(const RnsSet& s, const double* W, int mp, int kp, void* res, double* sa,
-                             cudaStream_t st);
+// Powers of two 2^de[k] that even out the columns of W [m][k] (row stride ldw): the residues are those of
+// W[r][k] 2^-de[k], the operand beside them is multiplied by 2^de[k].  Scratch: rns_even_scratch(k)
+// bytes.  *flags receives kRnsUneven where the rounding of a row would cost too much all the same (the
+// net's products then stay on the CUDA cores), kRnsScaled where de is needed (else
+// it is left out).
+constexpr int kRnsUneven = 1, kRnsScaled = 2;
+size_t rns_even_scratch(int k);
+cudaError_t rns_even_out(const RnsSet& s, const double* W, int ldw, int m, int k, void* scratch, int* de,
+                         int* flags, cudaStream_t st);
+
+// Weights W [mp][kp] (FP64): residues [set.n][mp][kp] of W 2^-de (de [kp] or NULL) with q folded in, and
+// the row scales sa[mp].
+cudaError_t rns_pack_weights(const RnsSet& s, const double* W, int mp, int kp, const int* de, void* res,
+                             double* sa, cudaStream_t st);
 
 // One layer's tangents, row by row (n rows of K = mp columns).
 struct RnsRows {
@@ -51,7 +62,8 @@ struct RnsRows {
   int n = 0, K = 0;             // K: columns handled (a multiple of 128)
   const double* s1 = nullptr;   // sigma' of the layer
   const double *c = nullptr, *rc = nullptr;   // curvature weight and sqrt|c|
-  void* At = nullptr;           // residues of s1 * Z [out.n][n][K], or NULL
+  const int* de = nullptr;      // the next layer's column exponents [K], or NULL
+  void* At = nullptr;           // residues of s1 * Z * 2^de [out.n][n][K], or NULL
   double* sat = nullptr;        // their row scales [n]
   void *Sa = nullptr, *Sb = nullptr;   // residues of rc Z (q folded in) and sign(c) rc Z, or NULL
   double* ss = nullptr;         // their row scales [n]
@@ -64,6 +76,7 @@ struct RnsRev {
   const unsigned char* C = nullptr;   // planes of rns_gemm on an rns_plan_rev plan, or NULL: seeds
   int chunks = 0, seeds = 0;          // seeds: rows of a plane (S rounded up to 16)
   const double* sb = nullptr;         // scales of the seeds that were multiplied [S]
+  const int* de = nullptr;            // column exponents of the weights that were multiplied [K], or NULL
   int K = 0, kvalid = 0, nJ = 0, lam_col = -1;
   const double *s1 = nullptr, *s2 = nullptr;   // of the layer that owns the K columns; NULL: x
   const double *lam = nullptr, *soft_p = nullptr;   // seeds (out_seed)
