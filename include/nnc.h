@@ -56,8 +56,9 @@ typedef enum {
  *                of a row, after powers of two have evened out the weights' columns, and the integer
  *                sums are exact.  The error of a column is that of an FP64 sum of normally distributed
  *                terms, whatever the units of inputs, hidden units and outputs.  Weights that powers of
- *                two do not even out, such as sparse ones, and nets whose residues do not fit in
- *                memory have FP64 products instead.
+ *                two do not even out, such as sparse ones, and nets whose residues (30 to 32 bytes
+ *                per weight) take more than an eighth of the device memory that is free at load, have
+ *                FP64 products instead, about 30 times slower on large nets: nnc_fp64_residues tells.
  *   NNC_FP32   : FP32 weights and tangents on CUDA cores, FP32 products, FP64 outputs.
  *   NNC_BF16   : value/Jacobian/adjoint in FP32; Hessian sweep on tcgen05 tensor cores with
  *                BF16 operands and FP32 accumulation (one product per tile).
@@ -255,6 +256,9 @@ const char* nnc_last_error(void);
 
 /* Query helpers (no device work). */
 int nnc_net_info(const nnc_net* net, int* n_layers, int* n_in, int* n_out, int* prec);
+/* 1 if the net's products run by residues on the tensor cores (see NNC_FP64 above), 0 if not (FP64
+ * products, or another form). */
+int nnc_fp64_residues(const nnc_net* net);
 /* Layer l (0-based) of the loaded net: its FP64 weights W (rows x cols, row-major, host, may be
  * NULL), bias b (rows, host, may be NULL; zeros if none was given), activation code, and shape
  * (rows = width of layer l+1, cols = width of layer l).  Synchronises the net's stream. */

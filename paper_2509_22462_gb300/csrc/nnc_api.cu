@@ -64,14 +64,14 @@ size_t elem_size(int prec) { return prec == NNC_FP64 ? 8 : prec == NNC_FP32 ? 4 
   } while (0)
 
 template <typename T>
-int dalloc(nnc_net* net, T** p, size_t n, bool zero = true) {
+int dalloc(nnc_net* net, T** p, size_t n) {
   void* q = nullptr;
   const size_t bytes = std::max<size_t>(n, 1) * sizeof(T);
   cudaError_t e = cudaMalloc(&q, bytes);
   if (e != cudaSuccess)
     return fail(NNC_ERR_OOM, std::string("cudaMalloc(") + std::to_string(bytes) + "): " +
                                  cudaGetErrorString(e));
-  if (zero) e = cudaMemsetAsync(q, 0, bytes, net->stream);
+  e = cudaMemsetAsync(q, 0, bytes, net->stream);
   net->allocs.push_back(q);
   if (e != cudaSuccess) return fail(NNC_ERR_CUDA, cudaGetErrorString(e));
   net->bytes += bytes;
@@ -82,12 +82,6 @@ int dalloc(nnc_net* net, T** p, size_t n, bool zero = true) {
 #define AL(p, n)                                    \
   do {                                              \
     int r_ = dalloc(net, &(p), (n));                \
-    if (r_ != NNC_OK) return r_;                    \
-  } while (0)
-// an array whose every element is written before it is read
-#define AL_RAW(p, n)                                \
-  do {                                              \
-    int r_ = dalloc(net, &(p), (n), false);         \
     if (r_ != NNC_OK) return r_;                    \
   } while (0)
 
@@ -714,6 +708,11 @@ int nnc_net_info(const nnc_net* net, int* n_layers, int* n_in, int* n_out, int* 
   return NNC_OK;
 }
 
+int nnc_fp64_residues(const nnc_net* net) {
+  if (!net) return fail(NNC_ERR_ARG, "net is NULL");
+  return net->rns ? 1 : 0;
+}
+
 int nnc_selftest_bounded_wait(int which, long long cycles, int* code) {
   if (code) *code = 0;
   if (which < 0 || which > 1 || cycles < 1 || cycles > 4000000000LL)
@@ -784,83 +783,118 @@ void nnc_free(nnc_net* net) {
   delete net;
 }
 
-// Buffers, residues and plans of the FP64 form's residue products.  They take 30 to 32 bytes per
-// weight beside the 8 of the FP64 weights; where that is more than half of the free memory, or where the
-// residues of the weights would keep too few bits (rns_even_out), the CUDA-core products stay in use
-// (net->rns false).
+// Buffers, residues and plans of the FP64 form's residue products, in one allocation of 30 to 32 bytes per
+// weight beside the 8 of the FP64 weights.  Where that is more than an eighth of the free memory (it is the
+// caller's, for more nets and other work), and where the residues of the weights would keep too few bits
+// (rns_even_out), the CUDA-core products stay in use (net->rns false).
 static int load_rns(nnc_net* net) {
-  const int n = net->n_in, L = net->L;
+  const int n = net->n_in, L = net->L, seeds = (net->S_max + 15) / 16 * 16;
   int planes = 0, k_max = net->n_in_pad;
-  size_t need = 0, cv = 0;
-  const int seeds = (net->S_max + 15) / 16 * 16;
-  for (int l = 0; l < L; ++l) {
-    LayerDev& Ly = net->layers[l];
+  for (auto& Ly : net->layers) {
     if (Ly.zy_off >= 0) Ly.h_plane = planes++;
     k_max = std::max(k_max, Ly.mp);
-    need += (size_t)Ly.mp * Ly.kp * 2 * kRnsMax;
-    cv = std::max(cv, (size_t)((Ly.mp + 1023) / 1024) * kRnsMax * seeds * Ly.kp);
   }
   net->h_planes = planes;
   net->zs_ld = k_max + kPad;
   net->u_ld = net->n_in_pad;
   net->rset = rns_set(net->zs_ld);
-  const size_t row_elems = (size_t)n * net->zs_ld, rs = net->rset.n;
-  need += row_elems * (kRnsMax * 7 + 16) + (size_t)planes * kRnsMax * n * net->u_ld + cv +
-          (size_t)seeds * k_max * (8 + 2 * kRnsMax);
+  const size_t rs = net->rset.n, row_elems = (size_t)n * net->zs_ld;
+  // offsets in the allocation; what has to start as zero comes first
+  size_t size = 0;
+  auto take = [&](size_t bytes) {
+    const size_t at = size;
+    size += (bytes + 1023) / 1024 * 1024;
+    return at;
+  };
+  const bool hess = planes > 0;
+  const size_t o_flags = take(sizeof(int) * L), o_even = take(rns_even_scratch(k_max));
+  const size_t o_c = take(8 * (size_t)std::max(net->K_total, kPad));
+  const size_t o_rc = take(8 * (size_t)std::max(net->K_total, kPad));
+  const size_t o_zv = take(8 * (size_t)seeds * k_max), o_zr = take(2 * rs * seeds * k_max);
+  const size_t o_zsc = take(8 * 96);
+  const size_t o_z1 = hess ? take(8 * (size_t)n * (net->layers[0].mp + kPad)) : 0;
+  const size_t o_zs = hess ? take(8 * row_elems) : 0;
+  const size_t o_rts = hess ? take(8 * (size_t)n) : 0, o_rus = hess ? take(8 * (size_t)planes * n) : 0;
+  std::vector<size_t> o_wr(L), o_ws(L), o_de(L);
+  for (int l = 0; l < L; ++l) {
+    o_ws[l] = take(8 * (size_t)net->layers[l].mp);
+    o_de[l] = take(sizeof(int) * net->layers[l].kp);
+  }
+  const size_t zeroed = size;
+  size_t cv = 0;
+  for (int l = 0; l < L; ++l) {
+    const LayerDev& Ly = net->layers[l];
+    o_wr[l] = take(2 * rs * Ly.mp * Ly.kp);
+    cv = std::max(cv, (size_t)((Ly.mp + 1023) / 1024) * rs * seeds * Ly.kp);
+  }
+  const size_t o_cv = take(cv);
+  size_t o_rt = 0, o_ra = 0, o_rb = 0, o_rcv = 0, o_ru = 0;
+  if (hess) {
+    o_rt = take(2 * rs * row_elems);
+    o_ra = take(2 * rs * row_elems);
+    o_rb = take(2 * rs * row_elems);
+    o_rcv = take(rs * row_elems);
+    o_ru = take((size_t)planes * kRnsMax * n * net->u_ld);
+  }
   size_t free_b = 0, total_b = 0;
   CK(cudaMemGetInfo(&free_b, &total_b));
-  if (need > free_b / 2) return NNC_OK;
-  unsigned char* p;
+  if (size > free_b / 8) return NNC_OK;
+  unsigned char* base = nullptr;
+  if (cudaMalloc(&base, size) != cudaSuccess) {
+    cudaGetLastError();   // taken by someone else meanwhile
+    return NNC_OK;
+  }
+  net->allocs.push_back(base);
+  net->bytes += size;
+  CK(cudaMemsetAsync(base, 0, zeroed, net->stream));
   // the layers' column exponents, and whether the weights are even enough
-  int *flags, *de;
-  std::vector<int> hflags(L);
-  AL(flags, L);
-  AL(p, rns_even_scratch(k_max));
+  int* flags = (int*)(base + o_flags);
   for (int l = 0; l < L; ++l) {
     LayerDev& Ly = net->layers[l];
-    AL(de, Ly.kp);
-    Ly.wr_de = de;
-    CK(rns_even_out(net->rset, Ly.W64, Ly.kp, Ly.m, Ly.k, p, de, flags + l, net->stream));
+    Ly.wr_de = (int*)(base + o_de[l]);
+    CK(rns_even_out(net->rset, Ly.W64, Ly.kp, Ly.m, Ly.k, base + o_even, Ly.wr_de, flags + l, net->stream));
   }
+  std::vector<int> hflags(L);
   CK(cudaMemcpyAsync(hflags.data(), flags, sizeof(int) * L, cudaMemcpyDeviceToHost, net->stream));
   CK(cudaStreamSynchronize(net->stream));
   for (int l = 0; l < L; ++l) {
-    if (hflags[l] & kRnsUneven) return NNC_OK;
+    if (hflags[l] & kRnsUneven) {
+      net->allocs.pop_back();
+      net->bytes -= size;
+      for (auto& Ly : net->layers) Ly.wr_de = nullptr;
+      CK(cudaFree(base));
+      return NNC_OK;
+    }
     if (!(hflags[l] & kRnsScaled)) net->layers[l].wr_de = nullptr;
   }
   net->rns = true;
-  AL(net->c64, std::max(net->K_total, kPad));
-  AL(net->rc64, std::max(net->K_total, kPad));
-  AL(net->Zv, (size_t)seeds * k_max);
-  AL(p, (size_t)seeds * k_max * 2 * rs);
-  net->Zr = p;
-  AL(net->zr_scale, 96);
-  AL_RAW(net->Cv, cv);
-  if (planes > 0) {
-    AL(net->Z1, (size_t)n * (net->layers[0].mp + kPad));
-    AL(net->Zs, row_elems);
-    AL_RAW(p, row_elems * 2 * rs);
-    net->Rt = p;
-    AL_RAW(p, row_elems * 2 * rs);
-    net->Ra = p;
-    AL_RAW(p, row_elems * 2 * rs);
-    net->Rb = p;
-    AL_RAW(net->Rc, row_elems * rs);
-    AL_RAW(net->Ru, (size_t)planes * kRnsMax * n * net->u_ld);
-    AL(net->rt_scale, n);
-    AL(net->ru_scale, (size_t)planes * n);
+  net->c64 = (double*)(base + o_c);
+  net->rc64 = (double*)(base + o_rc);
+  net->Zv = (double*)(base + o_zv);
+  net->Zr = base + o_zr;
+  net->zr_scale = (double*)(base + o_zsc);
+  net->Cv = base + o_cv;
+  if (hess) {
+    net->Z1 = (double*)(base + o_z1);
+    net->Zs = (double*)(base + o_zs);
+    net->Rt = base + o_rt;
+    net->Ra = base + o_ra;
+    net->Rb = base + o_rb;
+    net->Rc = base + o_rcv;
+    net->Ru = base + o_ru;
+    net->rt_scale = (double*)(base + o_rts);
+    net->ru_scale = (double*)(base + o_rus);
     LayerDev& L1 = net->layers[0];
     CK(launch_transpose_f64(L1.W64, L1.kp, L1.mp, n, net->Z1, L1.mp + kPad, net->stream));
   }
   for (int l = 0; l < L; ++l) {
     LayerDev& Ly = net->layers[l];
     if (Ly.zy_off >= 0) Ly.c = net->c64 + Ly.zy_off;
-    AL_RAW(p, rs * Ly.mp * Ly.kp * 2);
-    Ly.Wr = p;
-    AL(Ly.wr_scale, Ly.mp);
+    Ly.Wr = base + o_wr[l];
+    Ly.wr_scale = (double*)(base + o_ws[l]);
     CK(rns_pack_weights(net->rset, Ly.W64, Ly.mp, Ly.kp, Ly.wr_de, Ly.Wr, Ly.wr_scale, net->stream));
     int r = rns_plan_rev(Ly.plan_rr, Ly.Wr, Ly.mp, Ly.kp, net->Zr, net->S_max, net->rset.n);
-    if (r == NNC_OK && planes > 0 && l > 0)
+    if (r == NNC_OK && hess && l > 0)
       r = rns_plan(Ly.plan_rt, Ly.Wr, Ly.mp, net->Rt, n, Ly.mp, n, Ly.kp, net->rset.n, false);
     if (r == NNC_OK && Ly.zy_off >= 0)
       r = rns_plan(Ly.plan_rs, net->Ra, n, net->Rb, n, n, n,
@@ -975,9 +1009,6 @@ static int load_impl(nnc_net* net, int n_layers, const int* widths, const int* a
   }
   AL(net->ydev, net->n_out);
   AL(net->rdev, net->n_out);
-  AL(net->Zbar[0], (size_t)mp_max * net->S_max);
-  AL(net->Zbar[1], (size_t)mp_max * net->S_max);
-  AL(net->part, part_max);
   if (net->rev_stream) {
     AL(net->Zf[0], (size_t)mp_max * 16);
     AL(net->Zf[1], (size_t)mp_max * 16);
@@ -1014,6 +1045,11 @@ static int load_impl(nnc_net* net, int n_layers, const int* widths, const int* a
   if (prec == NNC_FP64) {
     int r = load_rns(net);
     if (r != NNC_OK) return r;
+  }
+  if (!net->rns) {
+    AL(net->Zbar[0], (size_t)mp_max * net->S_max);
+    AL(net->Zbar[1], (size_t)mp_max * net->S_max);
+    AL(net->part, part_max);
   }
   const size_t tan_elems = (size_t)n * mp_max;
   const size_t zy_elems = (size_t)n * std::max(net->K_total, kPad);

@@ -24,7 +24,7 @@ STATUS = {0: "NNC_OK", -1: "NNC_ERR_ARG", -2: "NNC_ERR_CUDA", -3: "NNC_ERR_NONFI
 EXPORTS = ["nnc_load_weights", "nnc_eval", "nnc_residual", "nnc_jacobian", "nnc_hessian_lag",
            "nnc_eval_batched", "nnc_eval_dev", "nnc_residual_dev", "nnc_jacobian_dev",
            "nnc_hessian_lag_dev", "nnc_eval_all_dev", "nnc_eval_kkt_dev", "nnc_eval_kkt", "nnc_free", "nnc_last_error",
-           "nnc_net_info", "nnc_launch_count", "nnc_profile", "nnc_profile_read",
+           "nnc_net_info", "nnc_fp64_residues", "nnc_launch_count", "nnc_profile", "nnc_profile_read",
            "nnc_ipm_default_options", "nnc_ipm_adversarial", "nnc_ipm_adversarial_l1",
            "nnc_ipm_adversarial_l1_fullspace", "nnc_layer_weights", "nnc_selftest_bounded_wait", "nnc_selftest_net_wait",
            "nnc_kkt_solve", "nnc_stage_kkt_solve",
@@ -112,6 +112,7 @@ def load_library(path: str = LIB_PATH):
     lib.nnc_ipm_default_options.restype = None
     lib.nnc_last_error.restype = ctypes.c_char_p
     lib.nnc_net_info.argtypes = [_P] + [ctypes.POINTER(ctypes.c_int)] * 4
+    lib.nnc_fp64_residues.argtypes = [_P]
     lib.nnc_launch_count.restype = ctypes.c_longlong
     lib.nnc_profile.argtypes = [_P, ctypes.c_int]
     lib.nnc_ipm_default_options.argtypes = [ctypes.POINTER(IpmOptions)]
@@ -252,6 +253,13 @@ class Net:
     @property
     def handle(self):
         return self._h
+
+    @property
+    def fp64_residues(self):
+        """True if the products of this FP64 net run by residues on the tensor cores (nnc_fp64_residues)."""
+        r = _lib.nnc_fp64_residues(self._h)
+        _check(min(r, 0))
+        return r == 1
 
     def free(self):
         if getattr(self, "_h", None) is not None and self._h.value:
