@@ -33,7 +33,8 @@ cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
   cfg.numAttrs = 1;
   const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
   note_launch();
-  return e != cudaSuccess ? e : cudaGetLastError();
+  const cudaError_t last = cudaGetLastError();   // cleared: the caller has to look at the result
+  return e != cudaSuccess ? e : last;
 }
 
 // sigma, sigma' and sigma'' of Eq. 3's activations, in FP64.  The derivatives follow from

@@ -34,8 +34,7 @@ __global__ void k_bx_scatter(const double* __restrict__ xcat, const int* __restr
 cudaError_t launch_bx_scatter(const double* xcat, const int* gn, const int* goff, int kp, int groups,
                               double* xs, float* xf, cudaStream_t st) {
   dim3 grid((kp + 255) / 256, groups);
-  launch_pdl(k_bx_scatter, grid, dim3(256), 0, st, xcat, gn, goff, kp, xs, xf);
-  return cudaGetLastError();
+  return launch_pdl(k_bx_scatter, grid, dim3(256), 0, st, xcat, gn, goff, kp, xs, xf);
 }
 
 
@@ -115,13 +114,9 @@ cudaError_t launch_bgemv_rev(const float* W, int ldw, int mp, int m, int groups,
   // threads: the row's 4-column groups, rounded up to whole warps, at most 256
   const int threads = std::min(256, (ldw / 4 + 31) / 32 * 32);
   dim3 grid((ldw + 4 * threads - 1) / (4 * threads), chunks, groups);
-  if (S <= 2)
-    launch_pdl(k_bgemv_rev<2>, grid, dim3(threads), 0, st, W, ldw, mp, m, Zbar, S, chunks, part, gcols);
-  else if (S <= 4)
-    launch_pdl(k_bgemv_rev<4>, grid, dim3(threads), 0, st, W, ldw, mp, m, Zbar, S, chunks, part, gcols);
-  else
-    return cudaErrorInvalidValue;
-  return cudaGetLastError();
+  if (S > 4) return cudaErrorInvalidValue;
+  return launch_pdl(S <= 2 ? k_bgemv_rev<2> : k_bgemv_rev<4>, grid, dim3(threads), 0, st, W, ldw, mp, m, Zbar, S,
+                    chunks, part, gcols);
 }
 
 int bgemv_rev_chunks(int m, int ldw) { return (m + brev_rows(ldw) - 1) / brev_rows(ldw); }
@@ -168,9 +163,8 @@ cudaError_t launch_brev_reduce(const float* part, int chunks, int kcols, int mp_
                                double* Zbar_out, double* c_out, float* c_f, const int* gn,
                                const int* goff, double* J_cat, double* g_cat, cudaStream_t st) {
   dim3 grid((kcols * S + 255) / 256, groups);
-  launch_pdl(k_brev_reduce, grid, dim3(256), 0, st, part, chunks, kcols, mp_out, S, s1, s2, lam_col,
+  return launch_pdl(k_brev_reduce, grid, dim3(256), 0, st, part, chunks, kcols, mp_out, S, s1, s2, lam_col,
              nJ, Zbar_out, c_out, c_f, gn, goff, J_cat, g_cat);
-  return cudaGetLastError();
 }
 
 // Output-layer seeds of every group (m = n_out rows per group, stacked with stride mp).
@@ -199,8 +193,7 @@ cudaError_t launch_brev_seed(int m, int mp, int groups, int S, int nJ, int lam_c
                              const double* s2, const double* lam, double* Zbar, double* c_out,
                              float* c_f, cudaStream_t st) {
   dim3 grid((m * S + 255) / 256, groups);
-  launch_pdl(k_brev_seed, grid, dim3(256), 0, st, m, mp, S, nJ, lam_col, s1, s2, lam, Zbar, c_out, c_f);
-  return cudaGetLastError();
+  return launch_pdl(k_brev_seed, grid, dim3(256), 0, st, m, mp, S, nJ, lam_col, s1, s2, lam, Zbar, c_out, c_f);
 }
 
 // First-layer tangents of every group: At[boff+n][m] = s1[m] W1_g[m][n], Zt/Yt likewise at
@@ -284,10 +277,9 @@ cudaError_t launch_bfirst_tangent(const float* W1, int ldw, int mp, int groups, 
       !al8(yt_hi) || !al8(yt_lo) || (zt_hi && !yt_hi))
     return cudaErrorInvalidValue;
   dim3 grid((n_max + 31) / 32, mp / 64, groups);
-  launch_pdl(k_bfirst_tangent, grid, dim3(256), 0, st, W1, ldw, mp, gn, goff, s1, c,
+  return launch_pdl(k_bfirst_tangent, grid, dim3(256), 0, st, W1, ldw, mp, gn, goff, s1, c,
              (__nv_bfloat16*)at_hi, (__nv_bfloat16*)at_lo, lda, (__nv_bfloat16*)zt_hi,
              (__nv_bfloat16*)zt_lo, (__nv_bfloat16*)yt_hi, (__nv_bfloat16*)yt_lo, ldz, x3 ? 1 : 0);
-  return cudaGetLastError();
 }
 
 // H_g[i][j] = sum_s Hp[s][g][max][min] for every group (row-major n_g x n_g at hoff[g]).
@@ -312,8 +304,7 @@ __global__ void k_bh_finish(const float* __restrict__ Hp, int splits, long long 
 cudaError_t launch_bh_finish(const float* Hp, int splits, long long ldh_split, int groups,
                              const int* gn, const long long* hoff, double* H, cudaStream_t st) {
   dim3 grid(32, groups);
-  launch_pdl(k_bh_finish, grid, dim3(256), 0, st, Hp, splits, ldh_split, gn, hoff, H);
-  return cudaGetLastError();
+  return launch_pdl(k_bh_finish, grid, dim3(256), 0, st, Hp, splits, ldh_split, gn, hoff, H);
 }
 
 // r_cat[g*m + i] = y_cat[g*m + i] - a[g*mp + i]
@@ -328,8 +319,7 @@ __global__ void k_bsub(const double* y, const double* a, int m, int mp, int grou
 
 cudaError_t launch_bsub(const double* y, const double* a, int m, int mp, int groups, double* r,
                         cudaStream_t st) {
-  launch_pdl(k_bsub, dim3((m * groups + 255) / 256), dim3(256), 0, st, y, a, m, mp, groups, r);
-  return cudaGetLastError();
+  return launch_pdl(k_bsub, dim3((m * groups + 255) / 256), dim3(256), 0, st, y, a, m, mp, groups, r);
 }
 
 // y_cat[g*m + i] = a[g*mp + i]
@@ -342,8 +332,7 @@ __global__ void k_bgather(const double* a, int m, int mp, int groups, double* y)
 }
 
 cudaError_t launch_bgather(const double* a, int m, int mp, int groups, double* y, cudaStream_t st) {
-  launch_pdl(k_bgather, dim3((m * groups + 255) / 256), dim3(256), 0, st, a, m, mp, groups, y);
-  return cudaGetLastError();
+  return launch_pdl(k_bgather, dim3((m * groups + 255) / 256), dim3(256), 0, st, a, m, mp, groups, y);
 }
 
 }  // namespace nnc

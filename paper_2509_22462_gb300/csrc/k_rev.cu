@@ -335,9 +335,8 @@ cudaError_t launch_rev_seed_f(int m, int S, int nJ, int lam_col, const double* s
                               const double* lam, const double* p, float* Zf, double* c_out,
                               float* c_f, cudaStream_t st) {
   const int SM = rev_stream_sm(S);
-  launch_pdl(k_rev_seed_f, dim3((m * SM + 255) / 256), dim3(256), 0, st, m, S, SM, nJ, lam_col, s1, s2,
+  return launch_pdl(k_rev_seed_f, dim3((m * SM + 255) / 256), dim3(256), 0, st, m, S, SM, nJ, lam_col, s1, s2,
              lam, p, Zf, c_out, c_f);
-  return cudaGetLastError();
 }
 
 cudaError_t launch_rev_stream(const CUtensorMap& map, int m, int kp, const float* Zf, int S,

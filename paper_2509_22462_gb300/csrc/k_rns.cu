@@ -1065,7 +1065,8 @@ cudaError_t rns_rev_rows(const RnsSet& s, const RnsRev& a, int S, cudaStream_t s
   cfg.numAttrs = 2;
   const cudaError_t e = cudaLaunchKernelEx(&cfg, a.C && a.de ? k_rns_rev_rows<true> : k_rns_rev_rows<false>, s, a);
   note_launch();
-  return e != cudaSuccess ? e : cudaGetLastError();
+  const cudaError_t last = cudaGetLastError();
+  return e != cudaSuccess ? e : last;
 }
 
 cudaError_t rns_softmax_ext(int n, int m, int col, const double* p, const double* lam, double* Z,

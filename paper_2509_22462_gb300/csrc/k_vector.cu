@@ -318,20 +318,11 @@ __global__ void k_softmax_ext(int n, int m, const double* __restrict__ p, const 
 
 cudaError_t launch_softmax_ext(Elem e, int n, int m, const double* p, const double* lam, TanBuf ZL,
                                TanBuf Zx, TanBuf Yx, int ldz, cudaStream_t st) {
-  const int blocks = (n + 127) / 128;
-  switch (e) {
-    case Elem::F64: launch_pdl(k_softmax_ext<Elem::F64>, dim3(blocks), dim3(128), 0, st, n, m, p, lam,
-                               ZL, Zx, Yx, ldz); break;
-    case Elem::F32: launch_pdl(k_softmax_ext<Elem::F32>, dim3(blocks), dim3(128), 0, st, n, m, p, lam,
-                               ZL, Zx, Yx, ldz); break;
-    case Elem::BF16: launch_pdl(k_softmax_ext<Elem::BF16>, dim3(blocks), dim3(128), 0, st, n, m, p,
-                                lam, ZL, Zx, Yx, ldz); break;
-    case Elem::BF16X3:
-      launch_pdl(k_softmax_ext<Elem::BF16X3>, dim3(blocks), dim3(128), 0, st, n, m, p, lam, ZL, Zx, Yx,
-                 ldz);
-      break;
-  }
-  return cudaGetLastError();
+  auto kernel = e == Elem::F64    ? k_softmax_ext<Elem::F64>
+                : e == Elem::F32  ? k_softmax_ext<Elem::F32>
+                : e == Elem::BF16 ? k_softmax_ext<Elem::BF16>
+                                  : k_softmax_ext<Elem::BF16X3>;
+  return launch_pdl(kernel, dim3((n + 127) / 128), dim3(128), 0, st, n, m, p, lam, ZL, Zx, Yx, ldz);
 }
 
 template <Elem E, typename TW>
@@ -545,13 +536,8 @@ cudaError_t launch_first_tangent_t(bool x3, const float* W1T, int ldt, int m_pad
                                    TanBuf Yt, int ldz, cudaStream_t st) {
   if (m_pad % 8 || ldt % 4 || lda % 8 || ldz % 8 || ((uintptr_t)W1T & 15)) return cudaErrorInvalidValue;
   const dim3 grid((m_pad / 8 + 255) / 256, (n + kFtN - 1) / kFtN);
-  if (x3)
-    launch_pdl(k_first_tangent_t<true>, grid, dim3(256), 0, st, W1T, ldt, m_pad, n, s1, c, At, lda, Yt,
-               ldz);
-  else
-    launch_pdl(k_first_tangent_t<false>, grid, dim3(256), 0, st, W1T, ldt, m_pad, n, s1, c, At, lda,
-               Yt, ldz);
-  return cudaGetLastError();
+  return launch_pdl(x3 ? k_first_tangent_t<true> : k_first_tangent_t<false>, grid, dim3(256), 0, st, W1T, ldt,
+                    m_pad, n, s1, c, At, lda, Yt, ldz);
 }
 
 // Ydot = c * Zdot over the columns [k0, k1) of the n x ldz operand blocks of the symmetric
@@ -636,26 +622,13 @@ cudaError_t launch_first_tangent(Elem e, const void* W1, int ldw, int m_pad, int
     return cudaGetLastError();
   }
   dim3 grid((n + 31) / 32, (m_pad + 31) / 32), block(32, 8);
-  const float* Wf = (const float*)W1;
-  switch (e) {
-    case Elem::F64:
-      launch_pdl(k_first_tangent<Elem::F64, double>, grid, block, 0, st, (const double*)W1, ldw, m_pad,
-                 n, s1, c, At, lda, Zt, Yt, ldz);
-      break;
-    case Elem::F32:
-      launch_pdl(k_first_tangent<Elem::F32, float>, grid, block, 0, st, Wf, ldw, m_pad, n, s1, c, At,
-                 lda, Zt, Yt, ldz);
-      break;
-    case Elem::BF16:
-      launch_pdl(k_first_tangent<Elem::BF16, float>, grid, block, 0, st, Wf, ldw, m_pad, n, s1, c, At,
-                 lda, Zt, Yt, ldz);
-      break;
-    case Elem::BF16X3:
-      launch_pdl(k_first_tangent<Elem::BF16X3, float>, grid, block, 0, st, Wf, ldw, m_pad, n, s1, c,
-                 At, lda, Zt, Yt, ldz);
-      break;
-  }
-  return cudaGetLastError();
+  if (e == Elem::F64)
+    return launch_pdl(k_first_tangent<Elem::F64, double>, grid, block, 0, st, (const double*)W1, ldw, m_pad, n,
+                      s1, c, At, lda, Zt, Yt, ldz);
+  auto kernel = e == Elem::F32    ? k_first_tangent<Elem::F32, float>
+                : e == Elem::BF16 ? k_first_tangent<Elem::BF16, float>
+                                  : k_first_tangent<Elem::BF16X3, float>;
+  return launch_pdl(kernel, grid, block, 0, st, (const float*)W1, ldw, m_pad, n, s1, c, At, lda, Zt, Yt, ldz);
 }
 
 // ------------------------------------------------------------------ Hessian finish
@@ -722,12 +695,11 @@ cudaError_t launch_h_finish(bool part_f32, const void* Hp, int splits, int n, in
                             cudaStream_t st) {
   const int T = (n + 31) / 32, tiles = T * (T + 1) / 2;
   const dim3 block(32, 8);
-  if (!part_f32) launch_pdl(k_h_finish<double, 4>, dim3(tiles), block, 0, st, (const double*)Hp,
-                            splits, n, ldp, H);
-  else if (splits > 16) launch_pdl(k_h_finish<float, 1>, dim3(4 * tiles), block, 0, st,
-                                   (const float*)Hp, splits, n, ldp, H);
-  else launch_pdl(k_h_finish<float, 4>, dim3(tiles), block, 0, st, (const float*)Hp, splits, n, ldp, H);
-  return cudaGetLastError();
+  if (!part_f32)
+    return launch_pdl(k_h_finish<double, 4>, dim3(tiles), block, 0, st, (const double*)Hp, splits, n, ldp, H);
+  if (splits > 16)
+    return launch_pdl(k_h_finish<float, 1>, dim3(4 * tiles), block, 0, st, (const float*)Hp, splits, n, ldp, H);
+  return launch_pdl(k_h_finish<float, 4>, dim3(tiles), block, 0, st, (const float*)Hp, splits, n, ldp, H);
 }
 
 __global__ void k_sub(const double* y, const double* a, double* r, int n) {
@@ -922,9 +894,8 @@ __global__ void k_rev_seed_t(int m, int S, int nJ, int lam_col, const double* __
 cudaError_t launch_rev_seed_t(int m, int S, int nJ, int lam_col, const double* s1, const double* s2,
                               const double* lam, const double* p, void* const z[3], int ld,
                               double* c_out, float* c_f, cudaStream_t st) {
-  launch_pdl(k_rev_seed_t, dim3((m * S + 255) / 256), dim3(256), 0, st, m, S, nJ, lam_col, s1, s2, lam,
+  return launch_pdl(k_rev_seed_t, dim3((m * S + 255) / 256), dim3(256), 0, st, m, S, nJ, lam_col, s1, s2, lam,
              p, (__nv_bfloat16*)z[0], (__nv_bfloat16*)z[1], (__nv_bfloat16*)z[2], ld, c_out, c_f);
-  return cudaGetLastError();
 }
 
 // Sum the split partials P[sp][k][0..bn) of W_l^T Zbar; then either the next seeds (transposed,
@@ -984,9 +955,8 @@ cudaError_t launch_rev_reduce_t(const float* P, int splits, int kcols, int bn, i
   __nv_bfloat16* z1 = z ? (__nv_bfloat16*)z[1] : nullptr;
   __nv_bfloat16* z2 = z ? (__nv_bfloat16*)z[2] : nullptr;
   const dim3 block = splits > 16 ? dim3(32, 8) : dim3(256, 1);
-  launch_pdl(k_rev_reduce_t, dim3((kcols * S + block.x - 1) / block.x), block, 0, st, P, splits, kcols,
+  return launch_pdl(k_rev_reduce_t, dim3((kcols * S + block.x - 1) / block.x), block, 0, st, P, splits, kcols,
              bn, S, kvalid, s1, s2, lam_col, nJ, z0, z1, z2, ld, c_out, c_f, J_out, g_out);
-  return cudaGetLastError();
 }
 
 }  // namespace nnc
@@ -1011,8 +981,7 @@ __global__ void k_split_df(const double* __restrict__ src, size_t n, float2* __r
 cudaError_t launch_split_df(const double* src, size_t n, void* dst, cudaStream_t st) {
   size_t blocks = (n + 255) / 256;
   if (blocks > 4096) blocks = 4096;
-  launch_pdl(k_split_df, dim3((unsigned)blocks), dim3(256), 0, st, src, n, (float2*)dst);
-  return cudaGetLastError();
+  return launch_pdl(k_split_df, dim3((unsigned)blocks), dim3(256), 0, st, src, n, (float2*)dst);
 }
 
 }  // namespace nnc

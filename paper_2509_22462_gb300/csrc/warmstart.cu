@@ -102,10 +102,10 @@ __global__ void __launch_bounds__(256) k_ws_gemm(const T* __restrict__ A, long s
 }
 
 template <typename T>
-void gemm(const T* A, long sam, long sak, const T* B, long sbk, long sbn, int M, int N, int K,
-          const float* bias, float* C, int ldc, cudaStream_t st) {
+cudaError_t gemm(const T* A, long sam, long sak, const T* B, long sbk, long sbn, int M, int N, int K,
+                 const float* bias, float* C, int ldc, cudaStream_t st) {
   dim3 grid((N + 31) / 32, (M + 31) / 32);
-  launch_pdl(k_ws_gemm<T>, grid, dim3(256), 0, st, A, sam, sak, B, sbk, sbn, M, N, K, bias, C, ldc);
+  return launch_pdl(k_ws_gemm<T>, grid, dim3(256), 0, st, A, sam, sak, B, sbk, sbn, M, N, K, bias, C, ldc);
 }
 
 template <typename T>
@@ -459,10 +459,9 @@ int make_plans(nnc_ws* s, int B) {
   } while (0)
 
 template <typename T>
-void gelu(nnc_ws* s, const float* Z, int B, int cols, void* Hl, float* D1, __nv_bfloat16* Ht) {
-  launch_pdl(k_ws_gelu<T>, dim3((B * cols + 63) / 64), dim3(64), 0, s->stream, Z, B * cols, (T*)Hl, D1,
-             cols, Ht,
-             s->cap);
+cudaError_t gelu(nnc_ws* s, const float* Z, int B, int cols, void* Hl, float* D1, __nv_bfloat16* Ht) {
+  return launch_pdl(k_ws_gelu<T>, dim3((B * cols + 63) / 64), dim3(64), 0, s->stream, Z, B * cols, (T*)Hl,
+                    D1, cols, Ht, s->cap);
 }
 
 // forward on the first B rows of s->Ul (operand type): P = net(U)
@@ -474,21 +473,21 @@ int forward(nnc_ws* s, int B) {
       int r = make_plans(s, B);
       if (r) return r;
       TCK(nnc::tc_plain(s->pl[0], s->w[1], s->Z1, s->h1, s->d_err, st));
-      gelu<T>(s, s->Z1, B, s->h1, s->H1l, s->D1, s->H1t);
+      TCK(gelu<T>(s, s->Z1, B, s->h1, s->H1l, s->D1, s->H1t));
       TCK(nnc::tc_plain(s->pl[1], s->w[3], s->Z2, s->h2, s->d_err, st));
-      gelu<T>(s, s->Z2, B, s->h2, s->H2l, s->D2, s->H2t);
+      TCK(gelu<T>(s, s->Z2, B, s->h2, s->H2l, s->D2, s->H2t));
       TCK(nnc::tc_plain(s->pl[2], s->w[5], s->P, s->n_out, s->d_err, st));
       return NNC_OK;
     }
   }
-  gemm<T>((const T*)s->Ul, s->n_in, 1, (const T*)s->wl[0], 1, s->n_in, B, s->h1, s->n_in, s->w[1], s->Z1,
-          s->h1, st);
-  gelu<T>(s, s->Z1, B, s->h1, s->H1l, s->D1, nullptr);
-  gemm<T>((const T*)s->H1l, s->h1, 1, (const T*)s->wl[2], 1, s->h1, B, s->h2, s->h1, s->w[3], s->Z2, s->h2,
-          st);
-  gelu<T>(s, s->Z2, B, s->h2, s->H2l, s->D2, nullptr);
-  gemm<T>((const T*)s->H2l, s->h2, 1, (const T*)s->wl[4], 1, s->h2, B, s->n_out, s->h2, s->w[5], s->P,
-          s->n_out, st);
+  TCK(gemm<T>((const T*)s->Ul, s->n_in, 1, (const T*)s->wl[0], 1, s->n_in, B, s->h1, s->n_in, s->w[1], s->Z1,
+          s->h1, st));
+  TCK(gelu<T>(s, s->Z1, B, s->h1, s->H1l, s->D1, nullptr));
+  TCK(gemm<T>((const T*)s->H1l, s->h1, 1, (const T*)s->wl[2], 1, s->h1, B, s->h2, s->h1, s->w[3], s->Z2, s->h2,
+          st));
+  TCK(gelu<T>(s, s->Z2, B, s->h2, s->H2l, s->D2, nullptr));
+  TCK(gemm<T>((const T*)s->H2l, s->h2, 1, (const T*)s->wl[4], 1, s->h2, B, s->n_out, s->h2, s->w[5], s->P,
+          s->n_out, st));
   return NNC_OK;
 }
 
@@ -503,35 +502,34 @@ int loss_grad(nnc_ws* s, int B, double* loss) {
   const bool tcb = !std::is_same<T, float>::value && s->tc && B % 64 == 0;
   __nv_bfloat16* dZt = tcb ? s->dZt : nullptr;
   auto back = [&](const float* D, int cols, float* db) {
-    launch_pdl(k_ws_gelu_back<T>, dim3((cols + 31) / 32), dim3(32), 0, st, s->dH, D, B, cols,
-               (T*)s->dZl, db, dZt,
-               s->cap);
+    return launch_pdl(k_ws_gelu_back<T>, dim3((cols + 31) / 32), dim3(32), 0, st, s->dH, D, B, cols,
+                      (T*)s->dZl, db, dZt, s->cap);
   };
-  launch_pdl(k_ws_loss<T>, dim3((s->n_out + 31) / 32), dim3(32), 0, st, s->P, s->Tt, B, s->n_out,
-             1.f / (float)nP, (T*)s->dPl, s->g[5], s->part, tcb ? s->dPp : nullptr, s->n_out_p,
-             tcb ? s->dPt : nullptr, s->cap);
+  TCK(launch_pdl(k_ws_loss<T>, dim3((s->n_out + 31) / 32), dim3(32), 0, st, s->P, s->Tt, B, s->n_out,
+                 1.f / (float)nP, (T*)s->dPl, s->g[5], s->part, tcb ? s->dPp : nullptr, s->n_out_p,
+                 tcb ? s->dPt : nullptr, s->cap));
   // layer by layer: dW = dZ^T H (db with dZ), dH = dZ W, dZ = dH * GELU'
   if (tcb) {
     TCK(nnc::tc_plain(s->pl[3], nullptr, s->g[4], s->h2, s->d_err, st));
     TCK(nnc::tc_plain(s->pl[4], nullptr, s->dH, s->h2, s->d_err, st));
-    back(s->D2, s->h2, s->g[3]);
+    TCK(back(s->D2, s->h2, s->g[3]));
     TCK(nnc::tc_plain(s->pl[5], nullptr, s->g[2], s->h1, s->d_err, st));
     TCK(nnc::tc_plain(s->pl[6], nullptr, s->dH, s->h1, s->d_err, st));
-    back(s->D1, s->h1, s->g[1]);
+    TCK(back(s->D1, s->h1, s->g[1]));
     TCK(nnc::tc_plain(s->pl[7], nullptr, s->g[0], s->n_in, s->d_err, st));
   } else {
-    gemm<T>((const T*)s->dPl, 1, s->n_out, (const T*)s->H2l, s->h2, 1, s->n_out, s->h2, B, nullptr, s->g[4],
-            s->h2, st);
-    gemm<T>((const T*)s->dPl, s->n_out, 1, (const T*)s->wl[4], s->h2, 1, B, s->h2, s->n_out, nullptr, s->dH,
-            s->h2, st);
-    back(s->D2, s->h2, s->g[3]);
-    gemm<T>((const T*)s->dZl, 1, s->h2, (const T*)s->H1l, s->h1, 1, s->h2, s->h1, B, nullptr, s->g[2], s->h1,
-            st);
-    gemm<T>((const T*)s->dZl, s->h2, 1, (const T*)s->wl[2], s->h1, 1, B, s->h1, s->h2, nullptr, s->dH, s->h1,
-            st);
-    back(s->D1, s->h1, s->g[1]);
-    gemm<T>((const T*)s->dZl, 1, s->h1, (const T*)s->Ul, s->n_in, 1, s->h1, s->n_in, B, nullptr, s->g[0],
-            s->n_in, st);
+    TCK(gemm<T>((const T*)s->dPl, 1, s->n_out, (const T*)s->H2l, s->h2, 1, s->n_out, s->h2, B, nullptr, s->g[4],
+            s->h2, st));
+    TCK(gemm<T>((const T*)s->dPl, s->n_out, 1, (const T*)s->wl[4], s->h2, 1, B, s->h2, s->n_out, nullptr, s->dH,
+            s->h2, st));
+    TCK(back(s->D2, s->h2, s->g[3]));
+    TCK(gemm<T>((const T*)s->dZl, 1, s->h2, (const T*)s->H1l, s->h1, 1, s->h2, s->h1, B, nullptr, s->g[2], s->h1,
+            st));
+    TCK(gemm<T>((const T*)s->dZl, s->h2, 1, (const T*)s->wl[2], s->h1, 1, B, s->h1, s->h2, nullptr, s->dH, s->h1,
+            st));
+    TCK(back(s->D1, s->h1, s->g[1]));
+    TCK(gemm<T>((const T*)s->dZl, 1, s->h1, (const T*)s->Ul, s->n_in, 1, s->h1, s->n_in, B, nullptr, s->g[0],
+            s->n_in, st));
   }
   if (loss) {
     std::vector<double> h(s->n_out);
@@ -545,7 +543,7 @@ int loss_grad(nnc_ws* s, int B, double* loss) {
 }
 
 template <typename T>
-void adam(nnc_ws* s, float lr, float b1, float b2, float eps) {
+cudaError_t adam(nnc_ws* s, float lr, float b1, float b2, float eps) {
   s->step += 1;
   AdamArgs p{};
   p.lr = lr;
@@ -562,18 +560,16 @@ void adam(nnc_ws* s, float lr, float b1, float b2, float eps) {
                      i == 2 ? s->h1 : i == 4 ? s->h2 : 1, i == 2 ? s->h2 : i == 4 ? s->n_out_p : 0, blocks};
     blocks += (s->sizes[i] + 255) / 256;
   }
-  launch_pdl(k_ws_adam<T>, dim3(blocks), dim3(256), 0, s->stream, p);
+  return launch_pdl(k_ws_adam<T>, dim3(blocks), dim3(256), 0, s->stream, p);
 }
 
 template <typename T>
-void stage_rows(nnc_ws* s, const float* U, const float* Tt, int B) {
-  // U (B x n_in) and T (B x n_out) already on the device in standardized FP32
-  if (U != s->U) cudaMemcpyAsync(s->U, U, sizeof(float) * B * s->n_in, cudaMemcpyDeviceToDevice, s->stream);
-  if (Tt && Tt != s->Tt)
-    cudaMemcpyAsync(s->Tt, Tt, sizeof(float) * B * s->n_out, cudaMemcpyDeviceToDevice, s->stream);
+cudaError_t stage_rows(nnc_ws* s, int B) {
+  // s->U (B x n_in) is on the device in standardized FP32
   k_ws_cast<T><<<(B * s->n_in + 255) / 256, 256, 0, s->stream>>>(s->U, B * s->n_in, (T*)s->Ul, s->n_in,
                                                                   s->tc ? s->Ut : nullptr, s->cap);
   note_launch();
+  return cudaGetLastError();
 }
 
 int upload_std(nnc_ws* s, const double* U, const double* Tt, int N, bool with_t) {
@@ -707,10 +703,10 @@ int nnc_ws_loss_grad(nnc_ws* s, const double* U, const double* Tt, int B, double
   int r = upload_std(s, U, Tt, B, true);
   if (r) return r;
   if (s->prec == NNC_FP32) {
-    stage_rows<float>(s, s->U, s->Tt, B);
+    WCK(stage_rows<float>(s, B));
     r = loss_grad<float>(s, B, loss);
   } else {
-    stage_rows<__nv_bfloat16>(s, s->U, s->Tt, B);
+    WCK(stage_rows<__nv_bfloat16>(s, B));
     r = loss_grad<__nv_bfloat16>(s, B, loss);
   }
   if (r) return r;
@@ -730,9 +726,8 @@ int nnc_ws_loss_grad(nnc_ws* s, const double* U, const double* Tt, int B, double
 
 int nnc_ws_adam_step(nnc_ws* s, double lr, double beta1, double beta2, double eps) {
   if (!s) return wfail(NNC_ERR_ARG, "ws is NULL");
-  if (s->prec == NNC_FP32) adam<float>(s, (float)lr, (float)beta1, (float)beta2, (float)eps);
-  else adam<__nv_bfloat16>(s, (float)lr, (float)beta1, (float)beta2, (float)eps);
-  WCK(cudaGetLastError());
+  WCK(s->prec == NNC_FP32 ? adam<float>(s, (float)lr, (float)beta1, (float)beta2, (float)eps)
+                          : adam<__nv_bfloat16>(s, (float)lr, (float)beta1, (float)beta2, (float)eps));
   return NNC_OK;
 }
 
@@ -755,6 +750,7 @@ int nnc_ws_train(nnc_ws* s, const double* U, const double* Tt, int N, int epochs
   k_ws_standardize<<<dim3(N, (n_in + 255) / 256), 256, 0, st>>>(s->Ur, n_in, mean, sd, s->Ud);
   k_ws_standardize<<<dim3(N, (n_out + 255) / 256), 256, 0, st>>>(s->Tr, n_out, mean + n_in, sd + n_in, s->Td);
   note_launch(4);
+  WCK(cudaGetLastError());
   std::vector<double> h(2 * (size_t)nc);
   WCK(cudaMemcpyAsync(h.data(), s->stats, sizeof(double) * h.size(), cudaMemcpyDeviceToHost, st));
   WCK(cudaStreamSynchronize(st));
@@ -774,19 +770,18 @@ int nnc_ws_train(nnc_ws* s, const double* U, const double* Tt, int N, int epochs
     for (int b0 = 0; b0 + B <= N; b0 += B) {
       const bool want = (e == epochs - 1) && (b0 + 2 * B > N);
       if (s->prec == NNC_FP32) {
-        launch_pdl(k_ws_gather<float>, gg, dim3(256), 0, st, s->Ud, s->Td, s->perm + b0, n_in, n_out,
-                   (float*)s->Ul,
-                   nullptr, 0, s->Tt);
+        WCK(launch_pdl(k_ws_gather<float>, gg, dim3(256), 0, st, s->Ud, s->Td, s->perm + b0, n_in, n_out,
+                       (float*)s->Ul, nullptr, 0, s->Tt));
         r = loss_grad<float>(s, B, want ? &last : nullptr);
-        adam<float>(s, (float)lr, (float)beta1, (float)beta2, (float)eps);
+        if (r) return r;
+        WCK(adam<float>(s, (float)lr, (float)beta1, (float)beta2, (float)eps));
       } else {
-        launch_pdl(k_ws_gather<__nv_bfloat16>, gg, dim3(256), 0, st, s->Ud, s->Td, s->perm + b0, n_in,
-                   n_out,
-                   (__nv_bfloat16*)s->Ul, s->tc ? s->Ut : nullptr, s->cap, s->Tt);
+        WCK(launch_pdl(k_ws_gather<__nv_bfloat16>, gg, dim3(256), 0, st, s->Ud, s->Td, s->perm + b0, n_in,
+                       n_out, (__nv_bfloat16*)s->Ul, s->tc ? s->Ut : nullptr, s->cap, s->Tt));
         r = loss_grad<__nv_bfloat16>(s, B, want ? &last : nullptr);
-        adam<__nv_bfloat16>(s, (float)lr, (float)beta1, (float)beta2, (float)eps);
+        if (r) return r;
+        WCK(adam<__nv_bfloat16>(s, (float)lr, (float)beta1, (float)beta2, (float)eps));
       }
-      if (r) return r;
     }
   }
   WCK(cudaStreamSynchronize(s->stream));
@@ -802,10 +797,10 @@ int nnc_ws_predict(nnc_ws* s, const double* U, int N, double* P) {
   int r = upload_std(s, U, nullptr, N, false);
   if (r) return r;
   if (s->prec == NNC_FP32) {
-    stage_rows<float>(s, s->U, nullptr, N);
+    WCK(stage_rows<float>(s, N));
     r = forward<float>(s, N);
   } else {
-    stage_rows<__nv_bfloat16>(s, s->U, nullptr, N);
+    WCK(stage_rows<__nv_bfloat16>(s, N));
     r = forward<__nv_bfloat16>(s, N);
   }
   if (r) return r;

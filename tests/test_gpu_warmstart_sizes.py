@@ -1,0 +1,54 @@
+"""The warm-start network at sizes past the limits of a launch's second grid dimension (65535 tiles of 32
+rows, 65535 blocks of 256 columns), against FP64: FP32 sums of k terms are held to 4 k 2^-24 of their
+terms' size."""
+import numpy as np
+import pytest
+
+from synth.rng import derive_key, normal
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def lib():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2509_22462_gb300 import build, nnc
+    build.build()
+    return nnc
+
+
+def params(n_in, h1, h2, n_out, scale=1.0):
+    out = []
+    for i, (m, k) in enumerate(((h1, n_in), (h2, h1), (n_out, h2))):
+        out += [scale * normal(derive_key(i, "wsz-w"), m * k).reshape(m, k) / np.sqrt(k),
+                0.1 * normal(derive_key(i, "wsz-b"), m)]
+    return out
+
+
+def gelu(z):
+    from scipy.special import erf
+    return 0.5 * z * (1.0 + erf(z / np.sqrt(2.0)))
+
+
+def many_rows(lib):
+    p = params(3, 5, 4, 2)
+    U = normal(derive_key(9, "wsz-u"), 3 * (65535 * 32 + 33)).reshape(-1, 3)
+    a = gelu(gelu(U @ p[0].T + p[1]) @ p[2].T + p[3]) @ p[4].T + p[5]
+    ws = lib.WarmStart(p, precision="fp32")
+    return ws, U, a
+
+
+def test_launches_that_fail_are_reported(lib):
+    """A call whose launches do not fit raises; it never returns what happened to lie in the buffers, and
+    the calls after it are none the wiser."""
+    ws, U, a = many_rows(lib)
+    try:
+        P = ws.predict(U)
+    except lib.NNCError:
+        P = a
+    assert np.max(np.abs(P - a)) < 1e-5
+    ws.free()
+    ws = lib.WarmStart(params(3, 5, 4, 2), precision="fp32")
+    assert np.max(np.abs(ws.predict(U[:100]) - a[:100])) < 1e-5
