@@ -13,6 +13,7 @@
 // weight-gradient products, widths that are not multiples of 64) and the FP32 form use a
 // shared-memory tiled CUDA-core kernel.
 #include <algorithm>
+#include <climits>
 #include <cmath>
 #include <cstring>
 #include <numeric>
@@ -51,7 +52,8 @@ __global__ void __launch_bounds__(256) k_ws_gemm(const T* __restrict__ A, long s
                                                  int N, int K, const float* __restrict__ bias,
                                                  float* __restrict__ C, int ldc) {
   __shared__ float As[32][33], Bs[32][33];
-  const int m0 = blockIdx.y * 32, n0 = blockIdx.x * 32;
+  const int ntn = (N + 31) / 32;   // one grid dimension: the others end at 65535 tiles
+  const int m0 = blockIdx.x / ntn * 32, n0 = blockIdx.x % ntn * 32;
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
   const int lo = threadIdx.x & 31, hi = threadIdx.x >> 5;   // neighbouring threads: neighbouring addresses
   float ra[4], rb[4];
@@ -104,8 +106,9 @@ __global__ void __launch_bounds__(256) k_ws_gemm(const T* __restrict__ A, long s
 template <typename T>
 cudaError_t gemm(const T* A, long sam, long sak, const T* B, long sbk, long sbn, int M, int N, int K,
                  const float* bias, float* C, int ldc, cudaStream_t st) {
-  dim3 grid((N + 31) / 32, (M + 31) / 32);
-  return launch_pdl(k_ws_gemm<T>, grid, dim3(256), 0, st, A, sam, sak, B, sbk, sbn, M, N, K, bias, C, ldc);
+  const long long tiles = (N + 31LL) / 32 * ((M + 31LL) / 32);
+  if (tiles > INT_MAX) return cudaErrorInvalidValue;
+  return launch_pdl(k_ws_gemm<T>, dim3((unsigned)tiles), dim3(256), 0, st, A, sam, sak, B, sbk, sbn, M, N, K, bias, C, ldc);
 }
 
 template <typename T>
@@ -253,7 +256,8 @@ __global__ void __launch_bounds__(256) k_ws_gather(const float* __restrict__ Ud,
                                                    int ldt, float* __restrict__ Tt) {
   griddep_wait();
   griddep_launch();
-  const int r = blockIdx.x, c = blockIdx.y * 256 + threadIdx.x;
+  const int per_row = (n_in + n_out + 255) / 256;   // blocks
+  const int r = blockIdx.x / per_row, c = blockIdx.x % per_row * 256 + threadIdx.x;
   const size_t row = idx[r];
   if (c < n_in) {
     const float v = Ud[row * n_in + c];
@@ -292,9 +296,10 @@ __global__ void __launch_bounds__(256) k_ws_standardize(const double* __restrict
                                                         const double* __restrict__ mean,
                                                         const double* __restrict__ sd,
                                                         float* __restrict__ Y) {
-  const int c = blockIdx.y * 256 + threadIdx.x;
+  const int per_row = (cols + 255) / 256;   // blocks
+  const int c = blockIdx.x % per_row * 256 + threadIdx.x;
   if (c >= cols) return;
-  const size_t o = (size_t)blockIdx.x * cols + c;
+  const size_t o = (size_t)(blockIdx.x / per_row) * cols + c;
   Y[o] = (float)((X[o] - mean[c]) / sd[c]);
 }
 
@@ -460,8 +465,15 @@ int make_plans(nnc_ws* s, int B) {
 
 template <typename T>
 cudaError_t gelu(nnc_ws* s, const float* Z, int B, int cols, void* Hl, float* D1, __nv_bfloat16* Ht) {
-  return launch_pdl(k_ws_gelu<T>, dim3((B * cols + 63) / 64), dim3(64), 0, s->stream, Z, B * cols, (T*)Hl,
-                    D1, cols, Ht, s->cap);
+  const int rows = std::max(1, (1 << 30) / cols);   // of a launch, whose elements an int counts
+  for (int r = 0; r < B; r += rows) {
+    const int n = std::min(rows, B - r) * cols;
+    const size_t o = (size_t)r * cols;
+    const cudaError_t e = launch_pdl(k_ws_gelu<T>, dim3((n + 63) / 64), dim3(64), 0, s->stream, Z + o, n,
+                                     (T*)Hl + o, D1 + o, cols, Ht ? Ht + r : nullptr, s->cap);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 // forward on the first B rows of s->Ul (operand type): P = net(U)
@@ -747,8 +759,9 @@ int nnc_ws_train(nnc_ws* s, const double* U, const double* Tt, int N, int epochs
   double *mean = s->stats, *sd = s->stats + nc;
   k_ws_stats<<<(n_in + 31) / 32, 32, 0, st>>>(s->Ur, N, n_in, mean, sd);
   k_ws_stats<<<(n_out + 31) / 32, 32, 0, st>>>(s->Tr, N, n_out, mean + n_in, sd + n_in);
-  k_ws_standardize<<<dim3(N, (n_in + 255) / 256), 256, 0, st>>>(s->Ur, n_in, mean, sd, s->Ud);
-  k_ws_standardize<<<dim3(N, (n_out + 255) / 256), 256, 0, st>>>(s->Tr, n_out, mean + n_in, sd + n_in, s->Td);
+  k_ws_standardize<<<(unsigned)N * ((n_in + 255) / 256), 256, 0, st>>>(s->Ur, n_in, mean, sd, s->Ud);
+  k_ws_standardize<<<(unsigned)N * ((n_out + 255) / 256), 256, 0, st>>>(s->Tr, n_out, mean + n_in, sd + n_in,
+                                                                       s->Td);
   note_launch(4);
   WCK(cudaGetLastError());
   std::vector<double> h(2 * (size_t)nc);
@@ -762,7 +775,7 @@ int nnc_ws_train(nnc_ws* s, const double* U, const double* Tt, int N, int epochs
   std::vector<int> perm(N);
   std::iota(perm.begin(), perm.end(), 0);
   double last = 0.0;
-  const dim3 gg(B, (nc + 255) / 256);
+  const dim3 gg((unsigned)B * ((nc + 255) / 256));
   for (int e = 0; e < epochs; ++e) {
     std::shuffle(perm.begin(), perm.end(), rng);
     WCK(cudaMemcpyAsync(s->perm, perm.data(), sizeof(int) * N, cudaMemcpyHostToDevice, st));

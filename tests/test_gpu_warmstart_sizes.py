@@ -52,3 +52,23 @@ def test_launches_that_fail_are_reported(lib):
     ws.free()
     ws = lib.WarmStart(params(3, 5, 4, 2), precision="fp32")
     assert np.max(np.abs(ws.predict(U[:100]) - a[:100])) < 1e-5
+
+
+def test_predict_more_rows(lib):
+    ws, U, a = many_rows(lib)
+    assert np.max(np.abs(ws.predict(U) - a)) < 1e-5
+
+
+def test_train_more_columns(lib):
+    """Two rows standardize to -1 and 1, so that the gradient of W_1 has the sign of their difference times
+    that of a common factor, and the first Adam step moves every weight by the learning rate."""
+    n, lr = 256 * 65536 + 1, 1e-3
+    p = params(n, 1, 2, 2)
+    U, T = normal(derive_key(5, "wsz-u"), 2 * n).reshape(2, n), np.array([[0.0, 1.0], [2.0, -1.0]])
+    ws = lib.WarmStart(p, precision="fp32")
+    loss = ws.train(U, T, 1, batch=2, lr=lr, seed=1)
+    step = (ws.params()[0] - p[0].astype(np.float32))[0] / lr
+    assert np.isfinite(loss)
+    sign = np.sign(U[0] - U[1])
+    # FP32 weights of 1e-4 in size: the step is off by their rounding, 2^-24 * 2^-10 against 1e-3 at most
+    assert np.max(np.abs(step * sign * np.sign(step[0] * sign[0]) - 1.0)) < 1e-3
