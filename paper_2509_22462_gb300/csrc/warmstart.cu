@@ -268,29 +268,32 @@ __global__ void __launch_bounds__(256) k_ws_gather(const float* __restrict__ Ud,
   }
 }
 
-// Mean and standard deviation of each column of X [N][cols], rows in order, 16 loads in flight.
-__global__ void __launch_bounds__(32) k_ws_stats(const double* __restrict__ X, int N, int cols,
-                                                 double* __restrict__ mean, double* __restrict__ sd) {
+// Mean and standard deviation of each column of X [N][cols], rows in order, 16 loads in flight.  The rows
+// may come in several parts, rows [r0, r0 + n) of N at a time: all of them with pass = 0, then again with
+// pass = 1.  With pass = 2 X is all N rows and one launch does both.
+__global__ void __launch_bounds__(32) k_ws_stats(const double* __restrict__ X, int pass, int r0, int n, int N,
+                                                 int cols, double* __restrict__ mean,
+                                                 double* __restrict__ sd) {
   const int j = blockIdx.x * 32 + threadIdx.x;
   if (j >= cols) return;
-  double mu = 0.0, sq = 0.0;
+  double mu = pass != 1 ? (r0 == 0 ? 0.0 : mean[j]) : mean[j], sq = pass != 1 || r0 == 0 ? 0.0 : sd[j];
 #pragma unroll 1
-  for (int pass = 0; pass < 2; ++pass) {
-    for (int r0 = 0; r0 < N; r0 += 16) {
+  for (int p = pass == 1; p < (pass == 0 ? 1 : 2); ++p) {
+    for (int b = 0; b < n; b += 16) {
       double v[16];
 #pragma unroll
-      for (int u = 0; u < 16; ++u) v[u] = r0 + u < N ? X[(size_t)(r0 + u) * cols + j] : 0.0;
+      for (int u = 0; u < 16; ++u) v[u] = b + u < n ? X[(size_t)(b + u) * cols + j] : 0.0;
 #pragma unroll
       for (int u = 0; u < 16; ++u) {
-        if (r0 + u >= N) break;
-        if (pass == 0) mu += v[u];
+        if (b + u >= n) break;
+        if (p == 0) mu += v[u];
         else sq += (v[u] - mu) * (v[u] - mu);
       }
     }
-    if (pass == 0) mu /= N;
+    if (p == 0 && r0 + n == N) mu /= N;
   }
   mean[j] = mu;
-  sd[j] = fmax(sqrt(sq / N), 1e-12);
+  if (pass != 0) sd[j] = r0 + n == N ? fmax(sqrt(sq / N), 1e-12) : sq;
 }
 __global__ void __launch_bounds__(256) k_ws_standardize(const double* __restrict__ X, int cols,
                                                         const double* __restrict__ mean,
@@ -342,12 +345,12 @@ struct nnc_ws {
         *P = nullptr, *dH = nullptr;   // D1, D2: GELU' of the two hidden layers
   void *Ul = nullptr, *H1l = nullptr, *H2l = nullptr, *dPl = nullptr, *dZl = nullptr;
   double* part = nullptr;   // [n_out] the loss's column sums
-  // training set on the device (capacity nd rows): as given, standardized, the epoch's order, and the
-  // means and deviations of the columns [2][n_in + n_out]
-  double *Ur = nullptr, *Tr = nullptr, *stats = nullptr;
+  // training set on the device (capacity nd rows): standardized, the epoch's order, the means and
+  // deviations of the columns [2][n_in + n_out], and nr rows of it as given
   float *Ud = nullptr, *Td = nullptr;
   int* perm = nullptr;
-  int nd = 0;
+  double *Ur = nullptr, *Tr = nullptr, *stats = nullptr;
+  int nd = 0, nr = 0;
   // tensor-core path (BF16 form with n_in, h1, h2 multiples of 64): transposed BF16 operand copies
   // (row stride cap), dP with its row stride padded to n_out_p, W2^T and W3^T, and the plans of
   // the eight products (built for `plan_rows` batch rows)
@@ -412,7 +415,8 @@ int ensure_cap(nnc_ws* s, int B) {
   return NNC_OK;
 }
 
-// training-set buffers for N rows; a larger set replaces them
+// training-set buffers for N rows; a larger set replaces them.  The FP64 rows as given are needed until they
+// are standardized: all at once where they take an eighth of the free memory or less, else in parts.
 int ensure_set(nnc_ws* s, int N) {
   if (N <= s->nd) return NNC_OK;
   WCK(cudaStreamSynchronize(s->stream));
@@ -425,12 +429,16 @@ int ensure_set(nnc_ws* s, int N) {
   s->Ud = s->Td = nullptr;
   s->perm = nullptr;
   s->nd = 0;
-  WAL(s->Ur, (size_t)N * s->n_in);
-  WAL(s->Tr, (size_t)N * s->n_out);
   WAL(s->Ud, (size_t)N * s->n_in);
   WAL(s->Td, (size_t)N * s->n_out);
   WAL(s->perm, N);
   if (!s->stats) WAL(s->stats, 2 * (size_t)(s->n_in + s->n_out));
+  size_t free_b = 0, total_b = 0;
+  WCK(cudaMemGetInfo(&free_b, &total_b));
+  const size_t row = sizeof(double) * ((size_t)s->n_in + s->n_out);
+  s->nr = (int)std::min<size_t>(N, std::max<size_t>(1, free_b / 8 / row));
+  WAL(s->Ur, (size_t)s->nr * s->n_in);
+  WAL(s->Tr, (size_t)s->nr * s->n_out);
   s->nd = N;
   return NNC_OK;
 }
@@ -753,17 +761,30 @@ int nnc_ws_train(nnc_ws* s, const double* U, const double* Tt, int N, int epochs
   if (r) return r;
   cudaStream_t st = s->stream;
   // the data set goes to the device as given and is standardized there, per coordinate; batches are
-  // gathered by index
-  WCK(cudaMemcpyAsync(s->Ur, U, sizeof(double) * (size_t)N * n_in, cudaMemcpyHostToDevice, st));
-  WCK(cudaMemcpyAsync(s->Tr, Tt, sizeof(double) * (size_t)N * n_out, cudaMemcpyHostToDevice, st));
+  // gathered by index.  A set that does not fit beside its standardized copy is sent three times in parts:
+  // for the means, the deviations and the standardized values.
   double *mean = s->stats, *sd = s->stats + nc;
-  k_ws_stats<<<(n_in + 31) / 32, 32, 0, st>>>(s->Ur, N, n_in, mean, sd);
-  k_ws_stats<<<(n_out + 31) / 32, 32, 0, st>>>(s->Tr, N, n_out, mean + n_in, sd + n_in);
-  k_ws_standardize<<<(unsigned)N * ((n_in + 255) / 256), 256, 0, st>>>(s->Ur, n_in, mean, sd, s->Ud);
-  k_ws_standardize<<<(unsigned)N * ((n_out + 255) / 256), 256, 0, st>>>(s->Tr, n_out, mean + n_in, sd + n_in,
-                                                                       s->Td);
-  note_launch(4);
-  WCK(cudaGetLastError());
+  const int part = std::min(s->nr, N);
+  for (int pass = part == N ? 2 : 0; pass <= 2; ++pass) {
+    for (int r0 = 0; r0 < N; r0 += part) {
+      const int n = std::min(part, N - r0);
+      const size_t ou = (size_t)r0 * n_in, ot = (size_t)r0 * n_out;
+      WCK(cudaMemcpyAsync(s->Ur, U + ou, sizeof(double) * (size_t)n * n_in, cudaMemcpyHostToDevice, st));
+      WCK(cudaMemcpyAsync(s->Tr, Tt + ot, sizeof(double) * (size_t)n * n_out, cudaMemcpyHostToDevice, st));
+      if (pass < 2 || part == N) {
+        k_ws_stats<<<(n_in + 31) / 32, 32, 0, st>>>(s->Ur, pass, r0, n, N, n_in, mean, sd);
+        k_ws_stats<<<(n_out + 31) / 32, 32, 0, st>>>(s->Tr, pass, r0, n, N, n_out, mean + n_in, sd + n_in);
+        note_launch(2);
+      }
+      if (pass == 2) {
+        k_ws_standardize<<<(unsigned)n * ((n_in + 255) / 256), 256, 0, st>>>(s->Ur, n_in, mean, sd, s->Ud + ou);
+        k_ws_standardize<<<(unsigned)n * ((n_out + 255) / 256), 256, 0, st>>>(s->Tr, n_out, mean + n_in,
+                                                                             sd + n_in, s->Td + ot);
+        note_launch(2);
+      }
+      WCK(cudaGetLastError());
+    }
+  }
   std::vector<double> h(2 * (size_t)nc);
   WCK(cudaMemcpyAsync(h.data(), s->stats, sizeof(double) * h.size(), cudaMemcpyDeviceToHost, st));
   WCK(cudaStreamSynchronize(st));

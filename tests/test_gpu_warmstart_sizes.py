@@ -72,3 +72,29 @@ def test_train_more_columns(lib):
     sign = np.sign(U[0] - U[1])
     # FP32 weights of 1e-4 in size: the step is off by their rounding, 2^-24 * 2^-10 against 1e-3 at most
     assert np.max(np.abs(step * sign * np.sign(step[0] * sign[0]) - 1.0)) < 1e-3
+
+
+@pytest.mark.parametrize("precision", ["bf16", "fp32"])
+def test_train_set_that_fills_the_memory(lib, precision):
+    """A data set whose standardized FP32 values fit trains, to the same bits as with room to spare: 33 MB
+    beside the 66 MB of the values as given, with 80 MB free."""
+    import torch
+    n, rows = 1024, 4001
+    p = params(n, 64, 64, n)
+    U = normal(derive_key(6, "wsz-u"), n * rows).reshape(rows, n)
+    T = U[:, ::-1] ** 2
+
+    def train(room):
+        ws = lib.WarmStart(p, precision=precision)
+        torch.cuda.empty_cache()
+        hold = torch.empty(max(torch.cuda.mem_get_info()[0] - room, 1), dtype=torch.uint8, device="cuda")
+        try:
+            out = [ws.train(U, T, 1, batch=64, seed=2)] + ws.params()
+        finally:
+            del hold
+            torch.cuda.empty_cache()
+            ws.free()
+        return out
+
+    for a, b in zip(train(8 << 30), train(80 << 20)):
+        assert np.array_equal(a, b)
