@@ -99,7 +99,10 @@ int balloc(nnc_batch* b, T** p, size_t n) {
   void* q = nullptr;
   const size_t bytes = std::max<size_t>(n, 1) * sizeof(T);
   cudaError_t e = cudaMalloc(&q, bytes);
-  if (e != cudaSuccess) return bfail(NNC_ERR_OOM, std::string("cudaMalloc: ") + cudaGetErrorString(e));
+  if (e != cudaSuccess) {
+    cudaGetLastError();   // reported here, not by the next launch
+    return bfail(NNC_ERR_OOM, std::string("cudaMalloc: ") + cudaGetErrorString(e));
+  }
   e = cudaMemsetAsync(q, 0, bytes, b->stream);
   if (e != cudaSuccess) return bfail(NNC_ERR_CUDA, cudaGetErrorString(e));
   b->allocs.push_back(q);

@@ -68,9 +68,11 @@ int dalloc(nnc_net* net, T** p, size_t n) {
   void* q = nullptr;
   const size_t bytes = std::max<size_t>(n, 1) * sizeof(T);
   cudaError_t e = cudaMalloc(&q, bytes);
-  if (e != cudaSuccess)
+  if (e != cudaSuccess) {
+    cudaGetLastError();   // reported here, not by the next launch
     return fail(NNC_ERR_OOM, std::string("cudaMalloc(") + std::to_string(bytes) + "): " +
                                  cudaGetErrorString(e));
+  }
   e = cudaMemsetAsync(q, 0, bytes, net->stream);
   net->allocs.push_back(q);
   if (e != cudaSuccess) return fail(NNC_ERR_CUDA, cudaGetErrorString(e));

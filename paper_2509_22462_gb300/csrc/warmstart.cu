@@ -368,7 +368,10 @@ namespace {
 template <typename X>
 int walloc(nnc_ws* s, X** p, size_t n) {
   void* q = nullptr;
-  if (cudaMalloc(&q, std::max<size_t>(n, 1) * sizeof(X)) != cudaSuccess) return wfail(NNC_ERR_OOM, "cudaMalloc failed");
+  if (cudaMalloc(&q, std::max<size_t>(n, 1) * sizeof(X)) != cudaSuccess) {
+    cudaGetLastError();   // reported here, not by the next launch
+    return wfail(NNC_ERR_OOM, "cudaMalloc failed");
+  }
   cudaMemsetAsync(q, 0, std::max<size_t>(n, 1) * sizeof(X), s->stream);
   s->allocs.push_back(q);
   *p = (X*)q;
