@@ -228,13 +228,13 @@ cudaError_t launch_sgemm_c(const SgArgs& a, int splits, cudaStream_t st) {
 }
 
 template <int EPI>
-cudaError_t launch_sgemm(const SgArgs& a, int splits, cudaStream_t st) {
+cudaError_t launch_sgemm(const SgArgs& a, int splits, int sm_count, cudaStream_t st) {
   // columns per lane: the least time of the busiest SM, tiles times 4 + C (the bound above)
   int best = 8;
   long long least = -1;
   for (int c : {8, 6, 4, 2}) {
     const long long t = (long long)((a.M + kSgM - 1) / kSgM) * ((a.N + 8 * c - 1) / (8 * c)) * splits;
-    const long long cost = (t + 151) / 152 * (4 + c);
+    const long long cost = (t + sm_count - 1) / sm_count * (4 + c);
     if (least < 0 || cost < least) {
       least = cost;
       best = c;
@@ -250,7 +250,7 @@ cudaError_t launch_sgemm(const SgArgs& a, int splits, cudaStream_t st) {
 
 cudaError_t launch_simt_tangent(bool fp64, const void* A, int lda, const void* B, int ldb, int M,
                                 int N, int K, const double* s1, const double* c, void* At, int ldo,
-                                void* Zt, void* Yt, int ldz, cudaStream_t st) {
+                                void* Zt, void* Yt, int ldz, int sm_count, cudaStream_t st) {
   if (fp64) {
     dim3 grid((N + 63) / 64, (M + 63) / 64, 1);
     k_simt_gemm<double, 4, 4, EPI_TANGENT><<<grid, 256, 0, st>>>(
@@ -259,14 +259,14 @@ cudaError_t launch_simt_tangent(bool fp64, const void* A, int lda, const void* B
   } else {
     return launch_sgemm<EPI_TANGENT>(SgArgs{(const float*)A, (const float*)B, lda, ldb, M, N, K, K, s1, c,
                                             (float*)At, (float*)Zt, (float*)Yt, ldo, ldz, nullptr},
-                                     1, st);
+                                     1, sm_count, st);
   }
   note_launch();
   return cudaGetLastError();
 }
 
 cudaError_t launch_simt_syrk(bool fp64, const void* Zt, const void* Yt, int ld, int n, int K,
-                             int splits, double* Hp, cudaStream_t st) {
+                             int splits, double* Hp, int sm_count, cudaStream_t st) {
   const int kps = ((K + splits - 1) / splits + 15) / 16 * 16;
   if (fp64) {
     dim3 grid((n + 63) / 64, (n + 63) / 64, splits);
@@ -276,7 +276,7 @@ cudaError_t launch_simt_syrk(bool fp64, const void* Zt, const void* Yt, int ld, 
   } else {
     return launch_sgemm<EPI_SYRK>(SgArgs{(const float*)Yt, (const float*)Zt, ld, ld, n, n, K, kps, nullptr,
                                          nullptr, nullptr, nullptr, nullptr, 0, 0, Hp},
-                                  splits, st);
+                                  splits, sm_count, st);
   }
   note_launch();
   return cudaGetLastError();

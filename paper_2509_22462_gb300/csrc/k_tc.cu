@@ -1650,7 +1650,7 @@ cudaError_t launch_gtan_mode(const TcPlan& p, const TcArgs& a, int groups, int g
 }
 
 int tc_plain_plan(PlainPlan& p, const void* A, int a_rows, int lda, const void* B, int b_rows,
-                  int ldb, int M, int N, int K) {
+                  int ldb, int M, int N, int K, int sm_count) {
   p = PlainPlan();
   if (M <= 0 || N <= 0 || K <= 0 || K % 64 != 0 || lda % 8 != 0 || ldb % 8 != 0 || !A || !B)
     return NNC_ERR_ARG;
@@ -1660,7 +1660,7 @@ int tc_plain_plan(PlainPlan& p, const void* A, int a_rows, int lda, const void* 
   p.ntm = (M + BM - 1) / BM;
   // small products are bound by latency, most of it one CTA's epilogue: 32-column tiles while they fit
   // the chip in one wave
-  p.bn = p.ntm * ((N + 31) / 32) <= 152 ? 32 : N <= 128 ? 128 : 256;
+  p.bn = p.ntm * ((N + 31) / 32) <= sm_count ? 32 : N <= 128 ? 128 : 256;
   p.ntn = (N + p.bn - 1) / p.bn;
   if (!make_map(&p.ta, A, a_rows, K, lda, BM, 64) || !make_map(&p.tb, B, b_rows, K, ldb, p.bn, 64))
     return NNC_ERR_CUDA;

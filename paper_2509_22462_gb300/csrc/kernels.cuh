@@ -81,10 +81,11 @@ cudaError_t launch_copy_pad(const double* src, double* dst, void* dst2, int n, i
 // Yt[n][m] = c[m] D (row stride ldz; both may be NULL)  for n < N.
 cudaError_t launch_simt_tangent(bool fp64, const void* A, int lda, const void* B, int ldb, int M,
                                 int N, int K, const double* s1, const double* c, void* At, int ldo,
-                                void* Zt, void* Yt, int ldz, cudaStream_t st);
-// Symmetric-product epilogue: Hp[s][i][j] += D over the lower-triangle tiles, split-K `splits`.
+                                void* Zt, void* Yt, int ldz, int sm_count, cudaStream_t st);
+// Symmetric product: partials Hp[s][i][j] of the lower-triangle tiles, split-K `splits`; FP64 adds to them,
+// FP32 stores them.
 cudaError_t launch_simt_syrk(bool fp64, const void* Zt, const void* Yt, int ld, int n, int K,
-                             int splits, double* Hp, cudaStream_t st);
+                             int splits, double* Hp, int sm_count, cudaStream_t st);
 
 }  // namespace nnc
 

@@ -415,7 +415,7 @@ int run_hessian(nnc_net* net, const double* lam, double* H, cudaStream_t st, boo
                              prec == NNC_FP64 ? (const void*)Ly.W64 : (const void*)Ly.W32, Ly.kp,
                              net->At[cur][0], Ly.kp, Ly.mp, n, Ly.kp, Ly.s1, Ly.c, Anext_hi, Ly.mp,
                              zoff(net->Zt[0], Ly.zy_off), zoff(net->Yt[0], Ly.zy_off),
-                             net->K_total, st));
+                             net->K_total, net->sm_count, st));
     }
     cur = 1 - cur;
   }
@@ -459,7 +459,7 @@ int run_hessian(nnc_net* net, const double* lam, double* H, cudaStream_t st, boo
       CK(tc_syrk(net->plan_syrk, (float*)net->Hp, net->dev_err, st));
     else
       CK(launch_simt_syrk(prec == NNC_FP64, net->Zt[0], net->Yt[0], net->K_total, n, net->K_total,
-                          net->h_splits, (double*)net->Hp, st));
+                          net->h_splits, (double*)net->Hp, net->sm_count, st));
   }
   {
     PROF(PK_OTHER);

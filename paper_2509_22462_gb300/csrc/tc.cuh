@@ -79,7 +79,7 @@ struct PlainPlan {
   bool ready = false;
 };
 int tc_plain_plan(PlainPlan& p, const void* A, int a_rows, int lda, const void* B, int b_rows,
-                  int ldb, int M, int N, int K);
+                  int ldb, int M, int N, int K, int sm_count);
 cudaError_t tc_plain(const PlainPlan& p, const float* bias, float* C, int ldc, int* err,
                      cudaStream_t st);
 

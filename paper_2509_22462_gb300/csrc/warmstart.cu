@@ -361,6 +361,7 @@ struct nnc_ws {
   int* d_err = nullptr;
   nnc::PlainPlan pl[8];
   int plan_rows = -1;
+  int sm_count = 0;
 };
 
 namespace {
@@ -450,19 +451,19 @@ int ensure_set(nnc_ws* s, int N) {
 int make_plans(nnc_ws* s, int B) {
   if (s->plan_rows == B) return NNC_OK;
   using nnc::tc_plain_plan;
-  const int cap = s->cap;
+  const int cap = s->cap, sms = s->sm_count;
   const __nv_bfloat16* w1 = (const __nv_bfloat16*)s->wl[0];
   const __nv_bfloat16* w2 = (const __nv_bfloat16*)s->wl[2];
   const __nv_bfloat16* w3 = (const __nv_bfloat16*)s->wl[4];
-  int r = tc_plain_plan(s->pl[0], s->Ul, B, s->n_in, w1, s->h1, s->n_in, B, s->h1, s->n_in);
-  if (!r) r = tc_plain_plan(s->pl[1], s->H1l, B, s->h1, w2, s->h2, s->h1, B, s->h2, s->h1);
-  if (!r) r = tc_plain_plan(s->pl[2], s->H2l, B, s->h2, w3, s->n_out, s->h2, B, s->n_out, s->h2);
+  int r = tc_plain_plan(s->pl[0], s->Ul, B, s->n_in, w1, s->h1, s->n_in, B, s->h1, s->n_in, sms);
+  if (!r) r = tc_plain_plan(s->pl[1], s->H1l, B, s->h1, w2, s->h2, s->h1, B, s->h2, s->h1, sms);
+  if (!r) r = tc_plain_plan(s->pl[2], s->H2l, B, s->h2, w3, s->n_out, s->h2, B, s->n_out, s->h2, sms);
   if (!r && B % 64 == 0) {
-    r = tc_plain_plan(s->pl[3], s->dPt, s->n_out, cap, s->H2t, s->h2, cap, s->n_out, s->h2, B);
-    if (!r) r = tc_plain_plan(s->pl[4], s->dPp, B, s->n_out_p, s->W3t, s->h2, s->n_out_p, B, s->h2, s->n_out_p);
-    if (!r) r = tc_plain_plan(s->pl[5], s->dZt, s->h2, cap, s->H1t, s->h1, cap, s->h2, s->h1, B);
-    if (!r) r = tc_plain_plan(s->pl[6], s->dZl, B, s->h2, s->W2t, s->h1, s->h2, B, s->h1, s->h2);
-    if (!r) r = tc_plain_plan(s->pl[7], s->dZt, s->h1, cap, s->Ut, s->n_in, cap, s->h1, s->n_in, B);
+    r = tc_plain_plan(s->pl[3], s->dPt, s->n_out, cap, s->H2t, s->h2, cap, s->n_out, s->h2, B, sms);
+    if (!r) r = tc_plain_plan(s->pl[4], s->dPp, B, s->n_out_p, s->W3t, s->h2, s->n_out_p, B, s->h2, s->n_out_p, sms);
+    if (!r) r = tc_plain_plan(s->pl[5], s->dZt, s->h2, cap, s->H1t, s->h1, cap, s->h2, s->h1, B, sms);
+    if (!r) r = tc_plain_plan(s->pl[6], s->dZl, B, s->h2, s->W2t, s->h1, s->h2, B, s->h1, s->h2, sms);
+    if (!r) r = tc_plain_plan(s->pl[7], s->dZt, s->h1, cap, s->Ut, s->n_in, cap, s->h1, s->n_in, B, sms);
   }
   if (r) return wfail(r, "warm start: tensor-core plan failed");
   s->plan_rows = B;
@@ -641,6 +642,12 @@ int nnc_ws_create(nnc_ws** out, int n_in, int h1, int h2, int n_out, const doubl
   s->h2 = h2;
   s->n_out = n_out;
   s->prec = prec;
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&s->sm_count, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+    delete s;
+    return wfail(NNC_ERR_CUDA, "no CUDA device");
+  }
   if (stream) s->stream = (cudaStream_t)stream;
   else {
     if (cudaStreamCreateWithFlags(&s->stream, cudaStreamNonBlocking) != cudaSuccess) {
