@@ -87,14 +87,9 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const void* map, uint3
       : "memory");
 }
 
-// Barrier among the first `threads` threads of the CTA (named barrier `id`, 1..15).
-__device__ __forceinline__ void named_sync(int id, int threads) {
-  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
-}
-
-// The same with the barrier's number known at compile time (a number in a register reserves all 16
-// barriers, which limits the CTAs of an SM), and arriving there without waiting: the thread's earlier
-// shared-memory accesses are seen after the barrier.
+// Barrier among `threads` threads of the CTA (named barrier ID, 1..15, known at compile time: a number in a
+// register reserves all 16 barriers, which limits the CTAs of an SM), and arriving there without waiting:
+// the thread's earlier shared-memory accesses are seen after the barrier.
 template <int ID>
 __device__ __forceinline__ void named_sync(int threads) {
   asm volatile("bar.sync %0, %1;" ::"n"(ID), "r"(threads) : "memory");

@@ -1,8 +1,8 @@
 // CUDA-core GEMMs of the FP64 and FP32 forms: the forward tangent sweep of the Hessian
 // (Zdot_l = W_l Adot_{l-1}, n_in tangent columns) and the symmetric product
 // H = sum_l Zdot_l^T diag(c_l) Zdot_l, every sum in order of k.  k_sgemm is the FP32 form's; k_simt_gemm
-// the FP64 form's, which comes here only when the residue products of k_rns.cu do not fit (their
-// residues take four times the memory of the FP64 weights).
+// the FP64 form's, which comes here only where the residue products of k_rns.cu do not serve: their residues
+// take four times the memory of the FP64 weights, and keep too few bits of uneven weights.
 #include <algorithm>
 
 #include "async.cuh"
@@ -12,48 +12,48 @@ namespace nnc {
 
 enum { EPI_TANGENT = 0, EPI_SYRK = 1 };
 
-// D[m][n] = sum_k A[m][k] B[n][k] on a (16*TM) x (16*TN) tile with 256 threads; thread (tx, ty)
+// FP64: D[m][n] = sum_k A[m][k] B[n][k] on a 64 x 64 tile with 256 threads; thread (tx, ty)
 // owns rows m0 + tx + 16 i and columns n0 + ty + 16 j.  K must be a multiple of 16 (all
 // packed dimensions are multiples of 128).
-template <typename T, int TM, int TN, int EPI>
-__global__ void __launch_bounds__(256) k_simt_gemm(const T* __restrict__ A, int lda,
-                                                   const T* __restrict__ B, int ldb, int M, int N,
+template <int EPI>
+__global__ void __launch_bounds__(256) k_simt_gemm(const double* __restrict__ A, int lda,
+                                                   const double* __restrict__ B, int ldb, int M, int N,
                                                    int K, int k_per_split,
                                                    const double* __restrict__ s1,
                                                    const double* __restrict__ c,
-                                                   T* __restrict__ At, T* __restrict__ Zt,
-                                                   T* __restrict__ Yt, int ldo, int ldz,
+                                                   double* __restrict__ At, double* __restrict__ Zt,
+                                                   double* __restrict__ Yt, int ldo, int ldz,
                                                    double* __restrict__ Hp) {
-  constexpr int BM = 16 * TM, BN = 16 * TN, BK = 16;
-  __shared__ T As[BK][BM + 1];
-  __shared__ T Bs[BK][BN + 1];
+  constexpr int TM = 4, TN = 4, BM = 16 * TM, BN = 16 * TN, BK = 16;
+  __shared__ double As[BK][BM + 1];
+  __shared__ double Bs[BK][BN + 1];
   const int bm = blockIdx.y, bn = blockIdx.x, split = blockIdx.z;
   if (EPI == EPI_SYRK && bn > bm) return;  // upper-triangle tiles are mirrored at the end
   const int m0 = bm * BM, n0 = bn * BN;
   const int kbeg = split * k_per_split;
   const int kend = min(K, kbeg + k_per_split);
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  T acc[TM][TN];
+  double acc[TM][TN];
 #pragma unroll
   for (int i = 0; i < TM; ++i)
 #pragma unroll
-    for (int j = 0; j < TN; ++j) acc[i][j] = T(0);
+    for (int j = 0; j < TN; ++j) acc[i][j] = 0.0;
 
   for (int k0 = kbeg; k0 < kend; k0 += BK) {
     for (int i = threadIdx.x; i < BM * BK; i += 256) {
       const int r = i >> 4, kk = i & 15;
       const int gm = m0 + r;
-      As[kk][r] = gm < M ? A[(size_t)gm * lda + k0 + kk] : T(0);
+      As[kk][r] = gm < M ? A[(size_t)gm * lda + k0 + kk] : 0.0;
     }
     for (int i = threadIdx.x; i < BN * BK; i += 256) {
       const int r = i >> 4, kk = i & 15;
       const int gn = n0 + r;
-      Bs[kk][r] = gn < N ? B[(size_t)gn * ldb + k0 + kk] : T(0);
+      Bs[kk][r] = gn < N ? B[(size_t)gn * ldb + k0 + kk] : 0.0;
     }
     __syncthreads();
 #pragma unroll
     for (int kk = 0; kk < BK; ++kk) {
-      T a[TM], b[TN];
+      double a[TM], b[TN];
 #pragma unroll
       for (int i = 0; i < TM; ++i) a[i] = As[kk][tx + 16 * i];
 #pragma unroll
@@ -76,12 +76,12 @@ __global__ void __launch_bounds__(256) k_simt_gemm(const T* __restrict__ A, int 
       for (int j = 0; j < TN; ++j) {
         const int n = n0 + ty + 16 * j;
         if (n >= N) continue;
-        const double v = (double)acc[i][j];
-        if (At) At[(size_t)n * ldo + m] = (T)(sm * v);
+        const double v = acc[i][j];
+        if (At) At[(size_t)n * ldo + m] = sm * v;
         if (Zt) {
           const size_t oz = (size_t)n * ldz + m;
-          Zt[oz] = (T)v;
-          Yt[oz] = (T)(cm * v);
+          Zt[oz] = v;
+          Yt[oz] = cm * v;
         }
       }
     }
@@ -95,7 +95,7 @@ __global__ void __launch_bounds__(256) k_simt_gemm(const T* __restrict__ A, int 
       for (int j = 0; j < TN; ++j) {
         const int n = n0 + ty + 16 * j;
         if (n >= N) continue;
-        hp[(size_t)m * N + n] += (double)acc[i][j];
+        hp[(size_t)m * N + n] += acc[i][j];
       }
     }
   }
@@ -253,7 +253,7 @@ cudaError_t launch_simt_tangent(bool fp64, const void* A, int lda, const void* B
                                 void* Zt, void* Yt, int ldz, int sm_count, cudaStream_t st) {
   if (fp64) {
     dim3 grid((N + 63) / 64, (M + 63) / 64, 1);
-    k_simt_gemm<double, 4, 4, EPI_TANGENT><<<grid, 256, 0, st>>>(
+    k_simt_gemm<EPI_TANGENT><<<grid, 256, 0, st>>>(
         (const double*)A, lda, (const double*)B, ldb, M, N, K, K, s1, c, (double*)At, (double*)Zt,
         (double*)Yt, ldo, ldz, nullptr);
   } else {
@@ -270,7 +270,7 @@ cudaError_t launch_simt_syrk(bool fp64, const void* Zt, const void* Yt, int ld, 
   const int kps = ((K + splits - 1) / splits + 15) / 16 * 16;
   if (fp64) {
     dim3 grid((n + 63) / 64, (n + 63) / 64, splits);
-    k_simt_gemm<double, 4, 4, EPI_SYRK><<<grid, 256, 0, st>>>(
+    k_simt_gemm<EPI_SYRK><<<grid, 256, 0, st>>>(
         (const double*)Zt, ld, (const double*)Yt, ld, n, n, K, kps, nullptr, nullptr, nullptr,
         nullptr, nullptr, 0, 0, Hp);
   } else {

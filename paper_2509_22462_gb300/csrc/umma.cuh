@@ -1,74 +1,28 @@
-// tcgen05 / TMEM / TMA / mbarrier primitives of the tensor-core kernels (inline PTX for sm_103a).
+// tcgen05 / TMEM primitives of the tensor-core kernels (inline PTX for sm_103a), beside async.cuh.
 #pragma once
 #include <cuda.h>
 #include <cuda_runtime.h>
 #include <cstdint>
 
+#include "async.cuh"
+
 namespace nnc {
 namespace umma {
 
-constexpr long long kWaitCycles = 4000000000LL;  // about two seconds at GB300 clocks
-
-__device__ __forceinline__ uint32_t smem_u32(const void* p) {
-  return (uint32_t)__cvta_generic_to_shared(p);
-}
-
-__device__ __forceinline__ void mbar_init(uint32_t a, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(a), "r"(count) : "memory");
-}
-
-__device__ __forceinline__ void mbar_expect_tx(uint32_t a, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(a), "r"(bytes)
-               : "memory");
-}
-
-__device__ __forceinline__ bool mbar_try(uint32_t a, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}\n"
-      : "=r"(ok)
-      : "r"(a), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
+using async::griddep_launch;
+using async::griddep_wait;
+using async::kWaitCycles;
+using async::mbar_arrive;
+using async::mbar_expect_tx;
+using async::mbar_init;
+using async::smem_u32;
+using async::tma_load_2d;
 
 // Bounded wait for the phase with the given parity.  Returns false if the CTA aborted or the
 // wait ran out (then the error word and the CTA's abort flag are set).
 __device__ __forceinline__ bool mbar_wait(uint32_t a, uint32_t parity, int* err, int code,
                                           volatile int* abort_flag, long long limit = kWaitCycles) {
-  if (mbar_try(a, parity)) return true;
-  const long long t0 = clock64();
-  while (true) {
-    if (mbar_try(a, parity)) return true;
-    if (*abort_flag) return false;
-    if (clock64() - t0 > limit) {
-      atomicCAS(err, 0, code);
-      *abort_flag = 1;
-      return false;
-    }
-  }
-}
-
-// Programmatic dependent launch: wait until the preceding kernel of the stream has completed and
-// its writes are visible; allow the next one to be scheduled.
-__device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void griddep_launch() {
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-}
-
-__device__ __forceinline__ void mbar_arrive(uint32_t a) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(a) : "memory");
-}
-
-__device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, uint32_t mbar,
-                                            int x, int y) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes"
-      " [%0], [%1, {%3, %4}], [%2];" ::"r"(dst),
-      "l"((uint64_t)map), "r"(mbar), "r"(x), "r"(y)
-      : "memory");
+  return async::mbar_wait_abort(a, parity, err, code, abort_flag, limit);
 }
 
 // Shared-memory matrix descriptor of tcgen05 for a K-major tile written by TMA with 128- or
