@@ -179,9 +179,10 @@ __device__ __forceinline__ int block_sum(int v, int* sh) {
 // what it is smaller by: inputs spread over 2^40 left 1e-6 of a column of J, where FP64 products leave
 // 2e-15.  2^de[k] is the geometric mean of column k's entries in units of the first column's, which sees
 // through rows of any size.  The mean is taken of 16 bits of mantissa behind the exponent, in integers, so
-// that the order of the sums does not matter.  A matrix whose means all lie within 2^2.5 of the first one,
-// as those of evenly scaled weights do, stays as it is (784 -> 128 x 2 -> 10 takes 129 us with its
-// exponents of -1, 0 and 1, 126 without).
+// that the order of the sums does not matter.  A matrix whose means all lie within 2^2.5 of the first one
+// (2^4.5 for less than 64 rows, whose means scatter more), as those of evenly scaled weights do, stays as it
+// is: 784 -> 128 x 2 -> 10 takes 129 us with its exponents of -1, 0 and 1, 126 without, and
+// 784 -> 4096 x 7 -> 10 3.87 ms with those of its last layer, 3.84 without.
 struct RnsEven {
   unsigned long long* sum;   // [k] of the nonzero entries' logarithms, times 2^16
   int *cnt, *small;          // [k] nonzero entries; entries in nonzero rows that are small there
@@ -223,8 +224,8 @@ __global__ void __launch_bounds__(256) k_rns_colsum(const double* __restrict__ W
   atomicAdd(e.cnt + col, cnt);
 }
 
-__global__ void __launch_bounds__(256) k_rns_colexp(int k, const RnsEven e, int* __restrict__ de,
-                                                    int* __restrict__ flags) {
+__global__ void __launch_bounds__(256) k_rns_colexp(int m, int k, const RnsEven e,
+                                                    int* __restrict__ de, int* __restrict__ flags) {
   const int col = blockIdx.x * 256 + threadIdx.x;
   if (col >= k) return;
   int q = 0;   // the first column that is not zero
@@ -236,7 +237,7 @@ __global__ void __launch_bounds__(256) k_rns_colexp(int k, const RnsEven e, int*
     d = (int)(num >= 0 ? num / (2 * den) : -((2 * den - 1 - num) / (2 * den)));
   }
   de[col] = d;
-  if (abs(d) > 2) atomicOr(flags, kRnsScaled);
+  if (abs(d) > (m >= 64 ? 2 : 4)) atomicOr(flags, kRnsScaled);
 }
 
 // How uneven W 2^-de is: an entry is small if it lies more than 2^(bits - 44) below its row's largest, so
@@ -1026,7 +1027,7 @@ cudaError_t rns_even_out(const RnsSet& s, const double* W, int ldw, int m, int k
   if (r != cudaSuccess) return r;
   k_rns_colsum<<<dim3((k + 31) / 32, (m + kEvenRows - 1) / kEvenRows), dim3(32, 8), 0, st>>>(W, ldw, m, k, e,
                                                                                              flags);
-  k_rns_colexp<<<(k + 255) / 256, 256, 0, st>>>(k, e, de, flags);
+  k_rns_colexp<<<(k + 255) / 256, 256, 0, st>>>(m, k, e, de, flags);
   k_rns_spread<<<m, 256, 0, st>>>(W, ldw, k, s.bits, de, e, flags);
   k_rns_colspread<<<(k + 255) / 256, 256, 0, st>>>(k, e, flags);
   note_launch(4);
