@@ -1095,8 +1095,11 @@ static int load_impl(nnc_net* net, int n_layers, const int* widths, const int* a
     for (int l = 1; l < n_layers; ++l) {
       LayerDev& Ly = net->layers[l];
       const int cur = (l - 1) % 2;
-      // split form, wide layers: SM pairs, each of which copies half of the tangent tile (784 -> 4096 x 7
-      // -> 10: 705 us against 717 with one SM per tile)
+      // split form, wide layers: SM pairs, each of which copies half of the tangent tile.  Evaluation, pairs
+      // against the best tile of one SM: 784 -> 2048 x 4 198 / 209 us, 784 -> 2304 x 4 219 / 237, 512 -> 4096 x 4
+      // 322 / 325, 600 -> 4096 x 4 336 / 349, 784 -> 4096 x 7 677 / 689, 784 -> 8192 x 3 799 / 836, 300 -> 8192 x 3
+      // 557 / 580; at 300 inputs the padding takes the gain away again (300 -> 2048 x 4 182 / 173, 300 -> 4096 x 4
+      // 297 / 291).
       const bool pair = prec == NNC_BF16X3 && Ly.mp % 256 == 0 && Ly.mp >= 2048 && n > 256;
       int r = prec == NNC_FP8
                   ? tc_plan_make(Ly.plan_tan, TC_TANGENT, prec, Ly.W8, nullptr, Ly.mp, Ly.kp, net->A8,
