@@ -52,12 +52,12 @@ typedef enum {
 /* Number format of the network evaluation (Section 5.1 leaves it unstated).
  *   NNC_FP64   : FP64 weights, value pass and outputs; the reference form.  The products of the
  *                Jacobian, the gradient and the Hessian run on the tensor cores by residues: operands
- *                are integers of 50 (65536-wide layers) to 57 bits (up to 1024) below the largest entry
+ *                are integers of 54 (65536-wide layers) to 58 bits (narrow ones) below the largest entry
  *                of a row, after powers of two have evened out the weights' columns, and the integer
- *                sums are exact.  The error of a column is that of an FP64 sum of normally distributed
- *                terms, whatever the units of inputs, hidden units and outputs.  Weights that powers of
- *                two do not even out, such as sparse ones, and nets whose residues (30 to 32 bytes
- *                per weight) take more than an eighth of the device memory that is free at load, have
+ *                sums are exact.  Column by column the error is no larger than that of FP64 sums,
+ *                whatever the units of inputs, hidden units and outputs.  Weights that powers of
+ *                two do not even out, such as sparse ones, and nets whose residues (32 bytes per
+ *                weight) take more than an eighth of the device memory that is free at load have
  *                FP64 products instead, about 30 times slower on large nets: nnc_fp64_residues tells.
  *   NNC_FP32   : FP32 weights and tangents on CUDA cores, FP32 products, FP64 outputs.
  *   NNC_BF16   : value/Jacobian/adjoint in FP32; Hessian sweep on tcgen05 tensor cores with

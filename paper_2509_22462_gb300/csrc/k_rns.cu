@@ -5,13 +5,12 @@
 // 104M-parameter evaluation in an FP64 GEMM on the CUDA cores.  The residue scheme of Ozaki, Uchino
 // and Imamura ("Ozaki scheme II", 2025) does them with integer products instead:
 //   - every row of either operand is scaled by a power of two and rounded to integers of at most
-//     `bits` + 1 bits below its largest entry (bits = 57 for K <= 1024 with 16 moduli, 52 for K = 4096
-//     with 15);
+//     `bits` + 1 bits below its largest entry (bits = 57 at K = 1024, 56 at 4096, 54 at 65664);
 //   - so an entry 2^j below its row's largest has j bits fewer.  Powers of two even out the columns of the
 //     weights beforehand (k_rns_colsum), which makes the rounding independent of the units in which
 //     inputs, hidden units and outputs are measured; weights that stay uneven (k_rns_spread) keep the
 //     FP64 products;
-//   - an integer is kept as its residues modulo 15 (or 16) pairwise coprime numbers p_i <= 256, each
+//   - an integer is kept as its residues modulo 16 pairwise coprime numbers p_i <= 256, each
 //     in [-p/2, p/2], which BF16 holds exactly;
 //   - one BF16 product per modulus gives the result's residue: products are at most 2^14, so 1024
 //     terms add up exactly in the tensor core's FP32 accumulator, which is reduced mod p_i after
@@ -23,14 +22,13 @@
 // FP64 FMAs per weight would be 2.5 ms of the same evaluation.
 // The only roundings are those of the operands and of the result, so the error does not grow with
 // K as a sum of FP64 products does.  Chosen over slicing into 8-bit digits, which needs 28 products
-// where this needs 15.  Rows holding a NaN or an infinity give NaN.
+// where this needs 16.  Rows holding a NaN or an infinity give NaN.
 //
 // Every kernel waits for the one before it itself (programmatic dependent launch): a small net's evaluation
 // is twenty short launches.
 //
-// Measured, residual + J + H + gradient at one iterate: 784 -> 4096 x 7 -> 10 181 -> 6.0 ms with the
-// Hessian's products, 4.1 ms with the reverse sweep's too and 3.84 ms with the integer helpers below (error of
-// H against 64-bit sums 5.7e-15 -> 4.1e-15), 784 -> 128 x 2 -> 10 912 -> 313 -> 182 -> 125 us (8e-16 both).
+// Measured, residual + J + H + gradient at one iterate: 784 -> 4096 x 7 -> 10 181 ms with FP64 products, 4.00 ms
+// so (error of H against 64-bit sums 5.7e-15, 3.5e-15), 784 -> 128 x 2 -> 10 912 and 113 us (8e-16, 7e-16).
 #include <cudaTypedefs.h>
 
 #include <algorithm>
@@ -46,7 +44,7 @@ using namespace umma;
 
 namespace {
 
-constexpr int kModuli[kRnsMax] = {256, 255, 253, 251, 247, 241, 239, 233,
+constexpr int kModuli[kRns] = {256, 255, 253, 251, 247, 241, 239, 233,
                                   229, 227, 223, 217, 211, 199, 197, 193};
 
 // ------------------------------------------------------------------ residue arithmetic
@@ -300,7 +298,7 @@ __global__ void __launch_bounds__(256) k_rns_pack(const __grid_constant__ RnsSet
 #pragma unroll
     for (int j = 0; j < 4; ++j) l[j] = rns_limbs(to_int(w[k + j], sc - (de ? de[k + j] : 0)));
 #pragma unroll 4
-    for (int i = 0; i < s.n; ++i) {
+    for (int i = 0; i < kRns; ++i) {
       float v[4];
 #pragma unroll
       for (int j = 0; j < 4; ++j) v[j] = rns_mod(rns_res(s, i, l[j]) * s.q[i], s.p[i], s.pinv[i]);
@@ -315,7 +313,7 @@ __global__ void __launch_bounds__(256) k_rns_pack(const __grid_constant__ RnsSet
 // the row's largest |sigma' z| and |sqrt|c| z| give its scales, and the residues of both are written:
 // the operand of the next layer's product and the two operands of the symmetric product, which
 // takes sqrt|c| z on both sides (sign(c) on one) so that one scale per row fits every column.
-// Bound: 90 bytes written per element (15 residues x 3 operands) and about 450 instructions; four of them
+// Bound: 96 bytes written per element (16 residues x 3 operands) and about 450 instructions; four of them
 // on the FP64 pipe.
 // DE: the next layer's weights have column exponents.
 template <bool CRT, bool DE>
@@ -334,8 +332,8 @@ __global__ void __launch_bounds__(256) k_rns_rows(const __grid_constant__ RnsSet
       Crt t[4];
       const unsigned char* c = a.C + (size_t)r * a.ldc + k;
       const size_t plane = (size_t)a.n * a.ldc;
-#pragma unroll 5
-      for (int i = 0; i < set.n; ++i) {
+#pragma unroll 4
+      for (int i = 0; i < kRns; ++i) {
         const unsigned y = __ldg(reinterpret_cast<const unsigned*>(c + i * plane));
         t[0].add(set, i, y & 0xFFu);
         t[1].add(set, i, (y >> 8) & 0xFFu);
@@ -383,8 +381,8 @@ __global__ void __launch_bounds__(256) k_rns_rows(const __grid_constant__ RnsSet
 #pragma unroll
       for (int j = 0; j < 4; ++j) l[j] = rns_limbs(to_int(__ldg(a.s1 + k + j) * z[j], sca + d[j]));
       __nv_bfloat16* dst = (__nv_bfloat16*)a.At + o;
-#pragma unroll 5
-      for (int i = 0; i < set.n; ++i)
+#pragma unroll 4
+      for (int i = 0; i < kRns; ++i)
         *reinterpret_cast<uint2*>(dst + i * plane) =
             make_uint2(bf2(rns_res(set, i, l[0]), rns_res(set, i, l[1])),
                        bf2(rns_res(set, i, l[2]), rns_res(set, i, l[3])));
@@ -403,8 +401,8 @@ __global__ void __launch_bounds__(256) k_rns_rows(const __grid_constant__ RnsSet
         neg1 = (s4[2] >> 16) | s4[3];
       }
       __nv_bfloat16 *da = (__nv_bfloat16*)a.Sa + o, *db = (__nv_bfloat16*)a.Sb + o;
-#pragma unroll 5
-      for (int i = 0; i < set.n; ++i) {
+#pragma unroll 4
+      for (int i = 0; i < kRns; ++i) {
         float v[4], w[4];
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
@@ -424,7 +422,7 @@ __global__ void __launch_bounds__(256) k_rns_rows(const __grid_constant__ RnsSet
 // for the output layer, the seeds), then sigma' Abar of the layer below as residues, one scale per
 // seed (the row scales of that layer's weights are multiplied in, since its product sums over rows).
 // First layer: J and the gradient instead.  Bound: latency, so a thread has one column up to 4096, and
-// its loads, twenty at a time, are in flight together.
+// its loads, 32 at a time, are in flight together.
 // DE: the weights just multiplied have column exponents.
 constexpr int kRevCl = 8;
 template <bool DE>
@@ -446,26 +444,23 @@ __global__ void __launch_bounds__(512) k_rns_rev_rows(const __grid_constant__ Rn
       Crt t;
       const unsigned char* c = a.C + (size_t)s * a.K + k;
       const size_t plane = (size_t)a.seeds * a.K;
-      for (int i0 = 0; i0 < set.n; i0 += 5) {
-        unsigned y[5] = {0, 0, 0, 0, 0};
+      for (int i0 = 0; i0 < kRns; i0 += 8) {
+        unsigned y[8] = {0, 0, 0, 0, 0, 0, 0, 0};
         for (int c0 = 0; c0 < a.chunks; c0 += 4) {
-          unsigned q[5][4];
+          unsigned q[8][4];
 #pragma unroll
-          for (int u = 0; u < 5; ++u)
+          for (int u = 0; u < 8; ++u)
 #pragma unroll
             for (int w = 0; w < 4; ++w)
-              q[u][w] = i0 + u < set.n && c0 + w < a.chunks
-                            ? __ldg(c + (size_t)((c0 + w) * set.n + i0 + u) * plane) : 0u;
+              q[u][w] = c0 + w < a.chunks ? __ldg(c + (size_t)((c0 + w) * kRns + i0 + u) * plane) : 0u;
 #pragma unroll
-          for (int u = 0; u < 5; ++u) y[u] += q[u][0] + q[u][1] + q[u][2] + q[u][3];
+          for (int u = 0; u < 8; ++u) y[u] += q[u][0] + q[u][1] + q[u][2] + q[u][3];
         }
 #pragma unroll
-        for (int u = 0; u < 5; ++u) {
-          if (i0 + u < set.n) {
-            float r = rns_mod((float)y[u], set.p[i0 + u], set.pinv[i0 + u]);
-            r += r < 0.f ? set.p[i0 + u] : 0.f;
-            t.add(set, i0 + u, __float_as_uint(r + 8388608.f) & 0x1FFu);
-          }
+        for (int u = 0; u < 8; ++u) {
+          float r = rns_mod((float)y[u], set.p[i0 + u], set.pinv[i0 + u]);
+          r += r < 0.f ? set.p[i0 + u] : 0.f;
+          t.add(set, i0 + u, __float_as_uint(r + 8388608.f) & 0x1FFu);
         }
       }
       double v = t.value() * (set.scale * a.sb[s]);
@@ -511,8 +506,8 @@ __global__ void __launch_bounds__(512) k_rns_rev_rows(const __grid_constant__ Rn
     const Limbs l = rns_limbs(to_int(k == k0 ? keep : zrow[k], sc));
     __nv_bfloat16* dst = (__nv_bfloat16*)a.Zr + (size_t)s * a.K + k;
     const size_t plane = (size_t)a.seeds * a.K;
-#pragma unroll 5
-    for (int i = 0; i < set.n; ++i)
+#pragma unroll 4
+    for (int i = 0; i < kRns; ++i)
       dst[i * plane] = __ushort_as_bfloat16((unsigned short)(__float_as_uint(rns_res(set, i, l)) >> 16));
   }
 }
@@ -561,11 +556,11 @@ __global__ void __launch_bounds__(256) k_rns_h(const __grid_constant__ RnsSet s,
   double v[4] = {0.0, 0.0, 0.0, 0.0};
   if (j < n && i < n) {
     for (int l = 0; l < layers; ++l) {
-      const unsigned char* u = U + ((size_t)l * kRnsMax * n + j) * ldu + i;
+      const unsigned char* u = U + ((size_t)l * kRns * n + j) * ldu + i;
       const size_t plane = (size_t)n * ldu;
       Crt r[4];
-#pragma unroll 5
-      for (int q = 0; q < s.n; ++q) {
+#pragma unroll 4
+      for (int q = 0; q < kRns; ++q) {
         const unsigned b = __ldg(reinterpret_cast<const unsigned*>(u + q * plane));
         r[0].add(s, q, b & 0xFFu);
         r[1].add(s, q, (b >> 8) & 0xFFu);
@@ -607,18 +602,18 @@ __global__ void __launch_bounds__(256) k_rns_h(const __grid_constant__ RnsSet s,
 // the same residue array read the other way round: its stages are two boxes of 64 rows x 64 columns,
 // which the MMA takes as an MN-major operand.  Each item is one 128-column strip of one modulus and
 // one chunk of up to 1024 rows, whose residues go to a plane of their own (the reader adds the
-// chunks).  Bound: HBM, 30 bytes per weight; up to 12 stages of 18 KB keep 200 KB per SM in flight.
+// chunks).  Bound: HBM, 32 bytes per weight; up to 12 stages of 18 KB keep 200 KB per SM in flight.
 constexpr int kGBM = 128, kGBK = 64;
 constexpr int kGThreads = 320;                 // producer, MMA, eight epilogue warps
 constexpr int kGChunk = 1024 / kGBK;           // K blocks that add up exactly
 
 struct RnsGemm {
   int chunks;            // REV: chunks of 1024 rows
-  int M, N, nkb, lower, ntm, ntn, tiles, n_mod, a_rows, b_rows;
+  int M, N, nkb, lower, ntm, ntn, tiles, a_rows, b_rows;
   unsigned char* C;
   int ldc;
   int* err;
-  float p[kRnsMax], pinv[kRnsMax];
+  float p[kRns], pinv[kRns];
 };
 
 template <int BN, bool REV>
@@ -657,7 +652,7 @@ __global__ void __launch_bounds__(kGThreads, 1)
   volatile int* consumed_sh = (volatile int*)(tmem_slot + 2);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int per_mod = g.tiles, total = g.tiles * g.n_mod;
+  const int per_mod = g.tiles, total = g.tiles * kRns;
   // REV: tn is the chunk of rows
   auto decode = [&](int t, int& mod, int& tm, int& tn) {
     mod = t / per_mod;
@@ -822,7 +817,7 @@ __global__ void __launch_bounds__(kGThreads, 1)
       }
       if (stop) break;
       const int n0 = (REV ? 0 : tn * BN) + half * NH;
-      const size_t plane = REV ? (size_t)(tn * g.n_mod + mod) * BN : (size_t)mod * g.N;
+      const size_t plane = REV ? (size_t)(tn * kRns + mod) * BN : (size_t)mod * g.N;
       unsigned char* dst = g.C + (plane + n0) * g.ldc + tm * kGBM + q * 32 + lane;
 #pragma unroll
       for (int j = 0; j < NH; ++j) {
@@ -894,23 +889,25 @@ cudaError_t launch_gemm(const RnsPlan& p, const RnsGemm& g, int grid, cudaStream
 }  // namespace
 
 RnsSet rns_set(int K) {
-  // 15 moduli leave 52 bits at K = 4096; products of fewer terms, whose FP64 sums round less often,
-  // take a 16th (57 bits at K = 1024): with even rows (k_rns_spread) the error stays near that of an FP64
-  // sum, and the added product costs 7 % where launches, not products, set the time.
+  // 16 moduli leave 57 bits at K = 1024, 56 at 4096 and 54 at 65664.  Error of J, the gradient and H against
+  // 128-bit sums, FP64 products / 15 moduli (four bits less) / 16: 30 -> 1100 x 2 -> 3 4.5e-16 1.2e-15 3.1e-16,
+  // 4.1e-16 1.3e-15 2.7e-16, 1.2e-15 1.3e-15 4.0e-16; 16 -> 4096 x 2 -> 3 5.9e-16 1.9e-15 3.0e-16, 5.3e-16
+  // 1.6e-15 2.5e-16, 1.8e-15 2.0e-15 3.6e-16.  So 15, with 784 -> 4096 x 7 -> 10 in 3.86 ms instead of 4.00, would
+  // be less exact than FP64 products.
   RnsSet s;
-  s.n = K <= 1024 ? 16 : 15;
-  double bits = 0.0, P = 1.0;
-  for (int i = 0; i < s.n; ++i) {
+  double bits = 0.0;
+  unsigned __int128 P = 1;   // below 2^126; a product in FP64 would round fifteen times, the same way for all
+  for (int i = 0; i < kRns; ++i) {
     bits += std::log2((double)kModuli[i]);
-    P *= kModuli[i];
+    P *= (unsigned)kModuli[i];
   }
-  s.scale = std::ldexp(P, -64);
+  s.scale = std::ldexp((double)P, -64);
   s.bits = std::min(60, (int)std::floor((bits - 1.0 - std::log2((double)K)) / 2.0 - 1e-9));
   auto sym = [](long long v, int p) {
     v %= p;
     return (float)(v > p / 2 ? v - p : v);
   };
-  for (int i = 0; i < s.n; ++i) {
+  for (int i = 0; i < kRns; ++i) {
     const int p = kModuli[i];
     s.p[i] = (float)p;
     s.pinv[i] = 1.0f / (float)p;
@@ -919,7 +916,7 @@ RnsSet rns_set(int K) {
     s.r32[i] = sym(r32, p);
     s.r48[i] = sym(r48, p);
     long long m = 1;
-    for (int j = 0; j < s.n; ++j)
+    for (int j = 0; j < kRns; ++j)
       if (j != i) m = m * (kModuli[j] % p) % p;
     long long inv = 1;
     while (m * inv % p != 1) ++inv;   // the moduli are pairwise coprime
@@ -933,7 +930,7 @@ RnsSet rns_set(int K) {
 }
 
 int rns_plan(RnsPlan& p, const void* A, int a_rows, const void* B, int b_rows, int M, int N, int K,
-             int n_mod, bool lower) {
+             bool lower) {
   p = RnsPlan();
   if (K % kGBK || K <= 0 || M <= 0 || N <= 0 || N > b_rows) return NNC_ERR_ARG;
   p.M = M;
@@ -956,14 +953,14 @@ int rns_plan(RnsPlan& p, const void* A, int a_rows, const void* B, int b_rows, i
       }
     }
   }
-  if (!rns_map(&p.ta, A, (long long)n_mod * a_rows, K, kGBM) ||
-      !rns_map(&p.tb, B, (long long)n_mod * b_rows, K, p.bn))
+  if (!rns_map(&p.ta, A, (long long)kRns * a_rows, K, kGBM) ||
+      !rns_map(&p.tb, B, (long long)kRns * b_rows, K, p.bn))
     return NNC_ERR_CUDA;
   p.ready = true;
   return NNC_OK;
 }
 
-int rns_plan_rev(RnsPlan& p, const void* W, int mp, int kp, const void* Z, int seeds, int n_mod) {
+int rns_plan_rev(RnsPlan& p, const void* W, int mp, int kp, const void* Z, int seeds) {
   p = RnsPlan();
   if (mp % 128 || kp % 128 || seeds < 1 || seeds > 48) return NNC_ERR_ARG;
   p.M = kp;
@@ -973,8 +970,8 @@ int rns_plan_rev(RnsPlan& p, const void* W, int mp, int kp, const void* Z, int s
   p.a_rows = mp;
   p.b_rows = p.bn;
   p.rev = 1;
-  if (!rns_map(&p.ta, W, (long long)n_mod * mp, kp, kGBK) ||
-      !rns_map(&p.tb, Z, (long long)n_mod * p.bn, mp, p.bn))
+  if (!rns_map(&p.ta, W, (long long)kRns * mp, kp, kGBK) ||
+      !rns_map(&p.tb, Z, (long long)kRns * p.bn, mp, p.bn))
     return NNC_ERR_CUDA;
   p.ready = true;
   return NNC_OK;
@@ -992,17 +989,16 @@ cudaError_t rns_gemm(const RnsPlan& p, const RnsSet& s, unsigned char* C, int ld
   g.nkb = p.nkb;
   g.lower = p.lower;
   g.tiles = p.lower ? g.ntm * (g.ntm + 1) / 2 : g.ntm * g.ntn;
-  g.n_mod = s.n;
   g.a_rows = p.a_rows;
   g.b_rows = p.b_rows;
   g.C = C;
   g.ldc = ldc;
   g.err = err;
-  for (int i = 0; i < s.n; ++i) {
+  for (int i = 0; i < kRns; ++i) {
     g.p[i] = s.p[i];
     g.pinv[i] = s.pinv[i];
   }
-  const int grid = std::min(sm_count, g.tiles * g.n_mod);
+  const int grid = std::min(sm_count, g.tiles * kRns);
   switch (p.rev ? -p.bn : p.bn) {
     case -16: return launch_gemm<16, true>(p, g, grid, st);
     case -32: return launch_gemm<32, true>(p, g, grid, st);

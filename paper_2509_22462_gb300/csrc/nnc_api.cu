@@ -521,7 +521,7 @@ int run_hessian_rns(nnc_net* net, const double* lam, double* H, cudaStream_t st)
     if (Ly.zy_off >= 0) {
       PROF(PK_SYRK);
       CK(rns_gemm(Ly.plan_rs, net->rset,
-                  net->Ru + (size_t)Ly.h_plane * kRnsMax * n * net->u_ld, net->u_ld, net->dev_err,
+                  net->Ru + (size_t)Ly.h_plane * kRns * n * net->u_ld, net->u_ld, net->dev_err,
                   net->sm_count, st));
     }
   }
@@ -785,7 +785,7 @@ void nnc_free(nnc_net* net) {
   delete net;
 }
 
-// Buffers, residues and plans of the FP64 form's residue products, in one allocation of 30 to 32 bytes per
+// Buffers, residues and plans of the FP64 form's residue products, in one allocation of 32 bytes per
 // weight beside the 8 of the FP64 weights.  Where that is more than an eighth of the free memory (it is the
 // caller's, for more nets and other work), and where the residues of the weights would keep too few bits
 // (rns_even_out), the CUDA-core products stay in use (net->rns false).
@@ -800,7 +800,7 @@ static int load_rns(nnc_net* net) {
   net->zs_ld = k_max + kPad;
   net->u_ld = net->n_in_pad;
   net->rset = rns_set(net->zs_ld);
-  const size_t rs = net->rset.n, row_elems = (size_t)n * net->zs_ld;
+  const size_t rs = kRns, row_elems = (size_t)n * net->zs_ld;
   // offsets in the allocation; what has to start as zero comes first
   size_t size = 0;
   auto take = [&](size_t bytes) {
@@ -836,7 +836,7 @@ static int load_rns(nnc_net* net) {
     o_ra = take(2 * rs * row_elems);
     o_rb = take(2 * rs * row_elems);
     o_rcv = take(rs * row_elems);
-    o_ru = take((size_t)planes * kRnsMax * n * net->u_ld);
+    o_ru = take((size_t)planes * kRns * n * net->u_ld);
   }
   size_t free_b = 0, total_b = 0;
   CK(cudaMemGetInfo(&free_b, &total_b));
@@ -895,12 +895,12 @@ static int load_rns(nnc_net* net) {
     Ly.Wr = base + o_wr[l];
     Ly.wr_scale = (double*)(base + o_ws[l]);
     CK(rns_pack_weights(net->rset, Ly.W64, Ly.mp, Ly.kp, Ly.wr_de, Ly.Wr, Ly.wr_scale, net->stream));
-    int r = rns_plan_rev(Ly.plan_rr, Ly.Wr, Ly.mp, Ly.kp, net->Zr, net->S_max, net->rset.n);
+    int r = rns_plan_rev(Ly.plan_rr, Ly.Wr, Ly.mp, Ly.kp, net->Zr, net->S_max);
     if (r == NNC_OK && hess && l > 0)
-      r = rns_plan(Ly.plan_rt, Ly.Wr, Ly.mp, net->Rt, n, Ly.mp, n, Ly.kp, net->rset.n, false);
+      r = rns_plan(Ly.plan_rt, Ly.Wr, Ly.mp, net->Rt, n, Ly.mp, n, Ly.kp, false);
     if (r == NNC_OK && Ly.zy_off >= 0)
       r = rns_plan(Ly.plan_rs, net->Ra, n, net->Rb, n, n, n,
-                   Ly.mp + (l == L - 1 && net->softmax ? kPad : 0), net->rset.n, true);
+                   Ly.mp + (l == L - 1 && net->softmax ? kPad : 0), true);
     if (r != NNC_OK) return fail(r, "plan of the residue products failed");
   }
   return NNC_OK;
