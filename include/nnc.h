@@ -54,7 +54,7 @@ typedef enum {
  *                Jacobian, the gradient and the Hessian run on the tensor cores by residues: operands
  *                are integers of 54 (65536-wide layers) to 58 bits (narrow ones) below the largest entry
  *                of a row, after powers of two have evened out the weights' columns, and the integer
- *                sums are exact.  Column by column the error is no larger than that of FP64 sums,
+ *                sums are exact.  Column by column the error is that of FP64 sums,
  *                whatever the units of inputs, hidden units and outputs.  Weights that powers of
  *                two do not even out, such as sparse ones, and nets whose residues (32 bytes per
  *                weight) take more than an eighth of the device memory that is free at load have
