@@ -242,7 +242,9 @@ __global__ void __launch_bounds__(256) k_rns_colexp(int m, int k, const RnsEven 
 // that fewer than 44 of its bits are kept.  Sums in which such entries are outnumbered lose nothing to
 // speak of (a few percent of normally distributed entries are small); a row or column that consists of
 // them would.  So of 64 entries or more in a row or a column at most a quarter may be small, of 16 or
-// more half, and of the whole matrix a quarter.  Rows and columns of zeros do not count.
+// more half, and of the whole matrix a quarter.  Rows and columns of zeros do not count.  No row's largest
+// entry may lie more than 2^(bits - 44) above the geometric mean of its nonzero ones either, however short the
+// row: its scale is multiplied into the seeds, and would push those of the other rows down.
 __device__ __forceinline__ bool rns_uneven(int small, int n) {
   return n >= 64 ? 4 * (long long)small > n : n >= 16 && 2 * small > n;
 }
@@ -256,10 +258,14 @@ __global__ void __launch_bounds__(256) k_rns_spread(const double* __restrict__ W
     if (expo(w[j]) > 0) ex = max(ex, expo(w[j]) - de[j]);
   ex = block_max(ex, sh);
   if (ex <= 0) return;   // a row of zeros
-  int small = 0, n = 0;
+  int small = 0, n = 0, nz = 0, below = 0;   // below: sum of log2(largest / entry) over the nonzero ones
   for (int j = threadIdx.x; j < k; j += 256) {
     if (e.cnt[j] == 0) continue;
     ++n;
+    if (expo(w[j]) > 0) {
+      ++nz;
+      below += ex - (expo(w[j]) - de[j]);
+    }
     if (expo(w[j]) == 0 || expo(w[j]) - de[j] < ex - (bits - 44)) {
       ++small;
       atomicAdd(e.small + j, 1);
@@ -267,8 +273,10 @@ __global__ void __launch_bounds__(256) k_rns_spread(const double* __restrict__ W
   }
   n = block_sum(n, sh);
   small = block_sum(small, sh);
+  nz = block_sum(nz, sh);
+  below = block_sum(below, sh);   // at most 65536 times 1200
   if (threadIdx.x == 0) {
-    if (rns_uneven(small, n)) atomicOr(flags, kRnsUneven);
+    if (rns_uneven(small, n) || below > (bits - 44) * nz) atomicOr(flags, kRnsUneven);
     atomicAdd(e.total, (unsigned long long)n);
     atomicAdd(e.total + 1, (unsigned long long)small);
     atomicAdd(e.total + 2, 1ull);

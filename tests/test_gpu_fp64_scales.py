@@ -149,3 +149,14 @@ def test_uneven_weights(lib, kind, layer):
     if kind == "outlier":
         x = x * 2.0 ** -30     # keeps the activations in range
     check(lib, MLP(mlp.spec, W, mlp.b), x, lam)
+
+
+@pytest.mark.parametrize("n", [2, 3, 6, 15])
+def test_outlier_of_few_inputs(lib, n):
+    """One weight far above the others of a short row: too few entries to count, and the row's scale would
+    push the seeds of all other rows down."""
+    mlp = make_mlp(MLPSpec([n, 160, 144, 3], ["softplus", "softplus", "identity"]), seed=n, tag="scales", bias_std=0.1)
+    W = [np.abs(w) for w in mlp.W]
+    W[0][53, n // 3] *= 2.0 ** 30
+    x, lam = uniform01(derive_key(n, "scale-x"), n) * 2.0 ** -30, 0.5 + uniform01(derive_key(n, "scale-lam"), 3)
+    check(lib, MLP(mlp.spec, W, mlp.b), x, lam)
